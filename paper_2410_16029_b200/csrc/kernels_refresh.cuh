@@ -55,6 +55,7 @@ struct CholProblem {
   int L;
   int pad;
   double tiny;  // pivot floor, written by chol_begin_kernel
+  const int* only_if = nullptr;  // chol_cta_kernel, conditional launch: factor only where this word is set
 };
 
 constexpr int kCholNB = 32;  // panel width
@@ -288,7 +289,7 @@ __device__ __noinline__ void chol_panel_row(T* p, int ldp, const T (*D)[kCholNB 
 // about 1e-2 on a unit diagonal, and about twice as fast (half the shared-memory traffic per multiply-add, twice
 // the arithmetic rate).
 template <typename T>
-__global__ void __launch_bounds__(kCholCtaThreads, 1) chol_cta_kernel(const CholProblem* probs) {
+__global__ void __launch_bounds__(kCholCtaThreads, 1) chol_cta_kernel(const CholProblem* probs, int conditional) {
   constexpr int NB = kCholNB;
   extern __shared__ __align__(16) unsigned char chol_ps_raw[];
   T* chol_ps = reinterpret_cast<T*>(chol_ps_raw);    // panel, k-major: chol_ps[k * ldp + (row - base)]
@@ -296,6 +297,7 @@ __global__ void __launch_bounds__(kCholCtaThreads, 1) chol_cta_kernel(const Chol
   __shared__ T rdiag[NB];          // reciprocals of the factor's diagonal
   __shared__ T s_tiny;
   const CholProblem p = probs[blockIdx.x];
+  if (conditional && *p.only_if == 0) return;
   T* C = reinterpret_cast<T*>(p.C);
   const int L = p.L;
   const int tid = threadIdx.x;
@@ -392,8 +394,9 @@ __global__ void __launch_bounds__(kCholCtaThreads, 1) chol_cta_kernel(const Chol
 
 // Factor n matrices, one CTA each (the list should start with the largest matrices: CTAs are handed out in order).
 template <typename T>
-inline cudaError_t chol_cta_launch(const CholProblem* d_probs, int n, int Lmax, cudaStream_t stream, int64_t* launches) {
-  chol_cta_kernel<T><<<n, kCholCtaThreads, chol_cta_smem_bytes<T>(Lmax), stream>>>(d_probs);
+inline cudaError_t chol_cta_launch(const CholProblem* d_probs, int n, int Lmax, cudaStream_t stream, int64_t* launches,
+                                   bool conditional = false) {
+  chol_cta_kernel<T><<<n, kCholCtaThreads, chol_cta_smem_bytes<T>(Lmax), stream>>>(d_probs, conditional ? 1 : 0);
   *launches += 1;
   return cudaGetLastError();
 }

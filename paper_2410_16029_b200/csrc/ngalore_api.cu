@@ -79,10 +79,10 @@ struct ngalore_state {
   std::vector<int> refresh_tc_idx, refresh_plain_idx;
   std::vector<const uint16_t*> refresh_tc_G;
   CholProblem* d_chol = nullptr;
-  // Rayleigh-Ritz rotation of the plain refresh path: X of the Jacobi kernels lives in Xa, V (fp64) in C
-  JacobiMat* d_jac = nullptr;
-  JacobiInit* d_jac_init = nullptr;
-  JacobiOut* d_jac_out = nullptr;
+  // Rayleigh-Ritz rotation of the plain refresh path, which works on one matrix at a time: the eigensolver's work
+  // space is shared by all of them
+  EigMat* d_eig = nullptr;
+  CholProblem* d_eig_chol = nullptr;
   int64_t k = 0;
   int64_t n_appended = 0;
   bool has_subspace = false;         // every matrix has a projector
@@ -294,7 +294,7 @@ ngalore_status finish_refresh(ngalore_state* st, const std::vector<int>& idx, bo
   return NGALORE_OK;
 }
 
-// Leading columns of the basis that the Rayleigh-Ritz rotation turns into Ritz vectors (see ritz_jacobi.cuh).
+// Leading columns of the basis that the Rayleigh-Ritz rotation turns into Ritz vectors (see ritz_eigen.cuh).
 inline int ritz_columns(const ngalore_state* st) {
   return st->opt.ritz_columns == 0 ? 256 : (st->opt.ritz_columns < 0 ? (1 << 20) : st->opt.ritz_columns);
 }
@@ -325,8 +325,7 @@ ngalore_status refresh_simt(ngalore_state* st, const uint16_t* const* G, const s
   // Second pass Yb -> Ya so that a clamped pivot of the first pass cannot leave P non-orthonormal.
   if ((rc = orthonormalise(st, idx, 0, false, stream))) return rc;
   // Rayleigh-Ritz rotation (Sec. 1: P holds the singular vectors): Z = G^T Q into Xa, C = Z^T Z (fp64) into C,
-  // eigenvectors V of C by Jacobi rotations (X in Xa; V, fp64, takes over the memory of C once C has been read),
-  // V with its columns in falling order of the eigenvalue into Xb (as fp32), Yb = Ya V, and a last
+  // eigenvectors V of C with its columns in falling order of the eigenvalue into Xb (as fp32), Yb = Ya V, and a last
   // orthonormalisation Yb -> Ya (its triangular factor is the identity to about 1e-6, so the columns keep their
   // directions).
   if ((rc = apply_gradient(st, idx, G, 1, BUF_YA, BUF_XA, stream))) return rc;
@@ -340,12 +339,8 @@ ngalore_status refresh_simt(ngalore_state* st, const uint16_t* const* G, const s
     g.epilogue = EPI_STORE;
     NG_CUDA(launch_simt_gemm<double>(g, stream));
     st->launches += 1;
-    jacobi_init_kernel<<<1, 256, 0, stream>>>(st->d_jac + i, st->d_jac_init + i);
-    st->launches += 1;
-    const int Lj = std::min(hm.rp, ritz_columns(st));
-    NG_CUDA(jacobi_batched_launch(st->d_jac + i, 1, stream, &st->launches));
-    jacobi_finish_kernel<<<dim3(1, kJacFinishSplit), 256, 0, stream>>>(st->d_jac + i, st->d_jac_out + i);
-    st->launches += 1;
+    NG_CUDA(eig_batched_launch(st->d_eig + i, st->d_eig_chol + i, 1, std::min(hm.rp, ritz_columns(st)), hm.rp, 1, stream,
+                               &st->launches));
     SimtGemm a{};
     a.m = hm.eM; a.n = hm.rp; a.k = hm.rp;
     a.A = hm.Ya; a.a_rs = hm.rp; a.a_cs = 1; a.a_dt = DT_F32;
@@ -681,10 +676,13 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   const size_t o_desc = take(sizeof(MatDesc) * n_matrices);
   const size_t o_chol = take(sizeof(CholProblem) * n_matrices);
   const size_t o_flags = take(sizeof(int) * 2 * n_matrices);
-  const size_t o_jac = take(sizeof(JacobiMat) * n_matrices);
-  const size_t o_jac_init = take(sizeof(JacobiInit) * n_matrices);
-  const size_t o_jac_out = take(sizeof(JacobiOut) * n_matrices);
-  const size_t o_jac_flags = take(sizeof(int) * kJacMaxSweeps * n_matrices);
+  const size_t o_eig = take(sizeof(EigMat) * n_matrices);
+  const size_t o_eig_chol = take(sizeof(CholProblem) * n_matrices);
+  const size_t o_eig_redo = take(sizeof(int) * n_matrices);
+  size_t eig_n = 1;
+  for (const HostMat& hm : st->mats) eig_n = std::max(eig_n, static_cast<size_t>(std::min(hm.rp, ritz_columns(st))));
+  const size_t eig_mat = align_up(sizeof(double) * eig_n * (eig_n + 1));
+  const size_t o_eig_work = take(3 * eig_mat + sizeof(double) * eig_tri_doubles(eig_n));
   int n_tiles = 0;
   std::vector<StreamTile> tiles;
   std::vector<int> tile0(n_matrices), ntl(n_matrices);
@@ -727,12 +725,10 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   st->d_tiles = reinterpret_cast<StreamTile*>(st->work + o_tiles);
   int* flags = reinterpret_cast<int*>(st->work + o_flags);
   st->d_flags = flags;
-  st->d_jac = reinterpret_cast<JacobiMat*>(st->work + o_jac);
-  st->d_jac_init = reinterpret_cast<JacobiInit*>(st->work + o_jac_init);
-  st->d_jac_out = reinterpret_cast<JacobiOut*>(st->work + o_jac_out);
-  std::vector<JacobiMat> jac(n_matrices);
-  std::vector<JacobiInit> jac_init(n_matrices);
-  std::vector<JacobiOut> jac_out(n_matrices);
+  st->d_eig = reinterpret_cast<EigMat*>(st->work + o_eig);
+  st->d_eig_chol = reinterpret_cast<CholProblem*>(st->work + o_eig_chol);
+  std::vector<EigMat> eig(n_matrices);
+  std::vector<CholProblem> eig_chol(n_matrices);
   st->subspace_set.assign(n_matrices, 0);
 
   st->h_desc.resize(n_matrices);
@@ -781,13 +777,15 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     hm.C = reinterpret_cast<double*>(st->work + woffs[i].C);
     if (hm.right) hm.Gt = reinterpret_cast<uint16_t*>(st->work + woffs[i].Gt);
     chol[i].C = hm.C; chol[i].L = hm.rp; chol[i].pad = 0; chol[i].tiny = 0.0;
-    // eN >= r' and a multiple of 8, so r' rows of ld <= eN floats fit in the eN x r' floats of Xa; V (r' x ld
-    // doubles) takes over C, which is allocated with that leading dimension
-    const int Lj = std::min(hm.rp, ritz_columns(st));
-    jac[i] = JacobiMat{hm.Xa, hm.C, Lj, (Lj + 3) & ~3, jacobi_blocks(Lj),
-                       reinterpret_cast<int*>(st->work + o_jac_flags) + kJacMaxSweeps * i};
-    jac_init[i] = JacobiInit{nullptr, hm.C, hm.rp};
-    jac_out[i] = JacobiOut{hm.Xb, hm.rp, nullptr, nullptr, 0, hm.rp};
+    {
+      const int Lj = std::min(hm.rp, ritz_columns(st));
+      char* wk = st->work + o_eig_work;
+      double* S = reinterpret_cast<double*>(wk + 2 * eig_mat);
+      int* redo = reinterpret_cast<int*>(st->work + o_eig_redo) + i;
+      eig[i] = EigMat{nullptr, hm.C, hm.rp, Lj, (Lj + 1) & ~1, reinterpret_cast<double*>(wk), reinterpret_cast<double*>(wk + eig_mat), S,
+                      reinterpret_cast<double*>(wk + 3 * eig_mat), redo, hm.Xb, hm.rp, nullptr, nullptr, 0, hm.rp};
+      eig_chol[i] = CholProblem{S, Lj, 0, 0.0, redo};
+    }
     if (s == 0 && cudaMemcpy(d.wsol, w_init.data(), sizeof(float) * kMaxHistory, cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(NGALORE_ERR_CUDA);
   }
@@ -795,9 +793,8 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
       cudaMemcpy(st->d_chol, chol.data(), sizeof(CholProblem) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(st->d_tiles, tiles.data(), sizeof(StreamTile) * n_tiles, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(st->d_hyper, &st->hyper, sizeof(Hyper), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(st->d_jac, jac.data(), sizeof(JacobiMat) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(st->d_jac_init, jac_init.data(), sizeof(JacobiInit) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(st->d_jac_out, jac_out.data(), sizeof(JacobiOut) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess)
+      cudaMemcpy(st->d_eig, eig.data(), sizeof(EigMat) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(st->d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess)
     return fail(NGALORE_ERR_CUDA);
   st->hyper_dirty = false;
 
@@ -805,8 +802,14 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   int max_rp = 0;
   for (const HostMat& hm : st->mats) max_rp = hm.rp > max_rp ? hm.rp : max_rp;
   if (orth_apply_smem_bytes(max_rp) > static_cast<size_t>(prop.sharedMemPerBlockOptin)) return fail(NGALORE_ERR_INVALID_ARG);
+  // (the limit of a kernel belongs to the process: it must hold for the widest state, whichever is created last)
   if (cudaFuncSetAttribute(orth_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(orth_apply_smem_bytes(max_rp))) != cudaSuccess)
+                           static_cast<int>(prop.sharedMemPerBlockOptin)) != cudaSuccess ||
+      cudaFuncSetAttribute(chol_cta_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(chol_cta_smem_bytes<double>(kEigMaxN))) != cudaSuccess ||
+      cudaFuncSetAttribute(chol_cta_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(chol_cta_smem_bytes<float>(kEigMaxN))) != cudaSuccess ||
+      eig_init(static_cast<int>(eig_n)) != cudaSuccess)
     return fail(NGALORE_ERR_CUDA);
 
   const bool allow_gram_fusion = st->opt.gemm_impl != 1 && st->opt.stream_impl != 1 && !hist16 && st->opt.gram_fusion == 1;

@@ -10,7 +10,7 @@
 // indefinite, and
 // Q = Y R^-1 is again a tensor-core GEMM with R^-1 split in two bf16 parts.  The last basis is then
 // orthonormalised exactly (Gram, Cholesky and triangular solve in fp64), rotated to the Ritz vectors of G inside
-// the subspace (Z = G^T Q, eigenvectors V of Z^T Z by the Jacobi kernels of ritz_jacobi.cuh, P = Q V on the tensor
+// the subspace (Z = G^T Q, eigenvectors V of Z^T Z by the kernels of ritz_eigen.cuh, P = Q V on the tensor
 // cores, columns in falling order of their singular value) and orthonormalised once more.
 #pragma once
 
@@ -21,7 +21,7 @@
 
 #include "gemm_tcgen05.cuh"
 #include "kernels_refresh.cuh"
-#include "ritz_jacobi.cuh"
+#include "ritz_eigen.cuh"
 
 namespace ngalore {
 
@@ -477,10 +477,11 @@ struct RefreshPlan {
   int n_syrk_tiles = 0;
   GramPrep64* d_prep64 = nullptr;
   SplitJob* d_split_z = nullptr;
-  // Rayleigh-Ritz rotation: the Jacobi kernels work in the T64 (X, fp32) and X64 (V, fp64) buffers
-  JacobiMat* d_jac = nullptr;
-  JacobiInit* d_jac_init = nullptr;
-  JacobiOut* d_jac_out = nullptr;
+  // Rayleigh-Ritz rotation: the eigensolver works in the X64, T64 and C64 buffers
+  EigMat* d_eig = nullptr;
+  CholProblem* d_eig_chol = nullptr;
+  int eig_max = 0;             // largest matrix it diagonalises
+  int sm_count = 0;
   NormJob* d_norm = nullptr;
   FillJob* d_fill = nullptr;   // the random start Z = Omega of every matrix
   ZeroJob* d_zero_d = nullptr;   // clears every matrix's D (as 16-byte words)
@@ -508,6 +509,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.encode = reinterpret_cast<EncodeTiledFn>(fn);
   const int n = static_cast<int>(mats.size());
   plan.n = n;
+  plan.sm_count = sm_count;
   plan.mats.resize(n);
   plan.last_G.assign(n, nullptr);
 
@@ -610,13 +612,14 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_sz = take(sizeof(SplitJob) * n);
   const size_t o_sy_rest = take(sizeof(SplitJob) * n);
   const size_t o_sz_rest = take(sizeof(SplitJob) * n);
-  const size_t o_jac = take(sizeof(JacobiMat) * n);
-  const size_t o_jac_init = take(sizeof(JacobiInit) * n);
-  const size_t o_jac_out = take(sizeof(JacobiOut) * n);
+  const size_t o_eig = take(sizeof(EigMat) * n);
+  const size_t o_eig_chol = take(sizeof(CholProblem) * n);
+  const size_t o_eig_redo = take(sizeof(int) * n);
   const size_t o_norm = take(sizeof(NormJob) * n);
   const size_t o_fill = take(sizeof(FillJob) * n);
   const size_t o_zero_d = take(sizeof(ZeroJob) * n);
-  const size_t o_jac_flags = take(sizeof(int) * kJacMaxSweeps * n);
+  std::vector<size_t> o_eig_tri(n);
+  for (int i = 0; i < n; ++i) o_eig_tri[i] = take(sizeof(double) * eig_tri_doubles(plan.mats[i].L));
   if (cudaMalloc(&plan.buf, off) != cudaSuccess) { plan.buf = nullptr; return NGALORE_ERR_ALLOC; }
   if (cudaMemset(plan.buf, 0, off) != cudaSuccess) return NGALORE_ERR_CUDA;
   plan.device_bytes = off;
@@ -629,9 +632,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   std::vector<SplitJob> sy(n), sz(n), sy_rest, sz_rest;
   std::vector<SyrkMat> syrk_m(n);
   std::vector<GramPrep64> prep64(n);
-  std::vector<JacobiMat> jac(n);
-  std::vector<JacobiInit> jac_init(n);
-  std::vector<JacobiOut> jac_out(n);
+  std::vector<EigMat> eig(n);
+  std::vector<CholProblem> eig_chol(n);
   std::vector<NormJob> norm(n);
   plan.h_maps.resize(static_cast<size_t>(RM_COUNT) * n);
   std::memset(plan.h_maps.data(), 0, sizeof(CUtensorMap) * plan.h_maps.size());
@@ -659,14 +661,14 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       sy_rest.push_back(sy[i]);
     if (std::find(plan.atomic_mats[RG_Z_FROM_Y].begin(), plan.atomic_mats[RG_Z_FROM_Y].end(), i) != plan.atomic_mats[RG_Z_FROM_Y].end())
       sz_rest.push_back(sz[i]);
-    // the Jacobi rotation keeps X (fp32) in the memory of T64 and V (fp64) in X64 (L is a multiple of 4 on this path)
-    // (width of the rotated part: all of the basis, or its leading ritz_columns, kept a multiple of 4)
+    // (the rotated part: all of the basis, or its leading ritz_columns, kept a multiple of 4)
     const int Lj = std::min(m.L, (ritz_columns + 3) & ~3);
-    jac[i] = JacobiMat{reinterpret_cast<float*>(m.T64), m.X64, Lj, Lj, jacobi_blocks(Lj),
-                       reinterpret_cast<int*>(plan.buf + o_jac_flags) + kJacMaxSweeps * i};
+    int* redo = reinterpret_cast<int*>(plan.buf + o_eig_redo) + i;
+    eig[i] = EigMat{m.C32, nullptr, m.L, Lj, Lj, m.X64, m.T64, m.C64, reinterpret_cast<double*>(plan.buf + o_eig_tri[i]),
+                    redo, nullptr, 0, m.Rhi, m.Rlo, m.ldl, m.L};
+    eig_chol[i] = CholProblem{m.C64, Lj, 0, 0.0, redo};
+    plan.eig_max = std::max(plan.eig_max, Lj);
     norm[i] = NormJob{m.Yf, m.D, m.M, m.L};   // the column-norm buffer of the orthonormalisations is free by then
-    jac_init[i] = JacobiInit{m.C32, nullptr, m.L};
-    jac_out[i] = JacobiOut{nullptr, 0, m.Rhi, m.Rlo, m.ldl, m.L};
     CUtensorMap* mp = &plan.h_maps[static_cast<size_t>(i) * RM_COUNT];
     const uint64_t sl = static_cast<uint64_t>(m.ldl) * 2;
     bool ok = true;
@@ -776,11 +778,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     std::stable_sort(sorted.begin(), sorted.end(), [](const CholProblem& a, const CholProblem& b) { return a.L > b.L; });
     if (cudaMemcpy(plan.d_chol_sorted, sorted.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess)
       return NGALORE_ERR_CUDA;
-    if (cudaFuncSetAttribute(chol_cta_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(chol_cta_smem_bytes<double>(plan.l_max))) != cudaSuccess ||
-        cudaFuncSetAttribute(chol_cta_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(chol_cta_smem_bytes<float>(plan.l_max))) != cudaSuccess)
-      return NGALORE_ERR_CUDA;
   }
   plan.d_tri = reinterpret_cast<TriInverse*>(plan.buf + o_tri);
   plan.d_split_y = reinterpret_cast<SplitJob*>(plan.buf + o_sy);
@@ -792,9 +789,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.d_split_z_rest = reinterpret_cast<SplitJob*>(plan.buf + o_sz_rest);
   plan.n_split_y_rest = static_cast<int>(sy_rest.size());
   plan.n_split_z_rest = static_cast<int>(sz_rest.size());
-  plan.d_jac = reinterpret_cast<JacobiMat*>(plan.buf + o_jac);
-  plan.d_jac_init = reinterpret_cast<JacobiInit*>(plan.buf + o_jac_init);
-  plan.d_jac_out = reinterpret_cast<JacobiOut*>(plan.buf + o_jac_out);
+  plan.d_eig = reinterpret_cast<EigMat*>(plan.buf + o_eig);
+  plan.d_eig_chol = reinterpret_cast<CholProblem*>(plan.buf + o_eig_chol);
+  std::stable_sort(eig_chol.begin(), eig_chol.end(), [](const CholProblem& a, const CholProblem& b) { return a.L > b.L; });
   plan.d_norm = reinterpret_cast<NormJob*>(plan.buf + o_norm);
   plan.d_fill = reinterpret_cast<FillJob*>(plan.buf + o_fill);
   {
@@ -821,9 +818,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_split_z, sz.data(), sizeof(SplitJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_y_rest, sy_rest.data(), sizeof(SplitJob) * sy_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_z_rest, sz_rest.data(), sizeof(SplitJob) * sz_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_jac, jac.data(), sizeof(JacobiMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_jac_init, jac_init.data(), sizeof(JacobiInit) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_jac_out, jac_out.data(), sizeof(JacobiOut) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(plan.d_eig, eig.data(), sizeof(EigMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(plan.d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_norm, norm.data(), sizeof(NormJob) * n, cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
 
@@ -1058,16 +1054,12 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
   // Rayleigh-Ritz: Z = G^T Q, C = Z^T Z (tensor cores: its entries are good to about 2^-17 of the diagonal, far
   // finer than the gaps that decide a Ritz vector), V = eigenvectors of C (or of its leading block, see
-  // ritz_jacobi.cuh), P = Q V.
+  // ritz_eigen.cuh), P = Q V.
   if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, d_ctrl, stream, launches))) return rc;
   if ((rc = refresh_tc_split(plan, false, stream, launches, true))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Z, d_ctrl, stream, launches))) return rc;
-  jacobi_init_kernel<<<plan.n, 256, 0, stream>>>(plan.d_jac, plan.d_jac_init);
-  *launches += 1;
-  if (jacobi_batched_launch(plan.d_jac, plan.n, stream, launches) != cudaSuccess)
+  if (eig_batched_launch(plan.d_eig, plan.d_eig_chol, plan.n, plan.eig_max, plan.l_max, plan.sm_count, stream, launches) != cudaSuccess)
     return NGALORE_ERR_CUDA;
-  jacobi_finish_kernel<<<dim3(plan.n, kJacFinishSplit), 256, 0, stream>>>(plan.d_jac, plan.d_jac_out);
-  *launches += 1;
   // Q orthonormal to about 1e-6 and V orthogonal: so is their product, once its columns are scaled back to unit norm
   if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches))) return rc;
   zero_jobs_kernel<<<dim3(1, plan.n), 256, 0, stream>>>(plan.d_zero_d);
