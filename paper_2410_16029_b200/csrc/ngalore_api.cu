@@ -807,9 +807,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
                            static_cast<int>(prop.sharedMemPerBlockOptin)) != cudaSuccess ||
       cudaFuncSetAttribute(chol_cta_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(chol_cta_smem_bytes<double>(kEigMaxN))) != cudaSuccess ||
-      cudaFuncSetAttribute(chol_cta_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(chol_cta_smem_bytes<float>(kEigMaxN))) != cudaSuccess ||
-      eig_init(static_cast<int>(eig_n)) != cudaSuccess)
+      tri_factor_init() != cudaSuccess || eig_init(static_cast<int>(eig_n)) != cudaSuccess)
     return fail(NGALORE_ERR_CUDA);
 
   const bool allow_gram_fusion = st->opt.gemm_impl != 1 && st->opt.stream_impl != 1 && !hist16 && st->opt.gram_fusion == 1;

@@ -22,6 +22,7 @@
 #include "gemm_tcgen05.cuh"
 #include "kernels_refresh.cuh"
 #include "ritz_eigen.cuh"
+#include "tri_factor.cuh"
 
 namespace ngalore {
 
@@ -90,45 +91,12 @@ __global__ void zero_jobs_kernel(const ZeroJob* jobs) {
     jb.p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-struct GramPrep {
-  const float* C32;  // L x L Gram matrix from the tensor cores
-  double* C64;       // L x L, lower triangle written: column-scaled, symmetrised Gram + shift I (as doubles, or
-                     // as L x L floats at the same address: gram_prep_kernel<float>)
-  double* D;         // L column norms d_i = sqrt(C_ii)
-  int L;
-};
-
-// Shift added to the unit-diagonal Gram matrix.  Each entry carries a relative error of at most about
-// 3 * 2^-18 from the two-part bf16 split (the dropped lo*lo product and the rounding of lo) plus the fp32
+// Shift added to the unit-diagonal Gram matrix: L / 65536 (tri_factor_kernel).  Each entry carries a relative error of at
+// most about 3 * 2^-18 from the two-part bf16 split (the dropped lo*lo product and the rounding of lo) plus the fp32
 // accumulation error, so the error matrix has norm below 2^-16 L; with this shift the Cholesky factorisation
 // cannot meet a negative pivot.  The price is that directions closer than sqrt(shift) are not pulled
-// apart, which is harmless between products.
-__host__ __device__ inline double gram_shift(int L) { return static_cast<double>(L) / 65536.0; }
-
-// One CTA per matrix: C64 = D^-1 ((C32 + C32^T) / 2) D^-1 + shift I with D = diag(sqrt(C_ii)).
-// Scaling the columns to unit norm first makes the shift act on every column alike, whatever its
-// norm, so weak directions are still orthogonalised against each other and re-normalised.
-// (blockIdx.y shares the entries of a matrix among several CTAs; each of them forms the column norms for itself)
-template <typename T>
-__global__ void __launch_bounds__(256) gram_prep_kernel(const GramPrep* probs, double shift_scale) {
-  __shared__ double Ds[880];
-  const GramPrep p = probs[blockIdx.x];
-  for (int i = threadIdx.x; i < p.L; i += 256) {
-    const double c = static_cast<double>(p.C32[static_cast<long long>(i) * p.L + i]);
-    Ds[i] = sqrt(fmax(c, 1e-60));
-    if (blockIdx.y == 0) p.D[i] = Ds[i];
-  }
-  __syncthreads();
-  const long long total = static_cast<long long>(p.L) * p.L;
-  for (long long x = blockIdx.y * 256 + threadIdx.x; x < total; x += 256ll * gridDim.y) {
-    const int i = static_cast<int>(x / p.L), j = static_cast<int>(x % p.L);
-    if (j > i) continue;
-    double v = 0.5 * (static_cast<double>(p.C32[x]) + static_cast<double>(p.C32[static_cast<long long>(j) * p.L + i]));
-    v /= Ds[i] * Ds[j];
-    if (i == j) v = 1.0 + shift_scale * gram_shift(p.L);
-    reinterpret_cast<T*>(p.C64)[x] = static_cast<T>(v);
-  }
-}
+// apart, which is harmless between products.  Scaling the columns to unit norm first makes the shift act on every
+// column alike, whatever its norm, so weak directions are still orthogonalised against each other and re-normalised.
 
 struct SyrkTile {
   int mat, ti, tj, k0;  // output tile (ti, tj <= ti) of 64 x 64, rows k0 .. k0 + kSyrkRows of Y
@@ -200,167 +168,26 @@ __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, cons
   }
 }
 
-struct GramPrep64 {
-  const double* G;  // L x L exact Gram matrix, lower triangle valid
-  double* C64;      // L x L out: column-scaled Gram + tiny shift, lower triangle
-  double* D;
-  int L;
-};
-
-// Column scaling for the exact pass; the shift only keeps a numerically rank-deficient basis factorisable.
-__global__ void __launch_bounds__(256) gram_prep64_kernel(const GramPrep64* probs) {
-  const GramPrep64 p = probs[blockIdx.x];
-  for (int i = threadIdx.x; i < p.L; i += 256) p.D[i] = sqrt(fmax(p.G[static_cast<long long>(i) * p.L + i], 1e-60));
-  __syncthreads();
-  const long long total = static_cast<long long>(p.L) * p.L;
-  for (long long x = threadIdx.x; x < total; x += 256) {
-    const int i = static_cast<int>(x / p.L), j = static_cast<int>(x % p.L);
-    if (j > i) continue;
-    p.C64[x] = (i == j) ? 1.0 + 1e-12 : p.G[x] / (p.D[i] * p.D[j]);
-  }
-}
-
-struct TriInverse {
-  const double* Lf;      // L x L lower Cholesky factor of the column-scaled Gram matrix (row-major)
-  const double* D;       // L column norms: R^-1 = D^-1 Lf^-T
-  double* X;             // L x L: X = Lf^-1 (lower triangular, upper part zero)
-  __nv_bfloat16* Rhi;    // L x ld: high part of R^-1 = Lf^-T (upper triangular)
-  __nv_bfloat16* Rlo;
+struct NewtonJob {
+  const float* C32;     // L x L, lower triangle valid
+  __nv_bfloat16 *Rhi, *Rlo;
   int L, ld;
 };
-
-// ---- blocked inverse of the lower Cholesky factor: X = Lf^-1 by recursive halving,
-//   [[A, 0], [C, B]]^-1 = [[A^-1, 0], [-B^-1 C A^-1, B^-1]],
-// leaves (<= 32 x 32) by forward substitution, inner nodes by two small batched fp64 GEMMs per level.
-
-// (the pointers of TriLeaf and TriGemm are those of elements of type T, whatever their declared type: the tables
-// exist once for matrices of doubles and once for the same buffers holding floats)
-struct TriLeaf {
-  const void* Lf;  // top-left element of the diagonal block inside the L x L factor
-  void* X;         // same position inside X
-  int ld, size;
-};
-
-// One warp per leaf; lane j solves column j of the block by forward substitution in shared memory.
-template <typename T>
-__global__ void __launch_bounds__(128) tri_leaf_kernel(const TriLeaf* leaves, int n_leaves) {
-  __shared__ T blk[4][32][33];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int id = blockIdx.x * 4 + warp;
-  if (id >= n_leaves) return;
-  const TriLeaf lf = leaves[id];
-  const T* Lf = static_cast<const T*>(lf.Lf);
-  T* X = static_cast<T*>(lf.X);
-  for (int i = 0; i < lf.size; ++i)
-    if (lane < lf.size) blk[warp][i][lane] = Lf[static_cast<long long>(i) * lf.ld + lane];
-  __syncwarp();
-  if (lane < lf.size) {
-    T x[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      T acc = (i == lane) ? T(1) : T(0);
-      if (i < lf.size && i >= lane) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (k < i && k >= lane) acc -= blk[warp][i][k] * x[k];
-        acc /= blk[warp][i][i];
-      } else {
-        acc = T(0);
-      }
-      x[i] = acc;
-      if (i < lf.size) X[static_cast<long long>(i) * lf.ld + lane] = acc;
-    }
-  }
-}
-
-struct TriGemm {
-  const void* A;  // m x k
-  const void* B;  // k x n
-  void* C;        // m x n = (negate ? -1 : 1) * A B
-  int lda, ldb, ldc, m, n, k, negate;
-};
-
-// Batched small GEMM: blockIdx.z selects the problem, (blockIdx.y, blockIdx.x) a 64 x 64 tile of it.
-template <typename T>
-__global__ void __launch_bounds__(256) tri_gemm_kernel(const TriGemm* probs) {
-  __shared__ T As[16][64 + 1];
-  __shared__ T Bs[16][64 + 1];
-  const TriGemm g = probs[blockIdx.z];
-  const T* gA = static_cast<const T*>(g.A);
-  const T* gB = static_cast<const T*>(g.B);
-  T* gC = static_cast<T*>(g.C);
-  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
-  if (i0 >= g.m || j0 >= g.n) return;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  for (int k0 = 0; k0 < g.k; k0 += 16) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int kk = t & 15, i = (t >> 4) + 16 * p;  // A: k contiguous
-      As[kk][i] = (i0 + i < g.m && k0 + kk < g.k) ? gA[static_cast<long long>(i0 + i) * g.lda + k0 + kk] : T(0);
-      const int j = t & 63, kb = (t >> 6) + 4 * p;   // B: n contiguous
-      Bs[kb][j] = (j0 + j < g.n && k0 + kb < g.k) ? gB[static_cast<long long>(k0 + kb) * g.ldb + j0 + j] : T(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) { a[x] = As[kk][ty * 4 + x]; b[x] = Bs[kk][tx * 4 + x]; }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int i = i0 + ty * 4 + x;
-    if (i >= g.m) continue;
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int j = j0 + tx * 4 + y;
-      if (j < g.n) gC[static_cast<long long>(i) * g.ldc + j] = g.negate ? -acc[x][y] : acc[x][y];
-    }
-  }
-}
-
-// R^-1 = D^-1 X^T (upper triangular) split into two bf16 parts; blockIdx.x = matrix, blockIdx.y = share of its entries.
-template <typename T>
-__global__ void __launch_bounds__(256) tri_convert_kernel(const TriInverse* probs) {
-  const TriInverse p = probs[blockIdx.x];
-  const T* X = reinterpret_cast<const T*>(p.X);
-  const long long total = static_cast<long long>(p.L) * p.L;
-  for (long long x = blockIdx.y * 256 + threadIdx.x; x < total; x += 256ll * gridDim.y) {
-    const int j = static_cast<int>(x / p.L), i = static_cast<int>(x % p.L);  // entry (j, i) of R^-1
-    const double v = (i >= j) ? static_cast<double>(X[static_cast<long long>(i) * p.L + j]) / p.D[j] : 0.0;
-    const float f = static_cast<float>(fmin(fmax(v, -1e30), 1e30));
-    const __nv_bfloat16 h = __float2bfloat16_rn(f);
-    p.Rhi[static_cast<long long>(j) * p.ld + i] = h;
-    p.Rlo[static_cast<long long>(j) * p.ld + i] = __float2bfloat16_rn(f - __bfloat162float(h));
-  }
-}
 
 // Second-order orthonormalisation of a basis that is orthonormal to first order already: with C = Q^T Q = I + E,
 // Q (I - E / 2) has Q^T Q = I + O(E^2).  C comes from the tensor cores (its error, about 1e-7 on an entry for columns
 // of unit norm, is what is left of E afterwards); S = I - E / 2 = 1.5 I - C / 2 is written in two bf16 parts where the
 // product Q = Y R^-1 expects R^-1.  blockIdx.x = matrix, blockIdx.y = share of its entries.
-__global__ void __launch_bounds__(256) newton_prep_kernel(const GramPrep* preps, const TriInverse* tris) {
-  const GramPrep g = preps[blockIdx.x];
-  const TriInverse t = tris[blockIdx.x];
-  const long long total = static_cast<long long>(g.L) * g.L;
-  for (long long x = blockIdx.y * 256 + threadIdx.x; x < total; x += 256ll * gridDim.y) {
-    const int j = static_cast<int>(x / g.L), i = static_cast<int>(x % g.L);
-    const float c = 0.5f * (g.C32[x] + g.C32[static_cast<long long>(i) * g.L + j]);
+__global__ void __launch_bounds__(256) newton_prep_kernel(const NewtonJob* jobs) {
+  const NewtonJob g = jobs[blockIdx.x];
+  const int total = g.L * g.L;
+  for (int x = blockIdx.y * 256 + threadIdx.x; x < total; x += 256 * gridDim.y) {
+    const int j = x / g.L, i = x % g.L;
+    const float c = g.C32[j >= i ? x : i * g.L + j];
     const float f = (i == j) ? 1.5f - 0.5f * c : -0.5f * c;
     const __nv_bfloat16 h = __float2bfloat16_rn(f);
-    t.Rhi[static_cast<long long>(j) * t.ld + i] = h;
-    t.Rlo[static_cast<long long>(j) * t.ld + i] = __float2bfloat16_rn(f - __bfloat162float(h));
+    g.Rhi[j * g.ld + i] = h;
+    g.Rlo[j * g.ld + i] = __float2bfloat16_rn(f - __bfloat162float(h));
   }
 }
 
@@ -411,11 +238,10 @@ __global__ void __launch_bounds__(256) column_scale_kernel(const NormJob* jobs) 
   for (int r = r0 + threadIdx.y; r < r1; r += 8) jb.Y[static_cast<long long>(r) * jb.L + col] *= f;
 }
 
-constexpr int kTriMaxLevels = 12;
-
 // ------------------------------------------------------------------------------------------ plan
 
-enum RefreshGemm { RG_Y_FROM_Z = 0, RG_Z_FROM_Y, RG_GRAM_Y, RG_GRAM_Z, RG_APPLY_Y, RG_COUNT };
+// RG_APPLY_TRI: RG_APPLY_Y with an upper triangular right operand (its blocks of zeros are left out)
+enum RefreshGemm { RG_Y_FROM_Z = 0, RG_Z_FROM_Y, RG_GRAM_Y, RG_GRAM_Z, RG_APPLY_Y, RG_APPLY_TRI, RG_COUNT };
 enum RefreshMap { RM_G_A = 0, RM_G_MN, RM_Z_B, RM_Z_B_LO, RM_Y_B, RM_Y_B_LO, RM_Y_A, RM_Y_A_LO,
                   RM_RINV, RM_RINV_LO, RM_COUNT };
 
@@ -443,7 +269,6 @@ struct RefreshPlan {
   std::vector<CUtensorMap> h_maps;  // RM_COUNT per matrix
   std::vector<const void*> last_G;
   char* buf = nullptr;
-  char* tri_tables[2] = {nullptr, nullptr};
   CUtensorMap* d_maps = nullptr;
   TcProblem* d_probs[RG_COUNT] = {};
   TcTile* d_tiles[RG_COUNT] = {};
@@ -454,18 +279,10 @@ struct RefreshPlan {
   ZeroJob* d_zero[RG_COUNT + 1] = {};
   int n_zero[RG_COUNT + 1] = {};
   char* zero_tables = nullptr;
-  GramPrep* d_prep = nullptr;
-  CholProblem* d_chol = nullptr;
-  CholProblem* d_chol_sorted = nullptr;  // the same problems, widest first (for the one-CTA-per-matrix kernel)
+  NewtonJob* d_newton = nullptr;
+  FactorMat* d_factor32 = nullptr;   // R^-1 from C32 (tri_factor.cuh), widest first
+  FactorMat* d_factor64 = nullptr;   // R^-1 from the exact Gram matrix in X64
   int l_max = 0;  // largest basis width L of the set
-  TriInverse* d_tri = nullptr;
-  TriLeaf* d_leaves[2] = {nullptr, nullptr};   // [0]: the buffers hold doubles, [1]: floats
-  int n_leaves = 0;
-  TriGemm* d_tg1[2][kTriMaxLevels] = {};
-  TriGemm* d_tg2[2][kTriMaxLevels] = {};
-  int n_tg[kTriMaxLevels] = {};
-  int tg_max[kTriMaxLevels] = {};
-  int tri_levels = 0;
   SplitJob* d_split_y = nullptr;
   // the matrices whose product with G splits K (their result arrives as fp32 and is split afterwards; all others
   // leave the product as bf16 parts already)
@@ -475,7 +292,6 @@ struct RefreshPlan {
   SyrkMat* d_syrk_mats = nullptr;
   SyrkTile* d_syrk_tiles = nullptr;
   int n_syrk_tiles = 0;
-  GramPrep64* d_prep64 = nullptr;
   SplitJob* d_split_z = nullptr;
   // Rayleigh-Ritz rotation: the eigensolver works in the X64, T64 and C64 buffers
   EigMat* d_eig = nullptr;
@@ -490,12 +306,9 @@ struct RefreshPlan {
 
 inline void refresh_plan_destroy(RefreshPlan& plan) {
   if (plan.buf) cudaFree(plan.buf);
-  for (int set = 0; set < 2; ++set)
-    if (plan.tri_tables[set]) cudaFree(plan.tri_tables[set]);
   if (plan.zero_tables) cudaFree(plan.zero_tables);
   plan.zero_tables = nullptr;
   plan.buf = nullptr;
-  plan.tri_tables[0] = plan.tri_tables[1] = nullptr;
   plan.ready = false;
 }
 
@@ -524,11 +337,13 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     const int kb_per = (kb_total + splits - 1) / splits;
     splits = (kb_total + kb_per - 1) / kb_per;
     if (splits > 1) plan.atomic_mats[g].push_back(i);
+    const bool symmetric = g == RG_GRAM_Y || g == RG_GRAM_Z;   // the lower triangle is enough
     for (int n0 = 0; n0 < out_cols; n0 += kRefBN)
       for (int sp = 0; sp < splits; ++sp)
-        for (int m0 = 0; m0 < out_rows; m0 += kTcBM) {
+        for (int m0 = symmetric ? n0 / kTcBM * kTcBM : 0; m0 < out_rows; m0 += kTcBM) {
           const int kb0 = sp * kb_per;
-          const int kbn = std::min(kb_per, kb_total - kb0);
+          int kbn = std::min(kb_per, kb_total - kb0);
+          if (g == RG_APPLY_TRI) kbn = std::min(kbn, (n0 + kRefBN) / kTcBK);
           tiles[g].push_back(TcTile{i, m0, n0, kb0 * kTcBK, kbn, splits > 1 ? 1 : 0, out_rows, out_cols});
         }
   };
@@ -549,7 +364,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     offs[i].C32 = take(sizeof(float) * m.L * m.L);
     offs[i].C64 = take(sizeof(double) * m.L * m.L);
     offs[i].X64 = take(sizeof(double) * m.L * m.L);
-    offs[i].T64 = take(sizeof(double) * m.L * m.L);
+    offs[i].T64 = take(sizeof(double) * std::max(static_cast<size_t>(m.L) * m.L, tf_spill_doubles(m.L)));
     offs[i].D = take(sizeof(double) * m.L);
     offs[i].Rhi = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
     offs[i].Rlo = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
@@ -568,7 +383,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         case RG_Z_FROM_Y: rows = m.N; cols = m.L; K = m.M; break;
         case RG_GRAM_Y: rows = m.L; cols = m.L; K = m.M; break;
         case RG_GRAM_Z: rows = m.L; cols = m.L; K = m.N; break;
-        default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y
+        default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y, RG_APPLY_TRI
       }
       total_kb += static_cast<long long>((rows + kTcBM - 1) / kTcBM) * ((cols + kRefBN - 1) / kRefBN) *
                   ((K + kTcBK - 1) / kTcBK);
@@ -583,7 +398,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         case RG_Z_FROM_Y: rows = m.N; cols = m.L; K = m.M; break;
         case RG_GRAM_Y: rows = m.L; cols = m.L; K = m.M; break;
         case RG_GRAM_Z: rows = m.L; cols = m.L; K = m.N; break;
-        default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y
+        default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y, RG_APPLY_TRI
       }
       add_tiles(g, i, rows, cols, K, target);
     }
@@ -593,10 +408,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     plan.n_tiles[g] = static_cast<int>(tiles[g].size());
     plan.grid[g] = std::min(plan.n_tiles[g], sm_count);
   }
-  const size_t o_prep = take(sizeof(GramPrep) * n);
-  const size_t o_chol = take(sizeof(CholProblem) * n);
-  const size_t o_chol_sorted = take(sizeof(CholProblem) * n);
-  const size_t o_tri = take(sizeof(TriInverse) * n);
+  const size_t o_newton = take(sizeof(NewtonJob) * n);
+  const size_t o_factor32 = take(sizeof(FactorMat) * n);
+  const size_t o_factor64 = take(sizeof(FactorMat) * n);
   std::vector<SyrkTile> syrk_tiles;
   for (int i = 0; i < n; ++i) {
     const int nt = (plan.mats[i].L + 63) / 64;
@@ -607,7 +421,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.n_syrk_tiles = static_cast<int>(syrk_tiles.size());
   const size_t o_syrk_m = take(sizeof(SyrkMat) * n);
   const size_t o_syrk_t = take(sizeof(SyrkTile) * syrk_tiles.size());
-  const size_t o_prep64 = take(sizeof(GramPrep64) * n);
   const size_t o_sy = take(sizeof(SplitJob) * n);
   const size_t o_sz = take(sizeof(SplitJob) * n);
   const size_t o_sy_rest = take(sizeof(SplitJob) * n);
@@ -624,14 +437,12 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   if (cudaMemset(plan.buf, 0, off) != cudaSuccess) return NGALORE_ERR_CUDA;
   plan.device_bytes = off;
 
-  std::vector<GramPrep> prep(n);
-  std::vector<CholProblem> chol(n);
+  std::vector<NewtonJob> newton(n);
+  std::vector<FactorMat> factor32(n), factor64(n);
   plan.l_max = 0;
   for (const RefreshMat& m : plan.mats) plan.l_max = m.L > plan.l_max ? m.L : plan.l_max;
-  std::vector<TriInverse> tri(n);
   std::vector<SplitJob> sy(n), sz(n), sy_rest, sz_rest;
   std::vector<SyrkMat> syrk_m(n);
-  std::vector<GramPrep64> prep64(n);
   std::vector<EigMat> eig(n);
   std::vector<CholProblem> eig_chol(n);
   std::vector<NormJob> norm(n);
@@ -650,11 +461,10 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     m.D = reinterpret_cast<double*>(plan.buf + offs[i].D);
     m.Rhi = reinterpret_cast<__nv_bfloat16*>(plan.buf + offs[i].Rhi);
     m.Rlo = reinterpret_cast<__nv_bfloat16*>(plan.buf + offs[i].Rlo);
-    prep[i] = GramPrep{m.C32, m.C64, m.D, m.L};
-    chol[i] = CholProblem{m.C64, m.L, 0, 0.0};
-    tri[i] = TriInverse{m.C64, m.D, m.X64, m.Rhi, m.Rlo, m.L, m.ldl};
+    newton[i] = NewtonJob{m.C32, m.Rhi, m.Rlo, m.L, m.ldl};
+    factor32[i] = FactorMat{m.C32, m.C64, nullptr, m.Rhi, m.Rlo, m.L, m.ldl};
+    factor64[i] = FactorMat{m.X64, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
     syrk_m[i] = SyrkMat{m.Yf, m.X64, m.M, m.L};
-    prep64[i] = GramPrep64{m.X64, m.C64, m.D, m.L};
     sy[i] = SplitJob{m.Yf, m.Yhi, m.Ylo, static_cast<long long>(m.M) * m.L, m.L, m.ldl};
     sz[i] = SplitJob{m.Zf, m.Zhi, m.Zlo, static_cast<long long>(m.N) * m.L, m.L, m.ldl};
     if (std::find(plan.atomic_mats[RG_Y_FROM_Z].begin(), plan.atomic_mats[RG_Y_FROM_Z].end(), i) != plan.atomic_mats[RG_Y_FROM_Z].end())
@@ -697,70 +507,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     probs[RG_GRAM_Y][i] = TcProblem{m.C32, m.L, m.L, m.L, base + RM_Y_B, base + RM_Y_B, 0};
     probs[RG_GRAM_Z][i] = TcProblem{m.C32, m.L, m.L, m.L, base + RM_Z_B, base + RM_Z_B, 0};
     probs[RG_APPLY_Y][i] = TcProblem{m.Yf, m.M, m.L, m.L, base + RM_Y_A, base + RM_RINV, 0};
-  }
-  // ---- tables of the blocked triangular inverse, for the buffers holding doubles (set 0) and floats (set 1)
-  for (int set = 0; set < 2; ++set) {
-    const size_t esz = set == 0 ? sizeof(double) : sizeof(float);
-    std::vector<TriLeaf> leaves;
-    std::vector<TriGemm> g1[kTriMaxLevels], g2[kTriMaxLevels];
-    int max_level = 0;
-    for (int i = 0; i < n; ++i) {
-      const RefreshMat& m = plan.mats[i];
-      // returns the height of the node covering [lo, hi)
-      struct Rec {
-        size_t esz;
-        void* at(double* buf, const RefreshMat& m, int row, int col) const {
-          return reinterpret_cast<char*>(buf) + esz * (static_cast<size_t>(row) * m.L + col);
-        }
-        int go(const RefreshMat& m, int lo, int hi, std::vector<TriLeaf>& leaves, std::vector<TriGemm>* g1,
-               std::vector<TriGemm>* g2) const {
-          const int len = hi - lo;
-          if (len <= 32) {
-            leaves.push_back(TriLeaf{at(m.C64, m, lo, lo), at(m.X64, m, lo, lo), m.L, len});
-            return 0;
-          }
-          const int mid = lo + ((len / 2 + 31) / 32) * 32;
-          const int ha = go(m, lo, mid, leaves, g1, g2), hb = go(m, mid, hi, leaves, g1, g2);
-          const int h = (ha > hb ? ha : hb) + 1;
-          // T = C A^-1 with C = Lf[mid:hi, lo:mid];  X[mid:hi, lo:mid] = -B^-1 T
-          void* T = at(m.T64, m, mid, lo);
-          g1[h].push_back(TriGemm{at(m.C64, m, mid, lo), at(m.X64, m, lo, lo), T, m.L, m.L, m.L, hi - mid, mid - lo,
-                                  mid - lo, 0});
-          g2[h].push_back(TriGemm{at(m.X64, m, mid, mid), T, at(m.X64, m, mid, lo), m.L, m.L, m.L, hi - mid, mid - lo,
-                                  hi - mid, 1});
-          return h;
-        }
-      };
-      const int h = Rec{esz}.go(m, 0, m.L, leaves, g1, g2);
-      if (h > max_level) max_level = h;
-    }
-    if (max_level >= kTriMaxLevels) return NGALORE_ERR_INVALID_ARG;
-    plan.tri_levels = max_level;
-    plan.n_leaves = static_cast<int>(leaves.size());
-    size_t bytes = sizeof(TriLeaf) * leaves.size();
-    for (int h = 1; h <= max_level; ++h) bytes += 2 * ((sizeof(TriGemm) * g1[h].size() + 255) / 256 * 256);
-    bytes = (bytes + 255) / 256 * 256 + 256;
-    char* tb = nullptr;
-    if (cudaMalloc(&tb, bytes) != cudaSuccess) return NGALORE_ERR_ALLOC;
-    plan.tri_tables[set] = tb;
-    plan.device_bytes += bytes;
-    size_t o = 0;
-    plan.d_leaves[set] = reinterpret_cast<TriLeaf*>(tb);
-    if (cudaMemcpy(tb, leaves.data(), sizeof(TriLeaf) * leaves.size(), cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
-    o = (sizeof(TriLeaf) * leaves.size() + 255) / 256 * 256;
-    for (int h = 1; h <= max_level; ++h) {
-      const size_t sz = sizeof(TriGemm) * g1[h].size();
-      plan.n_tg[h] = static_cast<int>(g1[h].size());
-      int mx = 1;
-      for (const TriGemm& g : g1[h]) { if (g.m > mx) mx = g.m; if (g.n > mx) mx = g.n; }
-      plan.tg_max[h] = mx;
-      plan.d_tg1[set][h] = reinterpret_cast<TriGemm*>(tb + o);
-      if (sz && cudaMemcpy(tb + o, g1[h].data(), sz, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
-      o += (sz + 255) / 256 * 256;
-      plan.d_tg2[set][h] = reinterpret_cast<TriGemm*>(tb + o);
-      if (sz && cudaMemcpy(tb + o, g2[h].data(), sz, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
-      o += (sz + 255) / 256 * 256;
-    }
+    probs[RG_APPLY_TRI][i] = probs[RG_APPLY_Y][i];
   }
   plan.d_maps = reinterpret_cast<CUtensorMap*>(plan.buf + o_maps);
   for (int g = 0; g < RG_COUNT; ++g) {
@@ -770,20 +517,15 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         cudaMemcpy(plan.d_tiles[g], tiles[g].data(), sizeof(TcTile) * tiles[g].size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return NGALORE_ERR_CUDA;
   }
-  plan.d_prep = reinterpret_cast<GramPrep*>(plan.buf + o_prep);
-  plan.d_chol = reinterpret_cast<CholProblem*>(plan.buf + o_chol);
-  plan.d_chol_sorted = reinterpret_cast<CholProblem*>(plan.buf + o_chol_sorted);
-  {
-    std::vector<CholProblem> sorted(chol);
-    std::stable_sort(sorted.begin(), sorted.end(), [](const CholProblem& a, const CholProblem& b) { return a.L > b.L; });
-    if (cudaMemcpy(plan.d_chol_sorted, sorted.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess)
-      return NGALORE_ERR_CUDA;
-  }
-  plan.d_tri = reinterpret_cast<TriInverse*>(plan.buf + o_tri);
+  plan.d_newton = reinterpret_cast<NewtonJob*>(plan.buf + o_newton);
+  plan.d_factor32 = reinterpret_cast<FactorMat*>(plan.buf + o_factor32);
+  plan.d_factor64 = reinterpret_cast<FactorMat*>(plan.buf + o_factor64);
+  auto wider = [](const FactorMat& a, const FactorMat& b) { return a.L > b.L; };
+  std::stable_sort(factor32.begin(), factor32.end(), wider);
+  std::stable_sort(factor64.begin(), factor64.end(), wider);
   plan.d_split_y = reinterpret_cast<SplitJob*>(plan.buf + o_sy);
   plan.d_syrk_mats = reinterpret_cast<SyrkMat*>(plan.buf + o_syrk_m);
   plan.d_syrk_tiles = reinterpret_cast<SyrkTile*>(plan.buf + o_syrk_t);
-  plan.d_prep64 = reinterpret_cast<GramPrep64*>(plan.buf + o_prep64);
   plan.d_split_z = reinterpret_cast<SplitJob*>(plan.buf + o_sz);
   plan.d_split_y_rest = reinterpret_cast<SplitJob*>(plan.buf + o_sy_rest);
   plan.d_split_z_rest = reinterpret_cast<SplitJob*>(plan.buf + o_sz_rest);
@@ -808,12 +550,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     }
     if (cudaMemcpy(plan.d_zero_d, zd.data(), sizeof(ZeroJob) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
   }
-  if (cudaMemcpy(plan.d_prep, prep.data(), sizeof(GramPrep) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_chol, chol.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_tri, tri.data(), sizeof(TriInverse) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+  if (cudaMemcpy(plan.d_newton, newton.data(), sizeof(NewtonJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(plan.d_factor32, factor32.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(plan.d_factor64, factor64.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_syrk_mats, syrk_m.data(), sizeof(SyrkMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_syrk_tiles, syrk_tiles.data(), sizeof(SyrkTile) * syrk_tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_prep64, prep64.data(), sizeof(GramPrep64) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_y, sy.data(), sizeof(SplitJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_z, sz.data(), sizeof(SplitJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_y_rest, sy_rest.data(), sizeof(SplitJob) * sy_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -838,7 +579,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         const RefreshMat& m = plan.mats[i];
         float* out; long long bytes;
         switch (g) {
-          case RG_Y_FROM_Z: case RG_APPLY_Y: out = m.Yf; bytes = 4ll * m.M * m.L; break;
+          case RG_Y_FROM_Z: case RG_APPLY_Y: case RG_APPLY_TRI: out = m.Yf; bytes = 4ll * m.M * m.L; break;
           case RG_Z_FROM_Y: out = m.Zf; bytes = 4ll * m.N * m.L; break;
           default: out = m.C32; bytes = 4ll * m.L * m.L; break;
         }
@@ -924,26 +665,6 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, Ctrl* d_ctrl, cu
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
-// X = Lf^-1 for every matrix (blocked), then R^-1 = D^-1 X^T in two bf16 parts.  T: what the buffers hold.
-template <typename T>
-inline ngalore_status refresh_tc_tri_inverse(RefreshPlan& plan, cudaStream_t stream, int64_t* launches) {
-  constexpr int set = sizeof(T) == 8 ? 0 : 1;
-  zero_jobs_kernel<<<dim3(32, plan.n_zero[RG_COUNT]), 256, 0, stream>>>(plan.d_zero[RG_COUNT]);
-  *launches += 1;
-  tri_leaf_kernel<T><<<(plan.n_leaves + 3) / 4, 128, 0, stream>>>(plan.d_leaves[set], plan.n_leaves);
-  *launches += 1;
-  for (int h = 1; h <= plan.tri_levels; ++h) {
-    if (plan.n_tg[h] == 0) continue;
-    const int tiles = (plan.tg_max[h] + 63) / 64;
-    tri_gemm_kernel<T><<<dim3(tiles, tiles, plan.n_tg[h]), 256, 0, stream>>>(plan.d_tg1[set][h]);
-    tri_gemm_kernel<T><<<dim3(tiles, tiles, plan.n_tg[h]), 256, 0, stream>>>(plan.d_tg2[set][h]);
-    *launches += 2;
-  }
-  tri_convert_kernel<T><<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_tri);
-  *launches += 1;
-  return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
-}
-
 // after_product: the iterate has just left a product with G, which wrote the bf16 parts itself except for the
 // matrices whose K it splits.
 inline ngalore_status refresh_tc_split(RefreshPlan& plan, bool y_side, cudaStream_t stream, int64_t* launches,
@@ -967,11 +688,8 @@ inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStrea
   if ((rc = refresh_tc_split(plan, true, stream, launches, true))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, d_ctrl, stream, launches))) return rc;
   // single precision from here to R^-1: the Gram matrix has 2^-17 of relative accuracy and a shift of about 1e-2
-  gram_prep_kernel<float><<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_prep, shift_scale);
-  *launches += 1;
-  if (chol_cta_launch<float>(plan.d_chol_sorted, plan.n, plan.l_max, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
-  if ((rc = refresh_tc_tri_inverse<float>(plan, stream, launches))) return rc;
-  if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches))) return rc;
+  if (tri_factor_launch<float>(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if ((rc = refresh_tc_gemm(plan, RG_APPLY_TRI, d_ctrl, stream, launches))) return rc;
   return refresh_tc_split(plan, true, stream, launches);
 }
 
@@ -985,11 +703,9 @@ inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStre
   zero_jobs_kernel<<<dim3(32, plan.n_zero[RG_COUNT]), 256, 0, stream>>>(plan.d_zero[RG_COUNT]);
   *launches += 1;
   syrk_f64_kernel<<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
-  gram_prep64_kernel<<<plan.n, 256, 0, stream>>>(plan.d_prep64);
-  *launches += 2;
-  if (chol_cta_launch<double>(plan.d_chol_sorted, plan.n, plan.l_max, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
-  if ((rc = refresh_tc_tri_inverse<double>(plan, stream, launches))) return rc;
-  return refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches);
+  *launches += 1;
+  if (tri_factor_launch<double>(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  return refresh_tc_gemm(plan, RG_APPLY_TRI, d_ctrl, stream, launches);
 }
 
 // Pass after refresh_tc_final: the basis is orthonormal to first order by then (1e-5, up to 1e-3 for a gradient of
@@ -999,7 +715,7 @@ inline ngalore_status refresh_tc_refine(RefreshPlan& plan, Ctrl* d_ctrl, cudaStr
   ngalore_status rc;
   if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, d_ctrl, stream, launches))) return rc;
-  newton_prep_kernel<<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_prep, plan.d_tri);
+  newton_prep_kernel<<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_newton);
   *launches += 1;
   return refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches);
 }
