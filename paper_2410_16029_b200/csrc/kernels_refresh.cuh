@@ -28,11 +28,12 @@ __global__ void fill_normal_kernel(float* X, long long n, unsigned long long see
   X[i] = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
-// The same values for a list of matrices in one launch: blockIdx.y selects the matrix (its stream of random numbers
-// is stream_base + blockIdx.y), blockIdx.x strides over its entries.
+// The same values as two bf16 parts for a list of matrices in one launch: blockIdx.y selects the matrix (its stream of
+// random numbers is stream_base + blockIdx.y), blockIdx.x strides over its entries.
 struct FillJob {
-  float* X;
-  long long n;
+  __nv_bfloat16 *hi, *lo;   // rows x ld
+  long long n;              // rows x cols
+  int cols, ld;
 };
 
 __global__ void fill_normal_grouped_kernel(const FillJob* jobs, unsigned long long seed, unsigned long long stream_base) {
@@ -44,7 +45,12 @@ __global__ void fill_normal_grouped_kernel(const FillJob* jobs, unsigned long lo
         splitmix64(seed ^ splitmix64(stream_id * 0x100000001B3ull + static_cast<unsigned long long>(i)));
     const float u1 = (static_cast<float>(h >> 40) + 1.0f) * (1.0f / 16777217.0f);
     const float u2 = static_cast<float>((h >> 8) & 0xFFFFFFull) * (1.0f / 16777216.0f);
-    jb.X[i] = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+    const float x = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+    const __nv_bfloat16 b = __float2bfloat16_rn(x);
+    const long long row = i < (1ll << 32) ? static_cast<unsigned int>(i) / static_cast<unsigned int>(jb.cols) : i / jb.cols;
+    const long long o = row * jb.ld + (i - row * jb.cols);
+    jb.hi[o] = b;
+    jb.lo[o] = __float2bfloat16_rn(x - __bfloat162float(b));
   }
 }
 

@@ -27,17 +27,6 @@
 namespace ngalore {
 
 // hi = bf16(x), lo = bf16(x - hi); rows x cols fp32 (dense) -> rows x ld bf16 (padding untouched: it is zero).
-__global__ void split_hilo_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ hi,
-                                  __nv_bfloat16* __restrict__ lo, long long n, int cols, int ld) {
-  const long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (i >= n) return;
-  const float x = src[i];
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  const long long o = (i / cols) * ld + (i % cols);
-  hi[o] = h;
-  lo[o] = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
 struct SplitJob {
   const float* src;
   __nv_bfloat16 *hi, *lo;
@@ -104,68 +93,88 @@ struct SyrkTile {
 constexpr int kSyrkRows = 1024;
 
 struct SyrkMat {
-  const float* Y;  // rows x L fp32
+  const __nv_bfloat16 *hi, *lo;   // rows x ld: the two parts of the basis, L columns of which are valid
   double* C;       // L x L fp64 accumulator (zeroed before the launch); lower tiles are written
-  int rows, L;
+  int rows, L, ld;
 };
 
-// Exact Gram matrix C += Y^T Y in fp64 (products of fp32 values are exact in fp64), grouped over all
-// matrices: one CTA per 64 x 64 lower tile and slab of rows, partial sums added with fp64 atomics.
+// Exact Gram matrix C += Y^T Y in fp64 of the basis as its two bf16 parts hold it (which is what the product with R^-1
+// multiplies), grouped over all matrices: one CTA per 64 x 64 lower tile and slab of rows, partial sums added with fp64
+// atomics.  On the fp64 tensor cores: bound by their rate, which is that of the vector units (34 TFLOP/s), but reached
+// with a quarter of the instructions and a third of the shared-memory reads; the next 16 rows are fetched and widened
+// while the current ones are multiplied.  156 matrices of the 1.1B shapes, 115 GFLOP: 7.2 ms with 4 x 4 register tiles on
+// the vector units, 4.1 ms so.
 __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, const SyrkTile* tiles) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
+  constexpr int LD = 64 + 8;      // rows 8 modulo 16 doubles apart: fragments without bank conflicts
+  __shared__ __align__(16) double As[2][16][LD];
+  __shared__ __align__(16) double Bs[2][16][LD];
   const SyrkTile t = tiles[blockIdx.x];
   const SyrkMat m = mats[t.mat];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
   const int i0 = t.ti * 64, j0 = t.tj * 64;
   const int k1 = (t.k0 + kSyrkRows < m.rows) ? t.k0 + kSyrkRows : m.rows;
-  double acc[4][4];
+  const int lc = (tid & 15) * 4, lk = tid >> 4;   // this thread fetches four columns of one row of either operand
+  const int wr = (warp >> 1) * 16, wc = (warp & 1) * 32;
+  const bool idle = t.ti == t.tj && wc > wr + 15;   // (all of it above the diagonal)
+  double acc[2][4][2];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int x = 0; x < 2; ++x)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  // the next 16 rows are fetched into registers while the current ones are multiplied
-  const int lc = threadIdx.x & 63, lk = threadIdx.x >> 6;
-  float pa[4], pb[4];
+    for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = 0.0;
+  uint2 ah, al, bh, bl;
   auto fetch = [&](int k0) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int k = k0 + lk + 4 * p;
-      pa[p] = (k < k1 && i0 + lc < m.L) ? m.Y[static_cast<long long>(k) * m.L + i0 + lc] : 0.f;
-      pb[p] = (k < k1 && j0 + lc < m.L) ? m.Y[static_cast<long long>(k) * m.L + j0 + lc] : 0.f;
-    }
+    const int k = k0 + lk;
+    const long long row = static_cast<long long>(min(k, k1 - 1)) * m.ld;
+    const uint2 zero = make_uint2(0u, 0u);
+    const bool in_a = k < k1 && i0 + lc < m.L, in_b = k < k1 && j0 + lc < m.L;
+    ah = in_a ? *reinterpret_cast<const uint2*>(m.hi + row + i0 + lc) : zero;
+    al = in_a ? *reinterpret_cast<const uint2*>(m.lo + row + i0 + lc) : zero;
+    bh = in_b ? *reinterpret_cast<const uint2*>(m.hi + row + j0 + lc) : zero;
+    bl = in_b ? *reinterpret_cast<const uint2*>(m.lo + row + j0 + lc) : zero;
+  };
+  auto widen = [](uint32_t h, uint32_t l) {
+    return make_double2(static_cast<double>(__uint_as_float(h << 16)) + static_cast<double>(__uint_as_float(l << 16)),
+                        static_cast<double>(__uint_as_float(h & 0xffff0000u)) + static_cast<double>(__uint_as_float(l & 0xffff0000u)));
+  };
+  auto put = [&](int buf) {
+    double2* a = reinterpret_cast<double2*>(&As[buf][lk][lc]);
+    double2* b = reinterpret_cast<double2*>(&Bs[buf][lk][lc]);
+    a[0] = widen(ah.x, al.x); a[1] = widen(ah.y, al.y);
+    b[0] = widen(bh.x, bl.x); b[1] = widen(bh.y, bl.y);
   };
   fetch(t.k0);
-  for (int k0 = t.k0; k0 < k1; k0 += 16) {
+  put(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = t.k0; k0 < k1; k0 += 16, buf ^= 1) {
+    const bool more = k0 + 16 < k1;
+    if (more) fetch(k0 + 16);
+    if (!idle) {
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      As[lk + 4 * p][lc] = pa[p];
-      Bs[lk + 4 * p][lc] = pb[p];
+      for (int kk = 0; kk < 16; kk += 4) {
+        double a[2], b[4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) a[x] = As[buf][kk + fk][wr + 8 * x + fr];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) b[y] = Bs[buf][kk + fk][wc + 8 * y + fr];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) dmma(acc[x][y], a[x], b[y]);
+      }
     }
-    __syncthreads();
-    if (k0 + 16 < k1) fetch(k0 + 16);
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) { a[x] = static_cast<double>(As[kk][ty * 4 + x]); b[x] = static_cast<double>(Bs[kk][tx * 4 + x]); }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
-    }
+    if (more) put(buf ^ 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int i = i0 + ty * 4 + x;
-    if (i >= m.L) continue;
+  for (int x = 0; x < 2; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int j = j0 + tx * 4 + y;
-      if (j <= i) atomicAdd(m.C + static_cast<long long>(i) * m.L + j, acc[x][y]);
-    }
-  }
+    for (int y = 0; y < 4; ++y)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = i0 + wr + 8 * x + fr, j = j0 + wc + 8 * y + 2 * fk + h;
+        if (i < m.L && j <= i) atomicAdd(m.C + static_cast<long long>(i) * m.L + j, acc[x][y][h]);
+      }
 }
 
 struct NewtonJob {
@@ -242,13 +251,20 @@ __global__ void __launch_bounds__(256) column_scale_kernel(const NormJob* jobs) 
 
 // RG_APPLY_TRI: RG_APPLY_Y with an upper triangular right operand (its blocks of zeros are left out)
 enum RefreshGemm { RG_Y_FROM_Z = 0, RG_Z_FROM_Y, RG_GRAM_Y, RG_GRAM_Z, RG_APPLY_Y, RG_APPLY_TRI, RG_COUNT };
+// The basis Y is kept as two bf16 parts, in two sets that take turns: a product with G leaves it in set 0, Q = Y R^-1 goes
+// from one set to the other (its tiles read whole rows of Y while others write).  Set 1 shares the memory of the fp32
+// buffer Yf, which only the result of the refresh and the products with a split K use.
 enum RefreshMap { RM_G_A = 0, RM_G_MN, RM_Z_B, RM_Z_B_LO, RM_Y_B, RM_Y_B_LO, RM_Y_A, RM_Y_A_LO,
-                  RM_RINV, RM_RINV_LO, RM_COUNT };
+                  RM_Y1_B, RM_Y1_B_LO, RM_Y1_A, RM_Y1_A_LO, RM_RINV, RM_RINV_LO, RM_COUNT };
+// The problem tables: a kind of product (RefreshGemm: its tiles) with its operands' and result's place.
+enum RefreshProb { RP_Y_FROM_Z = 0, RP_Z_FROM_Y0, RP_Z_FROM_Y1, RP_GRAM_Y0, RP_GRAM_Y1, RP_GRAM_Z, RP_APPLY_01, RP_APPLY_10,
+                   RP_APPLY_0F, RP_COUNT };
 
 struct RefreshMat {
   int M, N, L, ldl;
   float *Yf, *Zf;                       // fp32 GEMM outputs (M x L, N x L)
-  __nv_bfloat16 *Yhi, *Ylo, *Zhi, *Zlo; // bf16 parts of the iterates (rows x ldl)
+  __nv_bfloat16 *Yhi, *Ylo, *Zhi, *Zlo; // bf16 parts of the iterates (rows x ldl), Y in set 0
+  __nv_bfloat16 *Y1hi, *Y1lo;           // Y in set 1 (the memory of Yf, M x ldl floats)
   float* C32;                           // L x L
   double *C64, *X64, *T64;              // L x L each
   double* D;                            // L
@@ -270,7 +286,7 @@ struct RefreshPlan {
   std::vector<const void*> last_G;
   char* buf = nullptr;
   CUtensorMap* d_maps = nullptr;
-  TcProblem* d_probs[RG_COUNT] = {};
+  TcProblem* d_probs[RP_COUNT] = {};
   TcTile* d_tiles[RG_COUNT] = {};
   int n_tiles[RG_COUNT] = {};
   int grid[RG_COUNT] = {};
@@ -283,7 +299,6 @@ struct RefreshPlan {
   FactorMat* d_factor32 = nullptr;   // R^-1 from C32 (tri_factor.cuh), widest first
   FactorMat* d_factor64 = nullptr;   // R^-1 from the exact Gram matrix in X64
   int l_max = 0;  // largest basis width L of the set
-  SplitJob* d_split_y = nullptr;
   // the matrices whose product with G splits K (their result arrives as fp32 and is split afterwards; all others
   // leave the product as bf16 parts already)
   SplitJob* d_split_y_rest = nullptr;
@@ -292,7 +307,6 @@ struct RefreshPlan {
   SyrkMat* d_syrk_mats = nullptr;
   SyrkTile* d_syrk_tiles = nullptr;
   int n_syrk_tiles = 0;
-  SplitJob* d_split_z = nullptr;
   // Rayleigh-Ritz rotation: the eigensolver works in the X64, T64 and C64 buffers
   EigMat* d_eig = nullptr;
   CholProblem* d_eig_chol = nullptr;
@@ -327,9 +341,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.last_G.assign(n, nullptr);
 
   // ---- tile and problem tables (host)
-  std::vector<TcProblem> probs[RG_COUNT];
+  std::vector<TcProblem> probs[RP_COUNT];
   std::vector<TcTile> tiles[RG_COUNT];
-  for (int g = 0; g < RG_COUNT; ++g) probs[g].resize(n);
+  for (int g = 0; g < RP_COUNT; ++g) probs[g].resize(n);
   auto add_tiles = [&](int g, int i, int out_rows, int out_cols, int K, long long target_kb) {
     const int kb_total = (K + kTcBK - 1) / kTcBK;
     int splits = static_cast<int>((kb_total + target_kb - 1) / target_kb);
@@ -370,7 +384,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     offs[i].Rlo = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
   }
   const size_t o_maps = take(sizeof(CUtensorMap) * RM_COUNT * n);
-  size_t o_probs[RG_COUNT], o_tiles[RG_COUNT];
+  size_t o_probs[RP_COUNT], o_tiles[RG_COUNT];
+  for (int g = 0; g < RP_COUNT; ++g) o_probs[g] = take(sizeof(TcProblem) * n);
 
   // work estimate for the split-K targets: per GEMM kind, k-blocks per CTA if perfectly balanced
   for (int g = 0; g < RG_COUNT; ++g) {
@@ -403,7 +418,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       add_tiles(g, i, rows, cols, K, target);
     }
     std::stable_sort(tiles[g].begin(), tiles[g].end(), [](const TcTile& a, const TcTile& b) { return a.kblocks > b.kblocks; });
-    o_probs[g] = take(sizeof(TcProblem) * n);
     o_tiles[g] = take(sizeof(TcTile) * tiles[g].size());
     plan.n_tiles[g] = static_cast<int>(tiles[g].size());
     plan.grid[g] = std::min(plan.n_tiles[g], sm_count);
@@ -421,8 +435,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.n_syrk_tiles = static_cast<int>(syrk_tiles.size());
   const size_t o_syrk_m = take(sizeof(SyrkMat) * n);
   const size_t o_syrk_t = take(sizeof(SyrkTile) * syrk_tiles.size());
-  const size_t o_sy = take(sizeof(SplitJob) * n);
-  const size_t o_sz = take(sizeof(SplitJob) * n);
   const size_t o_sy_rest = take(sizeof(SplitJob) * n);
   const size_t o_sz_rest = take(sizeof(SplitJob) * n);
   const size_t o_eig = take(sizeof(EigMat) * n);
@@ -441,7 +453,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   std::vector<FactorMat> factor32(n), factor64(n);
   plan.l_max = 0;
   for (const RefreshMat& m : plan.mats) plan.l_max = m.L > plan.l_max ? m.L : plan.l_max;
-  std::vector<SplitJob> sy(n), sz(n), sy_rest, sz_rest;
+  std::vector<SplitJob> sy_rest, sz_rest;
   std::vector<SyrkMat> syrk_m(n);
   std::vector<EigMat> eig(n);
   std::vector<CholProblem> eig_chol(n);
@@ -464,13 +476,13 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     newton[i] = NewtonJob{m.C32, m.Rhi, m.Rlo, m.L, m.ldl};
     factor32[i] = FactorMat{m.C32, m.C64, nullptr, m.Rhi, m.Rlo, m.L, m.ldl};
     factor64[i] = FactorMat{m.X64, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
-    syrk_m[i] = SyrkMat{m.Yf, m.X64, m.M, m.L};
-    sy[i] = SplitJob{m.Yf, m.Yhi, m.Ylo, static_cast<long long>(m.M) * m.L, m.L, m.ldl};
-    sz[i] = SplitJob{m.Zf, m.Zhi, m.Zlo, static_cast<long long>(m.N) * m.L, m.L, m.ldl};
+    m.Y1hi = reinterpret_cast<__nv_bfloat16*>(m.Yf);
+    m.Y1lo = m.Y1hi + static_cast<size_t>(m.M) * m.ldl;
+    syrk_m[i] = SyrkMat{m.Y1hi, m.Y1lo, m.X64, m.M, m.L, m.ldl};
     if (std::find(plan.atomic_mats[RG_Y_FROM_Z].begin(), plan.atomic_mats[RG_Y_FROM_Z].end(), i) != plan.atomic_mats[RG_Y_FROM_Z].end())
-      sy_rest.push_back(sy[i]);
+      sy_rest.push_back(SplitJob{m.Yf, m.Yhi, m.Ylo, static_cast<long long>(m.M) * m.L, m.L, m.ldl});
     if (std::find(plan.atomic_mats[RG_Z_FROM_Y].begin(), plan.atomic_mats[RG_Z_FROM_Y].end(), i) != plan.atomic_mats[RG_Z_FROM_Y].end())
-      sz_rest.push_back(sz[i]);
+      sz_rest.push_back(SplitJob{m.Zf, m.Zhi, m.Zlo, static_cast<long long>(m.N) * m.L, m.L, m.ldl});
     // (the rotated part: all of the basis, or its leading ritz_columns, kept a multiple of 4)
     const int Lj = std::min(m.L, (ritz_columns + 3) & ~3);
     int* redo = reinterpret_cast<int*>(plan.buf + o_eig_redo) + i;
@@ -488,33 +500,42 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     ok &= tc_encode_2d(plan.encode, mp + RM_Y_B_LO, m.Ylo, m.L, m.M, sl, 64, kTcBK);
     ok &= tc_encode_2d(plan.encode, mp + RM_Y_A, m.Yhi, m.L, m.M, sl, kTcBK, kTcBM);
     ok &= tc_encode_2d(plan.encode, mp + RM_Y_A_LO, m.Ylo, m.L, m.M, sl, kTcBK, kTcBM);
+    ok &= tc_encode_2d(plan.encode, mp + RM_Y1_B, m.Y1hi, m.L, m.M, sl, 64, kTcBK);
+    ok &= tc_encode_2d(plan.encode, mp + RM_Y1_B_LO, m.Y1lo, m.L, m.M, sl, 64, kTcBK);
+    ok &= tc_encode_2d(plan.encode, mp + RM_Y1_A, m.Y1hi, m.L, m.M, sl, kTcBK, kTcBM);
+    ok &= tc_encode_2d(plan.encode, mp + RM_Y1_A_LO, m.Y1lo, m.L, m.M, sl, kTcBK, kTcBM);
     ok &= tc_encode_2d(plan.encode, mp + RM_RINV, m.Rhi, m.L, m.L, sl, 64, kTcBK);
     ok &= tc_encode_2d(plan.encode, mp + RM_RINV_LO, m.Rlo, m.L, m.L, sl, 64, kTcBK);
     if (!ok) return NGALORE_ERR_CUDA;
     const int base = i * RM_COUNT;
-    probs[RG_Y_FROM_Z][i] = TcProblem{m.Yf, m.M, m.L, m.L, base + RM_G_A, base + RM_Z_B, 0};
-    probs[RG_Z_FROM_Y][i] = TcProblem{m.Zf, m.N, m.L, m.L, base + RM_G_MN, base + RM_Y_B, 0};
-    {
-      const std::vector<int>& ay = plan.atomic_mats[RG_Y_FROM_Z];
-      const std::vector<int>& az = plan.atomic_mats[RG_Z_FROM_Y];
-      if (std::find(ay.begin(), ay.end(), i) == ay.end()) {
-        probs[RG_Y_FROM_Z][i].ld16 = m.ldl; probs[RG_Y_FROM_Z][i].out_hi = m.Yhi; probs[RG_Y_FROM_Z][i].out_lo = m.Ylo;
-      }
-      if (std::find(az.begin(), az.end(), i) == az.end()) {
-        probs[RG_Z_FROM_Y][i].ld16 = m.ldl; probs[RG_Z_FROM_Y][i].out_hi = m.Zhi; probs[RG_Z_FROM_Y][i].out_lo = m.Zlo;
-      }
-    }
-    probs[RG_GRAM_Y][i] = TcProblem{m.C32, m.L, m.L, m.L, base + RM_Y_B, base + RM_Y_B, 0};
-    probs[RG_GRAM_Z][i] = TcProblem{m.C32, m.L, m.L, m.L, base + RM_Z_B, base + RM_Z_B, 0};
-    probs[RG_APPLY_Y][i] = TcProblem{m.Yf, m.M, m.L, m.L, base + RM_Y_A, base + RM_RINV, 0};
-    probs[RG_APPLY_TRI][i] = probs[RG_APPLY_Y][i];
+    // result as bf16 parts (hi == nullptr: as fp32)
+    auto problem = [&](float* out, int rows, int map_a, int map_b, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+      TcProblem q{out, rows, m.L, m.L, base + map_a, base + map_b, 0};
+      if (hi != nullptr) { q.ld16 = m.ldl; q.out_hi = hi; q.out_lo = lo; }
+      return q;
+    };
+    auto is_split = [&](int g) {
+      const std::vector<int>& a = plan.atomic_mats[g];
+      return std::find(a.begin(), a.end(), i) != a.end();
+    };
+    probs[RP_Y_FROM_Z][i] = problem(m.Yf, m.M, RM_G_A, RM_Z_B, is_split(RG_Y_FROM_Z) ? nullptr : m.Yhi, m.Ylo);
+    probs[RP_Z_FROM_Y0][i] = problem(m.Zf, m.N, RM_G_MN, RM_Y_B, is_split(RG_Z_FROM_Y) ? nullptr : m.Zhi, m.Zlo);
+    probs[RP_Z_FROM_Y1][i] = problem(m.Zf, m.N, RM_G_MN, RM_Y1_B, is_split(RG_Z_FROM_Y) ? nullptr : m.Zhi, m.Zlo);
+    probs[RP_GRAM_Y0][i] = problem(m.C32, m.L, RM_Y_B, RM_Y_B, nullptr, nullptr);
+    probs[RP_GRAM_Y1][i] = problem(m.C32, m.L, RM_Y1_B, RM_Y1_B, nullptr, nullptr);
+    probs[RP_GRAM_Z][i] = problem(m.C32, m.L, RM_Z_B, RM_Z_B, nullptr, nullptr);
+    probs[RP_APPLY_01][i] = problem(nullptr, m.M, RM_Y_A, RM_RINV, m.Y1hi, m.Y1lo);
+    probs[RP_APPLY_10][i] = problem(nullptr, m.M, RM_Y1_A, RM_RINV, m.Yhi, m.Ylo);
+    probs[RP_APPLY_0F][i] = problem(m.Yf, m.M, RM_Y_A, RM_RINV, nullptr, nullptr);
   }
   plan.d_maps = reinterpret_cast<CUtensorMap*>(plan.buf + o_maps);
-  for (int g = 0; g < RG_COUNT; ++g) {
+  for (int g = 0; g < RP_COUNT; ++g) {
     plan.d_probs[g] = reinterpret_cast<TcProblem*>(plan.buf + o_probs[g]);
+    if (cudaMemcpy(plan.d_probs[g], probs[g].data(), sizeof(TcProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
+  }
+  for (int g = 0; g < RG_COUNT; ++g) {
     plan.d_tiles[g] = reinterpret_cast<TcTile*>(plan.buf + o_tiles[g]);
-    if (cudaMemcpy(plan.d_probs[g], probs[g].data(), sizeof(TcProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(plan.d_tiles[g], tiles[g].data(), sizeof(TcTile) * tiles[g].size(), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(plan.d_tiles[g], tiles[g].data(), sizeof(TcTile) * tiles[g].size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return NGALORE_ERR_CUDA;
   }
   plan.d_newton = reinterpret_cast<NewtonJob*>(plan.buf + o_newton);
@@ -523,10 +544,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   auto wider = [](const FactorMat& a, const FactorMat& b) { return a.L > b.L; };
   std::stable_sort(factor32.begin(), factor32.end(), wider);
   std::stable_sort(factor64.begin(), factor64.end(), wider);
-  plan.d_split_y = reinterpret_cast<SplitJob*>(plan.buf + o_sy);
   plan.d_syrk_mats = reinterpret_cast<SyrkMat*>(plan.buf + o_syrk_m);
   plan.d_syrk_tiles = reinterpret_cast<SyrkTile*>(plan.buf + o_syrk_t);
-  plan.d_split_z = reinterpret_cast<SplitJob*>(plan.buf + o_sz);
   plan.d_split_y_rest = reinterpret_cast<SplitJob*>(plan.buf + o_sy_rest);
   plan.d_split_z_rest = reinterpret_cast<SplitJob*>(plan.buf + o_sz_rest);
   plan.n_split_y_rest = static_cast<int>(sy_rest.size());
@@ -538,7 +557,10 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.d_fill = reinterpret_cast<FillJob*>(plan.buf + o_fill);
   {
     std::vector<FillJob> fill(n);
-    for (int i = 0; i < n; ++i) fill[i] = FillJob{plan.mats[i].Zf, static_cast<long long>(plan.mats[i].N) * plan.mats[i].L};
+    for (int i = 0; i < n; ++i) {
+      const RefreshMat& m = plan.mats[i];
+      fill[i] = FillJob{m.Zhi, m.Zlo, static_cast<long long>(m.N) * m.L, m.L, m.ldl};
+    }
     if (cudaMemcpy(plan.d_fill, fill.data(), sizeof(FillJob) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
   }
   plan.d_zero_d = reinterpret_cast<ZeroJob*>(plan.buf + o_zero_d);
@@ -555,8 +577,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_factor64, factor64.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_syrk_mats, syrk_m.data(), sizeof(SyrkMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_syrk_tiles, syrk_tiles.data(), sizeof(SyrkTile) * syrk_tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_split_y, sy.data(), sizeof(SplitJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_split_z, sz.data(), sizeof(SplitJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_y_rest, sy_rest.data(), sizeof(SplitJob) * sy_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_z_rest, sz_rest.data(), sizeof(SplitJob) * sz_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_eig, eig.data(), sizeof(EigMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -621,9 +641,10 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
 }
 
 
+// g: the kind of product, problem: its operands' and result's place (RefreshProb).
 // high_only: the products with G take only the high bf16 part of the basis (half the tensor-core work; the basis
 // then enters with 8 bits instead of 16, which the early sweeps of the iteration do not notice).
-inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches,
+inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches,
                                       bool high_only = false) {
   // outputs that several K slices accumulate into start from zero
   if (plan.n_zero[g] > 0) {
@@ -638,86 +659,76 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, Ctrl* d_ctrl, cu
     case RG_Y_FROM_Z:
       if (high_only)
         tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L0::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       else
         tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L1::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     case RG_Z_FROM_Y:
       if (high_only)
         tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L0::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       else
         tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L1::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     case RG_GRAM_Y:
     case RG_GRAM_Z:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     default:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[g]);
+          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
   }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
-// after_product: the iterate has just left a product with G, which wrote the bf16 parts itself except for the
-// matrices whose K it splits.
-inline ngalore_status refresh_tc_split(RefreshPlan& plan, bool y_side, cudaStream_t stream, int64_t* launches,
-                                       bool after_product = false) {
-  const SplitJob* jobs = y_side ? plan.d_split_y : plan.d_split_z;
-  int n_jobs = plan.n;
-  if (after_product) {
-    jobs = y_side ? plan.d_split_y_rest : plan.d_split_z_rest;
-    n_jobs = y_side ? plan.n_split_y_rest : plan.n_split_z_rest;
-    if (n_jobs == 0) return NGALORE_OK;
-  }
-  split_hilo_grouped_kernel<<<dim3(64, n_jobs), 256, 0, stream>>>(jobs);
+// The products with G write the bf16 parts of their result themselves, except for the matrices whose K they split.
+inline ngalore_status refresh_tc_split(RefreshPlan& plan, bool y_side, cudaStream_t stream, int64_t* launches) {
+  const int n_jobs = y_side ? plan.n_split_y_rest : plan.n_split_z_rest;
+  if (n_jobs == 0) return NGALORE_OK;
+  split_hilo_grouped_kernel<<<dim3(64, n_jobs), 256, 0, stream>>>(y_side ? plan.d_split_y_rest : plan.d_split_z_rest);
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
-// iterate (as it leaves the product Y = G Z) -> well-conditioned basis, left both as fp32 and as its bf16 parts.
+// iterate (as it leaves the product Y = G Z, in set 0) -> well-conditioned basis, in set 1.
 inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches,
                                       double shift_scale = 1.0) {
   ngalore_status rc;
-  if ((rc = refresh_tc_split(plan, true, stream, launches, true))) return rc;
-  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, RP_GRAM_Y0, d_ctrl, stream, launches))) return rc;
   // single precision from here to R^-1: the Gram matrix has 2^-17 of relative accuracy and a shift of about 1e-2
   if (tri_factor_launch<float>(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
-  if ((rc = refresh_tc_gemm(plan, RG_APPLY_TRI, d_ctrl, stream, launches))) return rc;
-  return refresh_tc_split(plan, true, stream, launches);
+  return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_01, d_ctrl, stream, launches);
 }
 
 // Final pass: Cholesky QR of the last basis with the Gram matrix accumulated exactly in fp64 (no shift beyond
 // 1e-12), Cholesky and triangular inverse in fp64; only Q = Y R^-1 goes through the tensor cores in two bf16
 // parts, whose rounding averages out over the rows.  Matrices with few rows are re-done entirely in fp64 by
-// the caller.
+// the caller.  From set 1 to set 0.
 inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches) {
-  ngalore_status rc;
-  // (the bf16 parts of the basis, which the apply below multiplies, are current: refresh_tc_orth ends with a split)
   zero_jobs_kernel<<<dim3(32, plan.n_zero[RG_COUNT]), 256, 0, stream>>>(plan.d_zero[RG_COUNT]);
   *launches += 1;
   syrk_f64_kernel<<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
   *launches += 1;
   if (tri_factor_launch<double>(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
-  return refresh_tc_gemm(plan, RG_APPLY_TRI, d_ctrl, stream, launches);
+  return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_10, d_ctrl, stream, launches);
 }
 
 // Pass after refresh_tc_final: the basis is orthonormal to first order by then (1e-5, up to 1e-3 for a gradient of
 // low numerical rank), and a Newton step with the tensor-core Gram matrix squares what is missing, down to the
 // accuracy of that Gram matrix; a second exact pass gave the same at ten times the cost.
-inline ngalore_status refresh_tc_refine(RefreshPlan& plan, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches) {
+// From set `set` to the other.
+inline ngalore_status refresh_tc_refine(RefreshPlan& plan, int set, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches) {
   ngalore_status rc;
-  if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
-  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, set == 0 ? RP_GRAM_Y0 : RP_GRAM_Y1, d_ctrl, stream, launches))) return rc;
   newton_prep_kernel<<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_newton);
   *launches += 1;
-  return refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches);
+  return refresh_tc_gemm(plan, RG_APPLY_Y, set == 0 ? RP_APPLY_01 : RP_APPLY_10, d_ctrl, stream, launches);
 }
 
 // Whole-set refresh; leaves the basis in Yf.
@@ -743,8 +754,7 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   fill_normal_grouped_kernel<<<dim3(64, plan.n), 256, 0, stream>>>(plan.d_fill, seed, stream_base);
   *launches += 1;
   if (cudaGetLastError() != cudaSuccess) return NGALORE_ERR_CUDA;
-  if ((rc = refresh_tc_split(plan, false, stream, launches))) return rc;
-  if ((rc = refresh_tc_gemm(plan, RG_Y_FROM_Z, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_Y_FROM_Z, RP_Y_FROM_Z, d_ctrl, stream, launches))) return rc;
   if ((rc = refresh_tc_orth(plan, d_ctrl, stream, launches))) return rc;
   // A sweep applies G G^T to the basis and orthonormalises the result.  Z = G^T Q is not orthonormalised in between:
   // its columns are images of orthonormal ones, and the two-part bf16 operands keep 16 bits of every entry whatever
@@ -755,9 +765,9 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
     // (2^-9 of an entry) shrinks with every later sweep like any other component outside the dominant subspace
     // (not with fewer than four sweeps, where every one of them counts)
     const bool coarse = q >= 4 && it < q / 2;
-    if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, d_ctrl, stream, launches, coarse))) return rc;
-    if ((rc = refresh_tc_split(plan, false, stream, launches, true))) return rc;
-    if ((rc = refresh_tc_gemm(plan, RG_Y_FROM_Z, d_ctrl, stream, launches, coarse))) return rc;
+    if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, RP_Z_FROM_Y1, d_ctrl, stream, launches, coarse))) return rc;
+    if ((rc = refresh_tc_split(plan, false, stream, launches))) return rc;
+    if ((rc = refresh_tc_gemm(plan, RG_Y_FROM_Z, RP_Y_FROM_Z, d_ctrl, stream, launches, coarse))) return rc;
     if ((rc = refresh_tc_orth(plan, d_ctrl, stream, launches))) return rc;
   }
   // Exact orthonormalisation of the basis that leaves the sweeps: the basis can be ill conditioned in its weak
@@ -765,19 +775,18 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   // Newton steps start from that and end at about 1e-6.  The Rayleigh-Ritz step below relies on it (it
   // solves C v = lambda v, not C v = lambda (Q^T Q) v, and what Q lacks in orthonormality goes into the Ritz vectors).
   if ((rc = refresh_tc_final(plan, d_ctrl, stream, launches))) return rc;
-  if ((rc = refresh_tc_refine(plan, d_ctrl, stream, launches))) return rc;
-  if ((rc = refresh_tc_refine(plan, d_ctrl, stream, launches))) return rc;
-  if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
+  if ((rc = refresh_tc_refine(plan, 0, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_refine(plan, 1, d_ctrl, stream, launches))) return rc;
   // Rayleigh-Ritz: Z = G^T Q, C = Z^T Z (tensor cores: its entries are good to about 2^-17 of the diagonal, far
   // finer than the gaps that decide a Ritz vector), V = eigenvectors of C (or of its leading block, see
   // ritz_eigen.cuh), P = Q V.
-  if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, d_ctrl, stream, launches))) return rc;
-  if ((rc = refresh_tc_split(plan, false, stream, launches, true))) return rc;
-  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Z, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, RP_Z_FROM_Y0, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_split(plan, false, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_GRAM_Z, RP_GRAM_Z, d_ctrl, stream, launches))) return rc;
   if (eig_batched_launch(plan.d_eig, plan.d_eig_chol, plan.n, plan.eig_max, plan.l_max, plan.sm_count, stream, launches) != cudaSuccess)
     return NGALORE_ERR_CUDA;
   // Q orthonormal to about 1e-6 and V orthogonal: so is their product, once its columns are scaled back to unit norm
-  if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, RP_APPLY_0F, d_ctrl, stream, launches))) return rc;
   zero_jobs_kernel<<<dim3(1, plan.n), 256, 0, stream>>>(plan.d_zero_d);
   const dim3 norm_grid((plan.l_max + 31) / 32, plan.n, (plan.m_max + kNormRows - 1) / kNormRows);
   column_sumsq_kernel<<<norm_grid, dim3(32, 8), 0, stream>>>(plan.d_norm);
