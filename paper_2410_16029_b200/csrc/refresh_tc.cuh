@@ -18,6 +18,7 @@
 #include <vector>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "gemm_tcgen05.cuh"
 #include "kernels_refresh.cuh"
@@ -272,6 +273,11 @@ struct RefreshMat {
 };
 
 constexpr int kRefBN = 128;
+// The products with G take tiles of 256 columns where most of the work has bases that wide: a 128 x 256 tile needs
+// three quarters of the shared-memory reads per multiply-add, and G is read half as often.
+constexpr int kRefWideBN = 256;
+constexpr int kRefWideStages1 = 2;  // NA = 1, NB = 2: 80 KB per stage
+constexpr int kRefWideStages0 = 4;  // NA = 1, NB = 1: 48 KB per stage
 constexpr int kRefStages1 = 4;  // NA = 1, NB = 2: 48 KB per stage
 constexpr int kRefStages0 = 6;  // NA = 1, NB = 1: 32 KB per stage
 constexpr int kRefStages2 = 3;  // NA = 2, NB = 2: 64 KB per stage
@@ -290,6 +296,7 @@ struct RefreshPlan {
   TcTile* d_tiles[RG_COUNT] = {};
   int n_tiles[RG_COUNT] = {};
   int grid[RG_COUNT] = {};
+  bool wide = false;           // the products with G take tiles of kRefWideBN columns
   std::vector<int> atomic_mats[RG_COUNT];  // matrices whose K is split for this GEMM (output must be zeroed)
   // buffers to clear before GEMM kind g (the outputs of atomic_mats[g]); entry RG_COUNT: every matrix's X64
   ZeroJob* d_zero[RG_COUNT + 1] = {};
@@ -344,6 +351,16 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   std::vector<TcProblem> probs[RP_COUNT];
   std::vector<TcTile> tiles[RG_COUNT];
   for (int g = 0; g < RP_COUNT; ++g) probs[g].resize(n);
+  {
+    double all = 0.0, wide = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const double w = static_cast<double>(mats[i].M) * mats[i].N * mats[i].rp;
+      all += w;
+      if (mats[i].rp > 192) wide += w;
+    }
+    plan.wide = 2.0 * wide >= all;
+  }
+  auto tile_cols = [&](int g) { return plan.wide && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? kRefWideBN : kRefBN; };
   auto add_tiles = [&](int g, int i, int out_rows, int out_cols, int K, long long target_kb) {
     const int kb_total = (K + kTcBK - 1) / kTcBK;
     int splits = static_cast<int>((kb_total + target_kb - 1) / target_kb);
@@ -352,7 +369,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     splits = (kb_total + kb_per - 1) / kb_per;
     if (splits > 1) plan.atomic_mats[g].push_back(i);
     const bool symmetric = g == RG_GRAM_Y || g == RG_GRAM_Z;   // the lower triangle is enough
-    for (int n0 = 0; n0 < out_cols; n0 += kRefBN)
+    for (int n0 = 0; n0 < out_cols; n0 += tile_cols(g))
       for (int sp = 0; sp < splits; ++sp)
         for (int m0 = symmetric ? n0 / kTcBM * kTcBM : 0; m0 < out_rows; m0 += kTcBM) {
           const int kb0 = sp * kb_per;
@@ -400,7 +417,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         case RG_GRAM_Z: rows = m.L; cols = m.L; K = m.N; break;
         default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y, RG_APPLY_TRI
       }
-      total_kb += static_cast<long long>((rows + kTcBM - 1) / kTcBM) * ((cols + kRefBN - 1) / kRefBN) *
+      total_kb += static_cast<long long>((rows + kTcBM - 1) / kTcBM) * ((cols + tile_cols(g) - 1) / tile_cols(g)) *
                   ((K + kTcBK - 1) / kTcBK);
     }
     long long target = (total_kb + sm_count - 1) / sm_count / 4;
@@ -623,7 +640,17 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   using L1 = TcSmem<kRefBN, 1, 2, kRefStages1, 4>;
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 4>;
   using L0 = TcSmem<kRefBN, 1, 1, kRefStages0, 4>;
-  if (cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, false>,
+  using LW1 = TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>;
+  using LW0 = TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>;
+  if (cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, false>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW0::kTotal) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, true>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW0::kTotal) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, false>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW1::kTotal) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, true>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW1::kTotal) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, false>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L0::kTotal) != cudaSuccess ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L0::kTotal) != cudaSuccess ||
@@ -651,27 +678,29 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     zero_jobs_kernel<<<dim3(32, plan.n_zero[g]), 256, 0, stream>>>(plan.d_zero[g]);
     *launches += 1;
   }
-  using L1 = TcSmem<kRefBN, 1, 2, kRefStages1, 4>;
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 4>;
   const int threads = 64 + 32 * 4;
-  using L0 = TcSmem<kRefBN, 1, 1, kRefStages0, 4>;
+  auto product = [&](auto a_mn) {   // a product with G; a_mn: with G^T
+    constexpr bool MN = decltype(a_mn)::value;
+    if (plan.wide) {
+      if (high_only)
+        tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>::kTotal, stream>>>(
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+      else
+        tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>::kTotal, stream>>>(
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+    } else {
+      if (high_only)
+        tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 1, kRefStages0, 4>::kTotal, stream>>>(
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+      else
+        tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 2, kRefStages1, 4>::kTotal, stream>>>(
+            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+    }
+  };
   switch (g) {
-    case RG_Y_FROM_Z:
-      if (high_only)
-        tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L0::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      else
-        tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L1::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      break;
-    case RG_Z_FROM_Y:
-      if (high_only)
-        tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L0::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      else
-        tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L1::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      break;
+    case RG_Y_FROM_Z: product(std::false_type{}); break;
+    case RG_Z_FROM_Y: product(std::true_type{}); break;
     case RG_GRAM_Y:
     case RG_GRAM_Z:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
