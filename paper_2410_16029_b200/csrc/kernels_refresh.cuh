@@ -518,43 +518,117 @@ __global__ void working_copies_kernel(const float* P32, uint16_t* P16, uint16_t*
   }
 }
 
-// The same for a list of matrices in one launch, reading the new basis where the refresh left it (src) and writing
-// the fp32 master as well.  CTA t works on a 32 x 32 tile; tile_start[j] is the first tile of job j (n_jobs + 1
-// entries, ascending).
+// The end of a refresh for a list of matrices in two launches, each reading the new basis once: the column norms, and the
+// master and working copies of the basis with its columns scaled to unit norm.  Scaling: the products of the refresh go
+// through operands split in two bf16 parts; the rounding of the diagonal of a triangular factor or of a rotation (a
+// relative 2^-17) scales a whole column, which is the largest part of what the last product leaves of
+// non-orthonormality.  The norms also tell a basis that is none (see basis_check_kernel): all of them zero, or one not
+// finite; such a matrix gets the first r' unit vectors, in the second case with its status word set.
+// CTAs take tiles of kEndRows rows (norms) and kEndRows x kEndCols entries (copies); tile_start[j] is the first tile of
+// job j (n_jobs + 1 entries, ascending).  Bound by memory traffic: 4 bytes an entry read, then 12.  They replaced five
+// kernels of five passes with one CTA count for every matrix, so that a 32000-row embedding took as many CTAs as a
+// 512-row matrix: 60M shapes 316 us, 130M 680 us, 1.1B 2620 us before, 48, 113 and 610 us now.
 struct WorkingJob {
-  const float* src;   // rows x rp, dense
+  const float* src;   // rows x rp, dense; rp a multiple of 4
+  double* sums;       // rp sums of squares (cleared beforehand)
   float* P32;
   uint16_t* P16;
   uint16_t* Pt16;
+  int* status;
   int rows, rp, ldp, ldpt;
   int p16_is_half;
   int tiles_x;        // tiles along the rp columns
 };
+constexpr int kEndRows = 128, kEndCols = 64;
 
-__global__ void working_copies_grouped_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
-  __shared__ float tile[32][33];
+__device__ __forceinline__ int end_job(const int* tile_start, int n_jobs) {
   int lo = 0, hi = n_jobs;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (tile_start[mid] <= static_cast<int>(blockIdx.x)) lo = mid; else hi = mid;
   }
-  const WorkingJob jb = jobs[lo];
-  const int t = static_cast<int>(blockIdx.x) - tile_start[lo];
-  const int i0 = (t / jb.tiles_x) * 32, j0 = (t % jb.tiles_x) * 32;
-  for (int a = threadIdx.y; a < 32; a += blockDim.y) {
-    const int i = i0 + a, j = j0 + threadIdx.x;
-    float val = 0.f;
-    if (i < jb.rows && j < jb.rp) {
-      val = jb.src[static_cast<long long>(i) * jb.rp + j];
-      jb.P32[static_cast<long long>(i) * jb.rp + j] = val;
-      jb.P16[static_cast<long long>(i) * jb.ldp + j] = working_bits(val, jb.p16_is_half != 0);
+  return lo;
+}
+
+__global__ void __launch_bounds__(256) basis_norms_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
+  const int j = end_job(tile_start, n_jobs);
+  const WorkingJob jb = jobs[j];
+  const int r0 = (static_cast<int>(blockIdx.x) - tile_start[j]) * kEndRows, r1 = min(r0 + kEndRows, jb.rows);
+  const int quads = jb.rp >> 2;
+  // thread: a column quad (there are at most 219) and every `groups`-th row
+  __shared__ double part[256][4];
+  const int groups = 256 / quads, g = threadIdx.x / quads, q = threadIdx.x % quads;
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  if (g < groups) {
+#pragma unroll 4
+    for (int r = r0 + g; r < r1; r += groups) {
+      const float4 x = *reinterpret_cast<const float4*>(jb.src + static_cast<long long>(r) * jb.rp + 4 * q);
+      s0 += static_cast<double>(x.x) * x.x; s1 += static_cast<double>(x.y) * x.y;
+      s2 += static_cast<double>(x.z) * x.z; s3 += static_cast<double>(x.w) * x.w;
     }
-    tile[a][threadIdx.x] = val;
+  }
+  part[threadIdx.x][0] = s0; part[threadIdx.x][1] = s1; part[threadIdx.x][2] = s2; part[threadIdx.x][3] = s3;
+  __syncthreads();
+  for (int c = threadIdx.x; c < jb.rp; c += 256) {
+    double t = 0.0;
+    for (int x = 0; x < groups; ++x) t += part[x * quads + (c >> 2)][c & 3];
+    atomicAdd(jb.sums + c, t);
+  }
+}
+
+__global__ void __launch_bounds__(256) working_copies_grouped_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
+  __shared__ uint16_t tile[kEndCols][kEndRows + 4];
+  const int j = end_job(tile_start, n_jobs);
+  const WorkingJob jb = jobs[j];
+  const int t = static_cast<int>(blockIdx.x) - tile_start[j];
+  const int i0 = (t / jb.tiles_x) * kEndRows, j0 = (t % jb.tiles_x) * kEndCols;
+  bool bad = false, any = false;
+  for (int c = threadIdx.x; c < jb.rp; c += 256) {
+    const double v = jb.sums[c];
+    bad = bad || !isfinite(v);
+    any = any || v > 0.0;
+  }
+  const bool nonfinite = __syncthreads_or(bad ? 1 : 0) != 0;
+  const bool repair = nonfinite || __syncthreads_or(any ? 1 : 0) == 0;
+  if (nonfinite && t == 0 && threadIdx.x == 0) atomicCAS(jb.status, 0, 7 /* NGALORE_ERR_NONFINITE */);
+  const int q = threadIdx.x & 15, c = j0 + 4 * q;
+  float f[4] = {0.f, 0.f, 0.f, 0.f};
+  if (c < jb.rp) {
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const double v = jb.sums[c + y];
+      f[y] = v > 0.0 ? static_cast<float>(1.0 / sqrt(v)) : 0.f;
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < kEndRows / 16; ++p) {
+    const int a = (threadIdx.x >> 4) + 16 * p, i = i0 + a;
+    if (i >= jb.rows || c >= jb.rp) continue;
+    const float4 x = *reinterpret_cast<const float4*>(jb.src + static_cast<long long>(i) * jb.rp + c);
+    float v[4] = {x.x * f[0], x.y * f[1], x.z * f[2], x.w * f[3]};
+    if (repair) {
+#pragma unroll
+      for (int y = 0; y < 4; ++y) v[y] = i == c + y ? 1.f : 0.f;
+    }
+    *reinterpret_cast<float4*>(jb.P32 + static_cast<long long>(i) * jb.rp + c) = make_float4(v[0], v[1], v[2], v[3]);
+    uint2 w;
+    w.x = working_bits(v[0], jb.p16_is_half != 0) | (static_cast<uint32_t>(working_bits(v[1], jb.p16_is_half != 0)) << 16);
+    w.y = working_bits(v[2], jb.p16_is_half != 0) | (static_cast<uint32_t>(working_bits(v[3], jb.p16_is_half != 0)) << 16);
+    *reinterpret_cast<uint2*>(jb.P16 + static_cast<long long>(i) * jb.ldp + c) = w;
+#pragma unroll
+    for (int y = 0; y < 4; ++y) tile[4 * q + y][a] = working_bits(v[y], jb.p16_is_half == 0);
   }
   __syncthreads();
-  for (int a = threadIdx.y; a < 32; a += blockDim.y) {
-    const int j = j0 + a, i = i0 + threadIdx.x;
-    if (i < jb.rows && j < jb.rp) jb.Pt16[static_cast<long long>(j) * jb.ldpt + i] = working_bits(tile[threadIdx.x][a], jb.p16_is_half == 0);
+  // the transposed copy: a warp writes 128 rows of a column, four a lane
+  const int lane = threadIdx.x & 31, i = i0 + 4 * lane;
+  for (int y = threadIdx.x >> 5; y < kEndCols; y += 8) {
+    if (j0 + y >= jb.rp || i >= jb.rows) continue;
+    uint16_t* dst = jb.Pt16 + static_cast<long long>(j0 + y) * jb.ldpt + i;
+    if (i + 3 < jb.rows) {
+      *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(&tile[y][4 * lane]);
+    } else {
+      for (int x = 0; x < 4 && i + x < jb.rows; ++x) dst[x] = tile[y][4 * lane + x];
+    }
   }
 }
 

@@ -95,15 +95,13 @@ struct ngalore_state {
   FusedPlan fused;
   // tensor-core refresh plan
   RefreshPlan refresh;
-  // check and repair of a refreshed basis (finish_refresh): one job per matrix, and the jobs of refresh_tc_idx again
-  // in that order
+  // check and repair of a basis refreshed on the plain path (finish_refresh): one job per matrix
   BasisJob* d_bjobs = nullptr;
-  BasisJob* d_bjobs_tc = nullptr;
   double* d_bacc = nullptr;
-  // working copies of the projectors of refresh_tc_idx in one launch (finish_refresh)
+  // column norms and working copies of the projectors of refresh_tc_idx (finish_refresh)
   WorkingJob* d_wjobs = nullptr;
-  int* d_wtile_start = nullptr;
-  int n_wjobs = 0, n_wtiles = 0;
+  int *d_ntile_start = nullptr, *d_wtile_start = nullptr;
+  int n_wjobs = 0, n_ntiles = 0, n_wtiles = 0;
   // small-rank path (every r' <= 8): the step as two bandwidth kernels
   SrPlan sr;
   // host-buffer staging; W travels in groups of matrices so that the copies in, the back-projection and the
@@ -251,32 +249,25 @@ ngalore_status apply_gradient(ngalore_state* st, const std::vector<int>& idx, co
 }
 
 // whole_set: this call completes a refresh of every matrix (even when idx lists only part of them).
-// tc_set: idx is the whole list of matrices refreshed on the tensor-core path (ngalore_state::refresh_tc_idx), for
-// which the copies of all projectors are one prepared launch.
+// tc_set: idx is the whole list of matrices refreshed on the tensor-core path (ngalore_state::refresh_tc_idx), whose
+// bases sit in Ya: norms and copies of all projectors are two prepared launches.
 ngalore_status finish_refresh(ngalore_state* st, const std::vector<int>& idx, bool basis_in_a, cudaStream_t stream,
                               bool whole_set, bool tc_set = false) {
   ngalore_status rc;
   // a basis of zeros (zero gradient) or with entries that are not finite becomes the first r' unit vectors
-  NG_CUDA(cudaMemsetAsync(st->d_bacc, 0, sizeof(double) * 2 * st->n, stream));
   if (tc_set) {
-    const dim3 grid(32, static_cast<unsigned>(idx.size()));
-    basis_check_kernel<<<grid, 256, 0, stream>>>(st->d_bjobs_tc, basis_in_a ? 1 : 0);
-    basis_repair_kernel<<<grid, 256, 0, stream>>>(st->d_bjobs_tc, basis_in_a ? 1 : 0);
+    basis_norms_kernel<<<st->n_ntiles, 256, 0, stream>>>(st->d_wjobs, st->d_ntile_start, st->n_wjobs);
+    working_copies_grouped_kernel<<<st->n_wtiles, 256, 0, stream>>>(st->d_wjobs, st->d_wtile_start, st->n_wjobs);
     st->launches += 2;
+    NG_CUDA(cudaGetLastError());
   } else {
+    NG_CUDA(cudaMemsetAsync(st->d_bacc, 0, sizeof(double) * 2 * st->n, stream));
     for (int i : idx) {
       basis_check_kernel<<<dim3(32, 1), 256, 0, stream>>>(st->d_bjobs + i, basis_in_a ? 1 : 0);
       basis_repair_kernel<<<dim3(32, 1), 256, 0, stream>>>(st->d_bjobs + i, basis_in_a ? 1 : 0);
       st->launches += 2;
     }
-  }
-  NG_CUDA(cudaGetLastError());
-  if (tc_set && basis_in_a && st->n_wjobs > 0) {
-    // the whole tensor-core set: master and working copies of every projector in one launch
-    working_copies_grouped_kernel<<<st->n_wtiles, dim3(32, 8), 0, stream>>>(st->d_wjobs, st->d_wtile_start, st->n_wjobs);
-    st->launches += 1;
     NG_CUDA(cudaGetLastError());
-  } else {
     for (int i : idx) {
       const HostMat& hm = st->mats[i];
       NG_CUDA(cudaMemcpyAsync(st->h_desc[i].P32, basis_in_a ? hm.Ya : hm.Yb, sizeof(float) * hm.eM * hm.rp,
@@ -837,38 +828,40 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
       rc = refresh_plan_create(st->refresh, eff, Yf, Zf, prop.multiProcessorCount, ritz_columns(st));
       if (rc != NGALORE_OK) return fail(rc);
       std::vector<WorkingJob> jobs;
-      std::vector<int> start(1, 0);
-      for (int i : st->refresh_tc_idx) {
+      std::vector<int> start(1, 0), nstart(1, 0);
+      for (size_t k = 0; k < st->refresh_tc_idx.size(); ++k) {
+        const int i = st->refresh_tc_idx[k];
         const HostMat& hm = st->mats[i];
         const MatDesc& d = st->h_desc[i];
-        const int tx = (hm.rp + 31) / 32, ty = (hm.eM + 31) / 32;
-        jobs.push_back(WorkingJob{hm.Ya, d.P32, d.P16, d.Pt16, hm.eM, hm.rp, d.ldp, d.ldpt, hm.right ? 0 : 1, tx});
+        const int tx = (hm.rp + kEndCols - 1) / kEndCols, ty = (hm.eM + kEndRows - 1) / kEndRows;
+        jobs.push_back(WorkingJob{hm.Ya, st->refresh.mats[k].D, d.P32, d.P16, d.Pt16, st->d_status + i, hm.eM, hm.rp, d.ldp, d.ldpt,
+                                  hm.right ? 0 : 1, tx});
         start.push_back(start.back() + tx * ty);
+        nstart.push_back(nstart.back() + ty);
       }
       st->n_wjobs = static_cast<int>(jobs.size());
       st->n_wtiles = start.back();
+      st->n_ntiles = nstart.back();
       if (cudaMalloc(&st->d_wjobs, sizeof(WorkingJob) * jobs.size()) != cudaSuccess ||
+          cudaMalloc(&st->d_ntile_start, sizeof(int) * nstart.size()) != cudaSuccess ||
           cudaMalloc(&st->d_wtile_start, sizeof(int) * start.size()) != cudaSuccess)
         return fail(NGALORE_ERR_ALLOC);
       if (cudaMemcpy(st->d_wjobs, jobs.data(), sizeof(WorkingJob) * jobs.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(st->d_ntile_start, nstart.data(), sizeof(int) * nstart.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
           cudaMemcpy(st->d_wtile_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(NGALORE_ERR_CUDA);
     }
   }
   {
     if (cudaMalloc(&st->d_bacc, sizeof(double) * 2 * n_matrices) != cudaSuccess ||
-        cudaMalloc(&st->d_bjobs, sizeof(BasisJob) * n_matrices) != cudaSuccess ||
-        cudaMalloc(&st->d_bjobs_tc, sizeof(BasisJob) * (st->refresh_tc_idx.size() + 1)) != cudaSuccess)
+        cudaMalloc(&st->d_bjobs, sizeof(BasisJob) * n_matrices) != cudaSuccess)
       return fail(NGALORE_ERR_ALLOC);
-    std::vector<BasisJob> jobs(n_matrices), jobs_tc;
+    std::vector<BasisJob> jobs(n_matrices);
     for (int i = 0; i < n_matrices; ++i) {
       const HostMat& hm = st->mats[i];
       jobs[i] = BasisJob{hm.Ya, hm.Yb, st->d_bacc + 2 * i, st->d_status + i, hm.eM, hm.rp};
     }
-    for (int i : st->refresh_tc_idx) jobs_tc.push_back(jobs[i]);
-    if (cudaMemcpy(st->d_bjobs, jobs.data(), sizeof(BasisJob) * jobs.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        (!jobs_tc.empty() && cudaMemcpy(st->d_bjobs_tc, jobs_tc.data(), sizeof(BasisJob) * jobs_tc.size(),
-                                        cudaMemcpyHostToDevice) != cudaSuccess))
+    if (cudaMemcpy(st->d_bjobs, jobs.data(), sizeof(BasisJob) * jobs.size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(NGALORE_ERR_CUDA);
   }
   for (int e = 0; e < 4; ++e)
@@ -899,9 +892,9 @@ void ngalore_destroy(ngalore_state* st) {
   if (st->stage) cudaFree(st->stage);
   if (st->work) cudaFree(st->work);
   if (st->d_bjobs) cudaFree(st->d_bjobs);
-  if (st->d_bjobs_tc) cudaFree(st->d_bjobs_tc);
   if (st->d_bacc) cudaFree(st->d_bacc);
   if (st->d_wjobs) cudaFree(st->d_wjobs);
+  if (st->d_ntile_start) cudaFree(st->d_ntile_start);
   if (st->d_wtile_start) cudaFree(st->d_wtile_start);
   if (st->arena) cudaFree(st->arena);
   delete st;

@@ -201,53 +201,6 @@ __global__ void __launch_bounds__(256) newton_prep_kernel(const NewtonJob* jobs)
   }
 }
 
-// Scale every column of Y (rows x L, fp32) to unit norm, the norm summed in fp64.  The products of the refresh go
-// through operands split in two bf16 parts; the rounding of the diagonal of a triangular factor or of a rotation
-// (a relative 2^-17) scales a whole column, which is the largest part of what the last product leaves of
-// non-orthonormality.  Two kernels: partial sums of squares per strip of 32 columns and chunk of rows (added to
-// `sums` with fp64 atomics; `sums` is cleared beforehand), then the scaling.  Block (32, 8): blockIdx.x = strip of
-// 32 columns, blockIdx.y = matrix, blockIdx.z = chunk of kNormRows rows.
-struct NormJob {
-  float* Y;
-  double* sums;   // L sums of squares
-  int rows, L;
-};
-constexpr int kNormRows = 1024;
-
-__global__ void __launch_bounds__(256) column_sumsq_kernel(const NormJob* jobs) {
-  __shared__ double part[8][33];
-  const NormJob jb = jobs[blockIdx.y];
-  const int col = blockIdx.x * 32 + threadIdx.x;
-  const int r0 = blockIdx.z * kNormRows;
-  if (blockIdx.x * 32 >= jb.L || r0 >= jb.rows) return;
-  const int r1 = min(jb.rows, r0 + kNormRows);
-  double s = 0.0;
-  if (col < jb.L)
-    for (int r = r0 + threadIdx.y; r < r1; r += 8) {
-      const double v = static_cast<double>(jb.Y[static_cast<long long>(r) * jb.L + col]);
-      s += v * v;
-    }
-  part[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && col < jb.L) {
-    double t = 0.0;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) t += part[g][threadIdx.x];
-    atomicAdd(jb.sums + col, t);
-  }
-}
-
-__global__ void __launch_bounds__(256) column_scale_kernel(const NormJob* jobs) {
-  const NormJob jb = jobs[blockIdx.y];
-  const int col = blockIdx.x * 32 + threadIdx.x;
-  const int r0 = blockIdx.z * kNormRows;
-  if (col >= jb.L || r0 >= jb.rows) return;
-  const int r1 = min(jb.rows, r0 + kNormRows);
-  const double t = jb.sums[col];
-  const float f = t > 0.0 ? static_cast<float>(1.0 / sqrt(t)) : 0.f;
-  for (int r = r0 + threadIdx.y; r < r1; r += 8) jb.Y[static_cast<long long>(r) * jb.L + col] *= f;
-}
-
 // ------------------------------------------------------------------------------------------ plan
 
 // RG_APPLY_TRI: RG_APPLY_Y with an upper triangular right operand (its blocks of zeros are left out)
@@ -268,7 +221,7 @@ struct RefreshMat {
   __nv_bfloat16 *Y1hi, *Y1lo;           // Y in set 1 (the memory of Yf, M x ldl floats)
   float* C32;                           // L x L
   double *C64, *X64, *T64;              // L x L each
-  double* D;                            // L
+  double* D;                            // L column norms (sums of squares) of the result
   __nv_bfloat16 *Rhi, *Rlo;             // L x ldl
 };
 
@@ -319,10 +272,8 @@ struct RefreshPlan {
   CholProblem* d_eig_chol = nullptr;
   int eig_max = 0;             // largest matrix it diagonalises
   int sm_count = 0;
-  NormJob* d_norm = nullptr;
   FillJob* d_fill = nullptr;   // the random start Z = Omega of every matrix
   ZeroJob* d_zero_d = nullptr;   // clears every matrix's D (as 16-byte words)
-  int m_max = 0;                 // most rows among the matrices
 };
 
 inline void refresh_plan_destroy(RefreshPlan& plan) {
@@ -457,7 +408,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_eig = take(sizeof(EigMat) * n);
   const size_t o_eig_chol = take(sizeof(CholProblem) * n);
   const size_t o_eig_redo = take(sizeof(int) * n);
-  const size_t o_norm = take(sizeof(NormJob) * n);
   const size_t o_fill = take(sizeof(FillJob) * n);
   const size_t o_zero_d = take(sizeof(ZeroJob) * n);
   std::vector<size_t> o_eig_tri(n);
@@ -474,7 +424,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   std::vector<SyrkMat> syrk_m(n);
   std::vector<EigMat> eig(n);
   std::vector<CholProblem> eig_chol(n);
-  std::vector<NormJob> norm(n);
   plan.h_maps.resize(static_cast<size_t>(RM_COUNT) * n);
   std::memset(plan.h_maps.data(), 0, sizeof(CUtensorMap) * plan.h_maps.size());
   for (int i = 0; i < n; ++i) {
@@ -507,7 +456,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
                     redo, nullptr, 0, m.Rhi, m.Rlo, m.ldl, m.L};
     eig_chol[i] = CholProblem{m.C64, Lj, 0, 0.0, redo};
     plan.eig_max = std::max(plan.eig_max, Lj);
-    norm[i] = NormJob{m.Yf, m.D, m.M, m.L};   // the column-norm buffer of the orthonormalisations is free by then
     CUtensorMap* mp = &plan.h_maps[static_cast<size_t>(i) * RM_COUNT];
     const uint64_t sl = static_cast<uint64_t>(m.ldl) * 2;
     bool ok = true;
@@ -570,7 +518,6 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.d_eig = reinterpret_cast<EigMat*>(plan.buf + o_eig);
   plan.d_eig_chol = reinterpret_cast<CholProblem*>(plan.buf + o_eig_chol);
   std::stable_sort(eig_chol.begin(), eig_chol.end(), [](const CholProblem& a, const CholProblem& b) { return a.L > b.L; });
-  plan.d_norm = reinterpret_cast<NormJob*>(plan.buf + o_norm);
   plan.d_fill = reinterpret_cast<FillJob*>(plan.buf + o_fill);
   {
     std::vector<FillJob> fill(n);
@@ -583,10 +530,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.d_zero_d = reinterpret_cast<ZeroJob*>(plan.buf + o_zero_d);
   {
     std::vector<ZeroJob> zd(n);
-    for (int i = 0; i < n; ++i) {
+    for (int i = 0; i < n; ++i)
       zd[i] = ZeroJob{reinterpret_cast<float4*>(plan.mats[i].D), static_cast<long long>(plan.mats[i].L) * 8 / 16};  // L is a multiple of 4
-      plan.m_max = std::max(plan.m_max, plan.mats[i].M);
-    }
     if (cudaMemcpy(plan.d_zero_d, zd.data(), sizeof(ZeroJob) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
   }
   if (cudaMemcpy(plan.d_newton, newton.data(), sizeof(NewtonJob) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -597,8 +542,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_split_y_rest, sy_rest.data(), sizeof(SplitJob) * sy_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_z_rest, sz_rest.data(), sizeof(SplitJob) * sz_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_eig, eig.data(), sizeof(EigMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_norm, norm.data(), sizeof(NormJob) * n, cudaMemcpyHostToDevice) != cudaSuccess)
+      cudaMemcpy(plan.d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
 
   // ---- tables of buffers to clear
@@ -815,12 +759,10 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   if (eig_batched_launch(plan.d_eig, plan.d_eig_chol, plan.n, plan.eig_max, plan.l_max, plan.sm_count, stream, launches) != cudaSuccess)
     return NGALORE_ERR_CUDA;
   // Q orthonormal to about 1e-6 and V orthogonal: so is their product, once its columns are scaled back to unit norm
+  // (with the working copies, see finish_refresh; their norms go to D)
   if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, RP_APPLY_0F, d_ctrl, stream, launches))) return rc;
   zero_jobs_kernel<<<dim3(1, plan.n), 256, 0, stream>>>(plan.d_zero_d);
-  const dim3 norm_grid((plan.l_max + 31) / 32, plan.n, (plan.m_max + kNormRows - 1) / kNormRows);
-  column_sumsq_kernel<<<norm_grid, dim3(32, 8), 0, stream>>>(plan.d_norm);
-  column_scale_kernel<<<norm_grid, dim3(32, 8), 0, stream>>>(plan.d_norm);
-  *launches += 3;
+  *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
