@@ -36,7 +36,7 @@ struct P2Smem {
 static_assert(P2Smem::kTotal <= 232448, "shared memory budget of one CTA");
 
 __global__ void __launch_bounds__(kP2Threads, 1)
-tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__ tiles, int n_tiles,
+tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__ tiles, const int* __restrict__ cta_first,
                    const MatDesc* __restrict__ mats, Ctrl* ctrl) {
   using L = P2Smem;
   extern __shared__ unsigned char tc_smem_raw[];
@@ -67,7 +67,7 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int stride = gridDim.x;
+  const int t_begin = cta_first[blockIdx.x], t_end = cta_first[blockIdx.x + 1];   // this CTA's tiles
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -75,7 +75,7 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += stride) {
+      for (int t = t_begin; t < t_end && ok; ++t) {
         const TcTile tile = tiles[t];
         const CUtensorMap* mapA = tmaps + tile.mat * kTcMapsPerMat + TC_MAP_A_PROJ;
         const CUtensorMap* mapB = tmaps + tile.mat * kTcMapsPerMat + TC_MAP_B_PROJ;
@@ -105,7 +105,7 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += stride, ++local) {
+      for (int t = t_begin; t < t_end && ok; ++t, ++local) {
         const TcTile tile = tiles[t];
         const int halves = (tile.rows - tile.m0 > kTcBM) ? 2 : 1;
         const int n_rem = tile.cols - tile.n0;
@@ -140,7 +140,7 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
     float* stg = reinterpret_cast<float*>(smem + L::kEpiOffset + (warp - 2) * L::kEpiWarpBytes);
     const int sub_row = lane >> 3, sub_q = lane & 7;
     int local = 0;
-    for (int t = blockIdx.x; t < n_tiles; t += stride, ++local) {
+    for (int t = t_begin; t < t_end; ++t, ++local) {
       const TcTile tile = tiles[t];
       const MatDesc& d = mats[tile.mat];
       float* out = current_gradient(d, ring_cur(ctrl, d.s));
@@ -235,12 +235,12 @@ inline ngalore_status tc_project(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ct
   }
   if (plan.tall_proj) {
     tc_project2_kernel<<<plan.grid_proj, kP2Threads, P2Smem::kTotal, stream>>>(plan.d_maps, plan.d_tiles_proj,
-                                                                              plan.n_tiles_proj, d_mats, d_ctrl);
+                                                                              plan.d_proj_first, d_mats, d_ctrl);
   } else {
     using LP = TcSmem<kProjBN, 1, 1, kProjStages, kProjEpiWarps>;
     tc_gemm_kernel<kProjBN, 1, 1, kProjStages, TC_EPI_PROJECT, kProjEpiWarps, false>
         <<<plan.grid_proj, 64 + 32 * kProjEpiWarps, LP::kTotal, stream>>>(plan.d_maps, plan.d_tiles_proj,
-                                                                          plan.n_tiles_proj, d_mats, d_ctrl, nullptr);
+                                                                          plan.d_proj_first, d_mats, d_ctrl, nullptr);
   }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;

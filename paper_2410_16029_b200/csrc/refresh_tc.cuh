@@ -247,6 +247,7 @@ struct RefreshPlan {
   CUtensorMap* d_maps = nullptr;
   TcProblem* d_probs[RP_COUNT] = {};
   TcTile* d_tiles[RG_COUNT] = {};
+  int* d_first[RG_COUNT] = {};   // first tile of every CTA
   int n_tiles[RG_COUNT] = {};
   int grid[RG_COUNT] = {};
   bool wide = false;           // the products with G take tiles of kRefWideBN columns
@@ -314,7 +315,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   auto tile_cols = [&](int g) { return plan.wide && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? kRefWideBN : kRefBN; };
   auto add_tiles = [&](int g, int i, int out_rows, int out_cols, int K, long long target_kb) {
     const int kb_total = (K + kTcBK - 1) / kTcBK;
-    int splits = static_cast<int>((kb_total + target_kb - 1) / target_kb);
+    // (to the nearest number: a K a little over the target costs less balance than two tiles cost atomics)
+    int splits = static_cast<int>((kb_total + target_kb / 2) / target_kb);
     if (splits < 1) splits = 1;
     const int kb_per = (kb_total + splits - 1) / splits;
     splits = (kb_total + kb_per - 1) / kb_per;
@@ -352,7 +354,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     offs[i].Rlo = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
   }
   const size_t o_maps = take(sizeof(CUtensorMap) * RM_COUNT * n);
-  size_t o_probs[RP_COUNT], o_tiles[RG_COUNT];
+  size_t o_probs[RP_COUNT], o_tiles[RG_COUNT], o_first[RG_COUNT];
+  std::vector<int> tile_first[RG_COUNT];
   for (int g = 0; g < RP_COUNT; ++g) o_probs[g] = take(sizeof(TcProblem) * n);
 
   // work estimate for the split-K targets: per GEMM kind, k-blocks per CTA if perfectly balanced
@@ -385,10 +388,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       }
       add_tiles(g, i, rows, cols, K, target);
     }
-    std::stable_sort(tiles[g].begin(), tiles[g].end(), [](const TcTile& a, const TcTile& b) { return a.kblocks > b.kblocks; });
     o_tiles[g] = take(sizeof(TcTile) * tiles[g].size());
     plan.n_tiles[g] = static_cast<int>(tiles[g].size());
     plan.grid[g] = std::min(plan.n_tiles[g], sm_count);
+    tc_assign_tiles(tiles[g], plan.grid[g], tile_first[g]);
+    o_first[g] = take(sizeof(int) * tile_first[g].size());
   }
   const size_t o_newton = take(sizeof(NewtonJob) * n);
   const size_t o_factor32 = take(sizeof(FactorMat) * n);
@@ -500,7 +504,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   }
   for (int g = 0; g < RG_COUNT; ++g) {
     plan.d_tiles[g] = reinterpret_cast<TcTile*>(plan.buf + o_tiles[g]);
-    if (cudaMemcpy(plan.d_tiles[g], tiles[g].data(), sizeof(TcTile) * tiles[g].size(), cudaMemcpyHostToDevice) != cudaSuccess)
+    plan.d_first[g] = reinterpret_cast<int*>(plan.buf + o_first[g]);
+    if (cudaMemcpy(plan.d_first[g], tile_first[g].data(), sizeof(int) * tile_first[g].size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(plan.d_tiles[g], tiles[g].data(), sizeof(TcTile) * tiles[g].size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return NGALORE_ERR_CUDA;
   }
   plan.d_newton = reinterpret_cast<NewtonJob*>(plan.buf + o_newton);
@@ -629,17 +635,17 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     if (plan.wide) {
       if (high_only)
         tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       else
         tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
     } else {
       if (high_only)
         tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 1, kRefStages0, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       else
         tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 2, kRefStages1, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
     }
   };
   switch (g) {
@@ -648,11 +654,11 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     case RG_GRAM_Y:
     case RG_GRAM_Z:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     default:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.n_tiles[g], nullptr, d_ctrl, plan.d_probs[problem]);
+          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
   }
   *launches += 1;
