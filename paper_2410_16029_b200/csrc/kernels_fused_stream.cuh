@@ -3,12 +3,13 @@
 //
 // Structure: one CTA per SM; a producer warp streams the history (and m, v) through a ring of
 // shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight consumer
-// warps compute from shared memory.  The producer runs ahead of the consumers across tile and
+// warps compute from shared memory, a finishing warp turns the partial sums of a Gram tile into its partial row
+// and, after a matrix's last one, solves its s x s system while the consumers go on with the next item.  The producer runs ahead of the consumers across tile and
 // matrix boundaries, so the SM always has several stages of loads in flight.
 //
 // Work items (Gram tiles and combination tiles of all matrices) are fetched in order from a global
-// counter by the producer.  Gram items never wait; the CTA that finishes a matrix's last Gram tile
-// solves its s x s system and publishes the weights; the consumers of a combination item wait
+// counter by the producer.  Gram items never wait; the finishing warp of the CTA that has a matrix's last Gram
+// tile solves its s x s system and publishes the weights; the consumers of a combination item wait
 // (bounded) for that flag.  Every item a combination item depends on sits earlier in the list and
 // has been fetched by a CTA that consumes its items in order, so the kernel cannot deadlock.
 // All Gram items precede all combination items, so the wait is short except at the very end of the Gram items.
@@ -58,7 +59,7 @@ struct FusedCfg {
   // consumer threads: the bf16 history costs more instructions per byte (conversion, two Gram rows), so it gets
   // sixteen warps where the registers allow it
   static constexpr int kConsumers = (HIST16 && SMAX <= 16) ? 512 : 256;
-  static constexpr int kThreads = kConsumers + 32;
+  static constexpr int kThreads = kConsumers + 64;  // and the producer and the finishing warp
   static constexpr int kHistBytes = SMAX * CE * (HIST16 ? 2 : 4);
   static constexpr int kCurOff = kHistBytes;                          // HIST16: fp32 gradient of this step
   static constexpr int kMOff = kHistBytes + (HIST16 ? CE * 4 : 0);
@@ -67,10 +68,10 @@ struct FusedCfg {
   static constexpr int kStages = HIST16 ? (SMAX <= 8 ? 3 : (SMAX <= 16 ? 2 : 5)) : (SMAX <= 8 ? 5 : 3);
   static constexpr int kBase = kStages * kStageBytes;
   static constexpr int kFullOff = kBase, kEmptyOff = kBase + 64, kMetaOff = kBase + 128, kFlagOff = kBase + 512;
-  static constexpr int kWOff = kBase + 640, kRedOff = kBase + 768;
+  static constexpr int kWOff = kBase + 640, kRedBarOff = kBase + 768, kRedMetaOff = kBase + 800, kRedOff = kBase + 896;
+  static constexpr int kRows = HIST16 ? 2 : 1;                  // Gram rows per tile
   static constexpr int kRedDoubles = (kConsumers / 32) * SMAX;  // one Gram row per consumer warp
-  static constexpr int kAOff = kRedOff + (HIST16 ? 2 : 1) * kRedDoubles * 8;
-  static constexpr int kTotal = kAOff + kMaxHistory * (kMaxHistory + 1) * 8;
+  static constexpr int kTotal = kRedOff + 2 * kRows * kRedDoubles * 8;   // (two tiles in flight to the finishing warp)
   static_assert(kStages * sizeof(StageMeta) <= 384, "stage metadata overflows its slot");
   static_assert(kTotal <= 232448, "shared memory budget of one CTA exceeded");
 };
@@ -81,6 +82,36 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+// Sums of S values over the 32 lanes of a warp: afterwards lane l holds the sum of value l / (32 / S).  S - 1 exchanges
+// instead of the 5 S of one butterfly per value: each step halves the values a lane is responsible for.
+template <int S>
+__device__ __forceinline__ double warp_sums(double (&v)[S]) {
+  const int lane = threadIdx.x & 31;
+  int n = S, off = 16;
+#pragma unroll
+  for (int step = 0; step < 5; ++step, off >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool upper = (lane & off) != 0;
+#pragma unroll
+      for (int i = 0; i < S / 2; ++i) {
+        if (i < n) {
+          const double mine = upper ? v[i + n] : v[i], other = upper ? v[i] : v[i + n];
+          v[i] = mine + __shfl_xor_sync(0xffffffffu, other, off);
+        }
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    }
+  }
+  return v[0];
+}
+
+// What the finishing warp needs to know about a finished Gram tile (mat < 0: the CTA has no more).
+struct RedMeta {
+  int mat, local, cur, c;
+};
+
 template <int THREADS>
 __device__ __forceinline__ void consumer_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
@@ -106,7 +137,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   using C = FusedCfg<SMAX, HIST16, MOM16>;
   constexpr int CE = C::CE;
   constexpr int kConsumerThreads = C::kConsumers;
-  constexpr int kGroups = kConsumerThreads / 32;
+  constexpr int kWarps = kConsumerThreads / 32;
   constexpr int VEC = CE / kConsumerThreads;  // 4 or 2 elements per thread and stage
   static_assert(VEC == 2 || VEC == 4, "a thread handles two or four elements of a stage");
   extern __shared__ __align__(128) unsigned char fs_smem[];
@@ -116,9 +147,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   volatile int* abort_flag = reinterpret_cast<volatile int*>(fs_smem + C::kFlagOff);
   volatile int* s_flag = abort_flag + 1;
   float* wsm = reinterpret_cast<float*>(fs_smem + C::kWOff);
-  double* red = reinterpret_cast<double*>(fs_smem + C::kRedOff);
-  double* red2 = red + C::kRedDoubles;  // HIST16 only: the second Gram row
-  double* Amat = reinterpret_cast<double*>(fs_smem + C::kAOff);
+  uint64_t* red_full = reinterpret_cast<uint64_t*>(fs_smem + C::kRedBarOff);   // [2] all consumer warps have left their sums
+  uint64_t* red_empty = red_full + 2;                                           // [2] the finishing warp has taken them
+  RedMeta* red_meta = reinterpret_cast<RedMeta*>(fs_smem + C::kRedMetaOff);     // [2]
+  double* red = reinterpret_cast<double*>(fs_smem + C::kRedOff);                // [2][rows][warps][SMAX]
 
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -126,6 +158,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       mbar_init(full_bar + s, 1);
       mbar_init(empty_bar + s, kConsumerThreads / 32);
     }
+    for (int b = 0; b < 2; ++b) { mbar_init(red_full + b, kWarps); mbar_init(red_empty + b, 1); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -133,7 +166,62 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   __syncthreads();
   const int tag = ctrl->epoch + 1;
 
-  if (tid >= kConsumerThreads) {
+  if (tid >= kConsumerThreads + 32) {
+    // ------------------------------------------------------------------ finishing warp
+    const int lane = tid & 31;
+    const double lambda = hyper->lambda;
+    for (unsigned int n = 0;; ++n) {
+      const int buf = n & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(red_full + buf, (n >> 1) & 1u, abort_flag))) break;
+      const RedMeta mt = red_meta[buf];
+      double part[C::kRows];
+#pragma unroll
+      for (int r = 0; r < C::kRows; ++r) {
+        part[r] = 0.0;
+        if (lane < SMAX) {
+          const double* src = red + (buf * C::kRows + r) * C::kRedDoubles + lane;
+          double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+          for (int w = 0; w < kWarps; w += 2) { t0 += src[w * SMAX]; t1 += src[(w + 1) * SMAX]; }
+          part[r] = t0 + t1;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(red_empty + buf);
+      if (mt.mat < 0) break;
+      const MatDesc& d = mats[mt.mat];
+      const int cur = mt.cur, c = mt.c;
+      // per-tile partial rows: [tile][s] (fp32 history) or [tile][2][s] (HIST16: row of `cur`, row of `prev`)
+      if (d.ntiles > 1) {
+        int last = 0;
+        if (lane < d.s) {
+#pragma unroll
+          for (int r = 0; r < C::kRows; ++r) __stcg(d.gpart + (static_cast<long long>(mt.local) * C::kRows + r) * d.s + lane, part[r]);
+          __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(d.gram_done, 1) == d.ntiles - 1 ? 1 : 0;
+        if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+        __threadfence();
+      }
+      // the matrix's last tile
+      double a[SMAX];
+      solve_load<SMAX>(d, c, a);
+      if (d.ntiles > 1) {
+#pragma unroll
+        for (int r = 0; r < C::kRows; ++r) part[r] = gram_row_sum(d, lane, c, C::kRows, r);
+      }
+      const bool two = HIST16 && c >= 2;
+      solve_matrix<SMAX>(d, cur, c, lambda, a, lane < c ? part[0] : 0.0, two, two ? (cur == 0 ? d.s : cur) - 1 : 0, part[C::kRows - 1]);
+      __threadfence();
+      __syncwarp();
+      if (lane == 0) {
+        *d.gram_done = 0;
+        __threadfence();
+        if (ctrl->debug_withhold != mt.mat + 1) atomicExch(d.w_ready, tag);
+      }
+    }
+  } else if (tid >= kConsumerThreads) {
     // ------------------------------------------------------------------ producer warp
     // Lane 0 claims items and arms the barriers; every lane issues the bulk copy of "its" slot (lane j copies
     // history slot j, the next two lanes m and v), so a stage's copies are issued in parallel.
@@ -206,6 +294,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const Hyper hp = *hyper;
     int stage = 0;
     uint32_t phase = 0;
+    unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
     float acc[SMAX];
     float acc2[HIST16 ? SMAX : 1];  // HIST16: inner products with the slot that was current one step ago
     float w[SMAX];
@@ -222,7 +311,16 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     while (true) {
       if (!mbar_wait(full_bar + stage, phase, abort_flag)) break;
       const StageMeta mt = meta[stage];
-      if (mt.kind < 0) break;
+      if (mt.kind < 0) {
+        // no more items: tell the finishing warp
+        const int buf = tiles_done & 1;
+        if (mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) {
+          if (tid == 0) red_meta[buf].mat = -1;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(red_full + buf);
+        }
+        break;
+      }
       const MatDesc& d = mats[mt.mat];
       const int cur = mt.cur, c = mt.c;
       const unsigned char* sbytes = fs_smem + stage * C::kStageBytes;
@@ -297,79 +395,20 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         __syncwarp();
         if (lane == 0) mbar_arrive(empty_bar + stage);
         if (mt.last) {
+          const int buf = tiles_done & 1;
+          if (!mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
+          ++tiles_done;
 #pragma unroll
-          for (int j = 0; j < SMAX; ++j) {
-            const double t = warp_sum(static_cast<double>(acc[j]));
-            if (lane == 0) red[warp * SMAX + j] = t;
-            if (HIST16) {
-              const double t2 = warp_sum(static_cast<double>(acc2[HIST16 ? j : 0]));
-              if (lane == 0) red2[warp * SMAX + j] = t2;
-            }
-          }
-          consumer_sync<kConsumerThreads>();
-          // per-tile partial rows: [tile][s] (fp32 history) or [tile][2][s] (HIST16: row of `cur`, row of `prev`)
-          constexpr int kRows = HIST16 ? 2 : 1;
-          if (tid < kRows * 32 && (tid & 31) < SMAX && (tid & 31) < d.s) {
-            const int row = tid >> 5, j = tid & 31;
-            const double* src = row == 0 ? red : red2;
-            double t = 0.0;
+          for (int r = 0; r < C::kRows; ++r) {
+            double v[SMAX];
 #pragma unroll
-            for (int ww = 0; ww < kConsumerThreads / 32; ++ww) t += src[ww * SMAX + j];
-            d.gpart[(static_cast<long long>(mt.local) * kRows + row) * d.s + j] = t;
-            __threadfence();
+            for (int j = 0; j < SMAX; ++j) v[j] = static_cast<double>(r == 0 ? acc[j] : acc2[HIST16 ? j : 0]);
+            const double t = warp_sums<SMAX>(v);
+            if ((lane & (32 / SMAX - 1)) == 0) red[((buf * C::kRows + r) * kWarps + warp) * SMAX + lane / (32 / SMAX)] = t;
           }
-          consumer_sync<kConsumerThreads>();
-          if (tid == 0) {
-            const int done = atomicAdd(d.gram_done, 1);
-            *s_flag = (done == d.ntiles - 1) ? 1 : 0;
-          }
-          consumer_sync<kConsumerThreads>();
-          if (*s_flag) {
-            // last Gram tile of this matrix: all consumers pre-sum the per-tile partials (fixed partition,
-            // so the result is reproducible), then one warp factors and solves
-            __threadfence();
-            const int j = tid & 31, g = tid >> 5;
-            if (j < SMAX) {
-#pragma unroll
-              for (int row = 0; row < kRows; ++row) {
-                double t0 = 0.0, t1 = 0.0;
-                if (j < d.s) {
-                  const double* gp = d.gpart + static_cast<long long>(row) * d.s + j;
-                  const long long tstride = static_cast<long long>(kRows) * d.s;
-                  int t = g;
-                  for (; t + kGroups < d.ntiles; t += 2 * kGroups) {
-                    t0 += __ldcg(gp + t * tstride);
-                    t1 += __ldcg(gp + (t + kGroups) * tstride);
-                  }
-                  if (t < d.ntiles) t0 += __ldcg(gp + t * tstride);
-                }
-                (row == 0 ? red : red2)[g * SMAX + j] = t0 + t1;
-              }
-            }
-            consumer_sync<kConsumerThreads>();
-            if (tid < 32) {
-              if (two_rows) {
-                // row and column `prev` of Kraw against the stored (rounded) values; its entry with `cur`
-                // is written with the rest of row `cur` below, from the same products
-                double rowp = 0.0;
-                if (tid < c && tid != cur) {
-                  for (int gg = 0; gg < kConsumerThreads / 32; ++gg) rowp += red2[gg * SMAX + tid];
-                  if (isfinite(rowp)) {
-                    d.Kraw[prev * d.s + tid] = rowp;
-                    d.Kraw[tid * d.s + prev] = rowp;
-                  }
-                }
-                __syncwarp();
-              }
-              solve_matrix(d, cur, c, hp.lambda, Amat, red, kConsumerThreads / 32, SMAX);
-              if (tid == 0) {
-                *d.gram_done = 0;
-                __threadfence();
-                if (ctrl->debug_withhold != mt.mat + 1) atomicExch(d.w_ready, tag);
-              }
-            }
-          }
-          consumer_sync<kConsumerThreads>();
+          if (tid == 0) red_meta[buf] = RedMeta{mt.mat, mt.local, cur, c};
+          __syncwarp();
+          if (lane == 0) mbar_arrive(red_full + buf);
         }
       } else {
         if (mt.first) {

@@ -56,96 +56,104 @@ __device__ __forceinline__ void gram_tile(const MatDesc& d, int local, int cur, 
   __syncthreads();
 }
 
-// One warp: finish the Gram row from the per-tile partials (fixed order, so the result is
-// reproducible), form lambda I + K with K = Kraw / c, factor it (Cholesky, fp64) and solve for
+// Lane j's share of the Gram row: the sum over the matrix's tiles of partial product j (fixed order, so the result is
+// reproducible).  rows: partial rows per tile, row: which of them.
+__device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c, int rows = 1, int row = 0) {
+  double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
+  if (lane < c) {
+    const double* gp = d.gpart + static_cast<long long>(row) * d.s + lane;
+    const long long st = static_cast<long long>(rows) * d.s;
+    int t = 0;
+    for (; t + 7 < d.ntiles; t += 8) {
+      double x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = __ldcg(gp + (t + q) * st);
+      t0 += x[0] + x[4]; t1 += x[1] + x[5]; t2 += x[2] + x[6]; t3 += x[3] + x[7];
+    }
+    for (; t < d.ntiles; ++t) t0 += __ldcg(gp + t * st);
+  }
+  return (t0 + t1) + (t2 + t3);
+}
+
+// One warp: put the new Gram row (lane j: <H_cur, H_j>) into Kraw, form lambda I + K with K = Kraw / c and solve for
 // the weights w of N~ = sum_i w_i H_i, i.e. (lambda I + K) w = e_cur.  This is F^-1 applied to the
 // current gradient by the Woodbury identity, written for the case where the current gradient is a
 // column of the stacked matrix; it avoids the cancellation of the two-term form.
-// A is warp-private shared memory of kMaxHistory x (kMaxHistory + 1) doubles.
-// presum (optional, shared memory): groups x stride partial sums of the Gram row, already reduced over
-// disjoint subsets of the tiles by the caller.
-__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double* A,
-                                             const double* presum = nullptr, int groups = 0, int stride = 0) {
+// Lane i keeps row i of the matrix in registers; the elimination (Gauss-Jordan without pivoting: the matrix is
+// symmetric positive definite, its pivots are the squares of Cholesky's, and the same pivots tell when it is not)
+// broadcasts row k by shuffles, so the chain per step is one shuffle, one reciprocal and one multiply-add.  In shared
+// memory with serial substitutions the solve took 9 us for s = 8 and 25 us for s = 16; so 2 and 4 us.
+// have_prev: lane j also holds <H_prev, H_j> for the slot that was current one step ago (bf16 history).
+// The rows of Kraw are loaded by solve_load, which the caller may run ahead of its own sums.
+template <int SMAX>
+__device__ __forceinline__ void solve_load(const MatDesc& d, int c, double (&a)[SMAX]) {
   const int lane = threadIdx.x & 31;
-  constexpr int LD = kMaxHistory + 1;
-  bool finite = true;
-  // Gram row: lane j sums tile partials of column j.
-  if (d.s > 0) {
-    double row = 0.0;
-    if (lane < c) {
-      if (presum != nullptr) {
-        for (int g = 0; g < groups; ++g) row += presum[g * stride + lane];
-      } else {
-        for (int t = 0; t < d.ntiles; ++t) row += __ldcg(d.gpart + static_cast<long long>(t) * d.s + lane);
-      }
-      if (!isfinite(row)) finite = false;
+#pragma unroll
+  for (int j = 0; j < SMAX; ++j) a[j] = (lane < c && j < c) ? __ldcg(d.Kraw + lane * d.s + j) : 0.0;
+}
+
+template <int SMAX>
+__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double (&a)[SMAX], double row,
+                                             bool have_prev = false, int prev = 0, double rowp = 0.0) {
+  const int lane = threadIdx.x & 31;
+  if (have_prev) {
+    // row and column `prev` against the stored (rounded) values; the entry with `cur` follows below
+    const int use = lane < c && lane != cur && isfinite(rowp) ? 1 : 0;
+    if (use) {
+      d.Kraw[prev * d.s + lane] = rowp;
+      d.Kraw[lane * d.s + prev] = rowp;
     }
-    finite = __all_sync(0xffffffffu, finite);
-    if (lane < c) {
-      const double val = finite ? row : 0.0;
-      d.Kraw[cur * d.s + lane] = val;
-      d.Kraw[lane * d.s + cur] = val;
+#pragma unroll
+    for (int j = 0; j < SMAX; ++j) {
+      const double v = __shfl_sync(0xffffffffu, rowp, j);
+      const int uj = __shfl_sync(0xffffffffu, use, j);
+      if (lane == prev && uj) a[j] = v;
+      if (j == prev && use) a[j] = rowp;
     }
-    __syncwarp();
   }
+  const bool finite = __all_sync(0xffffffffu, lane >= c || isfinite(row));
   int bad = finite ? 0 : 7 /* NGALORE_ERR_NONFINITE */;
-  // A = lambda I + Kraw / c on the c valid slots.
-  for (int i = 0; i < c; ++i) {
-    if (lane < c) {
-      double a = d.s > 0 ? d.Kraw[i * d.s + lane] / static_cast<double>(c) : 0.0;
-      if (i == lane) a += lambda;
-      A[i * LD + lane] = a;
-    }
+  const double val = finite && lane < c ? row : 0.0;
+  if (lane < c) {
+    d.Kraw[cur * d.s + lane] = val;
+    d.Kraw[lane * d.s + cur] = val;
   }
-  __syncwarp();
-  // Cholesky, lower factor stored in place; lane = row.
-  for (int k = 0; k < c && bad == 0; ++k) {
-    const double dkk = A[k * LD + k];
-    if (!(dkk > 0.0) || !isfinite(dkk)) {
-      bad = isfinite(dkk) ? 6 /* NGALORE_ERR_NOT_SPD */ : 7;
+  const double ic = 1.0 / static_cast<double>(c);
+#pragma unroll
+  for (int j = 0; j < SMAX; ++j) {
+    const double v = __shfl_sync(0xffffffffu, val, j);
+    if (lane == cur) a[j] = v;
+    if (j == cur) a[j] = val;
+    a[j] *= ic;
+    if (j == lane) a[j] += lambda;
+  }
+  double b = lane == cur ? 1.0 : 0.0, diag = 1.0;
+#pragma unroll
+  for (int k = 0; k < SMAX; ++k) {
+    if (k >= c || bad != 0) break;
+    const double p = __shfl_sync(0xffffffffu, a[k], k);
+    if (!(p > 0.0) || !isfinite(p)) {
+      bad = isfinite(p) ? 6 /* NGALORE_ERR_NOT_SPD */ : 7;
       break;
     }
-    const double lkk = sqrt(dkk);
-    __syncwarp();
-    if (lane == k) A[k * LD + k] = lkk;
-    if (lane > k && lane < c) A[lane * LD + k] /= lkk;
-    __syncwarp();
-    if (lane > k && lane < c) {
-      const double lik = A[lane * LD + k];
-      for (int j = k + 1; j <= lane; ++j) A[lane * LD + j] -= lik * A[j * LD + k];
-    }
-    __syncwarp();
+    if (lane == k) diag = p;
+    const double f = lane == k ? 0.0 : a[k] * (1.0 / p);
+#pragma unroll
+    for (int j = k + 1; j < SMAX; ++j) a[j] -= f * __shfl_sync(0xffffffffu, a[j], k);
+    b -= f * __shfl_sync(0xffffffffu, b, k);
   }
-  // Forward and backward substitution (serial; c <= 32).
+  d.wsol[lane] = bad == 0 && lane < c ? static_cast<float>(b / diag) : 0.f;
+  if (bad != 0 && lane < d.s) {
+    // The poisoned slot becomes a zero gradient: its Gram row and column vanish.
+    d.Kraw[cur * d.s + lane] = 0.0;
+    d.Kraw[lane * d.s + cur] = 0.0;
+  }
   if (lane == 0) {
-    if (bad == 0) {
-      double t[kMaxHistory], w[kMaxHistory];
-      for (int i = 0; i < c; ++i) {
-        double acc = (i == cur) ? 1.0 : 0.0;
-        for (int j = 0; j < i; ++j) acc -= A[i * LD + j] * t[j];
-        t[i] = acc / A[i * LD + i];
-      }
-      for (int i = c - 1; i >= 0; --i) {
-        double acc = t[i];
-        for (int j = i + 1; j < c; ++j) acc -= A[j * LD + i] * w[j];
-        w[i] = acc / A[i * LD + i];
-      }
-      for (int i = 0; i < kMaxHistory; ++i) d.wsol[i] = i < c ? static_cast<float>(w[i]) : 0.f;
-      *d.step_bad = 0;
-    } else {
-      for (int i = 0; i < kMaxHistory; ++i) d.wsol[i] = 0.f;
-      *d.step_bad = 1;
-      atomicCAS(d.status, 0, bad);
-      // The poisoned slot becomes a zero gradient: its Gram row and column vanish.
-      for (int j = 0; j < d.s; ++j) {
-        d.Kraw[cur * d.s + j] = 0.0;
-        d.Kraw[j * d.s + cur] = 0.0;
-      }
-    }
+    *d.step_bad = bad != 0 ? 1 : 0;
+    if (bad != 0) atomicCAS(d.status, 0, bad);
   }
   __syncwarp();
 }
-
 
 // N~ = sum_j w_j H_j, then the Adam moments as printed in Sec. 2.2 (eps inside the root, no bias
 // correction), then u rounded to fp16 for the back-projection GEMM.
@@ -209,13 +217,15 @@ __global__ void __launch_bounds__(kStreamThreads) gram_kernel(const MatDesc* mat
 
 __global__ void __launch_bounds__(128) solve_kernel(const MatDesc* mats, int n_mats, const Ctrl* ctrl,
                                                     const Hyper* hyper) {
-  __shared__ double A[4][kMaxHistory * (kMaxHistory + 1)];
   const int warp = threadIdx.x >> 5;
   const int mat = blockIdx.x * 4 + warp;
   if (mat >= n_mats) return;
   const MatDesc& d = mats[mat];
   if (d.s == 0) return;
-  solve_matrix(d, ring_cur(ctrl, d.s), ring_count(ctrl, d.s), hyper->lambda, A[warp]);
+  const int c = ring_count(ctrl, d.s);
+  double a[kMaxHistory];
+  solve_load<kMaxHistory>(d, c, a);
+  solve_matrix<kMaxHistory>(d, ring_cur(ctrl, d.s), c, hyper->lambda, a, gram_row_sum(d, threadIdx.x & 31, c));
 }
 
 template <int SMAX>

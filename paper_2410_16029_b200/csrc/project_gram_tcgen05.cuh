@@ -339,7 +339,6 @@ __global__ void __launch_bounds__(256) pg_solve_kernel(const MatDesc* __restrict
                                                        const double* __restrict__ part, const int* __restrict__ list,
                                                        const Ctrl* __restrict__ ctrl, const Hyper* __restrict__ hyper) {
   __shared__ double red[8 * 32];
-  __shared__ double A[kMaxHistory * (kMaxHistory + 1)];
   const int mat = list[blockIdx.x];
   const MatDesc& d = mats[mat];
   const PgMat pm = pgm[mat];
@@ -358,11 +357,14 @@ __global__ void __launch_bounds__(256) pg_solve_kernel(const MatDesc* __restrict
   red[g * 32 + j] = t0 + t1;
   __syncthreads();
   if (threadIdx.x < 32) {
-    solve_matrix(d, ring_cur(ctrl, d.s), ring_count(ctrl, d.s), hyper->lambda, A, red, 8, 32);
-    if (threadIdx.x == 0) {
-      __threadfence();
-      atomicExch(d.w_ready, ctrl->epoch + 1);
-    }
+    const int c = ring_count(ctrl, d.s);
+    double a[kPgSMax], row = 0.0;
+    solve_load<kPgSMax>(d, c, a);
+    for (int q = 0; q < 8; ++q) row += red[q * 32 + threadIdx.x];
+    solve_matrix<kPgSMax>(d, ring_cur(ctrl, d.s), c, hyper->lambda, a, row);
+    __threadfence();
+    __syncwarp();
+    if (threadIdx.x == 0) atomicExch(d.w_ready, ctrl->epoch + 1);
   }
 }
 
