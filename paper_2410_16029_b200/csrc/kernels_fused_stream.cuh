@@ -224,69 +224,103 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   } else if (tid >= kConsumerThreads) {
     // ------------------------------------------------------------------ producer warp
     // Lane 0 claims items and arms the barriers; every lane issues the bulk copy of "its" slot (lane j copies
-    // history slot j, the next two lanes m and v), so a stage's copies are issued in parallel.
-    {
-      const int lane = tid & 31;
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      while (ok) {
-        int it = 0;
-        if (lane == 0) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= n_items) {
-          if (lane == 0 && mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag)) {
-            meta[stage].kind = -1;
-            mbar_arrive(full_bar + stage);
-          }
-          break;
-        }
-        const FusedItem item = items[it];
-        const MatDesc& d = mats[item.mat];
-        const int c = ring_count(ctrl, d.s);
-        const int cur_slot = ring_cur(ctrl, d.s);
-        const int ncopies = c + (item.kind == 1 ? 2 : 0);
-        const long long e0 = static_cast<long long>(item.local) * d.te;
-        const long long e1 = (e0 + d.te < d.rn) ? e0 + d.te : d.rn;
-        for (long long e = e0; e < e1; e += CE) {
-          const int cnt = (e1 - e < CE) ? static_cast<int>(e1 - e) : CE;
-          int good = 1;
-          if (lane == 0) good = mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag) ? 1 : 0;
-          good = __shfl_sync(0xffffffffu, good, 0);
-          if (!good) { ok = false; break; }
-          unsigned char* sb = fs_smem + stage * C::kStageBytes;
-          const uint32_t bytes = static_cast<uint32_t>(cnt) * 4u;
-          if (lane == 0) {
-            StageMeta mt;
-            mt.mat = item.mat; mt.kind = item.kind; mt.local = item.local;
-            mt.first = (e == e0) ? 1 : 0; mt.last = (e + CE >= e1) ? 1 : 0; mt.count = cnt; mt.e0 = e;
-            mt.cur = cur_slot; mt.c = c;
-            meta[stage] = mt;
-            const uint32_t hist_bytes = HIST16 ? bytes * static_cast<uint32_t>(c) - (bytes / 2) * static_cast<uint32_t>(c - 1)
-                                               : bytes * static_cast<uint32_t>(c);
-            const uint32_t mom_bytes = item.kind == 1 ? (MOM16 ? bytes : 2u * bytes) : 0u;
-            mbar_expect_tx(full_bar + stage, hist_bytes + mom_bytes);
-          }
-          __syncwarp();
-          for (int j = lane; j < ncopies; j += 32) {
-            if (j < c) {
-              if (!HIST16)
-                bulk_load(sb + j * CE * 4, d.H + static_cast<long long>(j) * d.rn + e, bytes, full_bar + stage);
-              else if (j == cur_slot)
-                bulk_load(sb + C::kCurOff, d.H + e, bytes, full_bar + stage);
-              else
-                bulk_load(sb + j * CE * 2, d.H16 + static_cast<long long>(j) * d.rn + e, bytes / 2, full_bar + stage);
-            } else {
-              const int k = j - c;  // 0: m, 1: v
-              if (MOM16)
-                bulk_load(sb + (k == 0 ? C::kMOff : C::kVOff), (k == 0 ? d.m16 : d.v16) + e, bytes / 2, full_bar + stage);
-              else
-                bulk_load(sb + (k == 0 ? C::kMOff : C::kVOff), (k == 0 ? d.m : d.v) + e, bytes, full_bar + stage);
-            }
-          }
-          if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
-        }
+    // history slot j, the next two lanes m and v), so a stage's copies are issued in parallel.  The next item is
+    // claimed and its descriptor fetched while the stages of the current one go out, one round trip to memory per
+    // stage: three round trips in a row between two items cost more than streaming 4096 elements of eight slots.
+    const int lane = tid & 31;
+    const int s_all = mats[0].s;                       // (the same for every matrix, and so are ring position and count)
+    const int c = ring_count(ctrl, s_all), cur_slot = ring_cur(ctrl, s_all);
+    struct Source {
+      int mat, kind, local;
+      long long e0, e1;
+      const unsigned char* src[2];                     // this lane's copies: number lane, and lane + 32 where there is one
+    };
+    // copy number k of an item: history slot k, then m and v; its place in a stage and bytes per element
+    auto place = [&](int k) {
+      if (k < c) return !HIST16 ? k * CE * 4 : (k == cur_slot ? C::kCurOff : k * CE * 2);
+      return k == c ? C::kMOff : C::kVOff;
+    };
+    auto width = [&](int k) { return k < c ? (HIST16 && k != cur_slot ? 2 : 4) : (MOM16 ? 2 : 4); };
+    auto describe = [&](const FusedItem& item, Source& o) {
+      const MatDesc& d = mats[item.mat];
+      o.mat = item.mat; o.kind = item.kind; o.local = item.local;
+      o.e0 = static_cast<long long>(item.local) * d.te;
+      o.e1 = (o.e0 + d.te < d.rn) ? o.e0 + d.te : d.rn;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int k = lane + 32 * q;
+        const void* base = nullptr;
+        if (k < c) base = !HIST16 ? static_cast<const void*>(d.H + static_cast<long long>(k) * d.rn)
+                                  : (k == cur_slot ? static_cast<const void*>(d.H) : static_cast<const void*>(d.H16 + static_cast<long long>(k) * d.rn));
+        else if (k == c) base = MOM16 ? static_cast<const void*>(d.m16) : static_cast<const void*>(d.m);
+        else if (k == c + 1) base = MOM16 ? static_cast<const void*>(d.v16) : static_cast<const void*>(d.v);
+        o.src[q] = static_cast<const unsigned char*>(base);
       }
+    };
+    int stage = 0;
+    uint32_t phase = 0;
+    int it = 0;
+    FusedItem item{};
+    Source now{}, next{};
+    if (lane == 0) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
+    it = __shfl_sync(0xffffffffu, it, 0);
+    if (it < n_items) { item = items[it]; describe(item, now); }
+    while (true) {
+      if (it >= n_items) {
+        if (lane == 0 && mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag)) {
+          meta[stage].kind = -1;
+          mbar_arrive(full_bar + stage);
+        }
+        break;
+      }
+      const int ncopies = c + (now.kind == 1 ? 2 : 0);
+      int step = 0;   // how far the next item is known: 0 claimed, 1 fetched, 2 described
+      auto look_ahead = [&]() {
+        if (step == 0) {
+          if (lane == 0) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
+        } else if (step == 1) {
+          it = __shfl_sync(0xffffffffu, it, 0);
+          if (it < n_items) item = items[it];
+        } else if (step == 2) {
+          if (it < n_items) describe(item, next);
+        }
+        ++step;
+      };
+      bool ok = true;
+      for (long long e = now.e0; e < now.e1; e += CE) {
+        const int cnt = (now.e1 - e < CE) ? static_cast<int>(now.e1 - e) : CE;
+        int good = 1;
+        if (lane == 0) good = mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag) ? 1 : 0;
+        good = __shfl_sync(0xffffffffu, good, 0);
+        if (!good) { ok = false; break; }
+        unsigned char* sb = fs_smem + stage * C::kStageBytes;
+        const uint32_t bytes = static_cast<uint32_t>(cnt) * 4u;
+        if (lane == 0) {
+          StageMeta mt;
+          mt.mat = now.mat; mt.kind = now.kind; mt.local = now.local;
+          mt.first = (e == now.e0) ? 1 : 0; mt.last = (e + CE >= now.e1) ? 1 : 0; mt.count = cnt; mt.e0 = e;
+          mt.cur = cur_slot; mt.c = c;
+          meta[stage] = mt;
+          const uint32_t hist_bytes = HIST16 ? bytes * static_cast<uint32_t>(c) - (bytes / 2) * static_cast<uint32_t>(c - 1)
+                                             : bytes * static_cast<uint32_t>(c);
+          const uint32_t mom_bytes = now.kind == 1 ? (MOM16 ? bytes : 2u * bytes) : 0u;
+          mbar_expect_tx(full_bar + stage, hist_bytes + mom_bytes);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int k = lane + 32 * q;
+          if (k < ncopies) {
+            const int w = width(k);
+            bulk_load(sb + place(k), now.src[q] + e * w, static_cast<uint32_t>(cnt * w), full_bar + stage);
+          }
+        }
+        if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+        look_ahead();
+      }
+      if (!ok) break;
+      while (step < 3) look_ahead();
+      now = next;
     }
   } else {
     // ------------------------------------------------------------------ consumers (8 or 16 warps)
