@@ -122,6 +122,20 @@ __device__ __forceinline__ uint32_t float_to_bf16_bits(float x) {
   return static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(x)));
 }
 
+// Two floats in a 64-bit register, and the packed multiply-add on them.
+__device__ __forceinline__ uint64_t pack_pair(float lo, float hi) {
+  uint64_t p;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(lo), "f"(hi));
+  return p;
+}
+__device__ __forceinline__ void unpack_pair(uint64_t p, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p)); }
+__device__ __forceinline__ uint64_t widen_pair(uint32_t bf16x2) { return pack_pair(__uint_as_float(bf16x2 << 16), __uint_as_float(bf16x2 & 0xFFFF0000u)); }
+__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
 // HIST16: the ring holds bf16 values; the gradient of the current step is read in fp32 from its own buffer
 // (MatDesc::H) and its bf16 rounding is written into ring slot `cur` by the combination pass.  The Gram pass
 // then also recomputes the row of the slot that was current one step ago, now that it is a rounded value, so
@@ -324,27 +338,62 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     }
   } else {
     // ------------------------------------------------------------------ consumers (8 or 16 warps)
+    // One loop over the stages of an item for either kind, so that the sums of a Gram tile and the weights of a
+    // combination tile do not both occupy registers.
     const int warp = tid >> 5, lane = tid & 31;
     const Hyper hp = *hyper;
+    const int idx = tid * VEC;     // this thread's elements of a stage
     int stage = 0;
     uint32_t phase = 0;
     unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
-    float acc[SMAX];
-    float acc2[HIST16 ? SMAX : 1];  // HIST16: inner products with the slot that was current one step ago
-    float w[SMAX];
+    if (HIST16) {
+      // the current slot's place in a stage stays zero for the whole launch: its gradient takes part in fp32 instead
+      const int cur = ring_cur(ctrl, mats[0].s);
+      for (int x = 0; x < C::kStages; ++x)
+        for (int i = tid; i < CE / 2; i += kConsumerThreads)
+          reinterpret_cast<uint32_t*>(fs_smem + x * C::kStageBytes + cur * CE * 2)[i] = 0u;
+      consumer_sync<kConsumerThreads>();
+    }
+    // hand the stage back and go on to the next one of the item
+    auto release = [&]() {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty_bar + stage);
+      if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+    };
+    // this thread's elements of fp32 slot j, of bf16 slot j (as pairs), of the fp32 gradient of the step, of a moment
+    auto load32 = [&](int j, float (&h)[VEC]) {
+      const float* q = reinterpret_cast<const float*>(fs_smem + stage * C::kStageBytes) + j * CE + idx;
 #pragma unroll
-    for (int j = 0; j < SMAX; ++j) { acc[j] = 0.f; w[j] = 0.f; }
+      for (int x = 0; x < VEC; ++x) h[x] = q[x];
+    };
+    auto load16 = [&](int j, uint64_t (&h)[VEC / 2]) {
+      const uint32_t* q = reinterpret_cast<const uint32_t*>(fs_smem + stage * C::kStageBytes + (j * CE + idx) * 2);
 #pragma unroll
-    for (int j = 0; j < (HIST16 ? SMAX : 1); ++j) acc2[j] = 0.f;
-    bool item_bad = false, item_ok = true;
-    // per-item pointers of the combination pass, fetched once at the item's first stage
-    float *it_m = nullptr, *it_v = nullptr, *it_cur = nullptr;
-    __half* it_u = nullptr;
-    uint16_t *it_h16 = nullptr, *it_m16 = nullptr, *it_v16 = nullptr;
-    unsigned int it_mat = 0, it_step = 0;
+      for (int x = 0; x < VEC / 2; ++x) h[x] = widen_pair(q[x]);
+    };
+    auto load_current = [&](float (&h)[VEC]) {
+      const float* q = reinterpret_cast<const float*>(fs_smem + stage * C::kStageBytes + C::kCurOff) + idx;
+#pragma unroll
+      for (int x = 0; x < VEC; ++x) h[x] = q[x];
+    };
+    auto load_moment = [&](int off, float (&h)[VEC]) {
+      if (!MOM16) {
+        const float* q = reinterpret_cast<const float*>(fs_smem + stage * C::kStageBytes + off) + idx;
+#pragma unroll
+        for (int x = 0; x < VEC; ++x) h[x] = q[x];
+      } else {
+        const uint32_t* q = reinterpret_cast<const uint32_t*>(fs_smem + stage * C::kStageBytes + off + idx * 2);
+#pragma unroll
+        for (int x = 0; x < VEC; x += 2) {
+          const uint32_t pair = q[x >> 1];
+          h[x] = bf16_bits_to_float(pair & 0xFFFFu);
+          h[x + 1] = bf16_bits_to_float(pair >> 16);
+        }
+      }
+    };
     while (true) {
       if (!mbar_wait(full_bar + stage, phase, abort_flag)) break;
-      const StageMeta mt = meta[stage];
+      StageMeta mt = meta[stage];
       if (mt.kind < 0) {
         // no more items: tell the finishing warp
         const int buf = tiles_done & 1;
@@ -355,207 +404,245 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         }
         break;
       }
-      const MatDesc& d = mats[mt.mat];
       const int cur = mt.cur, c = mt.c;
-      const unsigned char* sbytes = fs_smem + stage * C::kStageBytes;
-      const int idx = tid * VEC;
-      // this thread's VEC elements of history slot j in this stage
-      auto load_hist = [&](int j, float (&h)[VEC]) {
-        if (!HIST16) {
-          const float* p = reinterpret_cast<const float*>(sbytes) + j * CE + idx;
-#pragma unroll
-          for (int q = 0; q < VEC; ++q) h[q] = p[q];
-        } else if (j == cur) {
-          const float* p = reinterpret_cast<const float*>(sbytes + C::kCurOff) + idx;
-#pragma unroll
-          for (int q = 0; q < VEC; ++q) h[q] = p[q];
-        } else {
-          const uint32_t* p = reinterpret_cast<const uint32_t*>(sbytes + (j * CE + idx) * 2);
-#pragma unroll
-          for (int q = 0; q < VEC; q += 2) {
-            const uint32_t pair = p[q >> 1];
-            h[q] = bf16_bits_to_float(pair & 0xFFFFu);
-            h[q + 1] = bf16_bits_to_float(pair >> 16);
-          }
-        }
-      };
-      // this thread's VEC elements of a moment in this stage
-      auto load_moment = [&](int off, float (&x)[VEC]) {
-        if (!MOM16) {
-          const float* p = reinterpret_cast<const float*>(sbytes + off) + idx;
-#pragma unroll
-          for (int q = 0; q < VEC; ++q) x[q] = p[q];
-        } else {
-          const uint32_t* p = reinterpret_cast<const uint32_t*>(sbytes + off + idx * 2);
-#pragma unroll
-          for (int q = 0; q < VEC; q += 2) {
-            const uint32_t pair = p[q >> 1];
-            x[q] = bf16_bits_to_float(pair & 0xFFFFu);
-            x[q + 1] = bf16_bits_to_float(pair >> 16);
-          }
-        }
-      };
-      const bool two_rows = HIST16 && c >= 2;
-      const int prev = two_rows ? (cur == 0 ? d.s : cur) - 1 : 0;
+      bool alive = true;
       if (mt.kind == 0) {
-        if (mt.first) {
+        // ---- Gram tile
+        const int buf = tiles_done & 1;
+        // this warp's sums of row r over its lanes, into the buffer of the finishing warp
+        auto hand_over = [&](int r, double (&v)[SMAX]) {
+          const double t = warp_sums<SMAX>(v);
+          if ((lane & (32 / SMAX - 1)) == 0) red[((buf * C::kRows + r) * kWarps + warp) * SMAX + lane / (32 / SMAX)] = t;
+        };
+        if constexpr (!HIST16) {
+          float acc[SMAX];
 #pragma unroll
           for (int j = 0; j < SMAX; ++j) acc[j] = 0.f;
-#pragma unroll
-          for (int j = 0; j < (HIST16 ? SMAX : 1); ++j) acc2[j] = 0.f;
-        }
-        if (idx < mt.count) {
-          float x[VEC], xp[VEC];
-          load_hist(cur, x);
-          if (two_rows) load_hist(prev, xp);
-#pragma unroll
-          for (int j = 0; j < SMAX; ++j) {
-            if (j < c) {
-              float h[VEC];
-              load_hist(j, h);
-              float t = 0.f;
-#pragma unroll
-              for (int q = 0; q < VEC; ++q) t += x[q] * h[q];
-              acc[j] += t;
-              if (HIST16 && two_rows) {
-                float t2 = 0.f;
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) t2 += xp[q] * h[q];
-                acc2[HIST16 ? j : 0] += t2;
-              }
-            }
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty_bar + stage);
-        if (mt.last) {
-          const int buf = tiles_done & 1;
-          if (!mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
-          ++tiles_done;
-#pragma unroll
-          for (int r = 0; r < C::kRows; ++r) {
-            double v[SMAX];
-#pragma unroll
-            for (int j = 0; j < SMAX; ++j) v[j] = static_cast<double>(r == 0 ? acc[j] : acc2[HIST16 ? j : 0]);
-            const double t = warp_sums<SMAX>(v);
-            if ((lane & (32 / SMAX - 1)) == 0) red[((buf * C::kRows + r) * kWarps + warp) * SMAX + lane / (32 / SMAX)] = t;
-          }
-          if (tid == 0) red_meta[buf] = RedMeta{mt.mat, mt.local, cur, c};
-          __syncwarp();
-          if (lane == 0) mbar_arrive(red_full + buf);
-        }
-      } else {
-        if (mt.first) {
-          item_ok = true;
-          if (d.s > 0) {
-            if (tid == 0) {
-              const volatile int* flag = d.w_ready;
-              const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
-              long long spins = 0;
-              int ok = 1;
-              while (*flag != tag) {
-                if (++spins > limit) { ok = 0; break; }
-                __nanosleep(100);
-              }
-              if (!ok) {
-                // The weights never came: this matrix takes no update in this step (the back-projection skips it)
-                // and says why.  Tiles of it that other CTAs did combine have advanced their part of m and v.
-                atomicExch(&ctrl->timeout_flag, 1);
-                atomicExch(d.step_bad, 1);
-                atomicCAS(d.status, 0, 8 /* NGALORE_ERR_TIMEOUT */);
-              }
-              *s_flag = ok;
-            }
-            consumer_sync<kConsumerThreads>();
-            item_ok = *s_flag != 0;
-            __threadfence();
-          }
-          if (tid < kMaxHistory) wsm[tid] = __ldcg(d.wsol + tid);
-          item_bad = __ldcg(d.step_bad) != 0;
-          it_m = d.m; it_v = d.v; it_u = d.u16;
-          it_m16 = d.m16; it_v16 = d.v16;
-          it_mat = static_cast<unsigned int>(d.index);
-          it_step = static_cast<unsigned int>(ctrl->k);
-          it_cur = current_gradient(d, cur);
-          it_h16 = HIST16 ? d.H16 + static_cast<long long>(cur) * d.rn : nullptr;
-          consumer_sync<kConsumerThreads>();
-#pragma unroll
-          for (int j = 0; j < SMAX; ++j) w[j] = wsm[j];
-        }
-        if (item_ok && idx < mt.count) {
-          const long long e = mt.e0 + idx;
-          if (item_bad) {
-            // The poisoned slot becomes a zero gradient; m, v are left alone and the update is zero.
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-              it_cur[e + q] = 0.f;
-              it_u[e + q] = __float2half_rn(0.f);
-              if (HIST16) it_h16[e + q] = 0;
-            }
-          } else {
-            float n[VEC], mm[VEC], vv[VEC], uu[VEC];
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) n[q] = 0.f;
-#pragma unroll
-            for (int j = 0; j < SMAX; ++j) {
-              if (j < c) {
-                float h[VEC];
-                load_hist(j, h);
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) n[q] = fmaf(w[j], h[q], n[q]);
-              }
-            }
-            if (HIST16) {
-              // from the next step on this gradient is an old one: store its bf16 rounding in the ring
+          while (true) {
+            if (idx < mt.count) {
               float x[VEC];
-              load_hist(cur, x);
-              uint32_t* dst = reinterpret_cast<uint32_t*>(it_h16 + e);
+              load32(cur, x);
 #pragma unroll
-              for (int q = 0; q < VEC; q += 2) dst[q >> 1] = float_to_bf16_bits(x[q]) | (float_to_bf16_bits(x[q + 1]) << 16);
+              for (int j = 0; j < SMAX; ++j) {
+                if (j >= c) break;
+                float h[VEC];
+                load32(j, h);
+                float t = 0.f;
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) t += x[q] * h[q];
+                acc[j] += t;
+              }
             }
-            load_moment(C::kMOff, mm);
-            load_moment(C::kVOff, vv);
+            const bool last = mt.last != 0;
+            release();
+            if (last) break;
+            if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+            mt = meta[stage];
+          }
+          if (!alive || !mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
+          double v[SMAX];
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-              mm[q] = hp.beta1 * mm[q] + (1.f - hp.beta1) * n[q];
-              vv[q] = hp.beta2 * vv[q] + (1.f - hp.beta2) * n[q] * n[q];
-              uu[q] = mm[q] / sqrtf(vv[q] + hp.eps);
-            }
-            if (MOM16) {
-              // elements 4 g .. 4 g + 3 take the upper halves of the four words of one generator call
-              uint32_t* dm = reinterpret_cast<uint32_t*>(it_m16 + e);
-              uint32_t* dv = reinterpret_cast<uint32_t*>(it_v16 + e);
+          for (int j = 0; j < SMAX; ++j) v[j] = static_cast<double>(acc[j]);
+          hand_over(0, v);
+        } else {
+          // rows of `cur` and of the slot that was current one step ago, in pairs: the inner loop is bound by the
+          // instructions it issues, and the packed multiply-add halves those
+          uint64_t acc[SMAX], acc2[SMAX];
+          float axx = 0.f, apx = 0.f;      // products with the fp32 gradient itself
 #pragma unroll
-              for (int q0 = 0; q0 < VEC; q0 += 4) {
-                const unsigned long long grp = static_cast<unsigned long long>(e + q0) >> 2;
-                const uint4 rnd = philox4x32_10(make_uint4(static_cast<unsigned int>(grp), static_cast<unsigned int>(grp >> 32),
-                                                           it_mat, it_step), hp.seed_lo, hp.seed_hi);
-                const unsigned int rb[4] = {rnd.x >> 16, rnd.y >> 16, rnd.z >> 16, rnd.w >> 16};
+          for (int j = 0; j < SMAX; ++j) acc[j] = acc2[j] = 0ull;
+          const int prev = c >= 2 ? (cur == 0 ? mats[mt.mat].s : cur) - 1 : cur;
+          while (true) {
+            if (idx < mt.count) {
+              float x[VEC];
+              uint64_t xx[VEC / 2], xp[VEC / 2];
+              load_current(x);
+              load16(prev, xp);            // (a single gradient: the zeros of its own place)
 #pragma unroll
-                for (int q = q0; q < q0 + 4 && q < VEC; q += 2) {
-                  // (VEC = 2: e is a multiple of 2, the pair is words 0, 1 or words 2, 3 of its group)
-                  const int w0 = VEC == 2 ? static_cast<int>(e & 2) : q - q0;
-                  dm[q >> 1] = float_to_bf16_bits(mm[q]) | (float_to_bf16_bits(mm[q + 1]) << 16);
-                  dv[q >> 1] = stochastic_bf16_bits(vv[q], rb[w0]) | (stochastic_bf16_bits(vv[q + 1], rb[w0 + 1]) << 16);
+              for (int q = 0; q < VEC / 2; ++q) {
+                xx[q] = pack_pair(x[2 * q], x[2 * q + 1]);
+                float p0, p1;
+                unpack_pair(xp[q], p0, p1);
+                axx += x[2 * q] * x[2 * q] + x[2 * q + 1] * x[2 * q + 1];
+                apx += x[2 * q] * p0 + x[2 * q + 1] * p1;
+              }
+#pragma unroll
+              for (int j = 0; j < SMAX; ++j) {
+                if (j >= c) break;
+                uint64_t h[VEC / 2];
+                load16(j, h);
+#pragma unroll
+                for (int q = 0; q < VEC / 2; ++q) {
+                  acc[j] = fma_pair(xx[q], h[q], acc[j]);
+                  acc2[j] = fma_pair(xp[q], h[q], acc2[j]);
                 }
               }
-              if (VEC == 4) *reinterpret_cast<uint2*>(it_u + e) = pack_f16x4(uu[0], uu[1], uu[2 % VEC], uu[3 % VEC]);
-              else *reinterpret_cast<uint32_t*>(it_u + e) = pack_f16x4(uu[0], uu[1], 0.f, 0.f).x;
-            } else if (VEC == 4) {
-              *reinterpret_cast<float4*>(it_m + e) = make_float4(mm[0], mm[1], mm[2 % VEC], mm[3 % VEC]);
-              *reinterpret_cast<float4*>(it_v + e) = make_float4(vv[0], vv[1], vv[2 % VEC], vv[3 % VEC]);
-              *reinterpret_cast<uint2*>(it_u + e) = pack_f16x4(uu[0], uu[1], uu[2 % VEC], uu[3 % VEC]);
-            } else {
-              *reinterpret_cast<float2*>(it_m + e) = make_float2(mm[0], mm[1]);
-              *reinterpret_cast<float2*>(it_v + e) = make_float2(vv[0], vv[1]);
-              *reinterpret_cast<uint32_t*>(it_u + e) = pack_f16x4(uu[0], uu[1], 0.f, 0.f).x;
             }
+            const bool last = mt.last != 0;
+            release();
+            if (last) break;
+            if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+            mt = meta[stage];
+          }
+          if (!alive || !mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
+          {
+            double v[SMAX];
+#pragma unroll
+            for (int j = 0; j < SMAX; ++j) {
+              float s0, s1;
+              unpack_pair(acc[j], s0, s1);
+              v[j] = static_cast<double>(j == cur ? axx : s0 + s1);
+            }
+            hand_over(0, v);
+          }
+          __syncwarp();
+          {
+            double v[SMAX];
+#pragma unroll
+            for (int j = 0; j < SMAX; ++j) {
+              float s0, s1;
+              unpack_pair(acc2[j], s0, s1);
+              v[j] = static_cast<double>(j == cur ? apx : s0 + s1);
+            }
+            hand_over(C::kRows - 1, v);
           }
         }
+        ++tiles_done;
+        if (tid == 0) red_meta[buf] = RedMeta{mt.mat, mt.local, cur, c};
         __syncwarp();
-        if (lane == 0) mbar_arrive(empty_bar + stage);
+        if (lane == 0) mbar_arrive(red_full + buf);
+      } else {
+        // ---- combination tile
+        const MatDesc& d = mats[mt.mat];
+        bool item_ok = true;
+        if (d.s > 0) {
+          if (tid == 0) {
+            const volatile int* flag = d.w_ready;
+            const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
+            long long spins = 0;
+            int ok = 1;
+            while (*flag != tag) {
+              if (++spins > limit) { ok = 0; break; }
+              __nanosleep(100);
+            }
+            if (!ok) {
+              // The weights never came: this matrix takes no update in this step (the back-projection skips it)
+              // and says why.  Tiles of it that other CTAs did combine have advanced their part of m and v.
+              atomicExch(&ctrl->timeout_flag, 1);
+              atomicExch(d.step_bad, 1);
+              atomicCAS(d.status, 0, 8 /* NGALORE_ERR_TIMEOUT */);
+            }
+            *s_flag = ok;
+          }
+          consumer_sync<kConsumerThreads>();
+          item_ok = *s_flag != 0;
+          __threadfence();
+        }
+        if (tid < kMaxHistory) wsm[tid] = __ldcg(d.wsol + tid);
+        const bool item_bad = __ldcg(d.step_bad) != 0;
+        float *const it_m = d.m, *const it_v = d.v, *const it_cur = current_gradient(d, cur);
+        __half* const it_u = d.u16;
+        uint16_t *const it_m16 = d.m16, *const it_v16 = d.v16;
+        uint16_t* const it_h16 = HIST16 ? d.H16 + static_cast<long long>(cur) * d.rn : nullptr;
+        const unsigned int it_mat = static_cast<unsigned int>(d.index), it_step = static_cast<unsigned int>(ctrl->k);
+        consumer_sync<kConsumerThreads>();
+        float w[SMAX];
+#pragma unroll
+        for (int j = 0; j < SMAX; ++j) w[j] = wsm[j];
+        const float wc = HIST16 ? wsm[cur] : 0.f;
+        while (true) {
+          if (item_ok && idx < mt.count) {
+            const long long e = mt.e0 + idx;
+            if (item_bad) {
+              // The poisoned slot becomes a zero gradient; m, v are left alone and the update is zero.
+#pragma unroll
+              for (int q = 0; q < VEC; ++q) {
+                it_cur[e + q] = 0.f;
+                it_u[e + q] = __float2half_rn(0.f);
+                if (HIST16) it_h16[e + q] = 0;
+              }
+            } else {
+              float n[VEC], mm[VEC], vv[VEC], uu[VEC];
+              if constexpr (!HIST16) {
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) n[q] = 0.f;
+#pragma unroll
+                for (int j = 0; j < SMAX; ++j) {
+                  if (j >= c) break;
+                  float h[VEC];
+                  load32(j, h);
+#pragma unroll
+                  for (int q = 0; q < VEC; ++q) n[q] = fmaf(w[j], h[q], n[q]);
+                }
+              } else {
+                float x[VEC];
+                load_current(x);
+                uint64_t np[VEC / 2];
+#pragma unroll
+                for (int q = 0; q < VEC / 2; ++q) np[q] = pack_pair(wc * x[2 * q], wc * x[2 * q + 1]);
+#pragma unroll
+                for (int j = 0; j < SMAX; ++j) {
+                  if (j >= c) break;
+                  uint64_t h[VEC / 2];
+                  load16(j, h);
+                  const uint64_t ww = pack_pair(w[j], w[j]);
+#pragma unroll
+                  for (int q = 0; q < VEC / 2; ++q) np[q] = fma_pair(ww, h[q], np[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < VEC / 2; ++q) unpack_pair(np[q], n[2 * q], n[2 * q + 1]);
+                // from the next step on this gradient is an old one: store its bf16 rounding in the ring
+                uint32_t* dst = reinterpret_cast<uint32_t*>(it_h16 + e);
+#pragma unroll
+                for (int q = 0; q < VEC; q += 2) dst[q >> 1] = float_to_bf16_bits(x[q]) | (float_to_bf16_bits(x[q + 1]) << 16);
+              }
+              load_moment(C::kMOff, mm);
+              load_moment(C::kVOff, vv);
+#pragma unroll
+              for (int q = 0; q < VEC; ++q) {
+                mm[q] = hp.beta1 * mm[q] + (1.f - hp.beta1) * n[q];
+                vv[q] = hp.beta2 * vv[q] + (1.f - hp.beta2) * n[q] * n[q];
+                uu[q] = mm[q] / sqrtf(vv[q] + hp.eps);
+              }
+              if (MOM16) {
+                // elements 4 g .. 4 g + 3 take the upper halves of the four words of one generator call
+                uint32_t* dm = reinterpret_cast<uint32_t*>(it_m16 + e);
+                uint32_t* dv = reinterpret_cast<uint32_t*>(it_v16 + e);
+#pragma unroll
+                for (int q0 = 0; q0 < VEC; q0 += 4) {
+                  const unsigned long long grp = static_cast<unsigned long long>(e + q0) >> 2;
+                  const uint4 rnd = philox4x32_10(make_uint4(static_cast<unsigned int>(grp), static_cast<unsigned int>(grp >> 32),
+                                                             it_mat, it_step), hp.seed_lo, hp.seed_hi);
+                  const unsigned int rb[4] = {rnd.x >> 16, rnd.y >> 16, rnd.z >> 16, rnd.w >> 16};
+#pragma unroll
+                  for (int q = q0; q < q0 + 4 && q < VEC; q += 2) {
+                    // (VEC = 2: e is a multiple of 2, the pair is words 0, 1 or words 2, 3 of its group)
+                    const int w0 = VEC == 2 ? static_cast<int>(e & 2) : q - q0;
+                    dm[q >> 1] = float_to_bf16_bits(mm[q]) | (float_to_bf16_bits(mm[q + 1]) << 16);
+                    dv[q >> 1] = stochastic_bf16_bits(vv[q], rb[w0]) | (stochastic_bf16_bits(vv[q + 1], rb[w0 + 1]) << 16);
+                  }
+                }
+                if (VEC == 4) *reinterpret_cast<uint2*>(it_u + e) = pack_f16x4(uu[0], uu[1], uu[2 % VEC], uu[3 % VEC]);
+                else *reinterpret_cast<uint32_t*>(it_u + e) = pack_f16x4(uu[0], uu[1], 0.f, 0.f).x;
+              } else if (VEC == 4) {
+                *reinterpret_cast<float4*>(it_m + e) = make_float4(mm[0], mm[1], mm[2 % VEC], mm[3 % VEC]);
+                *reinterpret_cast<float4*>(it_v + e) = make_float4(vv[0], vv[1], vv[2 % VEC], vv[3 % VEC]);
+                *reinterpret_cast<uint2*>(it_u + e) = pack_f16x4(uu[0], uu[1], uu[2 % VEC], uu[3 % VEC]);
+              } else {
+                *reinterpret_cast<float2*>(it_m + e) = make_float2(mm[0], mm[1]);
+                *reinterpret_cast<float2*>(it_v + e) = make_float2(vv[0], vv[1]);
+                *reinterpret_cast<uint32_t*>(it_u + e) = pack_f16x4(uu[0], uu[1], 0.f, 0.f).x;
+              }
+            }
+          }
+          const bool last = mt.last != 0;
+          release();
+          if (last) break;
+          if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+          mt = meta[stage];
+        }
+        if (!alive) break;
       }
-      if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
     }
   }
   __syncthreads();
