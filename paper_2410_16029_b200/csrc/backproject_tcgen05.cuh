@@ -62,7 +62,7 @@ __device__ __forceinline__ int bp_wchunks(const TcTile& tile) {
 template <int kBpStages, int kBpSlots>
 __global__ void __launch_bounds__(kBpThreads, 1)
 tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__ tiles, int n_tiles,
-                      const MatDesc* __restrict__ mats, Ctrl* ctrl, const Hyper* __restrict__ hyper) {
+                      const MatDesc* __restrict__ mats, Ctrl* ctrl, const Hyper* __restrict__ hyper, int advance) {
   using L = BpSmem<kBpStages, kBpSlots>;
   extern __shared__ unsigned char tc_smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
@@ -95,6 +95,9 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int stride = gridDim.x;
+  pdl_begin();
+  // the last launch of a step moves the step counters on (nothing in this kernel reads them)
+  if (advance && blockIdx.x == 0 && threadIdx.x == 32) advance_step(ctrl);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer of the operands
@@ -301,26 +304,28 @@ inline ngalore_status tc_backproject_init() {
   return NGALORE_OK;
 }
 
-// W <- (1 - lr wd) W - lr P u for the matrices [mat0, mat1), through the tensor maps tc_bind_buffers set up.
+// W <- (1 - lr wd) W - lr P u for the matrices [mat0, mat1), through the tensor maps tc_bind_buffers set up.  last: the
+// launch ends the step (it moves the counters on).  chained: nothing but the step's own kernels sits before it in the
+// stream (no event to wait for), so it may be a programmatic dependent launch.
 inline ngalore_status tc_backproject_range(TcPlan& plan, int mat0, int mat1, const MatDesc* d_mats, Ctrl* d_ctrl,
-                                           const Hyper* d_hyper, cudaStream_t stream, int64_t* launches) {
+                                           const Hyper* d_hyper, bool last, bool chained, cudaStream_t stream, int64_t* launches) {
   const int t0 = plan.back_tile0[mat0], t1 = plan.back_tile0[mat1];
   if (t1 <= t0) return NGALORE_OK;
   const int grid = (t1 - t0) < plan.grid_back ? (t1 - t0) : plan.grid_back;
-  if (plan.long_k_back)
-    tc_backproject_kernel<3, 5><<<grid, kBpThreads, BpSmem<3, 5>::kTotal, stream>>>(plan.d_maps, plan.d_tiles_back + t0,
-                                                                                   t1 - t0, d_mats, d_ctrl, d_hyper);
-  else
-    tc_backproject_kernel<2, 8><<<grid, kBpThreads, BpSmem<2, 8>::kTotal, stream>>>(plan.d_maps, plan.d_tiles_back + t0,
-                                                                                   t1 - t0, d_mats, d_ctrl, d_hyper);
+  auto launch = [&](auto kernel, size_t smem) {
+    launch_step(chained && plan.short_step, kernel, grid, kBpThreads, smem, stream, plan.d_maps, plan.d_tiles_back + t0, t1 - t0,
+                d_mats, d_ctrl, d_hyper, last ? 1 : 0);
+  };
+  if (plan.long_k_back) launch(tc_backproject_kernel<3, 5>, BpSmem<3, 5>::kTotal);
+  else launch(tc_backproject_kernel<2, 8>, BpSmem<2, 8>::kTotal);
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
-// W <- (1 - lr wd) W - lr P u for every matrix.
+// W <- (1 - lr wd) W - lr P u for every matrix, and the end of the step.
 inline ngalore_status tc_backproject(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
                                      cudaStream_t stream, int64_t* launches) {
-  return tc_backproject_range(plan, 0, plan.n_mats, d_mats, d_ctrl, d_hyper, stream, launches);
+  return tc_backproject_range(plan, 0, plan.n_mats, d_mats, d_ctrl, d_hyper, true, true, stream, launches);
 }
 
 }  // namespace ngalore

@@ -87,6 +87,43 @@ __device__ __forceinline__ unsigned int stochastic_bf16_bits(float x, unsigned i
   return (__float_as_uint(x) + bits16) >> 16;
 }
 
+// The end of a step: ring position, step counters and work counters move on.
+__device__ __forceinline__ void advance_step(Ctrl* ctrl) {
+  ctrl->n_appended += 1;
+  ctrl->k += 1;
+  ctrl->epoch += 1;
+  ctrl->work_counter = 0u;
+  ctrl->gemm_counter0 = 0u;
+  ctrl->gemm_counter1 = 0u;
+  ctrl->spin_limit = 0;
+  ctrl->debug_withhold = 0;
+}
+
+// Programmatic dependent launch, for the kernels of a short step: a kernel launched so may start while its predecessor in
+// the stream still runs.  pdl_begin lets the successor start in turn and then waits until the predecessor has finished
+// and its writes are visible; what comes before it (barriers, tensor memory) and the launch itself overlap the
+// predecessor's tail.  Every kernel that launch_step is given calls it before it touches global memory; after an ordinary
+// launch it returns at once.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_step(bool dependent, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 struct StreamTile {
   int mat;    // matrix index
   int local;  // tile index inside the matrix

@@ -214,6 +214,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
   const int t_begin = cta_first[blockIdx.x], t_end = cta_first[blockIdx.x + 1];   // this CTA's tiles
 
   if (warp == 0) {
@@ -415,6 +416,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
 
 // Zero the ring slot the projection is about to accumulate into, for the matrices whose K is split.
 __global__ void zero_split_slots_kernel(const MatDesc* mats, const int* split_mats, const Ctrl* ctrl) {
+  pdl_begin();
   const MatDesc& d = mats[split_mats[blockIdx.y]];
   float4* p = reinterpret_cast<float4*>(current_gradient(d, ring_cur(ctrl, d.s)));
   const long long n4 = d.rn / 4;
@@ -478,6 +480,11 @@ struct TcPlan {
   std::vector<int> rowsN;           // per matrix: M, N for re-encoding the maps of G and W
   std::vector<int> colsN;
   std::vector<int> right;           // per matrix: projected on the right
+  // Steps of at most about 0.3 ms (32 back-projection tiles a CTA) launch their kernels as programmatic dependents, which
+  // hides the 2 us between two kernels: 60M shapes 222 -> 214 us, encoder shapes at r = 8 189 -> 180, one matrix 54 -> 46.
+  // Longer ones do not: it changes which SM gets which CTA, and with it which tiles run side by side: 1.1B shapes 7.20 ->
+  // 7.32 ms, at r = 8 1.915 -> 1.957 ms, 130M and 350M the same either way.
+  bool short_step = false;
   bool tall_proj = false;           // projection tiles are 256 rows high (tc_project2_kernel)
   bool long_k_back = false;         // back-projection with three operand stages and a short W ring
   // Binding sets: the tensor maps of one particular array of G and W pointers, encoded once, kept in pinned host
@@ -673,6 +680,7 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
   std::vector<int> proj_first;
   tc_assign_tiles(proj, plan.grid_proj, proj_first);
   plan.grid_back = std::min(plan.n_tiles_back, sm_count);
+  plan.short_step = plan.n_tiles_back <= 32 * sm_count;
   plan.n_split = static_cast<int>(split_mats.size());
   plan.n_tiles_pg = static_cast<int>(pg.size());
   plan.grid_pg = std::min(plan.n_tiles_pg, sm_count);

@@ -178,6 +178,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  pdl_begin();
   const int tag = ctrl->epoch + 1;
 
   if (tid >= kConsumerThreads + 32) {
@@ -705,28 +706,28 @@ inline void fused_plan_destroy(FusedPlan& plan) {
 
 template <int SMAX, bool HIST16, bool MOM16>
 inline void fused_launch_one(const FusedPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
-                             cudaStream_t stream) {
+                             bool short_step, cudaStream_t stream) {
   using C = FusedCfg<SMAX, HIST16, MOM16>;
-  fused_stream_kernel<SMAX, HIST16, MOM16><<<plan.grid, C::kThreads, C::kTotal, stream>>>(d_mats, plan.d_items, plan.n_items,
-                                                                                         d_ctrl, d_hyper);
+  launch_step(short_step, fused_stream_kernel<SMAX, HIST16, MOM16>, plan.grid, C::kThreads, C::kTotal, stream, d_mats, plan.d_items,
+              plan.n_items, d_ctrl, d_hyper);
 }
 
 template <bool HIST16, bool MOM16>
 inline void fused_launch_for(const FusedPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper, int s,
-                             cudaStream_t stream) {
-  if (s <= 8) fused_launch_one<8, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, stream);
-  else if (s <= 16) fused_launch_one<16, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, stream);
-  else fused_launch_one<32, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, stream);
+                             bool short_step, cudaStream_t stream) {
+  if (s <= 8) fused_launch_one<8, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
+  else if (s <= 16) fused_launch_one<16, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
+  else fused_launch_one<32, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
 }
 
 inline ngalore_status fused_stream_launch(FusedPlan& plan, const MatDesc* d_mats, int /*n_mats*/, Ctrl* d_ctrl,
-                                          const Hyper* d_hyper, int s, cudaStream_t stream, int64_t* launches) {
+                                          const Hyper* d_hyper, int s, bool short_step, cudaStream_t stream, int64_t* launches) {
   if (plan.hist16) {
-    if (plan.mom16) fused_launch_for<true, true>(plan, d_mats, d_ctrl, d_hyper, s, stream);
-    else fused_launch_for<true, false>(plan, d_mats, d_ctrl, d_hyper, s, stream);
+    if (plan.mom16) fused_launch_for<true, true>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
+    else fused_launch_for<true, false>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
   } else {
-    if (plan.mom16) fused_launch_for<false, true>(plan, d_mats, d_ctrl, d_hyper, s, stream);
-    else fused_launch_for<false, false>(plan, d_mats, d_ctrl, d_hyper, s, stream);
+    if (plan.mom16) fused_launch_for<false, true>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
+    else fused_launch_for<false, false>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
   }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;

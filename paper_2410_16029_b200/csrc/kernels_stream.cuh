@@ -239,15 +239,6 @@ __global__ void __launch_bounds__(kStreamThreads) combine_kernel(const MatDesc* 
   combine_tile<SMAX>(d, t.local, ring_cur(ctrl, d.s), ring_count(ctrl, d.s), d.te, *hyper, wsm);
 }
 
-__global__ void advance_kernel(Ctrl* ctrl) {
-  ctrl->n_appended += 1;
-  ctrl->k += 1;
-  ctrl->epoch += 1;
-  ctrl->work_counter = 0u;
-  ctrl->gemm_counter0 = 0u;
-  ctrl->gemm_counter1 = 0u;
-  ctrl->spin_limit = 0;
-  ctrl->debug_withhold = 0;
-}
+__global__ void advance_kernel(Ctrl* ctrl) { advance_step(ctrl); }
 
 }  // namespace ngalore

@@ -458,7 +458,7 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
     else if (st->s <= 16) launch_plain_stream<16>(st, stream);
     else launch_plain_stream<32>(st, stream);
   } else {
-    if ((rc = fused_stream_launch(st->fused, st->d_desc, st->n, st->d_ctrl, st->d_hyper, st->s, stream, &st->launches))) return rc;
+    if ((rc = fused_stream_launch(st->fused, st->d_desc, st->n, st->d_ctrl, st->d_hyper, st->s, st->tc.short_step, stream, &st->launches))) return rc;
   }
   NG_CUDA(cudaGetLastError());
   if (st->profiling) NG_CUDA(cudaEventRecord(st->ev[2], stream));
@@ -489,22 +489,24 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
     for (size_t g = 0; g + 1 < st->group_first.size(); ++g) {
       NG_CUDA(cudaStreamWaitEvent(stream, st->ev_w_in[g], 0));
       if ((rc = tc_backproject_range(st->tc, st->group_first[g], st->group_first[g + 1], st->d_desc, st->d_ctrl,
-                                     st->d_hyper, stream, &st->launches)))
+                                     st->d_hyper, g + 2 == st->group_first.size(), false, stream, &st->launches)))
         return rc;
       NG_CUDA(cudaEventRecord(st->ev_w_done[g], stream));
     }
   } else if (st->upd_first.size() > 1) {
     for (size_t ug = 0; ug + 1 < st->upd_first.size(); ++ug) {
       if ((rc = tc_backproject_range(st->tc, st->upd_first[ug], st->upd_first[ug + 1], st->d_desc, st->d_ctrl,
-                                     st->d_hyper, stream, &st->launches)))
+                                     st->d_hyper, ug + 2 == st->upd_first.size(), false, stream, &st->launches)))
         return rc;
       NG_CUDA(cudaEventRecord(st->ev_upd[ug], stream));
     }
   } else {
     if ((rc = tc_backproject(st->tc, st->d_desc, st->d_ctrl, st->d_hyper, stream, &st->launches))) return rc;
   }
-  advance_kernel<<<1, 1, 0, stream>>>(st->d_ctrl);
-  st->launches += 1;
+  if (st->opt.gemm_impl == 1) {   // (the tensor-core back-projection moves the counters on itself)
+    advance_kernel<<<1, 1, 0, stream>>>(st->d_ctrl);
+    st->launches += 1;
+  }
   NG_CUDA(cudaGetLastError());
   if (st->profiling) {
     NG_CUDA(cudaEventRecord(st->ev[3], stream));

@@ -67,6 +67,7 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_begin();
   const int t_begin = cta_first[blockIdx.x], t_end = cta_first[blockIdx.x + 1];   // this CTA's tiles
 
   if (warp == 0) {
@@ -222,7 +223,7 @@ inline ngalore_status tc_project_init() {
 inline ngalore_status tc_project(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
                                  cudaStream_t stream, int64_t* launches) {
   if (plan.n_split > 0) {
-    zero_split_slots_kernel<<<dim3(64, plan.n_split), 256, 0, stream>>>(d_mats, plan.d_split_mats, d_ctrl);
+    launch_step(plan.short_step, zero_split_slots_kernel, dim3(64, plan.n_split), 256, 0, stream, d_mats, plan.d_split_mats, d_ctrl);
     *launches += 1;
   }
   if (plan.n_tiles_pg > 0) {
@@ -234,13 +235,12 @@ inline ngalore_status tc_project(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ct
     if (plan.n_tiles_proj == 0) return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
   }
   if (plan.tall_proj) {
-    tc_project2_kernel<<<plan.grid_proj, kP2Threads, P2Smem::kTotal, stream>>>(plan.d_maps, plan.d_tiles_proj,
-                                                                              plan.d_proj_first, d_mats, d_ctrl);
+    launch_step(plan.short_step, tc_project2_kernel, plan.grid_proj, kP2Threads, P2Smem::kTotal, stream, plan.d_maps,
+                plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl);
   } else {
     using LP = TcSmem<kProjBN, 1, 1, kProjStages, kProjEpiWarps>;
-    tc_gemm_kernel<kProjBN, 1, 1, kProjStages, TC_EPI_PROJECT, kProjEpiWarps, false>
-        <<<plan.grid_proj, 64 + 32 * kProjEpiWarps, LP::kTotal, stream>>>(plan.d_maps, plan.d_tiles_proj,
-                                                                          plan.d_proj_first, d_mats, d_ctrl, nullptr);
+    launch_step(plan.short_step, tc_gemm_kernel<kProjBN, 1, 1, kProjStages, TC_EPI_PROJECT, kProjEpiWarps, false>, plan.grid_proj,
+                64 + 32 * kProjEpiWarps, LP::kTotal, stream, plan.d_maps, plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl, nullptr);
   }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
