@@ -171,7 +171,7 @@ struct TcSmem {
   static constexpr int kBChunkBytes = 64 * kTcBK * 2;         // one 64-column chunk: 64 K rows x 128 B
   static constexpr int kBBytes = (BN / 64) * kBChunkBytes;    // per B operand
   static constexpr int kStageBytes = NA * kABytes + NB * kBBytes;
-  static constexpr int kEpiWarpBytes = 32 * 36 * 4;           // 32 rows x (32 + 4 pad) floats
+  static constexpr int kEpiWarpBytes = 32 * 32 * 4;           // 32 rows x 32 floats, 16-byte words swizzled by the row
   static constexpr int kBarOffset = STAGES * kStageBytes + NEPI * kEpiWarpBytes;
   static constexpr int kTotal = kBarOffset + 256 + 1024;      // barriers + slack for 1024-byte alignment
 };
@@ -223,21 +223,18 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      TcTile tile = tiles[t_begin];
+      auto map_a = [&](const TcTile& t) {
+        return tmaps + (EPI == TC_EPI_STORE ? probs[t.mat].map_a : t.mat * kTcMapsPerMat + TC_MAP_A_PROJ);
+      };
+      auto map_b = [&](const TcTile& t) {
+        return tmaps + (EPI == TC_EPI_STORE ? probs[t.mat].map_b : t.mat * kTcMapsPerMat + TC_MAP_B_PROJ);
+      };
+      const CUtensorMap *mapA = map_a(tile), *mapB0 = map_b(tile);
       for (int t = t_begin; t < t_end && ok; ++t) {
-        const TcTile tile = tiles[t];
-        const CUtensorMap *mapA, *mapB0;
-        int out_cols;
-        if (EPI == TC_EPI_STORE) {
-          const TcProblem pr = probs[tile.mat];
-          mapA = tmaps + pr.map_a;
-          mapB0 = tmaps + pr.map_b;
-          out_cols = pr.out_cols;
-        } else {
-          mapA = tmaps + tile.mat * kTcMapsPerMat + TC_MAP_A_PROJ;
-          mapB0 = tmaps + tile.mat * kTcMapsPerMat + TC_MAP_B_PROJ;
-          out_cols = tile.cols;
-        }
-        const int n_rem = out_cols - tile.n0;
+        // (the next tile is looked up while this one's loads go out)
+        const TcTile next = tiles[min(t + 1, t_end - 1)];
+        const int n_rem = tile.cols - tile.n0;
         const int n_eff = n_rem >= BN ? BN : ((n_rem + 15) & ~15);
         const int nchunks = (n_eff + 63) >> 6;
         const uint32_t bytes = NA * L::kABytes + NB * nchunks * L::kBChunkBytes;
@@ -263,6 +260,8 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
           }
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        if (next.mat != tile.mat) { mapA = map_a(next); mapB0 = map_b(next); }
+        tile = next;
       }
     }
   } else if (warp == 1) {
@@ -272,10 +271,11 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
+      TcTile next = tiles[t_begin];
       for (int t = t_begin; t < t_end && ok; ++t, ++local) {
-        const TcTile tile = tiles[t];
-        const int out_cols = (EPI == TC_EPI_STORE) ? probs[tile.mat].out_cols : tile.cols;
-        const int n_rem = out_cols - tile.n0;
+        const TcTile tile = next;
+        next = tiles[min(t + 1, t_end - 1)];
+        const int n_rem = tile.cols - tile.n0;
         const int n_eff = n_rem >= BN ? BN : ((n_rem + 15) & ~15);
         const uint32_t idesc = instr_desc(n_eff, A_MN, F16);
         const int buf = local & 1;
@@ -314,16 +314,18 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2 .. 2 + NEPI - 1)
     // With 8 epilogue warps there are two groups of four; group g drains accumulator buffer g, i.e. the
-    // tiles with (local & 1) == g.
+    // tiles with (local & 1) == g.  That is for tiles of few K blocks, whose epilogue takes longer than their MMAs
+    // (Q = Y R^-1 of the refresh, K = r': 58 matrices of r' = 128 33 -> 25 us, 84 of r' = 256 81 -> 67 us).
     const int quarter = warp & 3;  // TMEM lanes 32 * quarter .. + 31 belong to this warp
     constexpr int kGroups = NEPI / 4;
     const int group = (warp - 2) >> 2;
     float* stg = reinterpret_cast<float*>(smem + STAGES * L::kStageBytes + (warp - 2) * L::kEpiWarpBytes);
-    int local = 0;
     bool ok = true;
-    for (int t = t_begin; t < t_end && ok; ++t, ++local) {
-      if (kGroups == 2 && (local & 1) != group) continue;
-      const TcTile tile = tiles[t];
+    const int first = kGroups == 2 ? group : 0;
+    TcTile tile;
+    if (t_begin + first < t_end) tile = tiles[t_begin + first];
+    for (int local = first; t_begin + local < t_end && ok; local += kGroups) {
+      const TcTile next = tiles[min(t_begin + local + kGroups, t_end - 1)];
       float* out;
       __nv_bfloat16 *out_hi = nullptr, *out_lo = nullptr;
       int rows_total, out_cols, ld_out, ld16 = 0;
@@ -364,7 +366,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
           }
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(stg + lane * 36 + j * 4) =
+            *reinterpret_cast<float4*>(stg + lane * 32 + ((j ^ (lane & 7)) << 2)) =
                 make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
                             __uint_as_float(r[4 * j + 3]));
           __syncwarp();
@@ -375,7 +377,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
               const int rr = it * 4 + sub_row;
               const int row = row_base + rr;
               if (row < rows_total) {
-                const float4 acc = *reinterpret_cast<const float4*>(stg + rr * 36 + sub_col);
+                const float4 acc = *reinterpret_cast<const float4*>(stg + rr * 32 + (((lane ^ rr) & 7) << 2));
                 float* p = out + static_cast<long long>(row) * ld_out + col;
                 if (EPI == TC_EPI_STORE && out_hi != nullptr) {
                   const __nv_bfloat162 h01 = __floats2bfloat162_rn(acc.x, acc.y), h23 = __floats2bfloat162_rn(acc.z, acc.w);
@@ -398,6 +400,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
           __syncwarp();
         }
       }
+      tile = next;
     }
   }
 

@@ -588,7 +588,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   }
 
   using L1 = TcSmem<kRefBN, 1, 2, kRefStages1, 4>;
-  using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 4>;
+  using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
   using L0 = TcSmem<kRefBN, 1, 1, kRefStages0, 4>;
   using LW1 = TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>;
   using LW0 = TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>;
@@ -608,9 +608,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L1::kTotal) != cudaSuccess ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L1::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, false>,
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, true>,
+      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess)
     return NGALORE_ERR_CUDA;
   plan.ready = true;
@@ -628,7 +628,7 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     zero_jobs_kernel<<<dim3(32, plan.n_zero[g]), 256, 0, stream>>>(plan.d_zero[g]);
     *launches += 1;
   }
-  using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 4>;
+  using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
   const int threads = 64 + 32 * 4;
   auto product = [&](auto a_mn) {   // a product with G; a_mn: with G^T
     constexpr bool MN = decltype(a_mn)::value;
@@ -653,11 +653,11 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     case RG_Z_FROM_Y: product(std::true_type{}); break;
     case RG_GRAM_Y:
     case RG_GRAM_Z:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
+      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true><<<plan.grid[g], 64 + 32 * 8, L2::kTotal, stream>>>(
           plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     default:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 4, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
+      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false><<<plan.grid[g], 64 + 32 * 8, L2::kTotal, stream>>>(
           plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
   }
