@@ -89,9 +89,13 @@ __global__ void zero_jobs_kernel(const ZeroJob* jobs) {
 // column alike, whatever its norm, so weak directions are still orthogonalised against each other and re-normalised.
 
 struct SyrkTile {
-  int mat, ti, tj, k0;  // output tile (ti, tj <= ti) of 64 x 64, rows k0 .. k0 + kSyrkRows of Y
+  int mat, ti, tj, k0, k1;  // output tile (ti, tj <= ti) of 64 x 64, rows k0 .. k1 - 1 of Y
 };
-constexpr int kSyrkRows = 1024;
+// Rows of a slab: long ones save atomics, short ones balance the SMs where there are few tiles.  58 matrices of r' = 128
+// (232 tiles of 1024 rows) 138 us against 105 with 256 rows, 84 of r' = 256 (1080) 473 / 451 us, 156 of the 1.1B shapes
+// (15 thousand) 4.14 / 4.33 ms.
+constexpr int kSyrkRows = 1024, kSyrkRowsFew = 256;
+constexpr int kSyrkFewTiles = 16;   // per SM
 
 struct SyrkMat {
   const __nv_bfloat16 *hi, *lo;   // rows x ld: the two parts of the basis, L columns of which are valid
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, cons
   const SyrkMat m = mats[t.mat];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
   const int i0 = t.ti * 64, j0 = t.tj * 64;
-  const int k1 = (t.k0 + kSyrkRows < m.rows) ? t.k0 + kSyrkRows : m.rows;
+  const int k1 = t.k1;
   const int lc = (tid & 15) * 4, lk = tid >> 4;   // this thread fetches four columns of one row of either operand
   const int wr = (warp >> 1) * 16, wc = (warp & 1) * 32;
   const bool idle = t.ti == t.tj && wc > wr + 15;   // (all of it above the diagonal)
@@ -398,12 +402,17 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_factor32 = take(sizeof(FactorMat) * n);
   const size_t o_factor64 = take(sizeof(FactorMat) * n);
   std::vector<SyrkTile> syrk_tiles;
-  for (int i = 0; i < n; ++i) {
-    const int nt = (plan.mats[i].L + 63) / 64;
-    for (int k0 = 0; k0 < plan.mats[i].M; k0 += kSyrkRows)
-      for (int ti = 0; ti < nt; ++ti)
-        for (int tj = 0; tj <= ti; ++tj) syrk_tiles.push_back(SyrkTile{i, ti, tj, k0});
-  }
+  auto slabs = [&](int slab) {
+    syrk_tiles.clear();
+    for (int i = 0; i < n; ++i) {
+      const int nt = (plan.mats[i].L + 63) / 64;
+      for (int k0 = 0; k0 < plan.mats[i].M; k0 += slab)
+        for (int ti = 0; ti < nt; ++ti)
+          for (int tj = 0; tj <= ti; ++tj) syrk_tiles.push_back(SyrkTile{i, ti, tj, k0, std::min(k0 + slab, plan.mats[i].M)});
+    }
+  };
+  slabs(kSyrkRows);
+  if (static_cast<int>(syrk_tiles.size()) < kSyrkFewTiles * sm_count) slabs(kSyrkRowsFew);
   plan.n_syrk_tiles = static_cast<int>(syrk_tiles.size());
   const size_t o_syrk_m = take(sizeof(SyrkMat) * n);
   const size_t o_syrk_t = take(sizeof(SyrkTile) * syrk_tiles.size());
