@@ -61,7 +61,6 @@ struct CholProblem {
   int L;
   int pad;
   double tiny;  // pivot floor, written by chol_begin_kernel
-  const int* only_if = nullptr;  // chol_cta_kernel, conditional launch: factor only where this word is set
 };
 
 constexpr int kCholNB = 32;  // panel width
@@ -202,208 +201,6 @@ inline cudaError_t chol_batched_launch(CholProblem* d_probs, int n, int Lmax, cu
       *launches += 1;
     }
   }
-  return cudaGetLastError();
-}
-
-// The same factorisation with one CTA per matrix and no launches between the panels: for a batch of about as many
-// matrices as there are SMs this keeps every SM busy from the first panel to the last, where the launch-per-panel
-// version spends most of its time between kernels (a 512 x 512 factor is 16 panels, i.e. 32 launches of a few
-// tens of microseconds each, for 45 million multiply-adds).  Per panel: one warp factors the diagonal block in
-// registers, every thread solves one row of the panel against it (keeping the solved panel in shared memory,
-// column-major), and all threads update the trailing triangle in 4 x 4 register tiles straight in global memory
-// (the matrix stays in L2).  Shared memory: 32 x (L - 32) doubles for the panel.
-constexpr int kCholCtaThreads = 512;
-
-// Row length of the panel in shared memory: a multiple of 16 bytes, so that four consecutive rows load at once.
-template <typename T>
-__host__ __device__ inline int chol_cta_ldp(int trailing) {
-  return sizeof(T) == 8 ? trailing + 4 - (trailing & 1) : (trailing + 7) & ~3;
-}
-
-template <typename T>
-inline size_t chol_cta_smem_bytes(int Lmax) {
-  const int rows = Lmax > kCholNB ? Lmax - kCholNB : 0;
-  return sizeof(T) * static_cast<size_t>(kCholNB) * (chol_cta_ldp<T>(rows) + 4);
-}
-
-__device__ __forceinline__ void chol_load4(const double* p, double (&a)[4]) {
-  const double2 lo = *reinterpret_cast<const double2*>(p), hi = *reinterpret_cast<const double2*>(p + 2);
-  a[0] = lo.x; a[1] = lo.y; a[2] = hi.x; a[3] = hi.y;
-}
-__device__ __forceinline__ void chol_load4(const float* p, float (&a)[4]) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
-}
-
-// The diagonal block of a panel, by one warp: D (nbj x nbj, zero beyond) is replaced by its lower Cholesky factor
-// and rdiag receives the reciprocals of the factor's diagonal (zero beyond the block).  Lane i holds row i in
-// registers: step k takes the pivot from lane k, scales column k, and every lane subtracts its share of the
-// rank-one update with one shuffle per entry.  A function of its own so that its 32 row entries get registers
-// whatever the caller needs elsewhere.
-template <typename T>
-__device__ __noinline__ void chol_diag_block(T (*D)[kCholNB + 1], T* rdiag, int nbj, T tiny, int lane) {
-  constexpr int NB = kCholNB;
-  T r[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) r[j] = D[lane][j];
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    T dkk = __shfl_sync(0xffffffffu, r[k], k);
-    if (!(dkk > tiny)) dkk = tiny;
-    const T lkk = sqrt(dkk);
-    const T inv = T(1) / lkk;
-    if (lane == k) {
-      r[k] = lkk;
-      rdiag[k] = k < nbj ? inv : T(0);
-    }
-    if (lane > k) r[k] = r[k] * inv;
-    const T lik = r[k];
-#pragma unroll
-    for (int j = k + 1; j < NB; ++j) {
-      const T ljk = __shfl_sync(0xffffffffu, r[k], j);
-      if (lane >= j) r[j] -= lik * ljk;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < NB; ++j) D[lane][j] = (j <= lane && lane < nbj && j < nbj) ? r[j] : T(0);
-}
-
-// One row of the panel, held as entries p[jj * ldp] (jj = 0 .. 31) of the k-major panel in shared memory:
-// x D^T = c by forward substitution in place.  As soon as x_t is known every later entry takes its share of it, so
-// the dependent chain is one multiply and one multiply-add per t.
-template <typename T>
-__device__ __noinline__ void chol_panel_row(T* p, int ldp, const T (*D)[kCholNB + 1], const T* rdiag) {
-  constexpr int NB = kCholNB;
-  T a[NB];
-#pragma unroll
-  for (int jj = 0; jj < NB; ++jj) a[jj] = p[jj * ldp];
-#pragma unroll
-  for (int t = 0; t < NB; ++t) {
-    const T xt = a[t] * rdiag[t];
-    a[t] = xt;
-#pragma unroll
-    for (int jj = t + 1; jj < NB; ++jj) a[jj] -= xt * D[jj][t];
-    if ((t & 3) == 3) asm volatile("" ::: "memory");   // keeps the 496 loads of D from being lifted to the front
-  }
-#pragma unroll
-  for (int jj = 0; jj < NB; ++jj) p[jj * ldp] = a[jj];
-}
-
-// T = double: the factorisation as described.  T = float: the same on a matrix stored as L x L floats at the same
-// address (CholProblem::C reinterpreted); enough for the orthonormalisations between the products of the subspace
-// iteration, whose Gram matrices come from the tensor cores with 2^-17 of relative accuracy and carry a shift of
-// about 1e-2 on a unit diagonal, and about twice as fast (half the shared-memory traffic per multiply-add, twice
-// the arithmetic rate).
-template <typename T>
-__global__ void __launch_bounds__(kCholCtaThreads, 1) chol_cta_kernel(const CholProblem* probs, int conditional) {
-  constexpr int NB = kCholNB;
-  extern __shared__ __align__(16) unsigned char chol_ps_raw[];
-  T* chol_ps = reinterpret_cast<T*>(chol_ps_raw);    // panel, k-major: chol_ps[k * ldp + (row - base)]
-  __shared__ T D[NB][NB + 1];      // the diagonal block, then its lower Cholesky factor
-  __shared__ T rdiag[NB];          // reciprocals of the factor's diagonal
-  __shared__ T s_tiny;
-  const CholProblem p = probs[blockIdx.x];
-  if (conditional && *p.only_if == 0) return;
-  T* C = reinterpret_cast<T*>(p.C);
-  const int L = p.L;
-  const int tid = threadIdx.x;
-  // pivot floor from the diagonal (a pivot that is not above it is replaced by it, see chol_begin_kernel)
-  if (tid < 32) {
-    T md = 0;
-    for (int i = tid; i < L; i += 32) {
-      const T v = C[static_cast<long long>(i) * L + i];
-      md = v > md ? v : md;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const T v = __shfl_xor_sync(0xffffffffu, md, o);
-      md = v > md ? v : md;
-    }
-    if (tid == 0) s_tiny = sizeof(T) == 8 ? static_cast<T>(fmax(static_cast<double>(md) * 1e-28, 1e-300))
-                                          : static_cast<T>(fmax(static_cast<double>(md) * 1e-12, 1e-30));
-  }
-  __syncthreads();
-  const T tiny = s_tiny;
-  for (int j0 = 0; j0 < L; j0 += NB) {
-    const int nbj = (L - j0 < NB) ? (L - j0) : NB;
-    const int base = j0 + nbj;            // first row / column of the trailing part
-    const int Tn = L - base;              // its size
-    const int ldp = chol_cta_ldp<T>(Tn);
-    for (int x = tid; x < NB * NB; x += kCholCtaThreads) {
-      const int a = x / NB, b = x % NB;
-      D[a][b] = (a < nbj && b < nbj) ? C[static_cast<long long>(j0 + a) * L + j0 + b] : T(0);
-    }
-    __syncthreads();
-    if (tid < 32) chol_diag_block<T>(D, rdiag, nbj, tiny, tid);
-    __syncthreads();
-    for (int x = tid; x < NB * NB; x += kCholCtaThreads) {
-      const int a = x / NB, b = x % NB;
-      if (a < nbj && b <= a) C[static_cast<long long>(j0 + a) * L + j0 + b] = D[a][b];
-    }
-    // panel rows: x D^T = c.  The rows come in through shared memory (a warp reads one row of 32
-    // entries at a time, so that global memory sees whole lines), one thread per row then works in place on its
-    // column of the k-major panel, and the solved rows go out the same way.
-    {
-      const int warp = tid >> 5, lane = tid & 31;
-      for (int r = warp; r < Tn; r += kCholCtaThreads / 32)
-        chol_ps[lane * ldp + r] = (lane < nbj) ? C[static_cast<long long>(base + r) * L + j0 + lane] : T(0);
-      __syncthreads();
-      for (int r = tid; r < Tn; r += kCholCtaThreads) chol_panel_row<T>(chol_ps + r, ldp, D, rdiag);
-      __syncthreads();
-      for (int r = warp; r < Tn; r += kCholCtaThreads / 32)
-        if (lane < nbj) C[static_cast<long long>(base + r) * L + j0 + lane] = chol_ps[lane * ldp + r];
-    }
-    __syncthreads();
-    // trailing update on the lower triangle: C[i][j] -= sum_k panel[i][k] panel[j][k], 4 x 4 tiles
-    if (Tn > 0) {
-      const int nt = (Tn + 3) >> 2;
-      const int ntiles = nt * (nt + 1) / 2;
-      for (int t = tid; t < ntiles; t += kCholCtaThreads) {
-        int ti = static_cast<int>((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-        while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-        while (ti * (ti + 1) / 2 > t) --ti;
-        const int tj = t - ti * (ti + 1) / 2;
-        const int i0 = 4 * ti, c0 = 4 * tj;        // relative to base
-        T acc[4][4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int y = 0; y < 4; ++y) acc[x][y] = T(0);
-#pragma unroll 4
-        for (int k = 0; k < NB; ++k) {
-          const T* pk = chol_ps + k * ldp;
-          // (rows beyond the trailing part inside the last tile read the padding or the next column's start: finite
-          // values that the bounds check below keeps from being stored)
-          T a[4], b[4];
-          chol_load4(pk + i0, a);
-          chol_load4(pk + c0, b);
-#pragma unroll
-          for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
-        }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const int i = base + i0 + x;
-          if (i >= L) continue;
-#pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            const int j = base + c0 + y;
-            if (j <= i) C[static_cast<long long>(i) * L + j] -= acc[x][y];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Factor n matrices, one CTA each (the list should start with the largest matrices: CTAs are handed out in order).
-template <typename T>
-inline cudaError_t chol_cta_launch(const CholProblem* d_probs, int n, int Lmax, cudaStream_t stream, int64_t* launches,
-                                   bool conditional = false) {
-  chol_cta_kernel<T><<<n, kCholCtaThreads, chol_cta_smem_bytes<T>(Lmax), stream>>>(d_probs, conditional ? 1 : 0);
-  *launches += 1;
   return cudaGetLastError();
 }
 

@@ -82,7 +82,7 @@ struct ngalore_state {
   // Rayleigh-Ritz rotation of the plain refresh path, which works on one matrix at a time: the eigensolver's work
   // space is shared by all of them
   EigMat* d_eig = nullptr;
-  CholProblem* d_eig_chol = nullptr;
+  FactorMat* d_eig_factor = nullptr;
   int64_t k = 0;
   int64_t n_appended = 0;
   bool has_subspace = false;         // every matrix has a projector
@@ -330,7 +330,7 @@ ngalore_status refresh_simt(ngalore_state* st, const uint16_t* const* G, const s
     g.epilogue = EPI_STORE;
     NG_CUDA(launch_simt_gemm<double>(g, stream));
     st->launches += 1;
-    NG_CUDA(eig_batched_launch(st->d_eig + i, st->d_eig_chol + i, 1, std::min(hm.rp, ritz_columns(st)), hm.rp, 1, stream,
+    NG_CUDA(eig_batched_launch(st->d_eig + i, st->d_eig_factor + i, 1, std::min(hm.rp, ritz_columns(st)), hm.rp, 1, stream,
                                &st->launches));
     SimtGemm a{};
     a.m = hm.eM; a.n = hm.rp; a.k = hm.rp;
@@ -670,7 +670,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   const size_t o_chol = take(sizeof(CholProblem) * n_matrices);
   const size_t o_flags = take(sizeof(int) * 2 * n_matrices);
   const size_t o_eig = take(sizeof(EigMat) * n_matrices);
-  const size_t o_eig_chol = take(sizeof(CholProblem) * n_matrices);
+  const size_t o_eig_factor = take(sizeof(FactorMat) * n_matrices);
   const size_t o_eig_redo = take(sizeof(int) * n_matrices);
   size_t eig_n = 1;
   for (const HostMat& hm : st->mats) eig_n = std::max(eig_n, static_cast<size_t>(std::min(hm.rp, ritz_columns(st))));
@@ -719,9 +719,9 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   int* flags = reinterpret_cast<int*>(st->work + o_flags);
   st->d_flags = flags;
   st->d_eig = reinterpret_cast<EigMat*>(st->work + o_eig);
-  st->d_eig_chol = reinterpret_cast<CholProblem*>(st->work + o_eig_chol);
+  st->d_eig_factor = reinterpret_cast<FactorMat*>(st->work + o_eig_factor);
   std::vector<EigMat> eig(n_matrices);
-  std::vector<CholProblem> eig_chol(n_matrices);
+  std::vector<FactorMat> eig_factors(n_matrices);
   st->subspace_set.assign(n_matrices, 0);
 
   st->h_desc.resize(n_matrices);
@@ -777,7 +777,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
       int* redo = reinterpret_cast<int*>(st->work + o_eig_redo) + i;
       eig[i] = EigMat{nullptr, hm.C, hm.rp, Lj, (Lj + 1) & ~1, reinterpret_cast<double*>(wk), reinterpret_cast<double*>(wk + eig_mat), S,
                       reinterpret_cast<double*>(wk + 3 * eig_mat), redo, hm.Xb, hm.rp, nullptr, nullptr, 0, hm.rp};
-      eig_chol[i] = CholProblem{S, Lj, 0, 0.0, redo};
+      eig_factors[i] = eig_factor(eig[i]);
     }
     if (s == 0 && cudaMemcpy(d.wsol, w_init.data(), sizeof(float) * kMaxHistory, cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(NGALORE_ERR_CUDA);
@@ -787,7 +787,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
       cudaMemcpy(st->d_tiles, tiles.data(), sizeof(StreamTile) * n_tiles, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(st->d_hyper, &st->hyper, sizeof(Hyper), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(st->d_eig, eig.data(), sizeof(EigMat) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(st->d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess)
+      cudaMemcpy(st->d_eig_factor, eig_factors.data(), sizeof(FactorMat) * n_matrices, cudaMemcpyHostToDevice) != cudaSuccess)
     return fail(NGALORE_ERR_CUDA);
   st->hyper_dirty = false;
 
@@ -798,8 +798,6 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   // (the limit of a kernel belongs to the process: it must hold for the widest state, whichever is created last)
   if (cudaFuncSetAttribute(orth_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(prop.sharedMemPerBlockOptin)) != cudaSuccess ||
-      cudaFuncSetAttribute(chol_cta_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(chol_cta_smem_bytes<double>(kEigMaxN))) != cudaSuccess ||
       tri_factor_init() != cudaSuccess || eig_init(static_cast<int>(eig_n)) != cudaSuccess)
     return fail(NGALORE_ERR_CUDA);
 

@@ -274,7 +274,7 @@ struct RefreshPlan {
   int n_syrk_tiles = 0;
   // Rayleigh-Ritz rotation: the eigensolver works in the X64, T64 and C64 buffers
   EigMat* d_eig = nullptr;
-  CholProblem* d_eig_chol = nullptr;
+  FactorMat* d_eig_factor = nullptr;
   int eig_max = 0;             // largest matrix it diagonalises
   int sm_count = 0;
   FillJob* d_fill = nullptr;   // the random start Z = Omega of every matrix
@@ -351,8 +351,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     offs[i].Zlo = take(sizeof(__nv_bfloat16) * m.N * m.ldl);
     offs[i].C32 = take(sizeof(float) * m.L * m.L);
     offs[i].C64 = take(sizeof(double) * m.L * m.L);
-    offs[i].X64 = take(sizeof(double) * m.L * m.L);
-    offs[i].T64 = take(sizeof(double) * std::max(static_cast<size_t>(m.L) * m.L, tf_spill_doubles(m.L)));
+    const size_t l2 = std::max(static_cast<size_t>(m.L) * m.L, tf_spill_doubles(m.L));   // (both also hold the factor's rows)
+    offs[i].X64 = take(sizeof(double) * l2);
+    offs[i].T64 = take(sizeof(double) * l2);
     offs[i].D = take(sizeof(double) * m.L);
     offs[i].Rhi = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
     offs[i].Rlo = take(sizeof(__nv_bfloat16) * m.L * m.ldl);
@@ -419,7 +420,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_sy_rest = take(sizeof(SplitJob) * n);
   const size_t o_sz_rest = take(sizeof(SplitJob) * n);
   const size_t o_eig = take(sizeof(EigMat) * n);
-  const size_t o_eig_chol = take(sizeof(CholProblem) * n);
+  const size_t o_eig_factor = take(sizeof(FactorMat) * n);
   const size_t o_eig_redo = take(sizeof(int) * n);
   const size_t o_fill = take(sizeof(FillJob) * n);
   const size_t o_zero_d = take(sizeof(ZeroJob) * n);
@@ -436,7 +437,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   std::vector<SplitJob> sy_rest, sz_rest;
   std::vector<SyrkMat> syrk_m(n);
   std::vector<EigMat> eig(n);
-  std::vector<CholProblem> eig_chol(n);
+  std::vector<FactorMat> eig_factors(n);
   plan.h_maps.resize(static_cast<size_t>(RM_COUNT) * n);
   std::memset(plan.h_maps.data(), 0, sizeof(CUtensorMap) * plan.h_maps.size());
   for (int i = 0; i < n; ++i) {
@@ -467,7 +468,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     int* redo = reinterpret_cast<int*>(plan.buf + o_eig_redo) + i;
     eig[i] = EigMat{m.C32, nullptr, m.L, Lj, Lj, m.X64, m.T64, m.C64, reinterpret_cast<double*>(plan.buf + o_eig_tri[i]),
                     redo, nullptr, 0, m.Rhi, m.Rlo, m.ldl, m.L};
-    eig_chol[i] = CholProblem{m.C64, Lj, 0, 0.0, redo};
+    eig_factors[i] = eig_factor(eig[i]);
     plan.eig_max = std::max(plan.eig_max, Lj);
     CUtensorMap* mp = &plan.h_maps[static_cast<size_t>(i) * RM_COUNT];
     const uint64_t sl = static_cast<uint64_t>(m.ldl) * 2;
@@ -531,8 +532,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.n_split_y_rest = static_cast<int>(sy_rest.size());
   plan.n_split_z_rest = static_cast<int>(sz_rest.size());
   plan.d_eig = reinterpret_cast<EigMat*>(plan.buf + o_eig);
-  plan.d_eig_chol = reinterpret_cast<CholProblem*>(plan.buf + o_eig_chol);
-  std::stable_sort(eig_chol.begin(), eig_chol.end(), [](const CholProblem& a, const CholProblem& b) { return a.L > b.L; });
+  plan.d_eig_factor = reinterpret_cast<FactorMat*>(plan.buf + o_eig_factor);
+  std::stable_sort(eig_factors.begin(), eig_factors.end(), wider);
   plan.d_fill = reinterpret_cast<FillJob*>(plan.buf + o_fill);
   {
     std::vector<FillJob> fill(n);
@@ -557,7 +558,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_split_y_rest, sy_rest.data(), sizeof(SplitJob) * sy_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_split_z_rest, sz_rest.data(), sizeof(SplitJob) * sz_rest.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_eig, eig.data(), sizeof(EigMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(plan.d_eig_chol, eig_chol.data(), sizeof(CholProblem) * n, cudaMemcpyHostToDevice) != cudaSuccess)
+      cudaMemcpy(plan.d_eig_factor, eig_factors.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
 
   // ---- tables of buffers to clear
@@ -771,7 +772,7 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   if ((rc = refresh_tc_gemm(plan, RG_Z_FROM_Y, RP_Z_FROM_Y0, d_ctrl, stream, launches))) return rc;
   if ((rc = refresh_tc_split(plan, false, stream, launches))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Z, RP_GRAM_Z, d_ctrl, stream, launches))) return rc;
-  if (eig_batched_launch(plan.d_eig, plan.d_eig_chol, plan.n, plan.eig_max, plan.l_max, plan.sm_count, stream, launches) != cudaSuccess)
+  if (eig_batched_launch(plan.d_eig, plan.d_eig_factor, plan.n, plan.eig_max, plan.l_max, plan.sm_count, stream, launches) != cudaSuccess)
     return NGALORE_ERR_CUDA;
   // Q orthonormal to about 1e-6 and V orthogonal: so is their product, once its columns are scaled back to unit norm
   // (with the working copies, see finish_refresh; their norms go to D)

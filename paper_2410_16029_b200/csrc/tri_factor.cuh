@@ -40,6 +40,8 @@ struct FactorMat {
   __nv_bfloat16* Rhi;   // L x ld: high part of R^-1
   __nv_bfloat16* Rlo;
   int L, ld;
+  double* R64 = nullptr;         // if set: R^-1 goes here (L x L, fp64) instead; may be C, which is read before
+  const int* only_if = nullptr;  // conditional launches: nothing is done where this word is 0
 };
 
 // Shared memory without the blocks.
@@ -236,11 +238,12 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
 }
 
 template <typename T, bool S_GLOBAL>
-__global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorMat* mats, int smem_bytes, double shift_scale) {
+__global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorMat* mats, int smem_bytes, double shift_scale, int conditional) {
   constexpr int NB = kTfNB, LD = kTfLd, WARPS = kTfThreads / 32;
   extern __shared__ __align__(16) unsigned char tf_smem[];
   __shared__ int counter;
   const FactorMat m = mats[blockIdx.x];
+  if (conditional && *m.only_if == 0) return;
   const int L = m.L, nb = (L + NB - 1) / NB, np = nb * NB;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
   T* Inv0 = reinterpret_cast<T*>(tf_smem);            // [2][NB][LD]
@@ -321,7 +324,11 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
           const int kk = 8 * y + 2 * fk, col = k * NB + kk;
           S[row * LD + kk] = acc[x][y][0];
           S[row * LD + kk + 1] = acc[x][y][1];
-          if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
+          if (m.R64 != nullptr) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? static_cast<double>(acc[x][y][h] * scale) : 0.0;
+          } else if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
             float f[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -404,20 +411,20 @@ inline cudaError_t tri_factor_init() {
 // is added to the unit diagonal, for fp32 matrices in units of L / 65536.
 template <typename T>
 inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, double shift_scale, cudaStream_t stream,
-                                     int64_t* launches) {
+                                     int64_t* launches, bool conditional = false) {
   // as much shared memory as the widest matrix that fits with its blocks, and at least what the widest needs without
   size_t smem = tf_base_smem<T>(l_max, false);
   const bool s_global = smem > static_cast<size_t>(kTfSmemLimit);
   if (s_global) smem = tf_base_smem<T>(l_max, true);
-  for (int l = l_max; l >= 4; l -= 4) {
+  for (int l = l_max; l > 0; l -= 4) {
     const size_t need = tf_base_smem<T>(l, s_global) + tf_block_bytes<T>(l);
     if (need <= static_cast<size_t>(kTfSmemLimit)) { smem = need > smem ? need : smem; break; }
   }
   if (s_global) {
     if (sizeof(T) == 4) return cudaErrorInvalidValue;   // (an fp32 basis of 875 columns needs 147 KB)
-    tri_factor_kernel<double, true><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale);
+    tri_factor_kernel<double, true><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
   } else {
-    tri_factor_kernel<T, false><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale);
+    tri_factor_kernel<T, false><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
   }
   *launches += 1;
   return cudaGetLastError();

@@ -85,3 +85,20 @@ def test_gradient_of_low_rank(r):
     assert np.max(np.abs(P.T @ P - np.eye(r))) <= 1e-5
     R = G64 - P @ (P.T @ G64)
     assert np.linalg.norm(R) <= 1e-4 * np.linalg.norm(G64)
+
+
+def test_widest_bases_beside_narrow_ones():
+    """Above about 700 columns the factorisation of the Gram matrix of the vectors keeps its rows in global memory, for
+    every matrix of the launch."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    shapes = [(1448, 800), (160, 48), (600, 200), (4, 160)]
+    G = [_planted(M, N, min(M, N, 6), 700 + i, 2e-4) for i, (M, N) in enumerate(shapes)]
+    opt = NGaLore(shapes, 724, 0, 0, ritz_columns=-1)
+    opt.refresh_subspace(G)
+    torch.cuda.synchronize()
+    assert opt.poll_status()[0] == 0
+    for i, (M, N) in enumerate(shapes):
+        r = opt.rank(i)
+        assert r == min(M, N, 724)
+        _check(opt.get_subspace(i).double().cpu().numpy(), G[i] if not opt.projects_right(i) else G[i].T.contiguous(), r, min(r, 4))
