@@ -165,12 +165,12 @@ __device__ __forceinline__ uint32_t instr_desc(int n, bool a_mn_major, bool fp16
          (static_cast<uint32_t>(kTcBM >> 4) << 24);
 }
 
-template <int BN, int NA, int NB, int STAGES, int NEPI>
+template <int BN, int NA, int NB, int STAGES, int NEPI, int MT = 1>
 struct TcSmem {
   static constexpr int kABytes = kTcBM * kTcBK * 2;           // 16 KB
   static constexpr int kBChunkBytes = 64 * kTcBK * 2;         // one 64-column chunk: 64 K rows x 128 B
   static constexpr int kBBytes = (BN / 64) * kBChunkBytes;    // per B operand
-  static constexpr int kStageBytes = NA * kABytes + NB * kBBytes;
+  static constexpr int kStageBytes = MT * NA * kABytes + NB * kBBytes;
   static constexpr int kEpiWarpBytes = 32 * 32 * 4;           // 32 rows x 32 floats, 16-byte words swizzled by the row
   static constexpr int kBarOffset = STAGES * kStageBytes + NEPI * kEpiWarpBytes;
   static constexpr int kTotal = kBarOffset + 256 + 1024;      // barriers + slack for 1024-byte alignment
@@ -182,11 +182,14 @@ enum { TC_EPI_PROJECT = 0, TC_EPI_STORE = 2 };
 // hi*hi, hi*lo and lo*hi are accumulated (lo*lo is below fp32 resolution).  A_MN: A is stored with its
 // row index contiguous (A^T row-major), staged as two 64-row chunks like B.  F16: the operands are fp16
 // (otherwise bf16); TMA moves either as opaque 16-bit elements.
-template <int BN, int NA, int NB, int STAGES, int EPI, int NEPI, bool A_MN, bool F16 = false>
+// MT = 2: tiles of 256 rows, two accumulators that share the B operand.
+template <int BN, int NA, int NB, int STAGES, int EPI, int NEPI, bool A_MN, bool F16 = false, int MT = 1>
 __global__ void __launch_bounds__(64 + 32 * NEPI, 1)
 tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__ tiles, const int* __restrict__ cta_first,
                const MatDesc* __restrict__ mats, Ctrl* ctrl, const TcProblem* __restrict__ probs) {
-  using L = TcSmem<BN, NA, NB, STAGES, NEPI>;
+  using L = TcSmem<BN, NA, NB, STAGES, NEPI, MT>;
+  static_assert(MT == 1 || NEPI == 8, "a group of epilogue warps for each half of a tall tile");
+  constexpr int NBUF = 2 * MT * BN <= 512 ? 2 : 1;   // accumulator buffers
   extern __shared__ unsigned char tc_smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOffset);
@@ -200,7 +203,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar + s, 1); mbar_init(empty_bar + s, 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, 4 * MT); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -237,24 +240,27 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
         const int n_rem = tile.cols - tile.n0;
         const int n_eff = n_rem >= BN ? BN : ((n_rem + 15) & ~15);
         const int nchunks = (n_eff + 63) >> 6;
-        const uint32_t bytes = NA * L::kABytes + NB * nchunks * L::kBChunkBytes;
+        const int mts = MT == 2 && tile.rows - tile.m0 > kTcBM ? 2 : 1;
+        const uint32_t bytes = mts * NA * L::kABytes + NB * nchunks * L::kBChunkBytes;
         for (int kb = 0; kb < tile.kblocks; ++kb) {
           if (!mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag)) { ok = false; break; }
           unsigned char* sA = smem + stage * L::kStageBytes;
           mbar_expect_tx(full_bar + stage, bytes);
           const int k = tile.k0 + kb * kTcBK;
 #pragma unroll
-          for (int na = 0; na < NA; ++na) {
+          for (int x = 0; x < MT * NA; ++x) {
+            const int na = x % NA, m0 = tile.m0 + x / NA * kTcBM;
+            if (x >= mts * NA) break;
             if (A_MN) {
-              tma_load_2d(sA + na * L::kABytes, mapA + na, tile.m0, k, full_bar + stage);
-              tma_load_2d(sA + na * L::kABytes + L::kBChunkBytes, mapA + na, tile.m0 + 64, k, full_bar + stage);
+              tma_load_2d(sA + x * L::kABytes, mapA + na, m0, k, full_bar + stage);
+              tma_load_2d(sA + x * L::kABytes + L::kBChunkBytes, mapA + na, m0 + 64, k, full_bar + stage);
             } else {
-              tma_load_2d(sA + na * L::kABytes, mapA + na, k, tile.m0, full_bar + stage);
+              tma_load_2d(sA + x * L::kABytes, mapA + na, k, m0, full_bar + stage);
             }
           }
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb) {
-            unsigned char* sB = sA + NA * L::kABytes + nb * L::kBBytes;
+            unsigned char* sB = sA + MT * NA * L::kABytes + nb * L::kBBytes;
             for (int c = 0; c < nchunks; ++c)
               tma_load_2d(sB + c * L::kBChunkBytes, mapB0 + nb, tile.n0 + c * 64, k, full_bar + stage);
           }
@@ -278,30 +284,35 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
         const int n_rem = tile.cols - tile.n0;
         const int n_eff = n_rem >= BN ? BN : ((n_rem + 15) & ~15);
         const uint32_t idesc = instr_desc(n_eff, A_MN, F16);
-        const int buf = local & 1;
-        const uint32_t tphase = (local >> 1) & 1u;
+        const int mts = MT == 2 && tile.rows - tile.m0 > kTcBM ? 2 : 1;
+        const int buf = local % NBUF;
+        const uint32_t tphase = (local / NBUF) & 1u;
         if (!mbar_wait(tempty_bar + buf, tphase ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + buf * BN;
         for (int kb = 0; kb < tile.kblocks; ++kb) {
           if (!mbar_wait(full_bar + stage, phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint32_t aaddr0 = smem_u32(smem + stage * L::kStageBytes);
-          bool first = (kb == 0);
 #pragma unroll
-          for (int na = 0; na < NA; ++na) {
+          for (int mt = 0; mt < MT; ++mt) {
+            if (mt >= mts) break;
+            const uint32_t tmem_d = tmem_base + (buf * MT + mt) * BN;
+            bool first = (kb == 0);
 #pragma unroll
-            for (int nb = 0; nb < NB; ++nb) {
-              if (na == 1 && nb == 1) continue;  // lo * lo is dropped
-              const uint32_t aaddr = aaddr0 + na * L::kABytes;
-              const uint32_t baddr = aaddr0 + NA * L::kABytes + nb * L::kBBytes;
+            for (int na = 0; na < NA; ++na) {
 #pragma unroll
-              for (int kk = 0; kk < kTcBK / 16; ++kk) {
-                const uint64_t adesc = A_MN ? smem_desc(aaddr + kk * 2048, L::kBChunkBytes, 1024)
-                                            : smem_desc(aaddr + kk * 32, 16, 1024);
-                const uint64_t bdesc = smem_desc(baddr + kk * 2048, L::kBChunkBytes, 1024);
-                tc_mma(tmem_d, adesc, bdesc, idesc, first ? 0u : 1u);
-                first = false;
+              for (int nb = 0; nb < NB; ++nb) {
+                if (na == 1 && nb == 1) continue;  // lo * lo is dropped
+                const uint32_t aaddr = aaddr0 + (mt * NA + na) * L::kABytes;
+                const uint32_t baddr = aaddr0 + MT * NA * L::kABytes + nb * L::kBBytes;
+#pragma unroll
+                for (int kk = 0; kk < kTcBK / 16; ++kk) {
+                  const uint64_t adesc = A_MN ? smem_desc(aaddr + kk * 2048, L::kBChunkBytes, 1024)
+                                              : smem_desc(aaddr + kk * 32, 16, 1024);
+                  const uint64_t bdesc = smem_desc(baddr + kk * 2048, L::kBChunkBytes, 1024);
+                  tc_mma(tmem_d, adesc, bdesc, idesc, first ? 0u : 1u);
+                  first = false;
+                }
               }
             }
           }
@@ -321,11 +332,13 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
     const int group = (warp - 2) >> 2;
     float* stg = reinterpret_cast<float*>(smem + STAGES * L::kStageBytes + (warp - 2) * L::kEpiWarpBytes);
     bool ok = true;
-    const int first = kGroups == 2 ? group : 0;
+    // (of tall tiles, each group drains its half of all of them)
+    constexpr int kStep = MT == 2 ? 1 : kGroups;
+    const int first = kStep == 2 ? group : 0, half = MT == 2 ? group : 0;
     TcTile tile;
     if (t_begin + first < t_end) tile = tiles[t_begin + first];
-    for (int local = first; t_begin + local < t_end && ok; local += kGroups) {
-      const TcTile next = tiles[min(t_begin + local + kGroups, t_end - 1)];
+    for (int local = first; t_begin + local < t_end && ok; local += kStep) {
+      const TcTile next = tiles[min(t_begin + local + kStep, t_end - 1)];
       float* out;
       __nv_bfloat16 *out_hi = nullptr, *out_lo = nullptr;
       int rows_total, out_cols, ld_out, ld16 = 0;
@@ -347,17 +360,22 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       }
       const int n_rem = out_cols - tile.n0;
       const int n_eff = n_rem >= BN ? BN : ((n_rem + 15) & ~15);
-      const int buf = local & 1;
-      const uint32_t tphase = (local >> 1) & 1u;
-      const int row_base = tile.m0 + quarter * 32;
+      const int buf = local % NBUF;
+      const uint32_t tphase = (local / NBUF) & 1u;
+      const int row_base = tile.m0 + half * kTcBM + quarter * 32;
       const int sub_row = lane >> 3, sub_col = (lane & 7) * 4;
       if (!mbar_wait(tfull_bar + buf, tphase, abort_flag)) { ok = false; break; }
       tc_fence_after();
+      if (half == 1 && tile.rows - tile.m0 <= kTcBM) {   // nothing in this half
+        if (lane == 0) mbar_arrive(tempty_bar + buf);
+        tile = next;
+        continue;
+      }
 #pragma unroll
       for (int c0 = 0; c0 < BN; c0 += 32) {
         if (c0 < n_eff) {
           uint32_t r[32];
-          tc_ld32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * BN + c0), r);
+          tc_ld32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>((buf * MT + half) * BN + c0), r);
           tc_wait_ld();
           if (c0 + 32 >= n_eff) {
             // all TMEM reads of this tile are done: hand the buffer back before the global traffic

@@ -233,10 +233,14 @@ constexpr int kRefBN = 128;
 // The products with G take tiles of 256 columns where most of the work has bases that wide: a 128 x 256 tile needs
 // three quarters of the shared-memory reads per multiply-add, and G is read half as often.
 constexpr int kRefWideBN = 256;
-constexpr int kRefWideStages1 = 2;  // NA = 1, NB = 2: 80 KB per stage
-constexpr int kRefWideStages0 = 4;  // NA = 1, NB = 1: 48 KB per stage
-constexpr int kRefStages1 = 4;  // NA = 1, NB = 2: 48 KB per stage
-constexpr int kRefStages0 = 6;  // NA = 1, NB = 1: 32 KB per stage
+// A product with G (one part of A, NB parts of B): 192 KB of stages, as many as go.
+template <int BN, int NB, int MT, bool MN>
+struct RefProduct {
+  static constexpr int kEpiWarps = 4 * MT, kThreads = 64 + 32 * kEpiWarps;
+  static constexpr int kStages = 192 / (16 * MT + NB * BN / 8);
+  static constexpr int kSmem = TcSmem<BN, 1, NB, kStages, kEpiWarps, MT>::kTotal;
+  static constexpr auto kernel = tc_gemm_kernel<BN, 1, NB, kStages, TC_EPI_STORE, kEpiWarps, MN, false, MT>;
+};
 constexpr int kRefStages2 = 3;  // NA = 2, NB = 2: 64 KB per stage
 
 struct RefreshPlan {
@@ -254,7 +258,8 @@ struct RefreshPlan {
   int* d_first[RG_COUNT] = {};   // first tile of every CTA
   int n_tiles[RG_COUNT] = {};
   int grid[RG_COUNT] = {};
-  bool wide = false;           // the products with G take tiles of kRefWideBN columns
+  bool wide = false;           // the products with G take tiles of kRefWideBN columns ...
+  bool tall = false;           // ... and of 256 rows
   std::vector<int> atomic_mats[RG_COUNT];  // matrices whose K is split for this GEMM (output must be zeroed)
   // buffers to clear before GEMM kind g (the outputs of atomic_mats[g]); entry RG_COUNT: every matrix's X64
   ZeroJob* d_zero[RG_COUNT + 1] = {};
@@ -316,6 +321,22 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     }
     plan.wide = 2.0 * wide >= all;
   }
+  {
+    // Tiles of 256 rows: what bounds the products with G is the L2 bandwidth (10 TB/s), and two accumulators that share
+    // the basis halve its part of the traffic.  1.1B shapes, a product with two parts 1.86 -> 1.59 ms, with one 1.02 ->
+    // 0.94; 60M 44 -> 40 and 36 -> 34 us.  Not where that leaves SMs without a tile.  256 x 256 accumulators fill the
+    // tensor memory, so the epilogue of a tile is not hidden behind the next: of 15 K blocks a tile (130M shapes) 140 us
+    // become 146 (two parts) and 88 become 96 (one), of 40 (1.1B) it pays.
+    const int bn = plan.wide ? kRefWideBN : kRefBN;
+    long long tiles_tall = 0, blocks = 0;
+    for (const MatDesc& d : mats) {
+      const long long cols = (d.rp + bn - 1) / bn, ty = (d.M + 2 * kTcBM - 1) / (2 * kTcBM) * cols, tz = (d.N + 2 * kTcBM - 1) / (2 * kTcBM) * cols;
+      tiles_tall += ty + tz;
+      blocks += ty * ((d.N + kTcBK - 1) / kTcBK) + tz * ((d.M + kTcBK - 1) / kTcBK);
+    }
+    plan.tall = tiles_tall >= 2 * sm_count && (!plan.wide || blocks >= 24 * tiles_tall);
+  }
+  auto tile_rows = [&](int g) { return plan.tall && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? 2 * kTcBM : kTcBM; };
   auto tile_cols = [&](int g) { return plan.wide && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? kRefWideBN : kRefBN; };
   auto add_tiles = [&](int g, int i, int out_rows, int out_cols, int K, long long target_kb) {
     const int kb_total = (K + kTcBK - 1) / kTcBK;
@@ -328,7 +349,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     const bool symmetric = g == RG_GRAM_Y || g == RG_GRAM_Z;   // the lower triangle is enough
     for (int n0 = 0; n0 < out_cols; n0 += tile_cols(g))
       for (int sp = 0; sp < splits; ++sp)
-        for (int m0 = symmetric ? n0 / kTcBM * kTcBM : 0; m0 < out_rows; m0 += kTcBM) {
+        for (int m0 = symmetric ? n0 / kTcBM * kTcBM : 0; m0 < out_rows; m0 += tile_rows(g)) {
           const int kb0 = sp * kb_per;
           int kbn = std::min(kb_per, kb_total - kb0);
           if (g == RG_APPLY_TRI) kbn = std::min(kbn, (n0 + kRefBN) / kTcBK);
@@ -376,10 +397,10 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
         case RG_GRAM_Z: rows = m.L; cols = m.L; K = m.N; break;
         default: rows = m.M; cols = m.L; K = m.L; break;  // RG_APPLY_Y, RG_APPLY_TRI
       }
-      total_kb += static_cast<long long>((rows + kTcBM - 1) / kTcBM) * ((cols + tile_cols(g) - 1) / tile_cols(g)) *
+      total_kb += static_cast<long long>((rows + tile_rows(g) - 1) / tile_rows(g)) * ((cols + tile_cols(g) - 1) / tile_cols(g)) *
                   ((K + kTcBK - 1) / kTcBK);
     }
-    long long target = (total_kb + sm_count - 1) / sm_count / 4;
+    long long target = (total_kb * (tile_rows(g) / kTcBM) + sm_count - 1) / sm_count / 4;
     if (target < 16) target = 16;
     for (int i = 0; i < n; ++i) {
       const RefreshMat& m = plan.mats[i];
@@ -597,27 +618,17 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     plan.device_bytes += sizeof(ZeroJob) * (jobs.size() + 1);
   }
 
-  using L1 = TcSmem<kRefBN, 1, 2, kRefStages1, 4>;
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
-  using L0 = TcSmem<kRefBN, 1, 1, kRefStages0, 4>;
-  using LW1 = TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>;
-  using LW0 = TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>;
-  if (cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW0::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW0::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW1::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, LW1::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, L0::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, L0::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, L1::kTotal) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, L1::kTotal) != cudaSuccess ||
+  auto init = [](auto p) { return cudaFuncSetAttribute(p.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p.kSmem) == cudaSuccess; };
+  auto init_both = [&](auto p, auto q) { return init(p) && init(q); };
+  if (!init_both(RefProduct<kRefWideBN, 1, 1, false>{}, RefProduct<kRefWideBN, 1, 1, true>{}) ||
+      !init_both(RefProduct<kRefWideBN, 2, 1, false>{}, RefProduct<kRefWideBN, 2, 1, true>{}) ||
+      !init_both(RefProduct<kRefWideBN, 1, 2, false>{}, RefProduct<kRefWideBN, 1, 2, true>{}) ||
+      !init_both(RefProduct<kRefWideBN, 2, 2, false>{}, RefProduct<kRefWideBN, 2, 2, true>{}) ||
+      !init_both(RefProduct<kRefBN, 1, 1, false>{}, RefProduct<kRefBN, 1, 1, true>{}) ||
+      !init_both(RefProduct<kRefBN, 2, 1, false>{}, RefProduct<kRefBN, 2, 1, true>{}) ||
+      !init_both(RefProduct<kRefBN, 1, 2, false>{}, RefProduct<kRefBN, 1, 2, true>{}) ||
+      !init_both(RefProduct<kRefBN, 2, 2, false>{}, RefProduct<kRefBN, 2, 2, true>{}) ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true>,
@@ -639,23 +650,21 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     *launches += 1;
   }
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
-  const int threads = 64 + 32 * 4;
+  const int threads = 64 + 32 * 8;
   auto product = [&](auto a_mn) {   // a product with G; a_mn: with G^T
     constexpr bool MN = decltype(a_mn)::value;
-    if (plan.wide) {
-      if (high_only)
-        tc_gemm_kernel<kRefWideBN, 1, 1, kRefWideStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 1, kRefWideStages0, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      else
-        tc_gemm_kernel<kRefWideBN, 1, 2, kRefWideStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefWideBN, 1, 2, kRefWideStages1, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
+    auto run = [&](auto p) {
+      p.kernel<<<plan.grid[g], p.kThreads, p.kSmem, stream>>>(plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl,
+                                                              plan.d_probs[problem]);
+    };
+    if (plan.wide && plan.tall) {
+      if (high_only) run(RefProduct<kRefWideBN, 1, 2, MN>{}); else run(RefProduct<kRefWideBN, 2, 2, MN>{});
+    } else if (plan.wide) {
+      if (high_only) run(RefProduct<kRefWideBN, 1, 1, MN>{}); else run(RefProduct<kRefWideBN, 2, 1, MN>{});
+    } else if (plan.tall) {
+      if (high_only) run(RefProduct<kRefBN, 1, 2, MN>{}); else run(RefProduct<kRefBN, 2, 2, MN>{});
     } else {
-      if (high_only)
-        tc_gemm_kernel<kRefBN, 1, 1, kRefStages0, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 1, kRefStages0, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
-      else
-        tc_gemm_kernel<kRefBN, 1, 2, kRefStages1, TC_EPI_STORE, 4, MN><<<plan.grid[g], threads, TcSmem<kRefBN, 1, 2, kRefStages1, 4>::kTotal, stream>>>(
-            plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
+      if (high_only) run(RefProduct<kRefBN, 1, 1, MN>{}); else run(RefProduct<kRefBN, 2, 1, MN>{});
     }
   };
   switch (g) {
@@ -663,11 +672,11 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     case RG_Z_FROM_Y: product(std::true_type{}); break;
     case RG_GRAM_Y:
     case RG_GRAM_Z:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true><<<plan.grid[g], 64 + 32 * 8, L2::kTotal, stream>>>(
+      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
           plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
     default:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false><<<plan.grid[g], 64 + 32 * 8, L2::kTotal, stream>>>(
+      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
           plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
       break;
   }

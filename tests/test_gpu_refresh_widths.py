@@ -51,3 +51,34 @@ def test_mixed_widths():
         r = min(676, M, N)
         _check(opt, i, made[i][1], r, min(10, N // 2))
     assert opt.poll_status()[0] == 0
+
+
+@pytest.mark.parametrize("M,N,r", [(80072, 264, 64), (76904, 1560, 200)])
+def test_tall_tiles(M, N, r):
+    """Sets with at least two 256-row tiles of the products with G for every multiprocessor take such tiles (narrow bases,
+    and wide ones with long products).  Rows that end in the first or in the second half of a tile; P orthonormal, its
+    columns Ritz vectors of G (bounds as for smaller matrices: 1e-5 and 1e-4 of the larger diagonal entry) and the leading
+    ones the planted singular vectors."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    q = 6
+    U = torch.linalg.qr(torch.randn(M, q, generator=gen, device="cuda"))[0]
+    V = torch.linalg.qr(torch.randn(N, q, generator=gen, device="cuda"))[0]
+    G = ((U * 0.7 ** torch.arange(q, device="cuda")) @ V.T).add_(torch.randn(M, N, generator=gen, device="cuda"), alpha=2e-5).bfloat16()
+    opt = NGaLore([(M, N)], r, 0, 0, ritz_columns=-1)
+    opt.refresh_subspace([G])
+    torch.cuda.synchronize()
+    assert opt.poll_status()[0] == 0
+    P = opt.get_subspace(0).double()
+    G64 = G.double()
+    if opt.projects_right(0):
+        G64, U = G64.T, V
+    assert (P.T @ P - torch.eye(r, device="cuda")).abs().max().item() <= 1e-5
+    B = P.T @ G64
+    C = B @ B.T
+    d = torch.diagonal(C)
+    off = (C - torch.diag(d)).abs() / torch.sqrt(torch.maximum(d[:, None], d[None, :]) * d[0])
+    assert off.max().item() <= 1e-4
+    # (the bf16 rounding of G, 2^-9 of an entry at most, tilts its singular vectors from the planted ones)
+    assert (1.0 - (P[:, :q] * U.double()).sum(0).abs()).max().item() <= 1e-3
