@@ -452,8 +452,9 @@ __global__ void zero_split_slots_kernel(const MatDesc* mats, const int* split_ma
 // first[c] is the first of CTA c (grid + 1 entries).  A tile costs its K blocks and about three more for the start of its
 // pipeline.  (Strided over the sorted list instead, the first CTAs got the longest tile of every round: 1.1B shapes,
 // Z = G^T Q 2.2 -> 1.83 ms, step projection 0.92 -> 0.875; 130M 88 -> 82 us; 350M 218 -> 203 us.)
-inline void tc_assign_tiles(std::vector<TcTile>& tiles, int grid, std::vector<int>& first) {
-  std::stable_sort(tiles.begin(), tiles.end(), [](const TcTile& a, const TcTile& b) { return a.kblocks > b.kblocks; });
+// in_order: the tiles are handed out as they come, so that neighbours in the list run at about the same time.
+inline void tc_assign_tiles(std::vector<TcTile>& tiles, int grid, std::vector<int>& first, bool in_order = false) {
+  if (!in_order) std::stable_sort(tiles.begin(), tiles.end(), [](const TcTile& a, const TcTile& b) { return a.kblocks > b.kblocks; });
   std::vector<std::vector<TcTile>> of(grid);
   std::vector<std::pair<long long, int>> heap;   // (work so far, CTA), least on top
   for (int c = 0; c < grid; ++c) heap.push_back({0, c});
