@@ -163,18 +163,23 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
   __syncwarp();
 #pragma unroll 1
   for (int c0 = 0; c0 < kTfNB; c0 += 8) {
-    // the 8 x 8 block: its factor (lane = row), then the inverse of that (lane = column)
+    // the 8 x 8 block: every lane computes all of its factor (shuffles would double the length of the chain), then one
+    // column of the inverse
     {
-      T r[8], x[8], inv[8];
-      tf_load8(W + (c0 + (lane & 7)) * kTfLdW + c0, r);
+      T r[8][8], x[8], inv[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) tf_load8(W + (c0 + i) * kTfLdW + c0, r[i]);
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
-        T d = __shfl_sync(0xffffffffu, r[t], t, 8);
+        T d = r[t][t];
         if (!(d > tiny)) d = tiny;
         inv[t] = tf_rsqrt(d);
-        r[t] *= inv[t];
 #pragma unroll
-        for (int j = t + 1; j < 8; ++j) r[j] -= r[t] * __shfl_sync(0xffffffffu, r[t], j, 8);
+        for (int i = t + 1; i < 8; ++i) r[i][t] *= inv[t];
+#pragma unroll
+        for (int j = t + 1; j < 8; ++j)
+#pragma unroll
+          for (int i = j; i < 8; ++i) r[i][j] -= r[i][t] * r[j][t];
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) x[i] = i == (lane & 7) ? T(1) : T(0);
@@ -182,7 +187,7 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
       for (int t = 0; t < 8; ++t) {
         x[t] *= inv[t];
 #pragma unroll
-        for (int i = t + 1; i < 8; ++i) x[i] -= __shfl_sync(0xffffffffu, r[t], i, 8) * x[t];
+        for (int i = t + 1; i < 8; ++i) x[i] -= r[i][t] * x[t];
       }
       if (lane < 8) {
 #pragma unroll
