@@ -304,12 +304,11 @@ inline ngalore_status tc_backproject_init() {
   return NGALORE_OK;
 }
 
-// W <- (1 - lr wd) W - lr P u for the matrices [mat0, mat1), through the tensor maps tc_bind_buffers set up.  last: the
+// W <- (1 - lr wd) W - lr P u for the tiles [t0, t1) of TcPlan::d_tiles_back, through the tensor maps tc_bind_buffers set up.  last: the
 // launch ends the step (it moves the counters on).  chained: nothing but the step's own kernels sits before it in the
 // stream (no event to wait for), so it may be a programmatic dependent launch.
-inline ngalore_status tc_backproject_range(TcPlan& plan, int mat0, int mat1, const MatDesc* d_mats, Ctrl* d_ctrl,
+inline ngalore_status tc_backproject_range(TcPlan& plan, int t0, int t1, const MatDesc* d_mats, Ctrl* d_ctrl,
                                            const Hyper* d_hyper, bool last, bool chained, cudaStream_t stream, int64_t* launches) {
-  const int t0 = plan.back_tile0[mat0], t1 = plan.back_tile0[mat1];
   if (t1 <= t0) return NGALORE_OK;
   const int grid = (t1 - t0) < plan.grid_back ? (t1 - t0) : plan.grid_back;
   auto launch = [&](auto kernel, size_t smem) {
@@ -325,7 +324,7 @@ inline ngalore_status tc_backproject_range(TcPlan& plan, int mat0, int mat1, con
 // W <- (1 - lr wd) W - lr P u for every matrix, and the end of the step.
 inline ngalore_status tc_backproject(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
                                      cudaStream_t stream, int64_t* launches) {
-  return tc_backproject_range(plan, 0, plan.n_mats, d_mats, d_ctrl, d_hyper, true, true, stream, launches);
+  return tc_backproject_range(plan, 0, plan.n_tiles_back, d_mats, d_ctrl, d_hyper, true, true, stream, launches);
 }
 
 }  // namespace ngalore

@@ -104,11 +104,14 @@ struct ngalore_state {
   int n_wjobs = 0, n_ntiles = 0, n_wtiles = 0;
   // small-rank path (every r' <= 8): the step as two bandwidth kernels
   SrPlan sr;
-  // host-buffer staging; W travels in groups of matrices so that the copies in, the back-projection and the
-  // copies out of different groups overlap
+  // host-buffer staging (all G, then all W); W travels in groups of rows so that the copies in, the back-projection and
+  // the copies out of different groups overlap
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   cudaEvent_t ev_begin = nullptr, ev_G = nullptr, ev_out = nullptr;
-  std::vector<int> group_first;             // first matrix of every group, plus n
+  struct HostPart { int mat, row0, row1; };
+  std::vector<HostPart> host_parts;         // rows of W in the order of their transfer
+  std::vector<int> group_part, group_tile;  // first part, first back-projection tile of every group, plus the ends
+  PointerAttributeFn pointer_attribute = nullptr;
   std::vector<cudaEvent_t> ev_w_in, ev_w_done;
   char* stage = nullptr;
   size_t stage_bytes = 0;
@@ -387,7 +390,7 @@ ngalore_status refresh_impl(ngalore_state* st, const uint16_t* const* G_in, cons
   return finish_refresh(st, st->refresh_tc_idx, true, stream, true, true);
 }
 
-// grouped: the caller delivers W in the groups of ngalore_state::group_first; the back-projection of a group waits
+// grouped: the caller delivers W in the groups of ngalore_state::group_part; the back-projection of a group waits
 // for that group's event ev_w_in and records ev_w_done (host-buffer step, tensor-core path only).
 ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* const* G, cudaStream_t stream,
                          bool grouped = false) {
@@ -486,16 +489,16 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
         if (st->upd_first[ug + 1] == i + 1) NG_CUDA(cudaEventRecord(st->ev_upd[ug], stream));
     }
   } else if (grouped) {
-    for (size_t g = 0; g + 1 < st->group_first.size(); ++g) {
+    for (size_t g = 0; g + 1 < st->group_tile.size(); ++g) {
       NG_CUDA(cudaStreamWaitEvent(stream, st->ev_w_in[g], 0));
-      if ((rc = tc_backproject_range(st->tc, st->group_first[g], st->group_first[g + 1], st->d_desc, st->d_ctrl,
-                                     st->d_hyper, g + 2 == st->group_first.size(), false, stream, &st->launches)))
+      if ((rc = tc_backproject_range(st->tc, st->group_tile[g], st->group_tile[g + 1], st->d_desc, st->d_ctrl,
+                                     st->d_hyper, g + 2 == st->group_tile.size(), false, stream, &st->launches)))
         return rc;
       NG_CUDA(cudaEventRecord(st->ev_w_done[g], stream));
     }
   } else if (st->upd_first.size() > 1) {
     for (size_t ug = 0; ug + 1 < st->upd_first.size(); ++ug) {
-      if ((rc = tc_backproject_range(st->tc, st->upd_first[ug], st->upd_first[ug + 1], st->d_desc, st->d_ctrl,
+      if ((rc = tc_backproject_range(st->tc, st->tc.back_tile0[st->upd_first[ug]], st->tc.back_tile0[st->upd_first[ug + 1]], st->d_desc, st->d_ctrl,
                                      st->d_hyper, ug + 2 == st->upd_first.size(), false, stream, &st->launches)))
         return rc;
       NG_CUDA(cudaEventRecord(st->ev_upd[ug], stream));
@@ -933,14 +936,12 @@ ngalore_status ngalore_step_host(ngalore_state* st, float* const* W_host, const 
   DeviceGuard guard(st->device);
   if (!guard.ok) return NGALORE_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  auto host_elems = [&](int i) { return static_cast<size_t>(st->mats[i].M) * st->mats[i].N; };
   if (st->stage == nullptr) {
     size_t off = 0;
     std::vector<size_t> ow(st->n), og(st->n);
-    for (int i = 0; i < st->n; ++i) {
-      const size_t mn = static_cast<size_t>(st->mats[i].M) * st->mats[i].N;
-      ow[i] = off; off += align_up(mn * sizeof(float));
-      og[i] = off; off += align_up(mn * sizeof(uint16_t));
-    }
+    for (int i = 0; i < st->n; ++i) { og[i] = off; off += align_up(host_elems(i) * sizeof(uint16_t)); }
+    for (int i = 0; i < st->n; ++i) { ow[i] = off; off += align_up(host_elems(i) * sizeof(float)); }
     if (cudaMalloc(&st->stage, off) != cudaSuccess) { st->stage = nullptr; return NGALORE_ERR_ALLOC; }
     st->stage_bytes = off;
     st->stage_W.resize(st->n); st->stage_G.resize(st->n);
@@ -966,46 +967,107 @@ ngalore_status ngalore_step_host(ngalore_state* st, float* const* W_host, const 
     return NGALORE_OK;
   }
   // Pipelined: only the back-projection touches W, so the gradients go in first and the projection and the
-  // history phase run while W is still arriving; W then moves in about eight groups of matrices, each group's
-  // copy in, back-projection and copy out chained by events, so that the two directions of the link overlap.
+  // history phase run while W is still arriving; W then moves in groups of rows, each group's copy in, back-projection
+  // and copy out chained by events, so that the two directions of the link overlap.  What is left beside the copies in
+  // is the last group's way back, so a group is small: a 32nd of W, but at least 2 MB (a copy of 8 MB spends 3 % of its
+  // time on being issued).  Buffers that lie side by side, on either side of the link, travel in one copy.
+  // 60M shapes, 348 MB in and 232 MB out at 55 GB/s: 9.8 ms with a copy for each matrix and eight groups of whole
+  // matrices (the last of them a quarter of W), 7.7 ms so.
   if (st->copy_in == nullptr) {
     NG_CUDA(cudaStreamCreateWithFlags(&st->copy_in, cudaStreamNonBlocking));
     NG_CUDA(cudaStreamCreateWithFlags(&st->copy_out, cudaStreamNonBlocking));
     NG_CUDA(cudaEventCreateWithFlags(&st->ev_begin, cudaEventDisableTiming));
     NG_CUDA(cudaEventCreateWithFlags(&st->ev_G, cudaEventDisableTiming));
     NG_CUDA(cudaEventCreateWithFlags(&st->ev_out, cudaEventDisableTiming));
+    cudaDriverEntryPointQueryResult found;
+    void* fn = nullptr;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &fn, cudaEnableDefault, &found) == cudaSuccess)
+      st->pointer_attribute = reinterpret_cast<PointerAttributeFn>(fn);
     size_t total = 0;
-    for (const HostMat& hm : st->mats) total += static_cast<size_t>(hm.M) * hm.N;
-    const int want = st->n < 8 ? st->n : 8;
-    st->group_first.assign(1, 0);
+    for (int i = 0; i < st->n; ++i) total += host_elems(i) * sizeof(float);
+    const size_t size = std::max<size_t>(2 << 20, (total + 31) / 32);
+    st->group_part.assign(1, 0);
+    st->group_tile.assign(1, 0);
     size_t acc = 0;
     for (int i = 0; i < st->n; ++i) {
-      acc += static_cast<size_t>(st->mats[i].M) * st->mats[i].N;
-      const size_t done_groups = st->group_first.size();
-      if (i + 1 < st->n && static_cast<int>(done_groups) < want && acc * want >= total * done_groups)
-        st->group_first.push_back(i + 1);
+      const HostMat& hm = st->mats[i];
+      const int row_tiles = (hm.M + kTcBM - 1) / kTcBM;
+      const int across = (st->tc.back_tile0[i + 1] - st->tc.back_tile0[i]) / row_tiles;
+      int from = 0;
+      for (int t = 1; t <= row_tiles; ++t) {
+        const int row = std::min(t * kTcBM, hm.M);
+        acc += static_cast<size_t>(row - (t - 1) * kTcBM) * hm.N * sizeof(float);
+        const bool full = acc >= size;
+        if (!full && t < row_tiles) continue;
+        st->host_parts.push_back({i, from, row});
+        from = row;
+        if (full || i + 1 == st->n) {
+          st->group_part.push_back(static_cast<int>(st->host_parts.size()));
+          st->group_tile.push_back(st->tc.back_tile0[i] + t * across);
+          acc = 0;
+        }
+      }
     }
-    st->group_first.push_back(st->n);
-    const size_t ng = st->group_first.size() - 1;
+    const size_t ng = st->group_tile.size() - 1;
     st->ev_w_in.resize(ng); st->ev_w_done.resize(ng);
     for (size_t g = 0; g < ng; ++g) {
       NG_CUDA(cudaEventCreateWithFlags(&st->ev_w_in[g], cudaEventDisableTiming));
       NG_CUDA(cudaEventCreateWithFlags(&st->ev_w_done[g], cudaEventDisableTiming));
     }
   }
-  const size_t ng = st->group_first.size() - 1;
+  // Copies that continue the one before on both sides are joined, if the host memory is of one allocation (two that
+  // happen to be neighbours may not be copied across).
+  struct Run {
+    ngalore_state* st;
+    cudaMemcpyKind kind;
+    cudaStream_t stream;
+    char *dst = nullptr, *src = nullptr;
+    size_t bytes = 0;
+    bool same_allocation(const void* a, const void* b) const {
+      CUdeviceptr ra = 0, rb = 0;
+      return st->pointer_attribute != nullptr &&
+             st->pointer_attribute(&ra, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, reinterpret_cast<CUdeviceptr>(a)) == CUDA_SUCCESS &&
+             st->pointer_attribute(&rb, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, reinterpret_cast<CUdeviceptr>(b)) == CUDA_SUCCESS &&
+             ra != 0 && ra == rb;
+    }
+    cudaError_t flush() {
+      const size_t n = bytes;
+      bytes = 0;
+      return n > 0 ? cudaMemcpyAsync(dst, src, n, kind, stream) : cudaSuccess;
+    }
+    cudaError_t add(void* d, const void* s, size_t n) {
+      const bool in = kind == cudaMemcpyHostToDevice;
+      if (bytes > 0 && dst + bytes == d && src + bytes == s && same_allocation(in ? src : dst, in ? s : d)) {
+        bytes += n;
+        return cudaSuccess;
+      }
+      const cudaError_t e = flush();
+      dst = static_cast<char*>(d);
+      src = const_cast<char*>(static_cast<const char*>(s));
+      bytes = n;
+      return e;
+    }
+  };
+  Run in{st, cudaMemcpyHostToDevice, st->copy_in}, out{st, cudaMemcpyDeviceToHost, st->copy_out};
+  const size_t ng = st->group_tile.size() - 1;
   NG_CUDA(cudaEventRecord(st->ev_begin, s));
   NG_CUDA(cudaStreamWaitEvent(st->copy_in, st->ev_begin, 0));
-  for (int i = 0; i < st->n; ++i) {
-    const size_t mn = static_cast<size_t>(st->mats[i].M) * st->mats[i].N;
-    NG_CUDA(cudaMemcpyAsync(st->stage_G[i], G_host[i], mn * sizeof(uint16_t), cudaMemcpyHostToDevice, st->copy_in));
-  }
+  for (int i = 0; i < st->n; ++i) NG_CUDA(in.add(st->stage_G[i], G_host[i], host_elems(i) * sizeof(uint16_t)));
+  NG_CUDA(in.flush());
   NG_CUDA(cudaEventRecord(st->ev_G, st->copy_in));
-  for (size_t g = 0; g < ng; ++g) {
-    for (int i = st->group_first[g]; i < st->group_first[g + 1]; ++i) {
-      const size_t mn = static_cast<size_t>(st->mats[i].M) * st->mats[i].N;
-      NG_CUDA(cudaMemcpyAsync(st->stage_W[i], W_host[i], mn * sizeof(float), cudaMemcpyHostToDevice, st->copy_in));
+  auto group_copies = [&](Run& run, size_t g) {
+    for (int p = st->group_part[g]; p < st->group_part[g + 1]; ++p) {
+      const ngalore_state::HostPart& part = st->host_parts[p];
+      const size_t at = static_cast<size_t>(part.row0) * st->mats[part.mat].N;
+      const size_t n = static_cast<size_t>(part.row1 - part.row0) * st->mats[part.mat].N * sizeof(float);
+      float *dev = st->stage_W[part.mat] + at, *host = W_host[part.mat] + at;
+      const cudaError_t e = run.kind == cudaMemcpyHostToDevice ? run.add(dev, host, n) : run.add(host, dev, n);
+      if (e != cudaSuccess) return e;
     }
+    return run.flush();
+  };
+  for (size_t g = 0; g < ng; ++g) {
+    NG_CUDA(group_copies(in, g));
     NG_CUDA(cudaEventRecord(st->ev_w_in[g], st->copy_in));
   }
   NG_CUDA(cudaStreamWaitEvent(s, st->ev_G, 0));
@@ -1016,10 +1078,7 @@ ngalore_status ngalore_step_host(ngalore_state* st, float* const* W_host, const 
   }
   for (size_t g = 0; g < ng; ++g) {
     NG_CUDA(cudaStreamWaitEvent(st->copy_out, st->ev_w_done[g], 0));
-    for (int i = st->group_first[g]; i < st->group_first[g + 1]; ++i) {
-      const size_t mn = static_cast<size_t>(st->mats[i].M) * st->mats[i].N;
-      NG_CUDA(cudaMemcpyAsync(W_host[i], st->stage_W[i], mn * sizeof(float), cudaMemcpyDeviceToHost, st->copy_out));
-    }
+    NG_CUDA(group_copies(out, g));
   }
   NG_CUDA(cudaEventRecord(st->ev_out, st->copy_out));
   NG_CUDA(cudaStreamWaitEvent(s, st->ev_out, 0));

@@ -41,6 +41,39 @@ def test_step_host_equals_device_step():
     assert a.poll_status()[0] == 0 and b.poll_status()[0] == 0
 
 
+@pytest.mark.parametrize("layout", ["flat", "separate", "pageable"])
+def test_step_host_in_groups_of_rows(layout):
+    """W of more than 2 MB travels in groups that may end inside a matrix and hold several of them, and copies of
+    neighbouring buffers are joined: the step of the device all the same (to the order of the sums of a split K, a tenth
+    of the parity tolerance), for buffers side by side in one allocation, each in its own, and in pageable memory; a row
+    count that is no multiple of the 128-row tile."""
+    w = wl.tiny_workload([(1000, 1024), (72, 40), (2000, 768), (130, 264), (64, 64)], r=16, s=2, T=0, inner_rank=4, index=83)
+    dev = torch.device("cuda")
+    grads = _grads(w, 3, dev)
+    a, b = _make(w), _make(w)
+    a.refresh_subspace(grads[0])
+    torch.cuda.synchronize()
+    for i in range(w.n_matrices):
+        b.set_subspace(i, a.get_subspace(i))
+    Wd = [wl.initial_weight_device(w, i, dev) for i in range(w.n_matrices)]
+
+    def host(tensors):
+        if layout == "flat":
+            flat = torch.cat([t.flatten() for t in tensors]).cpu().pin_memory()
+            return list(p.view(t.shape) for p, t in zip(flat.split([t.numel() for t in tensors]), tensors))
+        return [t.cpu().pin_memory() if layout == "separate" else t.cpu() for t in tensors]
+
+    W0 = [t.cpu() for t in Wd]
+    Wh = host(Wd)
+    for k in range(3):
+        a.step(Wd, grads[k])
+        b.step_host(Wh, host(grads[k]))
+    torch.cuda.synchronize()
+    for x, y, z in zip(Wd, Wh, W0):
+        assert rel_err((y - z).numpy(), (x.cpu() - z).numpy()) <= 0.1 * TOL_UPDATE
+    assert a.poll_status()[0] == 0 and b.poll_status()[0] == 0
+
+
 def test_set_lr_scales_the_next_update_exactly():
     """W <- W - lr P u with W = 0 and wd = 0: doubling lr doubles every element (a power of two is exact in fp32),
     and the oracle with the new rate agrees."""
