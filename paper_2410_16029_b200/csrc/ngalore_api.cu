@@ -969,10 +969,11 @@ ngalore_status ngalore_step_host(ngalore_state* st, float* const* W_host, const 
   // Pipelined: only the back-projection touches W, so the gradients go in first and the projection and the
   // history phase run while W is still arriving; W then moves in groups of rows, each group's copy in, back-projection
   // and copy out chained by events, so that the two directions of the link overlap.  What is left beside the copies in
-  // is the last group's way back, so a group is small: a 32nd of W, but at least 2 MB (a copy of 8 MB spends 3 % of its
-  // time on being issued).  Buffers that lie side by side, on either side of the link, travel in one copy.
+  // is the last group's way back, so a group is small: a 16th of W, but at least 2 MB (a group costs about
+  // 20 us beside its copies: 60M shapes 7.39 ms, with 32 groups 7.70, with 64 8.37).  Buffers that lie side by side, on
+  // either side of the link, travel in one copy.
   // 60M shapes, 348 MB in and 232 MB out at 55 GB/s: 9.8 ms with a copy for each matrix and eight groups of whole
-  // matrices (the last of them a quarter of W), 7.7 ms so.
+  // matrices (the last of them a quarter of W), 7.4 ms so.
   if (st->copy_in == nullptr) {
     NG_CUDA(cudaStreamCreateWithFlags(&st->copy_in, cudaStreamNonBlocking));
     NG_CUDA(cudaStreamCreateWithFlags(&st->copy_out, cudaStreamNonBlocking));
@@ -985,7 +986,7 @@ ngalore_status ngalore_step_host(ngalore_state* st, float* const* W_host, const 
       st->pointer_attribute = reinterpret_cast<PointerAttributeFn>(fn);
     size_t total = 0;
     for (int i = 0; i < st->n; ++i) total += host_elems(i) * sizeof(float);
-    const size_t size = std::max<size_t>(2 << 20, (total + 31) / 32);
+    const size_t size = std::max<size_t>(2 << 20, (total + 15) / 16);
     st->group_part.assign(1, 0);
     st->group_tile.assign(1, 0);
     size_t acc = 0;
