@@ -92,8 +92,9 @@ struct SyrkTile {
   int mat, ti, tj, k0, k1;  // output tile (ti, tj <= ti) of 64 x 64, rows k0 .. k1 - 1 of Y
 };
 // Rows of a slab: long ones save atomics, short ones balance the SMs where there are few tiles.  58 matrices of r' = 128
-// (232 tiles of 1024 rows) 138 us against 105 with 256 rows, 84 of r' = 256 (1080) 473 / 451 us, 156 of the 1.1B shapes
+// (232 tiles of 1024 rows) 138 us against 117 with short ones, 84 of r' = 256 (1080) 473 / 448 us, 156 of the 1.1B shapes
 // (15 thousand) 4.14 / 4.33 ms.
+// Up to 2048 rows make no more than two slabs: two sums added to zero give the same bits in either order.
 constexpr int kSyrkRows = 1024, kSyrkRowsFew = 256;
 constexpr int kSyrkFewTiles = 16;   // per SM
 
@@ -352,6 +353,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     // (to the nearest number: a K a little over the target costs less balance than two tiles cost atomics)
     int splits = static_cast<int>((kb_total + target_kb / 2) / target_kb);
     if (splits < 1) splits = 1;
+    // Gram matrices have few tiles, of three products a K block: two halves from 16 blocks on (58 of r' = 128 24 -> 20.5 us; three
+    // sums and more would depend on the order of the atomics)
+    if ((g == RG_GRAM_Y || g == RG_GRAM_Z) && splits == 1 && kb_total >= 16 && target_kb == 16) splits = 2;
     const int kb_per = (kb_total + splits - 1) / splits;
     splits = (kb_total + kb_per - 1) / kb_per;
     if (splits > 1) plan.atomic_mats[g].push_back(i);
@@ -409,9 +413,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
                   ((K + kTcBK - 1) / kTcBK);
     }
     long long target = (total_kb * (tile_rows(g) / kTcBM) + sm_count - 1) / sm_count / 4;
-    // (Gram matrices have few tiles, of three products a K block: 58 of r' = 128 24 -> 20.5 us with 8 K blocks at least)
-    const long long least = g == RG_GRAM_Y || g == RG_GRAM_Z ? 8 : 16;
-    if (target < least) target = least;
+    if (target < 16) target = 16;
     for (int i = 0; i < n; ++i) {
       const RefreshMat& m = plan.mats[i];
       int rows, cols, K;
@@ -437,10 +439,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   auto slabs = [&](int slab) {
     syrk_tiles.clear();
     for (int i = 0; i < n; ++i) {
-      const int nt = (plan.mats[i].L + 63) / 64;
-      for (int k0 = 0; k0 < plan.mats[i].M; k0 += slab)
+      const int nt = (plan.mats[i].L + 63) / 64, rows = plan.mats[i].M;
+      const int step = rows <= 2 * kSyrkRows ? std::max(slab, (rows / 2 + 15) & ~15) : slab;
+      for (int k0 = 0; k0 < rows; k0 += step)
         for (int ti = 0; ti < nt; ++ti)
-          for (int tj = 0; tj <= ti; ++tj) syrk_tiles.push_back(SyrkTile{i, ti, tj, k0, std::min(k0 + slab, plan.mats[i].M)});
+          for (int tj = 0; tj <= ti; ++tj) syrk_tiles.push_back(SyrkTile{i, ti, tj, k0, std::min(k0 + step, rows)});
     }
   };
   slabs(kSyrkRows);
