@@ -284,6 +284,7 @@ struct RefreshPlan {
   int eig_max = 0;             // largest matrix it diagonalises
   int sm_count = 0;
   FillJob* d_fill = nullptr;   // the random start Z = Omega of every matrix
+  int fill_blocks = 1;         // blocks a matrix: eight entries a thread in the largest
   ZeroJob* d_zero_d = nullptr;   // clears every matrix's D (as 16-byte words)
 };
 
@@ -574,6 +575,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     for (int i = 0; i < n; ++i) {
       const RefreshMat& m = plan.mats[i];
       fill[i] = FillJob{m.Zhi, m.Zlo, static_cast<long long>(m.N) * m.L, m.L, m.ldl};
+      plan.fill_blocks = std::max(plan.fill_blocks, static_cast<int>(std::min<long long>(512, (fill[i].n + 2047) / 2048)));
     }
     if (cudaMemcpy(plan.d_fill, fill.data(), sizeof(FillJob) * n, cudaMemcpyHostToDevice) != cudaSuccess) return NGALORE_ERR_CUDA;
   }
@@ -769,7 +771,7 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
                                  cudaMemcpyHostToDevice, stream) != cudaSuccess)
     return NGALORE_ERR_CUDA;
   ngalore_status rc;
-  fill_normal_grouped_kernel<<<dim3(64, plan.n), 256, 0, stream>>>(plan.d_fill, seed, stream_base);
+  fill_normal_grouped_kernel<<<dim3(plan.fill_blocks, plan.n), 256, 0, stream>>>(plan.d_fill, seed, stream_base);
   *launches += 1;
   if (cudaGetLastError() != cudaSuccess) return NGALORE_ERR_CUDA;
   if ((rc = refresh_tc_gemm(plan, RG_Y_FROM_Z, RP_Y_FROM_Z, d_ctrl, stream, launches))) return rc;
