@@ -17,8 +17,8 @@
 // blocks live in shared memory where they fit (fp32: up to 256 columns, fp64: up to 160), else in L2.
 // It replaced a scaling kernel, a Cholesky factorisation with one CTA per matrix, a recursive triangular inverse (two
 // batched products per level) and a conversion: 12 launches.  Measured per orthonormalisation, fp32: 58 matrices of 128
-// columns 125 -> 43 us, 84 of 256 310 -> 94 us, 156 of up to 512 1600 -> 520 us; the fp64 pass of the same sets 190 -> 58,
-// 490 -> 166 and 2900 -> 900 us.  What is left is the chain of diagonal blocks up to 256 columns (8 000 cycles each) and
+// columns 125 -> 36 us, 84 of 256 310 -> 89 us, 156 of up to 512 1600 -> 493 us; the fp64 pass of the same sets 190 -> 52,
+// 490 -> 150 and 2900 -> 900 us.  What is left is the chain of diagonal blocks up to 256 columns (6 400 cycles each) and
 // the tensor cores' rate for TF32 beyond.
 #pragma once
 
