@@ -220,14 +220,12 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         __threadfence();
       }
       // the matrix's last tile
-      double a[SMAX];
-      solve_load<SMAX>(d, c, a);
       if (d.ntiles > 1) {
 #pragma unroll
-        for (int r = 0; r < C::kRows; ++r) part[r] = gram_row_sum(d, lane, c, C::kRows, r);
+        for (int r = 0; r < C::kRows; ++r) part[r] = gram_row_sum<SMAX>(d, lane, c, C::kRows, r);
       }
       const bool two = HIST16 && c >= 2;
-      solve_matrix<SMAX>(d, cur, c, lambda, a, lane < c ? part[0] : 0.0, two, two ? (cur == 0 ? d.s : cur) - 1 : 0, part[C::kRows - 1]);
+      solve_matrix<SMAX>(d, cur, c, lambda, lane < c ? part[0] : 0.0, two, two ? (cur == 0 ? d.s : cur) - 1 : 0, part[C::kRows - 1]);
       __threadfence();
       __syncwarp();
       if (lane == 0) {

@@ -56,23 +56,31 @@ __device__ __forceinline__ void gram_tile(const MatDesc& d, int local, int cur, 
   __syncthreads();
 }
 
-// Lane j's share of the Gram row: the sum over the matrix's tiles of partial product j (fixed order, so the result is
-// reproducible).  rows: partial rows per tile, row: which of them.
+// Lane j's share of the Gram row (zero from lane c on): the sum over the matrix's tiles of partial product j, in a fixed
+// order, so that the result is reproducible.  rows: partial rows per tile, row: which of them.
+// The partial rows of early tiles have left L2 by then, so it is the number of loads under way that decides: 32 / SMAX lanes
+// share a column, sixteen loads each (352 tiles, s = 16: 37 us with one lane a column and eight loads, 19 us so).
+template <int SMAX>
 __device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c, int rows = 1, int row = 0) {
-  double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-  if (lane < c) {
-    const double* gp = d.gpart + static_cast<long long>(row) * d.s + lane;
-    const long long st = static_cast<long long>(rows) * d.s;
-    int t = 0;
-    for (; t + 7 < d.ntiles; t += 8) {
-      double x[8];
+  constexpr int G = 32 / SMAX, U = 16;
+  const double* gp = d.gpart + static_cast<long long>(row) * d.s + min(lane % SMAX, c - 1);
+  const long long st = static_cast<long long>(rows) * d.s;
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int t0 = 0; t0 < d.ntiles; t0 += G * U) {
+    double x[U];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) x[q] = __ldcg(gp + (t + q) * st);
-      t0 += x[0] + x[4]; t1 += x[1] + x[5]; t2 += x[2] + x[6]; t3 += x[3] + x[7];
+    for (int q = 0; q < U; ++q) {
+      const int tile = t0 + q * G + lane / SMAX;
+      const double v = __ldcg(gp + min(tile, d.ntiles - 1) * st);
+      x[q] = tile < d.ntiles ? v : 0.0;
     }
-    for (; t < d.ntiles; ++t) t0 += __ldcg(gp + t * st);
+#pragma unroll
+    for (int q = 0; q < U; ++q) t[q & 3] += x[q];
   }
-  return (t0 + t1) + (t2 + t3);
+  double sum = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+  for (int o = SMAX; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return lane < c ? sum : 0.0;
 }
 
 // One warp: put the new Gram row (lane j: <H_cur, H_j>) into Kraw, form lambda I + K with K = Kraw / c and solve for
@@ -83,49 +91,47 @@ __device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c
 // symmetric positive definite, its pivots are the squares of Cholesky's, and the same pivots tell when it is not)
 // broadcasts row k by shuffles, so the chain per step is one shuffle, one reciprocal and one multiply-add.  In shared
 // memory with serial substitutions the solve took 9 us for s = 8 and 25 us for s = 16; so 2 and 4 us.
+// What bounds it is that the 32 lanes run together.  Lanes that a branch on the lane number has parted are not brought back
+// together by a shuffle that all of them take part in: each one then costs two turns of the scheduler, 500 cycles instead of
+// 30 (one 1024 x 1024 matrix, s = 20: 125 us a solve, 10 so).  So nothing ahead of the elimination, here and in
+// gram_row_sum, branches on the lane, and what is stored is stored after it.
 // have_prev: lane j also holds <H_prev, H_j> for the slot that was current one step ago (bf16 history).
-// The rows of Kraw are loaded by solve_load, which the caller may run ahead of its own sums.
 template <int SMAX>
-__device__ __forceinline__ void solve_load(const MatDesc& d, int c, double (&a)[SMAX]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int j = 0; j < SMAX; ++j) a[j] = (lane < c && j < c) ? __ldcg(d.Kraw + lane * d.s + j) : 0.0;
-}
-
-template <int SMAX>
-__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double (&a)[SMAX], double row,
+__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double row,
                                              bool have_prev = false, int prev = 0, double rowp = 0.0) {
   const int lane = threadIdx.x & 31;
-  if (have_prev) {
-    // row and column `prev` against the stored (rounded) values; the entry with `cur` follows below
-    const int use = lane < c && lane != cur && isfinite(rowp) ? 1 : 0;
-    if (use) {
-      d.Kraw[prev * d.s + lane] = rowp;
-      d.Kraw[lane * d.s + prev] = rowp;
+  __syncwarp();
+  double a[SMAX];
+  {
+    const double* old = d.Kraw + min(lane, c - 1) * d.s;
+#pragma unroll
+    for (int j = 0; j < SMAX; ++j) {
+      const double v = __ldcg(old + min(j, c - 1));
+      a[j] = lane < c && j < c ? v : 0.0;
     }
+  }
+  // row and column `prev` against the stored (rounded) values; the entry with `cur` follows below
+  const int use = have_prev && lane < c && lane != cur && isfinite(rowp) ? 1 : 0;
+  if (have_prev) {
 #pragma unroll
     for (int j = 0; j < SMAX; ++j) {
       const double v = __shfl_sync(0xffffffffu, rowp, j);
       const int uj = __shfl_sync(0xffffffffu, use, j);
-      if (lane == prev && uj) a[j] = v;
-      if (j == prev && use) a[j] = rowp;
+      a[j] = lane == prev && uj ? v : a[j];
+      a[j] = j == prev && use ? rowp : a[j];
     }
   }
   const bool finite = __all_sync(0xffffffffu, lane >= c || isfinite(row));
   int bad = finite ? 0 : 7 /* NGALORE_ERR_NONFINITE */;
   const double val = finite && lane < c ? row : 0.0;
-  if (lane < c) {
-    d.Kraw[cur * d.s + lane] = val;
-    d.Kraw[lane * d.s + cur] = val;
-  }
   const double ic = 1.0 / static_cast<double>(c);
 #pragma unroll
   for (int j = 0; j < SMAX; ++j) {
     const double v = __shfl_sync(0xffffffffu, val, j);
-    if (lane == cur) a[j] = v;
-    if (j == cur) a[j] = val;
+    a[j] = lane == cur ? v : a[j];
+    a[j] = j == cur ? val : a[j];
     a[j] *= ic;
-    if (j == lane) a[j] += lambda;
+    a[j] += j == lane ? lambda : 0.0;
   }
   double b = lane == cur ? 1.0 : 0.0, diag = 1.0;
 #pragma unroll
@@ -136,17 +142,23 @@ __device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, d
       bad = isfinite(p) ? 6 /* NGALORE_ERR_NOT_SPD */ : 7;
       break;
     }
-    if (lane == k) diag = p;
-    const double f = lane == k ? 0.0 : a[k] * (1.0 / p);
+    diag = lane == k ? p : diag;
+    const double ip = 1.0 / p;
+    const double f = lane == k ? 0.0 : a[k] * ip;
 #pragma unroll
     for (int j = k + 1; j < SMAX; ++j) a[j] -= f * __shfl_sync(0xffffffffu, a[j], k);
     b -= f * __shfl_sync(0xffffffffu, b, k);
   }
   d.wsol[lane] = bad == 0 && lane < c ? static_cast<float>(b / diag) : 0.f;
-  if (bad != 0 && lane < d.s) {
-    // The poisoned slot becomes a zero gradient: its Gram row and column vanish.
-    d.Kraw[cur * d.s + lane] = 0.0;
-    d.Kraw[lane * d.s + cur] = 0.0;
+  if (use) {
+    d.Kraw[prev * d.s + lane] = rowp;
+    d.Kraw[lane * d.s + prev] = rowp;
+  }
+  __syncwarp();
+  // (where the step is flagged the poisoned slot becomes a zero gradient: its Gram row and column vanish)
+  if (lane < (bad != 0 ? d.s : c)) {
+    d.Kraw[cur * d.s + lane] = bad != 0 ? 0.0 : val;
+    d.Kraw[lane * d.s + cur] = bad != 0 ? 0.0 : val;
   }
   if (lane == 0) {
     *d.step_bad = bad != 0 ? 1 : 0;
@@ -223,9 +235,7 @@ __global__ void __launch_bounds__(128) solve_kernel(const MatDesc* mats, int n_m
   const MatDesc& d = mats[mat];
   if (d.s == 0) return;
   const int c = ring_count(ctrl, d.s);
-  double a[kMaxHistory];
-  solve_load<kMaxHistory>(d, c, a);
-  solve_matrix<kMaxHistory>(d, ring_cur(ctrl, d.s), c, hyper->lambda, a, gram_row_sum(d, threadIdx.x & 31, c));
+  solve_matrix<kMaxHistory>(d, ring_cur(ctrl, d.s), c, hyper->lambda, gram_row_sum<kMaxHistory>(d, threadIdx.x & 31, c));
 }
 
 template <int SMAX>

@@ -358,10 +358,9 @@ __global__ void __launch_bounds__(256) pg_solve_kernel(const MatDesc* __restrict
   __syncthreads();
   if (threadIdx.x < 32) {
     const int c = ring_count(ctrl, d.s);
-    double a[kPgSMax], row = 0.0;
-    solve_load<kPgSMax>(d, c, a);
+    double row = 0.0;
     for (int q = 0; q < 8; ++q) row += red[q * 32 + threadIdx.x];
-    solve_matrix<kPgSMax>(d, ring_cur(ctrl, d.s), c, hyper->lambda, a, row);
+    solve_matrix<kPgSMax>(d, ring_cur(ctrl, d.s), c, hyper->lambda, row);
     __threadfence();
     __syncwarp();
     if (threadIdx.x == 0) atomicExch(d.w_ready, ctrl->epoch + 1);

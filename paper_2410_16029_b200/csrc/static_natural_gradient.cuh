@@ -57,9 +57,7 @@ __global__ void __launch_bounds__(kStreamThreads) static_gram_kernel(StaticArgs 
 
 __global__ void __launch_bounds__(32) static_solve_kernel(StaticArgs a) {
   const MatDesc d = static_desc(a);
-  double k[kMaxHistory];
-  solve_load<kMaxHistory>(d, a.count, k);
-  solve_matrix<kMaxHistory>(d, a.cur, a.count, a.lambda, k, gram_row_sum(d, threadIdx.x, a.count));
+  solve_matrix<kMaxHistory>(d, a.cur, a.count, a.lambda, gram_row_sum<kMaxHistory>(d, threadIdx.x, a.count));
 }
 
 // out = sum_j w_j H_j (zeros when the solve flagged the step).
