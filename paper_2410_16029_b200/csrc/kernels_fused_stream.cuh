@@ -447,7 +447,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           // rows of `cur` and of the slot that was current one step ago, in pairs: the inner loop is bound by the
           // instructions it issues, and the packed multiply-add halves those
           uint64_t acc[SMAX], acc2[SMAX];
-          float axx = 0.f, apx = 0.f;      // products with the fp32 gradient itself
+          // The product of the fp32 gradient with itself, in the operations and the order of the other products: a
+          // gradient that repeats bit for bit has to give an exactly singular Gram matrix, not one that a rounding makes
+          // indefinite.
+          uint64_t axx = 0ull;
 #pragma unroll
           for (int j = 0; j < SMAX; ++j) acc[j] = acc2[j] = 0ull;
           const int prev = c >= 2 ? (cur == 0 ? mats[mt.mat].s : cur) - 1 : cur;
@@ -460,10 +463,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
 #pragma unroll
               for (int q = 0; q < VEC / 2; ++q) {
                 xx[q] = pack_pair(x[2 * q], x[2 * q + 1]);
-                float p0, p1;
-                unpack_pair(xp[q], p0, p1);
-                axx += x[2 * q] * x[2 * q] + x[2 * q + 1] * x[2 * q + 1];
-                apx += x[2 * q] * p0 + x[2 * q + 1] * p1;
+                axx = fma_pair(xx[q], xx[q], axx);
               }
 #pragma unroll
               for (int j = 0; j < SMAX; ++j) {
@@ -489,8 +489,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
 #pragma unroll
             for (int j = 0; j < SMAX; ++j) {
               float s0, s1;
-              unpack_pair(acc[j], s0, s1);
-              v[j] = static_cast<double>(j == cur ? axx : s0 + s1);
+              unpack_pair(j == cur ? axx : acc[j], s0, s1);
+              v[j] = static_cast<double>(s0 + s1);
             }
             hand_over(0, v);
           }
@@ -501,7 +501,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
             for (int j = 0; j < SMAX; ++j) {
               float s0, s1;
               unpack_pair(acc2[j], s0, s1);
-              v[j] = static_cast<double>(j == cur ? apx : s0 + s1);
+              v[j] = static_cast<double>(s0 + s1);   // (entry `cur` is not used: row `cur` has it)
             }
             hand_over(C::kRows - 1, v);
           }

@@ -98,3 +98,24 @@ def test_option_is_rejected_where_it_cannot_work():
         NGaLore([(64, 64)], 8, 0, 0, history_bf16=True)                  # no history to narrow
     with pytest.raises(NGaLoreError):
         NGaLore([(64, 64)], 8, 4, 0, history_bf16=True, stream_impl=1)   # plain kernels read the fp32 ring
+
+
+@pytest.mark.parametrize("s", [2, 5, 12, 20])
+def test_repeated_gradient_gives_a_singular_gram_matrix_and_not_an_indefinite_one(s):
+    """The same gradient in every step, its projection exact in bf16 (a projector of unit vectors), lambda far below the
+    rounding of an fp32 inner product: all entries of K have to agree to the last bit, or a pivot can turn negative."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    gen = torch.Generator(device="cuda").manual_seed(s)
+    n, M, N, r = 8, 64, 1000 * 8, 32
+    for bf16 in (False, True):
+        opt = NGaLore([(M, N)] * n, r, s, 0, lam=1e-5, history_bf16=bf16)
+        G = [torch.randn(M, N, generator=gen, device="cuda").bfloat16() for _ in range(n)]
+        W = [torch.zeros(M, N, device="cuda") for _ in range(n)]
+        for i in range(n):
+            opt.set_subspace(i, torch.eye(M, device="cuda")[:, :r])
+        for _ in range(s + 2):
+            opt.step(W, G)
+        code, per = opt.poll_status()
+        assert code == 0, (bf16, per)
+        assert all(bool(torch.isfinite(w).all()) for w in W)
