@@ -345,6 +345,16 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     int stage = 0;
     uint32_t phase = 0;
     unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
+    // Tell the finishing warp that the CTA has no more of them (every Gram item is ahead of every combination item).  That
+    // is done as soon as it is known, so that none of its waits spans more than a Gram tile: a wait is given up after a
+    // time, and the combination items of a CTA may take longer than that without anything being wrong.
+    bool gram_open = true;
+    auto close_gram = [&]() {
+      if (tid == 0) red_meta[tiles_done & 1].mat = -1;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(red_full + (tiles_done & 1));
+      gram_open = false;
+    };
     if (HIST16) {
       // the current slot's place in a stage stays zero for the whole launch: its gradient takes part in fp32 instead
       const int cur = ring_cur(ctrl, mats[0].s);
@@ -393,14 +403,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     while (true) {
       if (!mbar_wait(full_bar + stage, phase, abort_flag)) break;
       StageMeta mt = meta[stage];
-      if (mt.kind < 0) {
-        // no more items: tell the finishing warp
-        const int buf = tiles_done & 1;
-        if (mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) {
-          if (tid == 0) red_meta[buf].mat = -1;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(red_full + buf);
-        }
+      if (mt.kind < 0) {   // no more items
+        if (gram_open && mbar_wait(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) close_gram();
         break;
       }
       const int cur = mt.cur, c = mt.c;
@@ -512,6 +516,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         if (lane == 0) mbar_arrive(red_full + buf);
       } else {
         // ---- combination tile
+        // (where the finishing warp still has two tiles to take, the next item will do)
+        if (gram_open && __all_sync(0xffffffffu, mbar_test(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u))) close_gram();
         const MatDesc& d = mats[mt.mat];
         bool item_ok = true;
         if (d.s > 0) {

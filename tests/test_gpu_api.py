@@ -301,6 +301,39 @@ def test_a_wait_that_runs_out_is_reported_and_skips_only_that_matrix():
         b.debug_withhold_solution(7, 20000)
 
 
+def test_waits_of_one_matrix_that_add_up_to_seconds_stay_its_own():
+    """Every combination tile of a matrix whose weights never come gives up for itself.  A CTA that meets eight of them spends
+    more than the two seconds after which a pipeline wait is abandoned, and is healthy all the same: the step ends
+    with that matrix's status, the other matrix as in a regular step, and the next step is regular for both."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    shapes = [(64, 4096), (64, 1000 * 152)]     # the last matrix: 1188 tiles on 148 multiprocessors
+    opts = [NGaLore(shapes, 64, 2, 0, lam=0.1) for _ in range(2)]
+    Ws = [[torch.zeros(s, device="cuda") for s in shapes] for _ in opts]
+    G = [[torch.randn(s, generator=gen, device="cuda").bfloat16() for s in shapes] for _ in range(4)]
+    for o, W in zip(opts, Ws):
+        for i in range(2):
+            o.set_subspace(i, torch.eye(64, device="cuda"))
+        for k in range(2):
+            o.step(W, G[k])
+    before = Ws[1][1].clone()
+    opts[1].debug_withhold_solution(1, 1000000)
+    begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    begin.record()
+    opts[1].step(Ws[1], G[2])
+    end.record()
+    opts[0].step(Ws[0], G[2])
+    torch.cuda.synchronize()
+    assert begin.elapsed_time(end) > 2100.0       # (measured: 2300)
+    assert opts[1].poll_status() == (8, [0, 8])
+    assert torch.equal(Ws[1][1], before) and torch.equal(Ws[1][0], Ws[0][0])
+    for o, W in zip(opts, Ws):
+        o.step(W, G[3])
+    torch.cuda.synchronize()
+    assert opts[1].poll_status() == (0, [0, 0]) and torch.equal(Ws[1][0], Ws[0][0]) and not torch.equal(Ws[1][1], before)
+
+
 def test_stepping_needs_a_projector_for_every_matrix():
     from paper_2410_16029_b200.ngalore import NGaLoreError
 
