@@ -376,7 +376,8 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       const uint32_t tphase = (local / NBUF) & 1u;
       const int row_base = tile.m0 + half * kTcBM + quarter * 32;
       const int sub_row = lane >> 3, sub_col = (lane & 7) * 4;
-      if (!mbar_wait(tfull_bar + buf, tphase, abort_flag)) { ok = false; break; }
+      // (every lane polls; the warp goes on only if all of them saw the barrier complete)
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar + buf, tphase, abort_flag))) { ok = false; break; }
       tc_fence_after();
       if (half == 1 && tile.rows - tile.m0 <= kTcBM) {   // nothing in this half
         if (lane == 0) mbar_arrive(tempty_bar + buf);

@@ -68,7 +68,7 @@ struct FusedCfg {
   static constexpr int kStages = HIST16 ? (SMAX <= 8 ? 3 : (SMAX <= 16 ? 2 : 5)) : (SMAX <= 8 ? 5 : 3);
   static constexpr int kBase = kStages * kStageBytes;
   static constexpr int kFullOff = kBase, kEmptyOff = kBase + 64, kMetaOff = kBase + 128, kFlagOff = kBase + 512;
-  static constexpr int kWOff = kBase + 640, kRedBarOff = kBase + 768, kRedMetaOff = kBase + 800, kRedOff = kBase + 896;
+  static constexpr int kMeetOff = kBase + 640, kRedBarOff = kBase + 768, kRedMetaOff = kBase + 800, kRedOff = kBase + 896;
   static constexpr int kRows = HIST16 ? 2 : 1;                  // Gram rows per tile
   static constexpr int kRedDoubles = (kConsumers / 32) * SMAX;  // one Gram row per consumer warp
   static constexpr int kTotal = kRedOff + 2 * kRows * kRedDoubles * 8;   // (two tiles in flight to the finishing warp)
@@ -105,6 +105,12 @@ __device__ __forceinline__ double warp_sums(double (&v)[S]) {
     }
   }
   return v[0];
+}
+
+// A wait of a whole warp: all lanes see the barrier complete, or all of them give up (lanes that part here could not come
+// together again in what follows).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
 
 // What the finishing warp needs to know about a finished Gram tile (mat < 0: the CTA has no more).
@@ -159,8 +165,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   uint64_t* empty_bar = reinterpret_cast<uint64_t*>(fs_smem + C::kEmptyOff);
   StageMeta* meta = reinterpret_cast<StageMeta*>(fs_smem + C::kMetaOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(fs_smem + C::kFlagOff);
-  volatile int* s_flag = abort_flag + 1;
-  float* wsm = reinterpret_cast<float*>(fs_smem + C::kWOff);
+  volatile int* s_flag = abort_flag + 1;                                        // [2] 1: the weights of a combination item came
+  uint64_t* meet_bar = reinterpret_cast<uint64_t*>(fs_smem + C::kMeetOff);      // all consumer warps
   uint64_t* red_full = reinterpret_cast<uint64_t*>(fs_smem + C::kRedBarOff);   // [2] all consumer warps have left their sums
   uint64_t* red_empty = red_full + 2;                                           // [2] the finishing warp has taken them
   RedMeta* red_meta = reinterpret_cast<RedMeta*>(fs_smem + C::kRedMetaOff);     // [2]
@@ -173,6 +179,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       mbar_init(empty_bar + s, kConsumerThreads / 32);
     }
     for (int b = 0; b < 2; ++b) { mbar_init(red_full + b, kWarps); mbar_init(red_empty + b, 1); }
+    mbar_init(meet_bar, kWarps);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -187,7 +194,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const double lambda = hyper->lambda;
     for (unsigned int n = 0;; ++n) {
       const int buf = n & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(red_full + buf, (n >> 1) & 1u, abort_flag))) break;
+      if (!mbar_wait_warp(red_full + buf, (n >> 1) & 1u, abort_flag)) break;
       const RedMeta mt = red_meta[buf];
       double part[C::kRows];
 #pragma unroll
@@ -345,6 +352,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     int stage = 0;
     uint32_t phase = 0;
     unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
+    unsigned int combined = 0;     // combination items whose weights have been waited for
     // Tell the finishing warp that the CTA has no more of them (every Gram item is ahead of every combination item).  That
     // is done as soon as it is known, so that none of its waits spans more than a Gram tile: a wait is given up after a
     // time, and the combination items of a CTA may take longer than that without anything being wrong.
@@ -401,10 +409,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       }
     };
     while (true) {
-      if (!mbar_wait(full_bar + stage, phase, abort_flag)) break;
+      if (!mbar_wait_warp(full_bar + stage, phase, abort_flag)) break;
       StageMeta mt = meta[stage];
       if (mt.kind < 0) {   // no more items
-        if (gram_open && mbar_wait(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) close_gram();
+        if (gram_open && mbar_wait_warp(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) close_gram();
         break;
       }
       const int cur = mt.cur, c = mt.c;
@@ -439,10 +447,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
             const bool last = mt.last != 0;
             release();
             if (last) break;
-            if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+            if (!mbar_wait_warp(full_bar + stage, phase, abort_flag)) { alive = false; break; }
             mt = meta[stage];
           }
-          if (!alive || !mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
+          if (!alive || !mbar_wait_warp(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
           double v[SMAX];
 #pragma unroll
           for (int j = 0; j < SMAX; ++j) v[j] = static_cast<double>(acc[j]);
@@ -484,10 +492,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
             const bool last = mt.last != 0;
             release();
             if (last) break;
-            if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+            if (!mbar_wait_warp(full_bar + stage, phase, abort_flag)) { alive = false; break; }
             mt = meta[stage];
           }
-          if (!alive || !mbar_wait(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
+          if (!alive || !mbar_wait_warp(red_empty + buf, ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) break;
           {
             double v[SMAX];
 #pragma unroll
@@ -521,6 +529,9 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         const MatDesc& d = mats[mt.mat];
         bool item_ok = true;
         if (d.s > 0) {
+          // One thread waits for the weights; the others meet it at a barrier that they leave, like every other wait, when
+          // one of the CTA's warps has given up.  (A bar.sync would wait for good for a warp that is gone.)  What it found
+          // goes through one of two places in turn: nobody is more than one item ahead.
           if (tid == 0) {
             const volatile int* flag = d.w_ready;
             const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
@@ -537,24 +548,26 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
               atomicExch(d.step_bad, 1);
               atomicCAS(d.status, 0, 8 /* NGALORE_ERR_TIMEOUT */);
             }
-            *s_flag = ok;
+            s_flag[combined & 1] = ok;
           }
-          consumer_sync<kConsumerThreads>();
-          item_ok = *s_flag != 0;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(meet_bar);
+          if (!mbar_wait_warp(meet_bar, combined & 1, abort_flag)) break;
+          item_ok = s_flag[combined & 1] != 0;
+          ++combined;
           __threadfence();
         }
-        if (tid < kMaxHistory) wsm[tid] = __ldcg(d.wsol + tid);
+        const float my_w = __ldcg(d.wsol + lane);
         const bool item_bad = __ldcg(d.step_bad) != 0;
         float *const it_m = d.m, *const it_v = d.v, *const it_cur = current_gradient(d, cur);
         __half* const it_u = d.u16;
         uint16_t *const it_m16 = d.m16, *const it_v16 = d.v16;
         uint16_t* const it_h16 = HIST16 ? d.H16 + static_cast<long long>(cur) * d.rn : nullptr;
         const unsigned int it_mat = static_cast<unsigned int>(d.index), it_step = static_cast<unsigned int>(ctrl->k);
-        consumer_sync<kConsumerThreads>();
         float w[SMAX];
 #pragma unroll
-        for (int j = 0; j < SMAX; ++j) w[j] = wsm[j];
-        const float wc = HIST16 ? wsm[cur] : 0.f;
+        for (int j = 0; j < SMAX; ++j) w[j] = __shfl_sync(0xffffffffu, my_w, j);
+        const float wc = HIST16 ? __shfl_sync(0xffffffffu, my_w, cur) : 0.f;
         while (true) {
           if (item_ok && idx < mt.count) {
             const long long e = mt.e0 + idx;
@@ -643,7 +656,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           const bool last = mt.last != 0;
           release();
           if (last) break;
-          if (!mbar_wait(full_bar + stage, phase, abort_flag)) { alive = false; break; }
+          if (!mbar_wait_warp(full_bar + stage, phase, abort_flag)) { alive = false; break; }
           mt = meta[stage];
         }
         if (!alive) break;
