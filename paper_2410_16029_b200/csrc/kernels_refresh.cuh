@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(256) basis_norms_kernel(const WorkingJob* jobs
 }
 
 __global__ void __launch_bounds__(256) working_copies_grouped_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
-  __shared__ uint16_t tile[kEndCols][kEndRows + 4];
+  __shared__ __align__(8) uint16_t tile[kEndCols][kEndRows + 4];   // (rows of 264 bytes, read eight at a time)
   const int j = end_job(tile_start, n_jobs);
   const WorkingJob jb = jobs[j];
   const int t = static_cast<int>(blockIdx.x) - tile_start[j];
