@@ -6,12 +6,11 @@
 // bf16 part (16 mantissa bits).  Between products the iterate only has to stay well conditioned, so
 // orth() is a *shifted* Cholesky QR: the Gram matrix Y^T Y comes from the tensor cores (three bf16
 // products, fp32 accumulation), its columns are scaled to unit norm and a small multiple of the identity
-// is added before the fp64 Cholesky factorisation so that the fp32 accumulation error cannot make it
-// indefinite, and
-// Q = Y R^-1 is again a tensor-core GEMM with R^-1 split in two bf16 parts.  The last basis is then
-// orthonormalised exactly (Gram, Cholesky and triangular solve in fp64), rotated to the Ritz vectors of G inside
-// the subspace (Z = G^T Q, eigenvectors V of Z^T Z by the kernels of ritz_eigen.cuh, P = Q V on the tensor
-// cores, columns in falling order of their singular value) and orthonormalised once more.
+// is added before the fp64 factorisation (tri_factor.cuh) so that the fp32 accumulation error cannot make it
+// indefinite, and Q = Y R^-1 is again a tensor-core GEMM with R^-1 split in two bf16 parts.  The last basis is then
+// orthonormalised exactly (Gram matrix, factorisation and triangular inverse in fp64) and by two Newton steps, and rotated to
+// the Ritz vectors of G inside the subspace (Z = G^T Q, eigenvectors V of Z^T Z by the kernels of ritz_eigen.cuh, P = Q V on
+// the tensor cores, columns in falling order of their singular value and scaled to unit norm).
 #pragma once
 
 #include <cstring>
@@ -489,8 +488,8 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     m.Rhi = reinterpret_cast<__nv_bfloat16*>(plan.buf + offs[i].Rhi);
     m.Rlo = reinterpret_cast<__nv_bfloat16*>(plan.buf + offs[i].Rlo);
     newton[i] = NewtonJob{m.C32, m.Rhi, m.Rlo, m.L, m.ldl};
-    factor32[i] = FactorMat{m.C32, m.C64, nullptr, m.Rhi, m.Rlo, m.L, m.ldl};
-    factor64[i] = FactorMat{m.X64, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
+    factor32[i] = FactorMat{m.C32, nullptr, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
+    factor64[i] = FactorMat{nullptr, m.X64, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
     m.Y1hi = reinterpret_cast<__nv_bfloat16*>(m.Yf);
     m.Y1lo = m.Y1hi + static_cast<size_t>(m.M) * m.ldl;
     syrk_m[i] = SyrkMat{m.Y1hi, m.Y1lo, m.X64, m.M, m.L, m.ldl};
@@ -721,8 +720,7 @@ inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStrea
   ngalore_status rc;
   if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, RP_GRAM_Y0, d_ctrl, stream, launches, false, true))) return rc;
-  // single precision from here to R^-1: the Gram matrix has 2^-17 of relative accuracy and a shift of about 1e-2
-  if (tri_factor_launch<float>(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_01, d_ctrl, stream, launches);
 }
 
@@ -735,7 +733,7 @@ inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStre
   *launches += 1;
   syrk_f64_kernel<<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
   *launches += 1;
-  if (tri_factor_launch<double>(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_10, d_ctrl, stream, launches);
 }
 

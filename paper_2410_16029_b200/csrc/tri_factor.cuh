@@ -10,16 +10,19 @@
 // one lower triangle of 32 x 32 blocks, and a step is a single symmetric-looking rank-32 update of it.  Row k of Lf^-1 is
 // final after its step and goes out as columns of R^-1.
 //
-// All products run on the tensor cores: fp64 matrices on the fp64 ones (which here have the rate of the vector units,
-// but need a fraction of the instructions and operand reads), fp32 matrices as three TF32 products of operands split in
-// two parts of eleven bits (2^-21 of a product is lost, with the Gram matrix good to 2^-17).  One warp factors and
-// inverts the next diagonal block as soon as that has its update, while the other fifteen update the rest.  The
-// blocks live in shared memory where they fit (fp32: up to 256 columns, fp64: up to 160), else in L2.
+// All of it is fp64, the products on the fp64 tensor cores (which here have the rate of the vector units, but need a
+// fraction of the instructions and operand reads), also where C comes as fp32 from the tensor cores: scaled, such a matrix has
+// a condition of up to 65536, which takes four digits off whatever precision the elimination has.  In fp32 with the
+// products as three TF32 products of operands in two parts it took two thirds of the time (58 matrices of 128
+// columns 35 us, 84 of 256 86, 156 of up to 512 493), but left R^-1 two to ten times as far from 64 bits as a plain fp32
+// factorisation does (the sums of the tensor cores are truncated); fp32 multiply-adds on the vector units take as long as
+// fp64 tensor cores and are no closer at 32 and 64 columns.  As it is, the two bf16 parts of the result are what decides.
+// One warp factors and inverts the next diagonal block as soon as that has its update, while the other fifteen update
+// the rest.  The blocks live in shared memory where they fit (up to 160 columns), else in L2.
 // It replaced a scaling kernel, a Cholesky factorisation with one CTA per matrix, a recursive triangular inverse (two
-// batched products per level) and a conversion: 12 launches.  Measured per orthonormalisation, fp32: 58 matrices of 128
-// columns 125 -> 36 us, 84 of 256 310 -> 89 us, 156 of up to 512 1600 -> 493 us; the fp64 pass of the same sets 190 -> 52,
-// 490 -> 150 and 2900 -> 900 us.  What is left is the chain of diagonal blocks up to 256 columns (6 400 cycles each) and
-// the tensor cores' rate for TF32 beyond.
+// batched products per level) and a conversion: 12 launches.  Measured per orthonormalisation: 58 matrices of 128 columns 50 us,
+// 84 of 256 150, 156 of up to 512 900 (those launches: in fp32 125, 310 and 1600 us, in fp64 190, 490 and 2900).  What is left
+// is the chain of diagonal blocks up to 256 columns (8 000 cycles each) and the fp64 tensor cores' rate beyond.
 #pragma once
 
 #include "common.cuh"
@@ -34,9 +37,10 @@ constexpr int kTfLdW = kTfNB + 8;    // row length of the diagonal block's work 
 constexpr int kTfLdS8 = 12;          // ... and of its operands
 
 struct FactorMat {
-  const void* C;        // L x L (T), lower triangle valid
-  void* work;           // blocks of the lower triangle, where they do not fit shared memory
-  void* spill;          // rows of S, where they do not fit shared memory
+  const float* C32;     // the Gram matrix, L x L, lower triangle valid: fp32 ...
+  const double* C64;    // ... or fp64
+  double* work;         // blocks of the lower triangle, where they do not fit shared memory
+  double* spill;        // rows of S, where they do not fit shared memory
   __nv_bfloat16* Rhi;   // L x ld: high part of R^-1
   __nv_bfloat16* Rlo;
   int L, ld;
@@ -45,56 +49,19 @@ struct FactorMat {
 };
 
 // Shared memory without the blocks.
-template <typename T>
 __host__ __device__ inline size_t tf_base_smem(int L, bool s_global) {
   const size_t np = static_cast<size_t>((L + kTfNB - 1) / kTfNB) * kTfNB;
-  return sizeof(T) * ((s_global ? 0 : np * kTfLd) + np + kTfNB * (2 * kTfLd + kTfLdW + kTfLdS8) + 64);
+  return sizeof(double) * ((s_global ? 0 : np * kTfLd) + np + kTfNB * (2 * kTfLd + kTfLdW + kTfLdS8) + 64);
 }
 // Rows of S in global memory.
 __host__ __device__ inline size_t tf_spill_doubles(int L) { return static_cast<size_t>((L + kTfNB - 1) / kTfNB) * kTfNB * kTfLd; }
-template <typename T>
 __host__ __device__ inline size_t tf_block_bytes(int L) {
   const size_t nb = (L + kTfNB - 1) / kTfNB;
-  return sizeof(T) * nb * (nb + 1) / 2 * kTfNB * kTfNB;
-}
-
-__device__ __forceinline__ void tf_mma(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-__device__ __forceinline__ void tf_split(float x, uint32_t& hi, uint32_t& lo) {
-  hi = __float_as_uint(x) & 0xffffe000u;
-  lo = __float_as_uint(x - __uint_as_float(hi));
+  return sizeof(double) * nb * (nb + 1) / 2 * kTfNB * kTfNB;
 }
 
 // acc[mt][nt][h] (entry (8 mt + lane / 4, 8 nt + 2 (lane % 4) + h) of a 32 x 32 block) += left(row, k) right(col, k),
 // summed over K values of k.
-template <int K, typename FL, typename FR>
-__device__ __forceinline__ void tf_product(float (&acc)[4][4][2], FL left, FR right, int fr, int fk) {
-#pragma unroll
-  for (int k0 = 0; k0 < K; k0 += 8) {
-    uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) tf_split(left(16 * m + 8 * (e & 1) + fr, k0 + 4 * (e >> 1) + fk), ah[m][e], al[m][e]);
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) tf_split(right(8 * n + fr, k0 + 4 * e + fk), bh[n][e], bl[n][e]);
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        float c[4] = {acc[2 * m][n][0], acc[2 * m][n][1], acc[2 * m + 1][n][0], acc[2 * m + 1][n][1]};
-        tf_mma(c, al[m], bh[n]);
-        tf_mma(c, ah[m], bl[n]);
-        tf_mma(c, ah[m], bh[n]);
-        acc[2 * m][n][0] = c[0]; acc[2 * m][n][1] = c[1]; acc[2 * m + 1][n][0] = c[2]; acc[2 * m + 1][n][1] = c[3];
-      }
-  }
-}
 template <int K, typename FL, typename FR>
 __device__ __forceinline__ void tf_product(double (&acc)[4][4][2], FL left, FR right, int fr, int fk) {
 #pragma unroll
@@ -114,47 +81,28 @@ __device__ __forceinline__ void tf_product(double (&acc)[4][4][2], FL left, FR r
 }
 
 __device__ __forceinline__ int tf_at(int row, int col) { return row * kTfNB + (col ^ ((row & 3) * 8)); }   // inside a block
-// 1 / sqrt(x): the approximation and one Newton step (fp32, to about one unit in the last place), the function (fp64).
-__device__ __forceinline__ float tf_rsqrt(float x) {
-  const float y = rsqrtf(x);
-  return y * (1.5f - 0.5f * x * y * y);
-}
-__device__ __forceinline__ double tf_rsqrt(double x) { return rsqrt(x); }
 
-template <typename T>
-struct alignas(16) TfVec { T v[16 / sizeof(T)]; };
 // Eight consecutive numbers.
-template <typename T>
-__device__ __forceinline__ void tf_load8(const T* p, T (&v)[8]) {
-  constexpr int N = 16 / sizeof(T);
+__device__ __forceinline__ void tf_load8(const double* p, double (&v)[8]) {
 #pragma unroll
-  for (int q = 0; q < 8 / N; ++q) {
-    const TfVec<T> x = reinterpret_cast<const TfVec<T>*>(p)[q];
-#pragma unroll
-    for (int y = 0; y < N; ++y) v[q * N + y] = x.v[y];
+  for (int q = 0; q < 4; ++q) {
+    const double2 x = reinterpret_cast<const double2*>(p)[q];
+    v[2 * q] = x.x; v[2 * q + 1] = x.y;
   }
 }
-template <typename T>
-__device__ __forceinline__ void tf_store8(T* p, const T (&v)[8]) {
-  constexpr int N = 16 / sizeof(T);
+__device__ __forceinline__ void tf_store8(double* p, const double (&v)[8]) {
 #pragma unroll
-  for (int q = 0; q < 8 / N; ++q) {
-    TfVec<T> x;
-#pragma unroll
-    for (int y = 0; y < N; ++y) x.v[y] = v[q * N + y];
-    reinterpret_cast<TfVec<T>*>(p)[q] = x;
-  }
+  for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(p)[q] = make_double2(v[2 * q], v[2 * q + 1]);
 }
 
 // One warp: Inv = inverse of the Cholesky factor of the 32 x 32 block at blk, by the elimination described at the top
 // once more, in blocks of eight.  A pivot that is not above tiny is replaced by it, so that the factor of a
 // rank-deficient matrix stays finite.  (Column by column, 32 steps of shuffle, square root, scaling and update, it took
 // 19 000 cycles and bounded the kernel.)
-template <typename T>
-__device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T* I8, T* Inv, int lane) {
+__device__ __forceinline__ void tf_diagonal(const double* blk, double tiny, double* W, double* S8, double* I8, double* Inv, int lane) {
   const int fr = lane >> 2, fk = lane & 3;
   {
-    T r[kTfNB];
+    double r[kTfNB];
 #pragma unroll
     for (int q = 0; q < kTfNB; ++q) r[q] = blk[tf_at(q, lane)];
 #pragma unroll
@@ -166,14 +114,14 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
     // the 8 x 8 block: every lane computes all of its factor (shuffles would double the length of the chain), then one
     // column of the inverse
     {
-      T r[8][8], x[8], inv[8];
+      double r[8][8], x[8], inv[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) tf_load8(W + (c0 + i) * kTfLdW + c0, r[i]);
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
-        T d = r[t][t];
+        double d = r[t][t];
         if (!(d > tiny)) d = tiny;
-        inv[t] = tf_rsqrt(d);
+        inv[t] = rsqrt(d);
 #pragma unroll
         for (int i = t + 1; i < 8; ++i) r[i][t] *= inv[t];
 #pragma unroll
@@ -182,7 +130,7 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
           for (int i = j; i < 8; ++i) r[i][j] -= r[i][t] * r[j][t];
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = i == (lane & 7) ? T(1) : T(0);
+      for (int i = 0; i < 8; ++i) x[i] = i == (lane & 7) ? 1.0 : 0.0;
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         x[t] *= inv[t];
@@ -197,33 +145,33 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
     __syncwarp();
     // the operands, lane = row, and rows c0 .. c0 + 7 of the result
     {
-      T v[8], o[8];
+      double v[8], o[8];
       if (lane >= c0 + 8) {
         tf_load8(W + lane * kTfLdW + c0, v);
       } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = lane < c0 ? W[(c0 + q) * kTfLdW + lane] : (lane == c0 + q ? T(1) : T(0));
+        for (int q = 0; q < 8; ++q) v[q] = lane < c0 ? W[(c0 + q) * kTfLdW + lane] : (lane == c0 + q ? 1.0 : 0.0);
       }
 #pragma unroll
       for (int n = 0; n < 8; ++n) {
-        T row[8];
+        double row[8];
         tf_load8(I8 + n * 8, row);
-        o[n] = T(0);
+        o[n] = 0.0;
 #pragma unroll
         for (int q = 0; q <= n; ++q) o[n] += row[q] * v[q];
-        Inv[(c0 + n) * kTfLd + lane] = lane < c0 + 8 ? o[n] : T(0);
+        Inv[(c0 + n) * kTfLd + lane] = lane < c0 + 8 ? o[n] : 0.0;
       }
       tf_store8(S8 + lane * kTfLdS8, o);
       __syncwarp();
       if (lane >= c0 + 8) {
-        const T zero[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+        const double zero[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         tf_store8(W + lane * kTfLdW + c0, zero);
       }
     }
     __syncwarp();
     if (c0 + 8 == kTfNB) break;
     // (rows up to c0 + 7 are not read any more: they may take part)
-    T acc[4][4][2];
+    double acc[4][4][2];
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -242,7 +190,7 @@ __device__ __forceinline__ void tf_diagonal(const T* blk, T tiny, T* W, T* S8, T
   }
 }
 
-template <typename T, bool S_GLOBAL>
+template <bool S_GLOBAL>
 __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorMat* mats, int smem_bytes, double shift_scale, int conditional) {
   constexpr int NB = kTfNB, LD = kTfLd, WARPS = kTfThreads / 32;
   extern __shared__ __align__(16) unsigned char tf_smem[];
@@ -251,25 +199,26 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
   if (conditional && *m.only_if == 0) return;
   const int L = m.L, nb = (L + NB - 1) / NB, np = nb * NB;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
-  T* Inv0 = reinterpret_cast<T*>(tf_smem);            // [2][NB][LD]
-  T* W = Inv0 + 2 * NB * LD;                           // work space of the diagonal block: [NB][kTfLdW],
-  T* S8 = W + NB * kTfLdW;                             // [NB][kTfLdS8],
-  T* I8 = S8 + NB * kTfLdS8;                           // [8][8]
-  T* rd = I8 + 64;                                     // [np] 1 / column norm
-  T* Ssh = rd + np;
-  T* S = S_GLOBAL ? static_cast<T*>(m.spill) : Ssh;    // [np][LD]
-  const bool resident = tf_base_smem<T>(L, S_GLOBAL) + tf_block_bytes<T>(L) <= static_cast<size_t>(smem_bytes);
-  T* B = resident ? (S_GLOBAL ? Ssh : Ssh + np * LD) : static_cast<T*>(m.work);
-  const T* C = static_cast<const T*>(m.C);
-  auto block = [&](int i, int j) -> T* { return B + (i * (i + 1) / 2 + j) * (NB * NB); };
-  const T tiny = sizeof(T) == 8 ? T(1e-28) : T(1e-12);
-  const T one = T(1.0 + (sizeof(T) == 8 ? shift_scale : shift_scale * static_cast<double>(L) / 65536.0));
+  double* Inv0 = reinterpret_cast<double*>(tf_smem);            // [2][NB][LD]
+  double* W = Inv0 + 2 * NB * LD;                           // work space of the diagonal block: [NB][kTfLdW],
+  double* S8 = W + NB * kTfLdW;                             // [NB][kTfLdS8],
+  double* I8 = S8 + NB * kTfLdS8;                           // [8][8]
+  double* rd = I8 + 64;                                     // [np] 1 / column norm
+  double* Ssh = rd + np;
+  double* S = S_GLOBAL ? m.spill : Ssh;    // [np][LD]
+  const bool resident = tf_base_smem(L, S_GLOBAL) + tf_block_bytes(L) <= static_cast<size_t>(smem_bytes);
+  double* B = resident ? (S_GLOBAL ? Ssh : Ssh + np * LD) : m.work;
+  auto gram = [&](int r, int c) {
+    const long long o = static_cast<long long>(r) * L + c;
+    return m.C32 != nullptr ? static_cast<double>(m.C32[o]) : m.C64[o];
+  };
+  auto block = [&](int i, int j) -> double* { return B + (i * (i + 1) / 2 + j) * (NB * NB); };
+  const double tiny = 1e-28, one = 1.0 + (m.C32 != nullptr ? shift_scale * static_cast<double>(L) / 65536.0 : shift_scale);
 
   for (int i = tid; i < np; i += kTfThreads) {
-    T d = i < L ? C[static_cast<long long>(i) * L + i] : T(1);
-    const T floor = sizeof(T) == 8 ? T(1e-60) : T(1e-37);
-    if (!(d > floor)) d = d == d ? floor : d;          // (a NaN stays one, and the basis check finds it)
-    rd[i] = tf_rsqrt(d);
+    double d = i < L ? gram(i, i) : 1.0;
+    if (!(d > 1e-60)) d = d == d ? 1e-60 : d;          // (a NaN stays one, and the basis check finds it)
+    rd[i] = rsqrt(d);
   }
   __syncthreads();
   // the scaled matrix (beyond L: the identity)
@@ -279,17 +228,17 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
     while (i * (i + 1) / 2 > b) --i;
     const int j = b - i * (i + 1) / 2;
     const int c = j * NB + lane;
-    T* dst = B + b * (NB * NB);
+    double* dst = B + b * (NB * NB);
 #pragma unroll 1
     for (int row0 = 0; row0 < NB; row0 += 16) {
-      T raw[16];
+      double raw[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) raw[q] = C[static_cast<long long>(min(i * NB + row0 + q, L - 1)) * L + min(c, L - 1)];
+      for (int q = 0; q < 16; ++q) raw[q] = gram(min(i * NB + row0 + q, L - 1), min(c, L - 1));
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         const int row = row0 + q, r = i * NB + row;
-        const T v = raw[q] * rd[r] * rd[c];
-        dst[tf_at(row, lane)] = r == c ? (r < L ? one : T(1)) : (r < L && c < r ? v : T(0));
+        const double v = raw[q] * rd[r] * rd[c];
+        dst[tf_at(row, lane)] = r == c ? (r < L ? one : 1.0) : (r < L && c < r ? v : 0.0);
       }
     }
   }
@@ -297,20 +246,20 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
   __syncthreads();
 
   for (int k = -1; k < nb; ++k) {
-    const T* Inv = Inv0 + (k & 1) * NB * LD;
+    const double* Inv = Inv0 + (k & 1) * NB * LD;
     // S, and block column k of R^-1
     for (int i = warp; i < nb && k >= 0; i += WARPS) {
-      T acc[4][4][2];
+      double acc[4][4][2];
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = T(0);
+        for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = 0.0;
       auto right = [&](int n, int kk) { return Inv[n * LD + kk]; };
       if (i > k) {
-        const T* blk = block(i, k);
+        const double* blk = block(i, k);
         tf_product<NB>(acc, [&](int r, int kk) { return blk[tf_at(r, kk)]; }, right, fr, fk);
       } else if (i < k) {
-        const T* blk = block(k, i);
+        const double* blk = block(k, i);
         tf_product<NB>(acc, [&](int r, int kk) { return blk[tf_at(kk, r)]; }, right, fr, fk);
       } else {
 #pragma unroll
@@ -323,7 +272,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         const int row = i * NB + 8 * x + fr;
-        const T scale = rd[row];
+        const double scale = rd[row];
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
           const int kk = 8 * y + 2 * fk, col = k * NB + kk;
@@ -332,7 +281,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
           if (m.R64 != nullptr) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-              if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? static_cast<double>(acc[x][y][h] * scale) : 0.0;
+              if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? acc[x][y][h] * scale : 0.0;
           } else if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
             float f[2];
 #pragma unroll
@@ -370,15 +319,15 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
         while ((i + 1) * (i + 2) / 2 <= t) ++i;
         while (i * (i + 1) / 2 > t) --i;
         const int j = t - i * (i + 1) / 2;
-        T* blk = block(i, j);
-        T acc[4][4][2];
+        double* blk = block(i, j);
+        double acc[4][4][2];
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
           for (int y = 0; y < 4; ++y)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) acc[x][y][h] = j == k ? T(0) : blk[tf_at(8 * x + fr, 8 * y + 2 * fk) + h];
-        const T *Si = S + i * NB * LD, *Sj = S + j * NB * LD;
+            for (int h = 0; h < 2; ++h) acc[x][y][h] = j == k ? 0.0 : blk[tf_at(8 * x + fr, 8 * y + 2 * fk) + h];
+        const double *Si = S + i * NB * LD, *Sj = S + j * NB * LD;
         tf_product<NB>(acc, [&](int r, int kk) { return -Si[r * LD + kk]; }, [&](int n, int kk) { return Sj[n * LD + kk]; }, fr, fk);
 #pragma unroll
         for (int x = 0; x < 4; ++x)
@@ -389,7 +338,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
       }
       if (first) {
         __syncwarp();
-        tf_diagonal<T>(block(k + 1, k + 1), tiny, W, S8, I8, Inv0 + ((k + 1) & 1) * NB * LD, lane);
+        tf_diagonal(block(k + 1, k + 1), tiny, W, S8, I8, Inv0 + ((k + 1) & 1) * NB * LD, lane);
         first = false;
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (k < 0) break;
@@ -405,32 +354,26 @@ constexpr int kTfSmemLimit = 232448 - 256;   // (the kernel has 128 bytes of its
 
 // (to their largest values: the limit of a kernel belongs to the process, not to one state)
 inline cudaError_t tri_factor_init() {
-  cudaError_t e;
   auto set = [](const void* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmemLimit); };
-  if ((e = set(reinterpret_cast<const void*>(tri_factor_kernel<float, false>))) != cudaSuccess) return e;
-  if ((e = set(reinterpret_cast<const void*>(tri_factor_kernel<double, false>))) != cudaSuccess) return e;
-  return set(reinterpret_cast<const void*>(tri_factor_kernel<double, true>));
+  const cudaError_t e = set(reinterpret_cast<const void*>(tri_factor_kernel<false>));
+  return e != cudaSuccess ? e : set(reinterpret_cast<const void*>(tri_factor_kernel<true>));
 }
 
 // Factor n matrices, the widest l_max wide (widest first in the list: CTAs are handed out in order).  shift_scale: what
 // is added to the unit diagonal, for fp32 matrices in units of L / 65536.
-template <typename T>
 inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, double shift_scale, cudaStream_t stream,
                                      int64_t* launches, bool conditional = false) {
   // as much shared memory as the widest matrix that fits with its blocks, and at least what the widest needs without
-  size_t smem = tf_base_smem<T>(l_max, false);
+  size_t smem = tf_base_smem(l_max, false);
   const bool s_global = smem > static_cast<size_t>(kTfSmemLimit);
-  if (s_global) smem = tf_base_smem<T>(l_max, true);
+  if (s_global) smem = tf_base_smem(l_max, true);
   for (int l = l_max; l > 0; l -= 4) {
-    const size_t need = tf_base_smem<T>(l, s_global) + tf_block_bytes<T>(l);
+    const size_t need = tf_base_smem(l, s_global) + tf_block_bytes(l);
     if (need <= static_cast<size_t>(kTfSmemLimit)) { smem = need > smem ? need : smem; break; }
   }
-  if (s_global) {
-    if (sizeof(T) == 4) return cudaErrorInvalidValue;   // (an fp32 basis of 875 columns needs 147 KB)
-    tri_factor_kernel<double, true><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
-  } else {
-    tri_factor_kernel<T, false><<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
-  }
+  auto run = [&](auto kernel) { kernel<<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0); };
+  if (s_global) run(tri_factor_kernel<true>);
+  else run(tri_factor_kernel<false>);
   *launches += 1;
   return cudaGetLastError();
 }
