@@ -801,7 +801,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   // (the limit of a kernel belongs to the process: it must hold for the widest state, whichever is created last)
   if (cudaFuncSetAttribute(orth_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(prop.sharedMemPerBlockOptin)) != cudaSuccess ||
-      tri_factor_init() != cudaSuccess || eig_init(static_cast<int>(eig_n)) != cudaSuccess)
+      !eig_fits(static_cast<int>(eig_n)))
     return fail(NGALORE_ERR_CUDA);
 
   const bool allow_gram_fusion = st->opt.gemm_impl != 1 && st->opt.stream_impl != 1 && !hist16 && st->opt.gram_fusion == 1;

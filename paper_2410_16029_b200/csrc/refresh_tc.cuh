@@ -639,16 +639,20 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   }
 
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
+  // (the four products with G that this plan takes: setting an attribute loads a kernel, the first state of a process would
+  // pay for all sixteen)
   auto init = [](auto p) { return cudaFuncSetAttribute(p.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p.kSmem) == cudaSuccess; };
-  auto init_both = [&](auto p, auto q) { return init(p) && init(q); };
-  if (!init_both(RefProduct<kRefWideBN, 1, 1, false>{}, RefProduct<kRefWideBN, 1, 1, true>{}) ||
-      !init_both(RefProduct<kRefWideBN, 2, 1, false>{}, RefProduct<kRefWideBN, 2, 1, true>{}) ||
-      !init_both(RefProduct<kRefWideBN, 1, 2, false>{}, RefProduct<kRefWideBN, 1, 2, true>{}) ||
-      !init_both(RefProduct<kRefWideBN, 2, 2, false>{}, RefProduct<kRefWideBN, 2, 2, true>{}) ||
-      !init_both(RefProduct<kRefBN, 1, 1, false>{}, RefProduct<kRefBN, 1, 1, true>{}) ||
-      !init_both(RefProduct<kRefBN, 2, 1, false>{}, RefProduct<kRefBN, 2, 1, true>{}) ||
-      !init_both(RefProduct<kRefBN, 1, 2, false>{}, RefProduct<kRefBN, 1, 2, true>{}) ||
-      !init_both(RefProduct<kRefBN, 2, 2, false>{}, RefProduct<kRefBN, 2, 2, true>{}) ||
+  auto init_all = [&](auto bn, auto mt) {
+    constexpr int BN = decltype(bn)::value, MT = decltype(mt)::value;
+    return init(RefProduct<BN, 1, MT, false>{}) && init(RefProduct<BN, 1, MT, true>{}) && init(RefProduct<BN, 2, MT, false>{}) &&
+           init(RefProduct<BN, 2, MT, true>{});
+  };
+  using Wide = std::integral_constant<int, kRefWideBN>;
+  using Narrow = std::integral_constant<int, kRefBN>;
+  using Tall = std::integral_constant<int, 2>;
+  using Flat = std::integral_constant<int, 1>;
+  if (!(plan.wide ? (plan.tall ? init_all(Wide{}, Tall{}) : init_all(Wide{}, Flat{}))
+                  : (plan.tall ? init_all(Narrow{}, Tall{}) : init_all(Narrow{}, Flat{}))) ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true>,

@@ -352,13 +352,6 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
 
 constexpr int kTfSmemLimit = 232448 - 256;   // (the kernel has 128 bytes of its own)
 
-// (to their largest values: the limit of a kernel belongs to the process, not to one state)
-inline cudaError_t tri_factor_init() {
-  auto set = [](const void* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmemLimit); };
-  const cudaError_t e = set(reinterpret_cast<const void*>(tri_factor_kernel<false>));
-  return e != cudaSuccess ? e : set(reinterpret_cast<const void*>(tri_factor_kernel<true>));
-}
-
 // Factor n matrices, the widest l_max wide (widest first in the list: CTAs are handed out in order).  shift_scale: what
 // is added to the unit diagonal, for fp32 matrices in units of L / 65536.
 inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, double shift_scale, cudaStream_t stream,
@@ -371,11 +364,16 @@ inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, 
     const size_t need = tf_base_smem(l, s_global) + tf_block_bytes(l);
     if (need <= static_cast<size_t>(kTfSmemLimit)) { smem = need > smem ? need : smem; break; }
   }
-  auto run = [&](auto kernel) { kernel<<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0); };
-  if (s_global) run(tri_factor_kernel<true>);
-  else run(tri_factor_kernel<false>);
-  *launches += 1;
-  return cudaGetLastError();
+  // (the limit to its largest value, since it belongs to the process and not to one state, and here, so that only a kernel
+  // that is launched gets loaded)
+  auto run = [&](auto kernel) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmemLimit);
+    if (e != cudaSuccess) return e;
+    kernel<<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
+    *launches += 1;
+    return cudaGetLastError();
+  };
+  return s_global ? run(tri_factor_kernel<true>) : run(tri_factor_kernel<false>);
 }
 
 }  // namespace ngalore
