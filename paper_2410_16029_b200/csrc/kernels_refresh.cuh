@@ -327,8 +327,9 @@ __global__ void working_copies_kernel(const float* P32, uint16_t* P16, uint16_t*
 // relative 2^-17) scales a whole column, which is the largest part of what the last product leaves of
 // non-orthonormality.  The norms also tell a basis that is none (see basis_check_kernel): all of them zero, or one not
 // finite; such a matrix gets the first r' unit vectors, in the second case with its status word set.
-// CTAs take tiles of kEndRows rows (norms) and kEndRows x kEndCols entries (copies); tile_start[j] is the first tile of
-// job j (n_jobs + 1 entries, ascending).  Bound by memory traffic: 4 bytes an entry read, then 12.  They replaced five
+// CTAs take tiles of norm_rows rows (norms) and kEndRows x kEndCols entries (copies); tile_start[j] is the first tile of
+// job j (n_jobs + 1 entries, ascending).  Up to 2048 rows make two tiles for the norms, whose sums give the same bits in either
+// order.  Bound by memory traffic: 4 bytes an entry read, then 12.  They replaced five
 // kernels of five passes with one CTA count for every matrix, so that a 32000-row embedding took as many CTAs as a
 // 512-row matrix: 60M shapes 316 us, 130M 680 us, 1.1B 2620 us before, 48, 113 and 610 us now.
 struct WorkingJob {
@@ -341,8 +342,10 @@ struct WorkingJob {
   int rows, rp, ldp, ldpt;
   int p16_is_half;
   int tiles_x;        // tiles along the rp columns
+  int norm_rows;      // rows of a tile for the norms (end_norm_rows)
 };
 constexpr int kEndRows = 128, kEndCols = 64;
+inline int end_norm_rows(int rows) { return rows <= 2048 && rows > 2 * kEndRows ? (rows + 1) / 2 : kEndRows; }
 
 __device__ __forceinline__ int end_job(const int* tile_start, int n_jobs) {
   int lo = 0, hi = n_jobs;
@@ -356,7 +359,7 @@ __device__ __forceinline__ int end_job(const int* tile_start, int n_jobs) {
 __global__ void __launch_bounds__(256) basis_norms_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
   const int j = end_job(tile_start, n_jobs);
   const WorkingJob jb = jobs[j];
-  const int r0 = (static_cast<int>(blockIdx.x) - tile_start[j]) * kEndRows, r1 = min(r0 + kEndRows, jb.rows);
+  const int r0 = (static_cast<int>(blockIdx.x) - tile_start[j]) * jb.norm_rows, r1 = min(r0 + jb.norm_rows, jb.rows);
   const int quads = jb.rp >> 2;
   // thread: a column quad (there are at most 219) and every `groups`-th row
   __shared__ double part[256][4];
