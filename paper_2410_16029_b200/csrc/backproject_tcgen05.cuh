@@ -305,8 +305,9 @@ inline ngalore_status tc_backproject_init() {
 }
 
 // W <- (1 - lr wd) W - lr P u for the tiles [t0, t1) of TcPlan::d_tiles_back, through the tensor maps tc_bind_buffers set up.  last: the
-// launch ends the step (it moves the counters on).  chained: nothing but the step's own kernels sits before it in the
-// stream (no event to wait for), so it may be a programmatic dependent launch.
+// launch ends the step (it moves the counters on).  chained: the step's stream kernel comes right before
+// it, so that an early start hides a launch; a launch that waits for a group's copies, or follows another one of this
+// kernel, has nothing to hide.
 inline ngalore_status tc_backproject_range(TcPlan& plan, int t0, int t1, const MatDesc* d_mats, Ctrl* d_ctrl,
                                            const Hyper* d_hyper, bool last, bool chained, cudaStream_t stream, int64_t* launches) {
   if (t1 <= t0) return NGALORE_OK;

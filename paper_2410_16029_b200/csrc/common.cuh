@@ -103,7 +103,8 @@ __device__ __forceinline__ void advance_step(Ctrl* ctrl) {
 // the stream still runs.  pdl_begin lets the successor start in turn and then waits until the predecessor has finished
 // and its writes are visible; what comes before it (barriers, tensor memory) and the launch itself overlap the
 // predecessor's tail.  Every kernel that launch_step is given calls it before it touches global memory; after an ordinary
-// launch it returns at once.
+// launch it returns at once.  What else the launch comes after in its stream, a wait for an event among it, stays a full
+// dependency, so the first kernel of a step may be launched so whatever the caller has put before it.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

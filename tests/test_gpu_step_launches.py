@@ -17,6 +17,9 @@ M, N, R, S = 2048, 2048, 64, 3      # 128 tiles a matrix
 
 
 def _run(n, how):
+    """how: waited (for every step), queued, graph (captured on one stream), joined and joined-graph (the gradients of a
+    step are written on a second stream, which the stepping stream waits for by an event just before the step; a wait
+    ahead of the write makes sure that it comes late)."""
     from paper_2410_16029_b200.ngalore import NGaLore
 
     gen = torch.Generator(device="cuda").manual_seed(7)
@@ -33,7 +36,31 @@ def _run(n, how):
         for i in range(3):
             buf[i].copy_(grads[k & 1][i])
 
-    if how == "graph":
+    side = torch.cuda.Stream()
+
+    def load_beside(k):
+        main = torch.cuda.current_stream()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(2000000)      # about a millisecond
+            load(k)
+        main.wait_event(side.record_event())
+
+    if how == "joined-graph":
+        load(0)
+        opt.step(W, G)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for k in (1, 0, 0):
+                load_beside(k)
+                opt.step(W, G)
+        graph.replay()
+    elif how == "joined":
+        for k in (0, 1, 0, 0):
+            load_beside(k)
+            opt.step(W, G)
+    elif how == "graph":
         load(0)
         opt.step(W, G)                      # binds the buffers
         load(1)
@@ -59,7 +86,7 @@ def _run(n, how):
 @pytest.mark.parametrize("n", [1, 37, 38])
 def test_queued_and_captured_steps_equal_waited_ones(n):
     want = _run(n, "waited")
-    for how in ("queued", "graph"):
+    for how in ("queued", "graph", "joined", "joined-graph"):
         got = _run(n, how)
         for i in range(n):
             err = (torch.linalg.norm(got[i] - want[i]) / torch.linalg.norm(want[i])).item()
