@@ -516,8 +516,8 @@ struct TcPlan {
   std::vector<int> rowsN;           // per matrix: M, N for re-encoding the maps of G and W
   std::vector<int> colsN;
   std::vector<int> right;           // per matrix: projected on the right
-  // Steps of at most about 0.3 ms (32 back-projection tiles a CTA) launch their kernels as programmatic dependents, which
-  // hides the 2 us between two kernels: 60M shapes 222 -> 214 us, encoder shapes at r = 8 189 -> 180, one matrix 54 -> 46.
+  // Steps of at most 32 back-projection tiles a CTA (the 130M shapes have 28) launch their kernels as programmatic dependents,
+  // which hides the 2 us between two kernels: 60M shapes 222 -> 214 us, encoder shapes at r = 8 189 -> 180, one matrix 54 -> 46.
   // Longer ones do not: it changes which SM gets which CTA, and with it which tiles run side by side: 1.1B shapes 7.20 ->
   // 7.32 ms, at r = 8 1.915 -> 1.957 ms, 130M and 350M the same either way.
   bool short_step = false;
