@@ -4,6 +4,8 @@
 // the Gram matrix and the factorisation in fp64).
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace ngalore {
@@ -327,7 +329,7 @@ __global__ void working_copies_kernel(const float* P32, uint16_t* P16, uint16_t*
 // relative 2^-17) scales a whole column, which is the largest part of what the last product leaves of
 // non-orthonormality.  The norms also tell a basis that is none (see basis_check_kernel): all of them zero, or one not
 // finite; such a matrix gets the first r' unit vectors, in the second case with its status word set.
-// CTAs take tiles of norm_rows rows (norms) and kEndRows x kEndCols entries (copies); tile_start[j] is the first tile of
+// CTAs take tiles of norm_rows x kEndCols (norms) and kEndRows x kEndCols entries (copies); tile_start[j] is the first tile of
 // job j (n_jobs + 1 entries, ascending).  Up to 2048 rows make two tiles for the norms, whose sums give the same bits in either
 // order.  Bound by memory traffic: 4 bytes an entry read, then 12.  They replaced five
 // kernels of five passes with one CTA count for every matrix, so that a 32000-row embedding took as many CTAs as a
@@ -345,7 +347,7 @@ struct WorkingJob {
   int norm_rows;      // rows of a tile for the norms (end_norm_rows)
 };
 constexpr int kEndRows = 128, kEndCols = 64;
-inline int end_norm_rows(int rows) { return rows <= 2048 && rows > 2 * kEndRows ? (rows + 1) / 2 : kEndRows; }
+inline int end_norm_rows(int rows) { return rows <= 2048 ? std::max((rows + 1) / 2, kEndRows) : 2 * kEndRows; }
 
 __device__ __forceinline__ int end_job(const int* tile_start, int n_jobs) {
   int lo = 0, hi = n_jobs;
@@ -359,26 +361,29 @@ __device__ __forceinline__ int end_job(const int* tile_start, int n_jobs) {
 __global__ void __launch_bounds__(256) basis_norms_kernel(const WorkingJob* jobs, const int* tile_start, int n_jobs) {
   const int j = end_job(tile_start, n_jobs);
   const WorkingJob jb = jobs[j];
-  const int r0 = (static_cast<int>(blockIdx.x) - tile_start[j]) * jb.norm_rows, r1 = min(r0 + jb.norm_rows, jb.rows);
-  const int quads = jb.rp >> 2;
-  // thread: a column quad (there are at most 219) and every `groups`-th row
-  __shared__ double part[256][4];
-  const int groups = 256 / quads, g = threadIdx.x / quads, q = threadIdx.x % quads;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  if (g < groups) {
-#pragma unroll 4
-    for (int r = r0 + g; r < r1; r += groups) {
-      const float4 x = *reinterpret_cast<const float4*>(jb.src + static_cast<long long>(r) * jb.rp + 4 * q);
-      s0 += static_cast<double>(x.x) * x.x; s1 += static_cast<double>(x.y) * x.y;
-      s2 += static_cast<double>(x.z) * x.z; s3 += static_cast<double>(x.w) * x.w;
+  const int t = static_cast<int>(blockIdx.x) - tile_start[j];
+  const int r0 = (t / jb.tiles_x) * jb.norm_rows, r1 = min(r0 + jb.norm_rows, jb.rows);
+  // thread: four neighbouring columns and every sixteenth row
+  __shared__ double part[16][kEndCols + 2];
+  const int q = threadIdx.x & 15, g = threadIdx.x >> 4, c = (t % jb.tiles_x) * kEndCols + 4 * q;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  if (c < jb.rp) {
+#pragma unroll 8
+    for (int r = r0 + g; r < r1; r += 16) {
+      const float4 x = *reinterpret_cast<const float4*>(jb.src + static_cast<long long>(r) * jb.rp + c);
+      s[0] += static_cast<double>(x.x) * x.x; s[1] += static_cast<double>(x.y) * x.y;
+      s[2] += static_cast<double>(x.z) * x.z; s[3] += static_cast<double>(x.w) * x.w;
     }
   }
-  part[threadIdx.x][0] = s0; part[threadIdx.x][1] = s1; part[threadIdx.x][2] = s2; part[threadIdx.x][3] = s3;
+#pragma unroll
+  for (int y = 0; y < 4; ++y) part[g][4 * q + y] = s[y];
   __syncthreads();
-  for (int c = threadIdx.x; c < jb.rp; c += 256) {
-    double t = 0.0;
-    for (int x = 0; x < groups; ++x) t += part[x * quads + (c >> 2)][c & 3];
-    atomicAdd(jb.sums + c, t);
+  const int col = (t % jb.tiles_x) * kEndCols + threadIdx.x;
+  if (threadIdx.x < kEndCols && col < jb.rp) {
+    double sum = 0.0;
+#pragma unroll
+    for (int x = 0; x < 16; ++x) sum += part[x][threadIdx.x];
+    atomicAdd(jb.sums + col, sum);
   }
 }
 

@@ -840,7 +840,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
         jobs.push_back(WorkingJob{hm.Ya, st->refresh.mats[k].D, d.P32, d.P16, d.Pt16, st->d_status + i, hm.eM, hm.rp, d.ldp, d.ldpt,
                                   hm.right ? 0 : 1, tx, end_norm_rows(hm.eM)});
         start.push_back(start.back() + tx * ty);
-        nstart.push_back(nstart.back() + (hm.eM + end_norm_rows(hm.eM) - 1) / end_norm_rows(hm.eM));
+        nstart.push_back(nstart.back() + tx * ((hm.eM + end_norm_rows(hm.eM) - 1) / end_norm_rows(hm.eM)));
       }
       st->n_wjobs = static_cast<int>(jobs.size());
       st->n_wtiles = start.back();
