@@ -333,7 +333,7 @@ __global__ void working_copies_kernel(const float* P32, uint16_t* P16, uint16_t*
 // job j (n_jobs + 1 entries, ascending).  Up to 2048 rows make two tiles for the norms, whose sums give the same bits in either
 // order.  Bound by memory traffic: 4 bytes an entry read, then 12.  They replaced five
 // kernels of five passes with one CTA count for every matrix, so that a 32000-row embedding took as many CTAs as a
-// 512-row matrix: 60M shapes 316 us, 130M 680 us, 1.1B 2620 us before, 48, 113 and 610 us now.
+// 512-row matrix: 60M shapes 316 us, 130M 680 us, 1.1B 2620 us before, 52, 121 and 596 us now.
 struct WorkingJob {
   const float* src;   // rows x rp, dense; rp a multiple of 4
   double* sums;       // rp sums of squares (cleared beforehand)

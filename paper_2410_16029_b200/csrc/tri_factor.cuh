@@ -21,7 +21,7 @@
 // the rest.  The blocks live in shared memory where they fit (up to 160 columns), else in L2.
 // It replaced a scaling kernel, a Cholesky factorisation with one CTA per matrix, a recursive triangular inverse (two
 // batched products per level) and a conversion: 12 launches.  Measured per orthonormalisation: 58 matrices of 128 columns 50 us,
-// 84 of 256 150, 156 of up to 512 900 (those launches: in fp32 125, 310 and 1600 us, in fp64 190, 490 and 2900).  What is left
+// 86 of 256 150, 156 of up to 512 840 (those launches: in fp32 125, 310 and 1600 us, in fp64 190, 490 and 2900).  What is left
 // is the chain of diagonal blocks up to 256 columns (8 000 cycles each) and the fp64 tensor cores' rate beyond.
 #pragma once
 
