@@ -109,7 +109,7 @@ __device__ __forceinline__ double warp_sums(double (&v)[S]) {
 
 // A wait of a whole warp: all lanes see the barrier complete, or all of them give up (lanes that part here could not come
 // together again in what follows).  The vote costs the bf16 history 2 % of the kernel (350M shapes, s = 16: 887 -> 907 us),
-// the fp32 history nothing; put off to the release of the stage, or with one lane polling for all, it costs more.
+// the fp32 history half a percent at most; put off to the release of the stage, or with one lane polling for all, it costs more.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
