@@ -2,7 +2,7 @@
 // the s x s solves, and the natural-gradient combination with the Adam moments (Sec. 2.4, 2.2).
 //
 // Structure: one CTA per SM; a producer warp streams the history (and m, v) through a ring of
-// shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight consumer
+// shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight or sixteen consumer
 // warps compute from shared memory, a finishing warp turns the partial sums of a Gram tile into its partial row
 // and, after a matrix's last one, solves its s x s system while the consumers go on with the next item.  The producer runs ahead of the consumers across tile and
 // matrix boundaries, so the SM always has several stages of loads in flight.
@@ -56,9 +56,12 @@ struct FusedCfg {
   // and the per-stage bookkeeping of a consumer thread weighs as much as its arithmetic on two elements, so its
   // stages are twice as long (four elements per thread) even though only two or three of them fit.
   static constexpr int CE = SMAX <= 16 ? (HIST16 ? 2048 : 1024) : 512;
-  // consumer threads: the bf16 history costs more instructions per byte (conversion, two Gram rows), so it gets
-  // sixteen warps where the registers allow it
-  static constexpr int kConsumers = (HIST16 && SMAX <= 16) ? 512 : 256;
+  // Consumer threads: a warp issues the 100 to 250 instructions of a stage one after another, so eight warps take 1 us for it
+  // whatever it holds.  The bf16 history costs more instructions per byte (conversion, two Gram rows), and a stage of
+  // eight slots at most holds as little as 12 KB (history and moments of s = 0) to 40 KB, which arrive in 0.3 to 0.9 us; they get
+  // sixteen warps.  Measured, eight against sixteen, stream phase: s = 5, 11 M elements, 154 -> 125 us; s = 0 on the 60M
+  // shapes 39 -> 35; s = 8 on them 88 either way, as sixteen slots (1.1B shapes, 4.16 ms), which stay with eight warps.
+  static constexpr int kConsumers = SMAX <= 8 || (HIST16 && SMAX <= 16) ? 512 : 256;
   static constexpr int kThreads = kConsumers + 64;  // and the producer and the finishing warp
   static constexpr int kHistBytes = SMAX * CE * (HIST16 ? 2 : 4);
   static constexpr int kCurOff = kHistBytes;                          // HIST16: fp32 gradient of this step
