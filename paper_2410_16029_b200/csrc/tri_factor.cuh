@@ -17,12 +17,16 @@
 // columns 35 us, 84 of 256 86, 156 of up to 512 493), but left R^-1 two to ten times as far from 64 bits as a plain fp32
 // factorisation does (the sums of the tensor cores are truncated); fp32 multiply-adds on the vector units take as long as
 // fp64 tensor cores and are no closer at 32 and 64 columns.  As it is, the two bf16 parts of the result are what decides.
-// One warp factors and inverts the next diagonal block as soon as that has its update, while the other fifteen update
+// One warp factors and inverts the next diagonal block as soon as that has its update, while the others update
 // the rest.  The blocks live in shared memory where they fit (up to 160 columns), else in L2.
 // It replaced a scaling kernel, a Cholesky factorisation with one CTA per matrix, a recursive triangular inverse (two
-// batched products per level) and a conversion: 12 launches.  Measured per orthonormalisation: 58 matrices of 128 columns 50 us,
-// 86 of 256 150, 156 of up to 512 840 (those launches: in fp32 125, 310 and 1600 us, in fp64 190, 490 and 2900).  What is left
-// is the chain of diagonal blocks up to 256 columns (8 000 cycles each) and the fp64 tensor cores' rate beyond.
+// batched products per level) and a conversion: 12 launches, in fp32 125, 310 and 1600 us for 58 matrices of 128 columns, 86 of 256 and
+// 156 of up to 512, in fp64 190, 490 and 2900.  As first built 49, 148 and 827 us: a step waited for all of S before the next
+// diagonal block had its update, one warp formed that (2 000 cycles) and took 8 000 for its factor, a square root and a
+// round through shared memory for each pivot, and the load took one entry at a time.  Now 31, 120 and 708 us: 9 000 cycles a step up
+// to 128 columns, two thirds of them the chain of pivots; beyond, the fp64 tensor cores are busy for half of the time, which neither
+// more of the blocks in shared memory, nor halves of blocks sent for ahead of time (123 and 760 us), nor columns collected in
+// registers (183 and 1070 us) changed.
 #pragma once
 
 #include "common.cuh"
@@ -33,8 +37,7 @@ namespace ngalore {
 constexpr int kTfThreads = 512;
 constexpr int kTfNB = 32;
 constexpr int kTfLd = kTfNB + 4;     // row length of the operands in shared memory (fragments without bank conflicts)
-constexpr int kTfLdW = kTfNB + 8;    // row length of the diagonal block's work space
-constexpr int kTfLdS8 = 12;          // ... and of its operands
+constexpr int kTfLdS8 = 12;          // ... and of an 8 x 8 tile
 
 struct FactorMat {
   const float* C32;     // the Gram matrix, L x L, lower triangle valid: fp32 ...
@@ -51,7 +54,7 @@ struct FactorMat {
 // Shared memory without the blocks.
 __host__ __device__ inline size_t tf_base_smem(int L, bool s_global) {
   const size_t np = static_cast<size_t>((L + kTfNB - 1) / kTfNB) * kTfNB;
-  return sizeof(double) * ((s_global ? 0 : np * kTfLd) + np + kTfNB * (2 * kTfLd + kTfLdW + kTfLdS8) + 64);
+  return sizeof(double) * ((s_global ? 0 : np * kTfLd) + np + 3 * kTfNB * kTfLd + 8 * kTfLdS8);
 }
 // Rows of S in global memory.
 __host__ __device__ inline size_t tf_spill_doubles(int L) { return static_cast<size_t>((L + kTfNB - 1) / kTfNB) * kTfNB * kTfLd; }
@@ -60,136 +63,131 @@ __host__ __device__ inline size_t tf_block_bytes(int L) {
   return sizeof(double) * nb * (nb + 1) / 2 * kTfNB * kTfNB;
 }
 
-// acc[mt][nt][h] (entry (8 mt + lane / 4, 8 nt + 2 (lane % 4) + h) of a 32 x 32 block) += left(row, k) right(col, k),
-// summed over K values of k.
-template <int K, typename FL, typename FR>
-__device__ __forceinline__ void tf_product(double (&acc)[4][4][2], FL left, FR right, int fr, int fk) {
-#pragma unroll
-  for (int k0 = 0; k0 < K; k0 += 4) {
-    double a[4], b[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) a[m] = left(8 * m + fr, k0 + fk);
-#pragma unroll
-    for (int n = 0; n < 4; ++n) b[n] = right(8 * n + fr, k0 + fk);
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-#pragma unroll
-      for (int n = 0; n < 4; ++n)
-        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                     : "+d"(acc[m][n][0]), "+d"(acc[m][n][1]) : "d"(a[m]), "d"(b[n]));
-  }
-}
-
 __device__ __forceinline__ int tf_at(int row, int col) { return row * kTfNB + (col ^ ((row & 3) * 8)); }   // inside a block
 
-// Eight consecutive numbers.
-__device__ __forceinline__ void tf_load8(const double* p, double (&v)[8]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const double2 x = reinterpret_cast<const double2*>(p)[q];
-    v[2 * q] = x.x; v[2 * q + 1] = x.y;
-  }
-}
-__device__ __forceinline__ void tf_store8(double* p, const double (&v)[8]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(p)[q] = make_double2(v[2 * q], v[2 * q + 1]);
+// fp64 tensor-core product of 8 x 4 (row = lane / 4, k = lane % 4) and 4 x 8 (k = lane % 4, column = lane / 4); the result's row is
+// lane / 4, its columns 2 (lane % 4) and the next.
+__device__ __forceinline__ void tf_dmma(double (&c)[2], double a, double b) {
+  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
 }
 
-// One warp: Inv = inverse of the Cholesky factor of the 32 x 32 block at blk, by the elimination described at the top
-// once more, in blocks of eight.  A pivot that is not above tiny is replaced by it, so that the factor of a
-// rank-deficient matrix stays finite.  (Column by column, 32 steps of shuffle, square root, scaling and update, it took
-// 19 000 cycles and bounded the kernel.)
-__device__ __forceinline__ void tf_diagonal(const double* blk, double tiny, double* W, double* S8, double* I8, double* Inv, int lane) {
+// 1 / d and 1 / sqrt(d) for d > 0 far from the ends of the range: the hardware's approximation (20 bits) and one step of
+// Householder's third-order iteration, y (1 + e + e^2) with e = 1 - d y and y (1 + e / 2 + 3 e^2 / 8) with e = 1 - d y^2, whose error is
+// of the order of e^3.  No branches, so that the pivots of a block and their square roots overlap.
+__device__ __forceinline__ double tf_reciprocal(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double tf_inverse_root(double d) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+
+// One warp: Inv = inverse of the Cholesky factor of the 32 x 32 block in W (row length kTfLd, lower triangle), by the elimination
+// described at the top once more, in blocks of eight.  The ten 8 x 8 tiles of the lower triangle stay in registers: tile (i, j) is that of
+// the matrix until step j and from then on that of the right-hand side, transposed.  So a tile of S is computed from tiles in
+// the layout of a result, and is both operands of the update in that layout (the index of summation may be permuted at
+// will): only the diagonal tile, which every lane factors for itself, and its inverse go through shared memory (I8).
+// A pivot that is not above tiny is replaced by it, so that the factor of a rank-deficient matrix stays finite.
+// What bounds it is the chain of 32 pivots, a reciprocal and two multiply-adds each; their square roots are taken beside it.
+// (With the block in shared memory and the square roots in the chain 8 000 cycles; column by column, 32 steps, 19 000.)
+__device__ __forceinline__ void tf_diagonal(const double* W, double tiny, double* I8, double* Inv, int lane) {
   const int fr = lane >> 2, fk = lane & 3;
-  {
-    double r[kTfNB];
+  double acc[4][4][2];
 #pragma unroll
-    for (int q = 0; q < kTfNB; ++q) r[q] = blk[tf_at(q, lane)];
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int q = 0; q < kTfNB; ++q) W[q * kTfLdW + lane] = r[q];
-  }
-  __syncwarp();
-#pragma unroll 1
-  for (int c0 = 0; c0 < kTfNB; c0 += 8) {
-    // the 8 x 8 block: every lane computes all of its factor (shuffles would double the length of the chain), then one
-    // column of the inverse
-    {
-      double r[8][8], x[8], inv[8];
+    for (int j = 0; j <= i; ++j) {
+      const double2 v = *reinterpret_cast<const double2*>(W + (8 * i + fr) * kTfLd + 8 * j + 2 * fk);
+      acc[i][j][0] = v.x; acc[i][j][1] = v.y;
+    }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) tf_load8(W + (c0 + i) * kTfLdW + c0, r[i]);
+  for (int s = 0; s < 4; ++s) {
+    __syncwarp();
+    *reinterpret_cast<double2*>(I8 + fr * kTfLdS8 + 2 * fk) = make_double2(acc[s][s][0], acc[s][s][1]);
+    __syncwarp();
+    // U D U^T of the tile, then column lane % 8 of D^-1/2 U^-1
+    double r[8][8], x[8], d[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        double d = r[t][t];
-        if (!(d > tiny)) d = tiny;
-        inv[t] = rsqrt(d);
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int i = t + 1; i < 8; ++i) r[i][t] *= inv[t];
-#pragma unroll
-        for (int j = t + 1; j < 8; ++j)
-#pragma unroll
-          for (int i = j; i < 8; ++i) r[i][j] -= r[i][t] * r[j][t];
+      for (int j = 0; j <= i; j += 2) {
+        const double2 v = *reinterpret_cast<const double2*>(I8 + i * kTfLdS8 + j);
+        r[i][j] = v.x; r[i][j + 1] = v.y;
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = i == (lane & 7) ? 1.0 : 0.0;
+    for (int t = 0; t < 8; ++t) {
+      d[t] = r[t][t] > tiny ? r[t][t] : tiny;
+      const double ip = tf_reciprocal(d[t]);
+      double l[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        x[t] *= inv[t];
+      for (int i = t + 1; i < 8; ++i) l[i] = r[i][t] * ip;
 #pragma unroll
-        for (int i = t + 1; i < 8; ++i) x[i] -= r[i][t] * x[t];
-      }
-      if (lane < 8) {
+      for (int j = t + 1; j < 8; ++j)
 #pragma unroll
-        for (int t = 0; t < 8; ++t) I8[t * 8 + lane] = x[t];
-      }
+        for (int i = j; i < 8; ++i) r[i][j] -= l[i] * r[j][t];
+#pragma unroll
+      for (int i = t + 1; i < 8; ++i) r[i][t] = l[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = i == (lane & 7) ? 1.0 : 0.0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+      for (int i = t + 1; i < 8; ++i) x[i] -= r[i][t] * x[t];
+    __syncwarp();
+    if (lane < 8) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) I8[t * kTfLdS8 + lane] = x[t] * tf_inverse_root(d[t]);
     }
     __syncwarp();
-    // the operands, lane = row, and rows c0 .. c0 + 7 of the result
-    {
-      double v[8], o[8];
-      if (lane >= c0 + 8) {
-        tf_load8(W + lane * kTfLdW + c0, v);
+    const double2 b = *reinterpret_cast<const double2*>(I8 + fr * kTfLdS8 + 2 * fk);
+    double S[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j == s) {
+        S[j][0] = I8[2 * fk * kTfLdS8 + fr];
+        S[j][1] = I8[(2 * fk + 1) * kTfLdS8 + fr];
       } else {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = lane < c0 ? W[(c0 + q) * kTfLdW + lane] : (lane == c0 + q ? 1.0 : 0.0);
-      }
-#pragma unroll
-      for (int n = 0; n < 8; ++n) {
-        double row[8];
-        tf_load8(I8 + n * 8, row);
-        o[n] = 0.0;
-#pragma unroll
-        for (int q = 0; q <= n; ++q) o[n] += row[q] * v[q];
-        Inv[(c0 + n) * kTfLd + lane] = lane < c0 + 8 ? o[n] : 0.0;
-      }
-      tf_store8(S8 + lane * kTfLdS8, o);
-      __syncwarp();
-      if (lane >= c0 + 8) {
-        const double zero[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        tf_store8(W + lane * kTfLdW + c0, zero);
+        double (&from)[2] = j > s ? acc[j][s] : acc[s][j];
+        S[j][0] = S[j][1] = 0.0;
+        tf_dmma(S[j], from[0], b.x);
+        tf_dmma(S[j], from[1], b.y);
       }
     }
-    __syncwarp();
-    if (c0 + 8 == kTfNB) break;
-    // (rows up to c0 + 7 are not read any more: they may take part)
-    double acc[4][4][2];
+    // the tiles right of s first: the next diagonal tile is one of them
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+    for (int i = s + 1; i < 4; ++i)
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
+      for (int j = s + 1; j <= i; ++j) {
+        tf_dmma(acc[i][j], -S[i][0], S[j][0]);
+        tf_dmma(acc[i][j], -S[i][1], S[j][1]);
+      }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) acc[x][y][h] = W[(8 * x + fr) * kTfLdW + 8 * y + 2 * fk + h];
-    tf_product<8>(acc, [&](int r, int kk) { return -S8[r * kTfLdS8 + kk]; }, [&](int n, int kk) { return S8[n * kTfLdS8 + kk]; }, fr, fk);
-    __syncwarp();
+    for (int i = s + 1; i < 4; ++i)
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+      for (int j = 0; j <= s; ++j) {
+        if (j == s) acc[i][j][0] = acc[i][j][1] = 0.0;
+        tf_dmma(acc[i][j], -S[j][0], S[i][0]);
+        tf_dmma(acc[i][j], -S[j][1], S[i][1]);
+      }
+    // rows 8 s .. 8 s + 7 of the result
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) W[(8 * x + fr) * kTfLdW + 8 * y + 2 * fk + h] = acc[x][y][h];
-    __syncwarp();
+      for (int h = 0; h < 2; ++h) Inv[(8 * s + 2 * fk + h) * kTfLd + 8 * j + fr] = j <= s ? S[j][h] : 0.0;
   }
 }
 
+// Warp 0 is the chain: it factors diagonal block k + 1 (tf_diagonal) while the others do the rest of step k.  Warps 1 to 3, which sit
+// on other schedulers, help it to get there: the four form a quarter each of S_(k+1) and of the update of block
+// (k + 1, k + 1), before anything else takes the tensor cores.  Then the twelve warps that do not share warp 0's scheduler form the
+// rest of S, a quarter of a block row at a time, and update the rest of the matrix; warps 4, 8 and 12, which would hold up the chain
+// (a multiply-add of it waits for every product that is under way), join them when it has ended, and so does warp 0.
 template <bool S_GLOBAL>
 __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorMat* mats, int smem_bytes, double shift_scale, int conditional) {
   constexpr int NB = kTfNB, LD = kTfLd, WARPS = kTfThreads / 32;
@@ -200,153 +198,196 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
   const int L = m.L, nb = (L + NB - 1) / NB, np = nb * NB;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
   double* Inv0 = reinterpret_cast<double*>(tf_smem);            // [2][NB][LD]
-  double* W = Inv0 + 2 * NB * LD;                           // work space of the diagonal block: [NB][kTfLdW],
-  double* S8 = W + NB * kTfLdW;                             // [NB][kTfLdS8],
-  double* I8 = S8 + NB * kTfLdS8;                           // [8][8]
-  double* rd = I8 + 64;                                     // [np] 1 / column norm
+  double* W = Inv0 + 2 * NB * LD;                           // [NB][LD] the next diagonal block
+  double* I8 = W + NB * LD;                                 // [8][kTfLdS8]
+  double* rd = I8 + 8 * kTfLdS8;                            // [np] 1 / column norm
   double* Ssh = rd + np;
   double* S = S_GLOBAL ? m.spill : Ssh;    // [np][LD]
   const bool resident = tf_base_smem(L, S_GLOBAL) + tf_block_bytes(L) <= static_cast<size_t>(smem_bytes);
   double* B = resident ? (S_GLOBAL ? Ssh : Ssh + np * LD) : m.work;
-  auto gram = [&](int r, int c) {
-    const long long o = static_cast<long long>(r) * L + c;
-    return m.C32 != nullptr ? static_cast<double>(m.C32[o]) : m.C64[o];
-  };
   auto block = [&](int i, int j) -> double* { return B + (i * (i + 1) / 2 + j) * (NB * NB); };
   const double tiny = 1e-28, one = 1.0 + (m.C32 != nullptr ? shift_scale * static_cast<double>(L) / 65536.0 : shift_scale);
+  if (tid == 0) counter = 0;
 
-  for (int i = tid; i < np; i += kTfThreads) {
-    double d = i < L ? gram(i, i) : 1.0;
-    if (!(d > 1e-60)) d = d == d ? 1e-60 : d;          // (a NaN stays one, and the basis check finds it)
-    rd[i] = rsqrt(d);
-  }
-  __syncthreads();
-  // the scaled matrix (beyond L: the identity)
-  for (int b = warp; b < nb * (nb + 1) / 2; b += WARPS) {
-    int i = static_cast<int>((sqrtf(8.f * b + 1.f) - 1.f) * 0.5f);
-    while ((i + 1) * (i + 2) / 2 <= b) ++i;
-    while (i * (i + 1) / 2 > b) --i;
-    const int j = b - i * (i + 1) / 2;
-    const int c = j * NB + lane;
-    double* dst = B + b * (NB * NB);
-#pragma unroll 1
-    for (int row0 = 0; row0 < NB; row0 += 16) {
-      double raw[16];
+  // the scaled matrix (beyond L: the identity), 16 rows of a block at a time; a warp's first ones are under way while the norms are
+  // worked out
+  {
+    double raw[16];
+    int i = 0, j = 0, row0 = 0;
+    auto fetch = [&](int u) {
+      const int b = u >> 1;
+      i = static_cast<int>((sqrtf(8.f * b + 1.f) - 1.f) * 0.5f);
+      while ((i + 1) * (i + 2) / 2 <= b) ++i;
+      while (i * (i + 1) / 2 > b) --i;
+      j = b - i * (i + 1) / 2;
+      row0 = (u & 1) * 16;
+      const int c = min(j * NB + lane, L - 1), r = i * NB + row0;
+      auto rows = [&](const auto* p) {
 #pragma unroll
-      for (int q = 0; q < 16; ++q) raw[q] = gram(min(i * NB + row0 + q, L - 1), min(c, L - 1));
+        for (int q = 0; q < 16; ++q) raw[q] = static_cast<double>(p[static_cast<long long>(min(r + q, L - 1)) * L + c]);
+      };
+      if (m.C32 != nullptr) rows(m.C32); else rows(m.C64);
+    };
+    const int units = nb * (nb + 1);
+    if (warp < units) fetch(warp);
+    for (int x = tid; x < np; x += kTfThreads) {
+      const long long o = static_cast<long long>(min(x, L - 1)) * (L + 1);
+      double d = m.C32 != nullptr ? static_cast<double>(m.C32[o]) : m.C64[o];
+      if (x >= L) d = 1.0;
+      if (!(d > 1e-60)) d = d == d ? 1e-60 : d;          // (a NaN stays one, and the basis check finds it)
+      rd[x] = rsqrt(d);
+    }
+    __syncthreads();
+    for (int u = warp; u < units;) {
+      const int c = j * NB + lane;
+      double* dst = B + (u >> 1) * (NB * NB);
+      const double scale = rd[c];
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         const int row = row0 + q, r = i * NB + row;
-        const double v = raw[q] * rd[r] * rd[c];
+        const double v = raw[q] * rd[r] * scale;
         dst[tf_at(row, lane)] = r == c ? (r < L ? one : 1.0) : (r < L && c < r ? v : 0.0);
       }
+      u += WARPS;
+      if (u < units) fetch(u);
     }
   }
-  if (tid == 0) counter = 0;
   __syncthreads();
 
   for (int k = -1; k < nb; ++k) {
     const double* Inv = Inv0 + (k & 1) * NB * LD;
-    // S, and block column k of R^-1
-    for (int i = warp; i < nb && k >= 0; i += WARPS) {
-      double acc[4][4][2];
+    // rows 8 q .. 8 q + 7 of S_i, and of the block (i, k) of R^-1
+    auto form = [&](int i, int q) {
+      double acc[4][2];
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int y = 0; y < 4; ++y) acc[y][0] = acc[y][1] = 0.0;
+      if (i != k) {
+        const double* blk = i > k ? block(i, k) : block(k, i);
+        double a[8];
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = 0.0;
-      auto right = [&](int n, int kk) { return Inv[n * LD + kk]; };
-      if (i > k) {
-        const double* blk = block(i, k);
-        tf_product<NB>(acc, [&](int r, int kk) { return blk[tf_at(r, kk)]; }, right, fr, fk);
-      } else if (i < k) {
-        const double* blk = block(k, i);
-        tf_product<NB>(acc, [&](int r, int kk) { return blk[tf_at(kk, r)]; }, right, fr, fk);
+        for (int kk = 0; kk < 8; ++kk) a[kk] = blk[i > k ? tf_at(8 * q + fr, 4 * kk + fk) : tf_at(4 * kk + fk, 8 * q + fr)];
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)
+#pragma unroll
+          for (int y = kk / 2; y < 4; ++y) tf_dmma(acc[y], a[kk], Inv[(8 * y + fr) * LD + 4 * kk + fk]);   // (Inv is lower triangular)
       } else {
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+        for (int y = 0; y < 4; ++y)
 #pragma unroll
-          for (int y = 0; y < 4; ++y)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) acc[x][y][h] = Inv[(8 * y + 2 * fk + h) * LD + 8 * x + fr];
+          for (int h = 0; h < 2; ++h) acc[y][h] = Inv[(8 * y + 2 * fk + h) * LD + 8 * q + fr];
       }
+      const int row = i * NB + 8 * q + fr;
+      const double scale = rd[row];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int row = i * NB + 8 * x + fr;
-        const double scale = rd[row];
+      for (int y = 0; y < 4; ++y) {
+        const int kk = 8 * y + 2 * fk, col = k * NB + kk;
+        *reinterpret_cast<double2*>(S + row * LD + kk) = make_double2(acc[y][0], acc[y][1]);
+        if (m.R64 != nullptr) {
 #pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const int kk = 8 * y + 2 * fk, col = k * NB + kk;
-          S[row * LD + kk] = acc[x][y][0];
-          S[row * LD + kk + 1] = acc[x][y][1];
-          if (m.R64 != nullptr) {
+          for (int h = 0; h < 2; ++h)
+            if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? acc[y][h] * scale : 0.0;
+        } else if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
+          float f[2];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-              if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? acc[x][y][h] * scale : 0.0;
-          } else if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
-            float f[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const float v = i <= k ? static_cast<float>(acc[x][y][h] * scale) : 0.f;
-              f[h] = v == v ? fminf(fmaxf(v, -1e30f), 1e30f) : v;
-            }
-            const __nv_bfloat162 hv = __floats2bfloat162_rn(f[0], f[1]);
-            const __nv_bfloat162 lv = __floats2bfloat162_rn(f[0] - __low2float(hv), f[1] - __high2float(hv));
-            const long long o = static_cast<long long>(row) * m.ld + col;
-            *reinterpret_cast<__nv_bfloat162*>(m.Rhi + o) = hv;
-            *reinterpret_cast<__nv_bfloat162*>(m.Rlo + o) = lv;
+          for (int h = 0; h < 2; ++h) {
+            const float v = i <= k ? static_cast<float>(acc[y][h] * scale) : 0.f;
+            f[h] = v == v ? fminf(fmaxf(v, -1e30f), 1e30f) : v;
           }
+          const __nv_bfloat162 hv = __floats2bfloat162_rn(f[0], f[1]);
+          const __nv_bfloat162 lv = __floats2bfloat162_rn(f[0] - __low2float(hv), f[1] - __high2float(hv));
+          const long long o = static_cast<long long>(row) * m.ld + col;
+          *reinterpret_cast<__nv_bfloat162*>(m.Rhi + o) = hv;
+          *reinterpret_cast<__nv_bfloat162*>(m.Rlo + o) = lv;
         }
       }
+    };
+    if (k + 1 == nb) {   // the last block column of R^-1
+      for (int t = warp; t < 4 * nb; t += WARPS) form(t >> 2, t & 3);
+      break;
     }
-    __syncthreads();
-    if (k + 1 == nb) break;
-    // block (i, j) -= S_i S_j^T; block column k starts from zero (its old contents were the panel).  Warp 0 begins with
-    // the next diagonal block, the others take the rest in order.
     const int t0 = (k + 1) * (k + 2) / 2, t1 = nb * (nb + 1) / 2, td = t0 + k + 1;   // td: block (k + 1, k + 1)
+    const bool beside = (warp & 3) != 0;   // not on the scheduler of the chain
+    if (warp < 4) {
+      double acc[4][2];
+      const double* blk = block(k + 1, k + 1);
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const double2 v = *reinterpret_cast<const double2*>(blk + tf_at(8 * warp + fr, 8 * y + 2 * fk));
+        acc[y][0] = v.x; acc[y][1] = v.y;
+      }
+      if (k >= 0) {
+        form(k + 1, warp);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        const double* Sk = S + (k + 1) * NB * LD;
+#pragma unroll
+        for (int kk = 0; kk < NB; kk += 4) {
+          const double a = -Sk[(8 * warp + fr) * LD + kk + fk];
+#pragma unroll
+          for (int y = 0; y < 4; ++y)
+            if (y <= warp) tf_dmma(acc[y], a, Sk[(8 * y + fr) * LD + kk + fk]);
+        }
+      }
+#pragma unroll
+      for (int y = 0; y < 4; ++y)
+        *reinterpret_cast<double2*>(W + (8 * warp + fr) * LD + 8 * y + 2 * fk) = make_double2(acc[y][0], acc[y][1]);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (warp == 0) tf_diagonal(W, tiny, I8, Inv0 + ((k + 1) & 1) * NB * LD, lane);
+    }
+    if (k >= 0) {
+      if (beside) {
+        for (int t = warp - 1 - (warp >> 2); t < 4 * (nb - 1); t += 12) {
+          const int i = t >> 2;
+          form(i > k ? i + 1 : i, t & 3);
+        }
+        asm volatile("bar.arrive 3, %0;" ::"n"(kTfThreads) : "memory");
+        asm volatile("bar.sync 2, 384;" ::: "memory");
+      } else {
+        asm volatile("bar.sync 3, %0;" ::"n"(kTfThreads) : "memory");   // (S is complete, and so is the chain's step)
+      }
+    }
+    // block (i, j) -= S_i S_j^T; block column k starts from zero (its old contents were the panel)
     auto next = [&]() {
       int t = 0;
       if (lane == 0) t = atomicAdd(&counter, 1);
       return __shfl_sync(0xffffffffu, t, 0) + t0;
     };
-    // (warps 4, 8 and 12 sit on the scheduler of warp 0, whose diagonal block the next step waits for: they rest
-    // until it is done)
-    if (warp != 0 && (warp & 3) == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-    int t = warp == 0 ? td : (k >= 0 ? next() : t1);
-    bool first = warp == 0;
-    while (t < t1) {
-      if (k >= 0 && (first || t != td)) {
-        int i = static_cast<int>((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-        while ((i + 1) * (i + 2) / 2 <= t) ++i;
-        while (i * (i + 1) / 2 > t) --i;
-        const int j = t - i * (i + 1) / 2;
-        double* blk = block(i, j);
-        double acc[4][4][2];
+    for (int t = k >= 0 ? next() : t1; t < t1; t = next()) {
+      if (t == td) continue;
+      int i = static_cast<int>((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while ((i + 1) * (i + 2) / 2 <= t) ++i;
+      while (i * (i + 1) / 2 > t) --i;
+      const int j = t - i * (i + 1) / 2;
+      double* blk = block(i, j);
+      double acc[4][4][2];
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < 4; ++x)
 #pragma unroll
-          for (int y = 0; y < 4; ++y)
+        for (int y = 0; y < 4; ++y) {
+          const double2 v = j == k ? make_double2(0.0, 0.0) : *reinterpret_cast<const double2*>(blk + tf_at(8 * x + fr, 8 * y + 2 * fk));
+          acc[x][y][0] = v.x; acc[x][y][1] = v.y;
+        }
+      const double *Si = S + i * NB * LD + fr * LD + fk, *Sj = S + j * NB * LD + fr * LD + fk;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) acc[x][y][h] = j == k ? 0.0 : blk[tf_at(8 * x + fr, 8 * y + 2 * fk) + h];
-        const double *Si = S + i * NB * LD, *Sj = S + j * NB * LD;
-        tf_product<NB>(acc, [&](int r, int kk) { return -Si[r * LD + kk]; }, [&](int n, int kk) { return Sj[n * LD + kk]; }, fr, fk);
+      for (int k0 = 0; k0 < NB; k0 += 4) {
+        double a[4], b[4];
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < 4; ++x) { a[x] = -Si[8 * x * LD + k0]; b[x] = Sj[8 * x * LD + k0]; }
 #pragma unroll
-          for (int y = 0; y < 4; ++y)
+        for (int y = 0; y < 4; ++y) {
+          if (j == k && k0 < 8 * y) continue;     // (S_k is the transpose of Inv, upper triangular)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) blk[tf_at(8 * x + fr, 8 * y + 2 * fk) + h] = acc[x][y][h];
+          for (int x = 0; x < 4; ++x)
+            if (x >= y || i != j) tf_dmma(acc[x][y], a[x], b[y]);   // (the upper part of a diagonal block is not used)
+        }
       }
-      if (first) {
-        __syncwarp();
-        tf_diagonal(block(k + 1, k + 1), tiny, W, S8, I8, Inv0 + ((k + 1) & 1) * NB * LD, lane);
-        first = false;
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (k < 0) break;
-      }
-      t = next();
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          *reinterpret_cast<double2*>(blk + tf_at(8 * x + fr, 8 * y + 2 * fk)) = make_double2(acc[x][y][0], acc[x][y][1]);
     }
     __syncthreads();
-    if (tid == 0) counter = 0;   // (read again only after the next barrier)
+    if (tid == 0) counter = 0;   // (read again only after the next barriers)
   }
 }
 
