@@ -2,7 +2,7 @@
 // the s x s solves, and the natural-gradient combination with the Adam moments (Sec. 2.4, 2.2).
 //
 // Structure: one CTA per SM; a producer warp streams the history (and m, v) through a ring of
-// shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight or sixteen consumer
+// shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight to sixteen consumer
 // warps compute from shared memory, a finishing warp turns the partial sums of a Gram tile into its partial row
 // and, after a matrix's last one, solves its s x s system while the consumers go on with the next item.  The producer runs ahead of the consumers across tile and
 // matrix boundaries, so the SM always has several stages of loads in flight.
@@ -54,21 +54,22 @@ template <int SMAX, bool HIST16, bool MOM16 = false>
 struct FusedCfg {
   // Elements per stage and slot.  The bf16 history costs more instructions per byte (conversion, two Gram rows),
   // and the per-stage bookkeeping of a consumer thread weighs as much as its arithmetic on two elements, so its
-  // stages are twice as long (four elements per thread) even though only two or three of them fit.
-  static constexpr int CE = SMAX <= 16 ? (HIST16 ? 2048 : 1024) : 512;
+  // threads take four, and its stages are as long as three of them fit: with two, a stage of which is worked on, the SM has too little
+  // under way.  350M shapes, s = 16, bf16 moments: two stages of 2048 elements 950 us, three of 1792 (14 warps) 805.
+  static constexpr int CE = !HIST16 ? (SMAX <= 16 ? 1024 : 512) : (SMAX <= 8 ? 2048 : (SMAX <= 16 ? (MOM16 ? 1792 : 1536) : 512));
   // Consumer threads: a warp issues the 100 to 250 instructions of a stage one after another, so eight warps take 1 us for it
   // whatever it holds.  The bf16 history costs more instructions per byte (conversion, two Gram rows), and a stage of
   // eight slots at most holds as little as 12 KB (history and moments of s = 0) to 40 KB, which arrive in 0.3 to 0.9 us; they get
   // sixteen warps.  Measured, eight against sixteen, stream phase: s = 5, 11 M elements, 154 -> 125 us; s = 0 on the 60M
   // shapes 39 -> 35; s = 8 on them 88 either way, as sixteen slots (1.1B shapes, 4.16 ms), which stay with eight warps.
-  static constexpr int kConsumers = SMAX <= 8 || (HIST16 && SMAX <= 16) ? 512 : 256;
+  static constexpr int kConsumers = HIST16 && SMAX <= 16 ? CE / 4 : (SMAX <= 8 ? 512 : 256);
   static constexpr int kThreads = kConsumers + 64;  // and the producer and the finishing warp
   static constexpr int kHistBytes = SMAX * CE * (HIST16 ? 2 : 4);
   static constexpr int kCurOff = kHistBytes;                          // HIST16: fp32 gradient of this step
   static constexpr int kMOff = kHistBytes + (HIST16 ? CE * 4 : 0);
   static constexpr int kVOff = kMOff + CE * (MOM16 ? 2 : 4);
   static constexpr int kStageBytes = kVOff + CE * (MOM16 ? 2 : 4);
-  static constexpr int kStages = HIST16 ? (SMAX <= 8 ? 3 : (SMAX <= 16 ? 2 : 5)) : (SMAX <= 8 ? 5 : 3);
+  static constexpr int kStages = HIST16 ? (SMAX <= 16 ? 3 : 5) : (SMAX <= 8 ? 5 : 3);
   static constexpr int kBase = kStages * kStageBytes;
   static constexpr int kFullOff = kBase, kEmptyOff = kBase + 64, kMetaOff = kBase + 128, kFlagOff = kBase + 512;
   static constexpr int kMeetOff = kBase + 640, kRedBarOff = kBase + 768, kRedMetaOff = kBase + 800, kRedOff = kBase + 896;
@@ -347,7 +348,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       now = next;
     }
   } else {
-    // ------------------------------------------------------------------ consumers (8 or 16 warps)
+    // ------------------------------------------------------------------ consumers (8 to 16 warps)
     // One loop over the stages of an item for either kind, so that the sums of a Gram tile and the weights of a
     // combination tile do not both occupy registers.
     const int warp = tid >> 5, lane = tid & 31;
