@@ -51,7 +51,7 @@ struct TcTile {
   int k0;          // first K element
   int kblocks;     // number of 64-wide K blocks
   int atomic;      // 1: K is split, accumulate into the output with atomics
-  int rows, cols;  // extent of the output the tile belongs to
+  int rows, cols;  // extent of the output the tile belongs to (in the step's tables a narrow tile ends at cols)
 };
 
 // Tensor maps of the step GEMMs, kTcMapsPerMat consecutive entries per matrix.
@@ -366,7 +366,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       } else {
         const MatDesc& d = mats[tile.mat];
         out_cols = tile.cols;
-        ld_out = tile.cols;
+        ld_out = d.lr_cols;
         out = current_gradient(d, ring_cur(ctrl, d.s));
         rows_total = tile.rows;
       }
@@ -651,6 +651,21 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
     plan.long_k_back = work_long_k * 10 >= work_all * 9;
   }
   const int proj_bm = plan.tall_proj ? 2 * kTcBM : kTcBM;
+  // Tiles of 128 or 64 columns where every one of them still has an SM to itself: with fewer tiles than SMs a step is
+  // the latency of one tile, and half the columns are two thirds of its operands and half of its epilogue.  One 512 x 1376 matrix,
+  // r = 128 (6 projection tiles of 256 columns, 22 of 64; 24 and 88 of the back-projection): 32.7 -> 26.4 us a step.
+  auto tile_width = [&](int widest, auto rows_of, auto cols_of) {
+    int width = widest;
+    while (width > 64) {
+      long long tiles = 0;
+      for (const MatDesc& d : mats) tiles += static_cast<long long>((rows_of(d) + kTcBM - 1) / kTcBM) * ((cols_of(d) + width / 2 - 1) / (width / 2));
+      if (tiles > sm_count) break;
+      width /= 2;
+    }
+    return width;
+  };
+  const int proj_bn = plan.tall_proj ? kProjBN : tile_width(kProjBN, [](const MatDesc& d) { return d.lr_rows; }, [](const MatDesc& d) { return d.lr_cols; });
+  const int back_bn = tile_width(kTcBackBN, [](const MatDesc& d) { return d.M; }, [](const MatDesc& d) { return d.N; });
   std::vector<TcTile> proj, back;
   long long total_kb = 0;
   for (int i = 0; i < n; ++i) {
@@ -692,12 +707,12 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
       continue;
     }
     if (splits > 1) split_mats.push_back(i);
-    for (int n0 = 0; n0 < d.lr_cols; n0 += kProjBN)
+    for (int n0 = 0; n0 < d.lr_cols; n0 += proj_bn)
       for (int sp = 0; sp < splits; ++sp)
         for (int m0 = 0; m0 < d.lr_rows; m0 += proj_bm) {
           const int kb0 = sp * kb_per;
           const int kbn = std::min(kb_per, kb_total - kb0);
-          proj.push_back(TcTile{i, m0, n0, kb0 * kTcBK, kbn, splits > 1 ? 1 : 0, d.lr_rows, d.lr_cols});
+          proj.push_back(TcTile{i, m0, n0, kb0 * kTcBK, kbn, splits > 1 ? 1 : 0, d.lr_rows, plan.tall_proj ? d.lr_cols : std::min(d.lr_cols, n0 + proj_bn)});
         }
   }
   std::stable_sort(pg.begin(), pg.end(), [](const TcTile& a, const TcTile& b) { return a.kblocks > b.kblocks; });
@@ -707,7 +722,7 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
     plan.back_tile0[i] = static_cast<int>(back.size());
     const int kbn = (d.rp + kTcBK - 1) / kTcBK;
     for (int m0 = 0; m0 < d.M; m0 += kTcBM)
-      for (int n0 = 0; n0 < d.N; n0 += kTcBackBN) back.push_back(TcTile{i, m0, n0, 0, kbn, 0, d.M, d.N});
+      for (int n0 = 0; n0 < d.N; n0 += back_bn) back.push_back(TcTile{i, m0, n0, 0, kbn, 0, d.M, std::min(d.N, n0 + back_bn)});
   }
   plan.back_tile0[n] = static_cast<int>(back.size());
   plan.n_tiles_proj = static_cast<int>(proj.size());

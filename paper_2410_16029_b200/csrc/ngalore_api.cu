@@ -623,10 +623,11 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   // Stream tiles: two per SM and pass on large workloads.  Where that would make them short, one per SM: every tile
   // ends with a block-wide reduction and a handful of global round trips, which on small workloads weigh as much
   // as its traffic (measured, stream phase: RoBERTa-base shapes r = 8 / r = 4 68 -> 44 us / 52 -> 39 us, 60M shapes
-  // 116 -> 106 us; the 130M shapes and larger are 2 % better with two).
+  // 116 -> 106 us; the 130M shapes and larger are 2 % better with two).  At least 4096 elements, or less where the set has not as
+  // many for every SM: a stage then waits for none before it (one 512 x 1376 matrix, r = 128: 28.2 -> 26.4 us a step).
   long long te_all = total_rn / (2ll * prop.multiProcessorCount) / 1024 * 1024;
   if (te_all < 32768) te_all *= 2;
-  if (te_all < 4096) te_all = 4096;
+  if (te_all < 4096) te_all = std::min(4096ll, std::max(1024ll, (total_rn / prop.multiProcessorCount + 1023) / 1024 * 1024));
   if (te_all > 131072) te_all = 131072;
   std::vector<int> tile_elems(n_matrices, static_cast<int>(te_all));
   // The matrices at the end of the item list get tiles a quarter of the size, so that the last wave of the
