@@ -52,8 +52,8 @@ struct Ctrl {
   int epoch;                  // increments every step; flags of the fused kernel compare against it
   int timeout_flag;           // set when a bounded wait ran out
   unsigned int work_counter;  // dynamic tile counter of the fused streaming kernel
-  unsigned int gemm_counter0; // item counter of the small-rank projection
-  unsigned int gemm_counter1; // item counter of the small-rank update
+  unsigned int gemm_counter0; // item counter of the small-rank projection; of the projection: pieces of ring slots claimed for clearing
+  unsigned int gemm_counter1; // item counter of the small-rank update; of the projection: pieces that are clear
   // Testing aids, both cleared at the end of every step.  They exist so that a test can make a bounded wait run
   // out without hanging or trapping anything: the solution of one matrix is computed but not published, and the
   // tiles that wait for it give up after a few polls.

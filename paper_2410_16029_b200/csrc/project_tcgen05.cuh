@@ -37,7 +37,7 @@ static_assert(P2Smem::kTotal <= 232448, "shared memory budget of one CTA");
 
 __global__ void __launch_bounds__(kP2Threads, 1)
 tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__ tiles, const int* __restrict__ cta_first,
-                   const MatDesc* __restrict__ mats, Ctrl* ctrl) {
+                   const MatDesc* __restrict__ mats, Ctrl* ctrl, const ClearJob* __restrict__ clear, int n_clear) {
   using L = P2Smem;
   extern __shared__ unsigned char tc_smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~uintptr_t(1023));
@@ -140,6 +140,8 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
     const int half = (warp - 2) >> 2;  // which 128-row half of the tile this warp drains
     float* stg = reinterpret_cast<float*>(smem + L::kEpiOffset + (warp - 2) * L::kEpiWarpBytes);
     const int sub_row = lane >> 3, sub_q = lane & 7;
+    bool cleared = n_clear == 0;
+    if (!cleared) clear_split_slots(mats, clear, n_clear, ctrl);
     int local = 0;
     for (int t = t_begin; t < t_end; ++t, ++local) {
       const TcTile tile = tiles[t];
@@ -151,6 +153,10 @@ tc_project2_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restri
       const int row_base = tile.m0 + half * kTcBM + quarter * 32;
       if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar, local & 1u, abort_flag))) break;
       tc_fence_after();
+      if (tile.atomic && !cleared) {
+        if (!wait_split_slots(n_clear, ctrl, abort_flag)) break;
+        cleared = true;
+      }
       if (half >= halves) {
         // nothing of this warp's half exists in the tile; it only has to hand the accumulators back
         tc_fence_before();
@@ -222,10 +228,6 @@ inline ngalore_status tc_project_init() {
 // from Ctrl), through the tensor maps tc_bind_buffers set up.
 inline ngalore_status tc_project(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
                                  cudaStream_t stream, int64_t* launches) {
-  if (plan.n_split > 0) {
-    launch_step(plan.short_step, zero_split_slots_kernel, dim3(64, plan.n_split), 256, 0, stream, d_mats, plan.d_split_mats, d_ctrl);
-    *launches += 1;
-  }
   if (plan.n_tiles_pg > 0) {
     // the matrices whose Gram row comes out of the projection's epilogue, then their s x s solves
     tc_project_gram_kernel<<<plan.grid_pg, kPgThreads, PgSmem::kTotal, stream>>>(
@@ -236,11 +238,12 @@ inline ngalore_status tc_project(TcPlan& plan, const MatDesc* d_mats, Ctrl* d_ct
   }
   if (plan.tall_proj) {
     launch_step(plan.short_step, tc_project2_kernel, plan.grid_proj, kP2Threads, P2Smem::kTotal, stream, plan.d_maps,
-                plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl);
+                plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl, plan.d_clear, plan.n_clear);
   } else {
     using LP = TcSmem<kProjBN, 1, 1, kProjStages, kProjEpiWarps>;
     launch_step(plan.short_step, tc_gemm_kernel<kProjBN, 1, 1, kProjStages, TC_EPI_PROJECT, kProjEpiWarps, false>, plan.grid_proj,
-                64 + 32 * kProjEpiWarps, LP::kTotal, stream, plan.d_maps, plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl, nullptr);
+                64 + 32 * kProjEpiWarps, LP::kTotal, stream, plan.d_maps, plan.d_tiles_proj, plan.d_proj_first, d_mats, d_ctrl, nullptr,
+                plan.d_clear, plan.n_clear);
   }
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;

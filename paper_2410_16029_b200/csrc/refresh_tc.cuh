@@ -680,7 +680,7 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     constexpr bool MN = decltype(a_mn)::value;
     auto run = [&](auto p) {
       p.kernel<<<plan.grid[g], p.kThreads, p.kSmem, stream>>>(plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl,
-                                                              plan.d_probs[problem]);
+                                                              plan.d_probs[problem], nullptr, 0);
     };
     if (plan.wide && plan.tall) {
       if (high_only) run(RefProduct<kRefWideBN, 1, 2, MN>{}); else run(RefProduct<kRefWideBN, 2, 2, MN>{});
@@ -698,11 +698,11 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     case RG_GRAM_Y:
     case RG_GRAM_Z:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
+          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
       break;
     default:
       tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem]);
+          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
       break;
   }
   *launches += 1;
