@@ -95,6 +95,9 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int stride = gridDim.x;
+  // (what the plan has laid out for good is read ahead of the wait for the kernel before)
+  const TcTile tile0 = tiles[min(static_cast<int>(blockIdx.x), n_tiles - 1)];
+  if (threadIdx.x < 4) tensormap_prefetch(tmaps + tile0.mat * kTcMapsPerMat + TC_MAP_A_BACK + threadIdx.x);   // (A, B, W in, W out)
   pdl_begin();
   // the last launch of a step moves the step counters on (nothing in this kernel reads them)
   if (advance && blockIdx.x == 0 && threadIdx.x == 32) advance_step(ctrl);
@@ -104,7 +107,7 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
     if (lane == 0 && static_cast<int>(blockIdx.x) < n_tiles) {
       int stage = 0;
       uint32_t phase = 0;
-      TcTile tile = tiles[blockIdx.x];
+      TcTile tile = tile0;
       for (int t = blockIdx.x; t < n_tiles; t += stride) {
         const int tn = t + stride;
         const TcTile next = tiles[tn < n_tiles ? tn : t];  // fetched early: its latency hides behind this tile
@@ -134,7 +137,7 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
     if (lane == 0 && static_cast<int>(blockIdx.x) < n_tiles) {
       int slot = 0;
       uint32_t phase = 0;
-      TcTile tile = tiles[blockIdx.x];
+      TcTile tile = tile0;
       for (int t = blockIdx.x; t < n_tiles; t += stride) {
         const int tn = t + stride;
         const TcTile next = tiles[tn < n_tiles ? tn : t];
@@ -157,7 +160,7 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
-      TcTile tile = tiles[blockIdx.x];
+      TcTile tile = tile0;
       for (int t = blockIdx.x; t < n_tiles; t += stride, ++local) {
         const int tn = t + stride;
         const TcTile next = tiles[tn < n_tiles ? tn : t];
@@ -198,7 +201,7 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
     uint32_t phase = 0;
     int pending_slot = -1;               // slot whose store was issued last and is not yet released
     if (static_cast<int>(blockIdx.x) < n_tiles) {
-      TcTile tile = tiles[blockIdx.x];
+      TcTile tile = tile0;
       int bad = __ldcg(mats[tile.mat].step_bad);
       int local = 0;
       bool ok = true;

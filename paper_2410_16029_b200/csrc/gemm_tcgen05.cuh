@@ -129,6 +129,10 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
+// A map on its way to the SM before its first use (its memory must not change any more).
+__device__ __forceinline__ void tensormap_prefetch(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
@@ -274,8 +278,14 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_begin();
+  // (what the plan has laid out for good is read ahead of the wait for the kernel before)
   const int t_begin = cta_first[blockIdx.x], t_end = cta_first[blockIdx.x + 1];   // this CTA's tiles
+  const TcTile tile0 = tiles[t_begin];
+  if (EPI == TC_EPI_PROJECT && threadIdx.x == 0) {
+    tensormap_prefetch(tmaps + tile0.mat * kTcMapsPerMat + TC_MAP_A_PROJ);
+    tensormap_prefetch(tmaps + tile0.mat * kTcMapsPerMat + TC_MAP_B_PROJ);
+  }
+  pdl_begin();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -283,7 +293,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      TcTile tile = tiles[t_begin];
+      TcTile tile = tile0;
       auto map_a = [&](const TcTile& t) {
         return tmaps + (EPI == TC_EPI_STORE ? probs[t.mat].map_a : t.mat * kTcMapsPerMat + TC_MAP_A_PROJ);
       };
@@ -334,7 +344,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
-      TcTile next = tiles[t_begin];
+      TcTile next = tile0;
       for (int t = t_begin; t < t_end && ok; ++t, ++local) {
         const TcTile tile = next;
         next = tiles[min(t + 1, t_end - 1)];
@@ -393,8 +403,8 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
     // (of tall tiles, each group drains its half of all of them)
     constexpr int kStep = MT == 2 ? 1 : kGroups;
     const int first = kStep == 2 ? group : 0, half = MT == 2 ? group : 0;
-    TcTile tile;
-    if (t_begin + first < t_end) tile = tiles[t_begin + first];
+    TcTile tile = tile0;
+    if (first > 0 && t_begin + first < t_end) tile = tiles[t_begin + first];
     for (int local = first; t_begin + local < t_end && ok; local += kStep) {
       const TcTile next = tiles[min(t_begin + local + kStep, t_end - 1)];
       float* out;

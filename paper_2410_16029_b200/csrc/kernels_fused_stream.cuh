@@ -190,6 +190,13 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  // (The tables are laid out for good: the item that this CTA will probably claim first, and its matrix, come to the SM ahead of
+  // the wait for the kernel before.  It is claimed like the others all the same: an item that belonged to a CTA which another kernel
+  // keeps from starting could be waited for by that kernel's neighbours for good.)
+  if (tid == kConsumerThreads && static_cast<int>(blockIdx.x) < n_items) {
+    const MatDesc& d0 = mats[items[blockIdx.x].mat];
+    asm volatile("" ::"l"(d0.H), "l"(d0.m), "r"(d0.te), "r"(mats[0].s));
+  }
   pdl_begin();
   const int tag = ctrl->epoch + 1;
 
