@@ -239,6 +239,28 @@ struct TcSmem {
 
 enum { TC_EPI_PROJECT = 0, TC_EPI_STORE = 2 };
 
+// Four neighbouring results of a row on their way out: as two bf16 parts, added to what is there, or as they are.
+template <int EPI>
+__device__ __forceinline__ void store_result(float4 acc, int row, int col, float* out, int ld_out, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo,
+                                             int ld16, int atomic) {
+  float* p = out + static_cast<long long>(row) * ld_out + col;
+  if (EPI == TC_EPI_STORE && out_hi != nullptr) {
+    const __nv_bfloat162 h01 = __floats2bfloat162_rn(acc.x, acc.y), h23 = __floats2bfloat162_rn(acc.z, acc.w);
+    const __nv_bfloat162 l01 = __floats2bfloat162_rn(acc.x - __low2float(h01), acc.y - __high2float(h01));
+    const __nv_bfloat162 l23 = __floats2bfloat162_rn(acc.z - __low2float(h23), acc.w - __high2float(h23));
+    uint2 hv, lv;
+    hv.x = *reinterpret_cast<const uint32_t*>(&h01); hv.y = *reinterpret_cast<const uint32_t*>(&h23);
+    lv.x = *reinterpret_cast<const uint32_t*>(&l01); lv.y = *reinterpret_cast<const uint32_t*>(&l23);
+    const long long o = static_cast<long long>(row) * ld16 + col;
+    *reinterpret_cast<uint2*>(out_hi + o) = hv;
+    *reinterpret_cast<uint2*>(out_lo + o) = lv;
+  } else if (atomic) {
+    atomicAdd(reinterpret_cast<float4*>(p), acc);
+  } else {
+    *reinterpret_cast<float4*>(p) = acc;
+  }
+}
+
 // NA / NB: number of 16-bit parts of A / B (1, or 2 = high and low part).  With NA = NB = 2 the products
 // hi*hi, hi*lo and lo*hi are accumulated (lo*lo is below fp32 resolution).  A_MN: A is stored with its
 // row index contiguous (A^T row-major), staged as two 64-row chunks like B.  F16: the operands are fp16
@@ -469,22 +491,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
               const int row = row_base + rr;
               if (row < rows_total) {
                 const float4 acc = *reinterpret_cast<const float4*>(stg + rr * 32 + (((lane ^ rr) & 7) << 2));
-                float* p = out + static_cast<long long>(row) * ld_out + col;
-                if (EPI == TC_EPI_STORE && out_hi != nullptr) {
-                  const __nv_bfloat162 h01 = __floats2bfloat162_rn(acc.x, acc.y), h23 = __floats2bfloat162_rn(acc.z, acc.w);
-                  const __nv_bfloat162 l01 = __floats2bfloat162_rn(acc.x - __low2float(h01), acc.y - __high2float(h01));
-                  const __nv_bfloat162 l23 = __floats2bfloat162_rn(acc.z - __low2float(h23), acc.w - __high2float(h23));
-                  uint2 hv, lv;
-                  hv.x = *reinterpret_cast<const uint32_t*>(&h01); hv.y = *reinterpret_cast<const uint32_t*>(&h23);
-                  lv.x = *reinterpret_cast<const uint32_t*>(&l01); lv.y = *reinterpret_cast<const uint32_t*>(&l23);
-                  const long long o = static_cast<long long>(row) * ld16 + col;
-                  *reinterpret_cast<uint2*>(out_hi + o) = hv;
-                  *reinterpret_cast<uint2*>(out_lo + o) = lv;
-                } else if (tile.atomic) {
-                  atomicAdd(reinterpret_cast<float4*>(p), acc);
-                } else {
-                  *reinterpret_cast<float4*>(p) = acc;
-                }
+                store_result<EPI>(acc, row, col, out, ld_out, out_hi, out_lo, ld16, tile.atomic);
               }
             }
           }

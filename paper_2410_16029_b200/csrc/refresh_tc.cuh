@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "gemm_pair_tcgen05.cuh"
 #include "gemm_tcgen05.cuh"
 #include "kernels_refresh.cuh"
 #include "ritz_eigen.cuh"
@@ -283,6 +284,7 @@ struct RefreshPlan {
   int grid[RG_COUNT] = {};
   bool wide = false;           // the products with G take tiles of kRefWideBN columns ...
   bool tall = false;           // ... and of 256 rows
+  bool pair = false;           // ... on pairs of SMs
   std::vector<int> atomic_mats[RG_COUNT];  // matrices whose K is split for this GEMM (output must be zeroed)
   // buffers to clear before GEMM kind g (the outputs of atomic_mats[g]); entry RG_COUNT: every matrix's X64
   ZeroJob* d_zero[RG_COUNT + 1] = {};
@@ -345,6 +347,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     }
     plan.wide = 2.0 * wide >= all;
   }
+  int pairs = 0;
   {
     // Tiles of 256 rows: what bounds the products with G is the L2 bandwidth (10 TB/s), and two accumulators that share
     // the basis halve its part of the traffic.  1.1B shapes, a product with two parts 1.86 -> 1.59 ms, with one 1.02 ->
@@ -359,8 +362,14 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       blocks += ty * ((d.N + kTcBK - 1) / kTcBK) + tz * ((d.M + kTcBK - 1) / kTcBK);
     }
     plan.tall = tiles_tall >= 2 * sm_count && (!plan.wide || blocks >= 24 * tiles_tall);
+    // 256 x 256 tiles on pairs of SMs (gemm_pair_tcgen05.cuh, which has the figures) where they are too short for the two
+    // accumulators of one CTA, and enough of them to balance the pairs.
+    if (plan.wide && !plan.tall && tiles_tall >= 2 * sm_count) {
+      pairs = std::min(tc_pair_init(), sm_count / 2);
+      plan.pair = 2 * pairs >= sm_count - 4;
+    }
   }
-  auto tile_rows = [&](int g) { return plan.tall && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? 2 * kTcBM : kTcBM; };
+  auto tile_rows = [&](int g) { return (plan.tall || plan.pair) && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? 2 * kTcBM : kTcBM; };
   auto tile_cols = [&](int g) { return plan.wide && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? kRefWideBN : kRefBN; };
   auto add_tiles = [&](int g, int i, int out_rows, int out_cols, int K, long long target_kb) {
     const int kb_total = (K + kTcBK - 1) / kTcBK;
@@ -451,7 +460,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     }
     o_tiles[g] = take(sizeof(TcTile) * tiles[g].size());
     plan.n_tiles[g] = static_cast<int>(tiles[g].size());
-    plan.grid[g] = std::min(plan.n_tiles[g], sm_count);
+    plan.grid[g] = std::min(plan.n_tiles[g], plan.pair && (g == RG_Y_FROM_Z || g == RG_Z_FROM_Y) ? pairs : sm_count);   // (CTAs, or pairs)
     tc_assign_tiles(tiles[g], plan.grid[g], tile_first[g], g == RG_APPLY_Y || g == RG_APPLY_TRI);
     o_first[g] = take(sizeof(int) * tile_first[g].size());
   }
@@ -674,9 +683,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   using Narrow = std::integral_constant<int, kRefBN>;
   using Tall = std::integral_constant<int, 2>;
   using Flat = std::integral_constant<int, 1>;
-  if (!(plan.wide ? (plan.tall ? init_all(Wide{}, Tall{}) : init_all(Wide{}, Flat{}))
-                  : (plan.tall ? init_all(Narrow{}, Tall{}) : init_all(Narrow{}, Flat{}))) ||
-      cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>,
+  if (!plan.pair &&
+      !(plan.wide ? (plan.tall ? init_all(Wide{}, Tall{}) : init_all(Wide{}, Flat{}))
+                  : (plan.tall ? init_all(Narrow{}, Tall{}) : init_all(Narrow{}, Flat{}))))
+    return NGALORE_ERR_CUDA;
+  if (cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess ||
       cudaFuncSetAttribute(tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, L2::kTotal) != cudaSuccess)
@@ -699,13 +710,19 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
   }
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
   const int threads = 64 + 32 * 8;
+  cudaError_t pair_err = cudaSuccess;
   auto product = [&](auto a_mn) {   // a product with G; a_mn: with G^T
     constexpr bool MN = decltype(a_mn)::value;
     auto run = [&](auto p) {
       p.kernel<<<plan.grid[g], p.kThreads, p.kSmem, stream>>>(plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl,
                                                               plan.d_probs[problem], nullptr, 0);
     };
-    if (plan.wide && plan.tall) {
+    if (plan.pair) {
+      auto pair = [&](auto parts) {
+        pair_err = tc_pair_launch<decltype(parts)::value, MN>(plan.grid[g], stream, plan.d_maps, plan.d_tiles[g], plan.d_first[g], d_ctrl, plan.d_probs[problem]);
+      };
+      if (high_only) pair(std::integral_constant<int, 1>{}); else pair(std::integral_constant<int, 2>{});
+    } else if (plan.wide && plan.tall) {
       if (high_only) run(RefProduct<kRefWideBN, 1, 2, MN>{}); else run(RefProduct<kRefWideBN, 2, 2, MN>{});
     } else if (plan.wide) {
       if (high_only) run(RefProduct<kRefWideBN, 1, 1, MN>{}); else run(RefProduct<kRefWideBN, 2, 1, MN>{});
@@ -729,7 +746,7 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
       break;
   }
   *launches += 1;
-  return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
+  return pair_err == cudaSuccess && cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
 // The products with G write the bf16 parts of their result themselves, except for the matrices whose K they split.
