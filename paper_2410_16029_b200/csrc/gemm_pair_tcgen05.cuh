@@ -8,8 +8,8 @@
 // the tile, 256 columns, twice, so that the epilogue overlaps the next tile's MMAs.
 // 86 matrices of the 130M shapes, r = 256 (12 to 32 K blocks a tile): two parts 141 -> 107 us a product, one 88 -> 81.
 // Where K is long the epilogue matters less and the pairs lose: with them a refresh of the 1.1B shapes took 52.0 ms, with two
-// accumulators a CTA 51.3 although that still had a slower factorisation.  Tried for the projection of a step as well: 350M shapes 225 -> 199 us, 130M shapes 94 -> 99 us, the steps as
-// they were to half a percent; not taken.
+// accumulators a CTA 51.3 although that still had a slower factorisation.  Tried for the projection of a step as well: 350M
+// shapes 225 -> 199 us, 130M shapes 94 -> 99 us, the steps as they were to half a percent; not taken.
 //
 // Both CTAs of a pair walk the same tiles.  In each: warp 0 loads (the transaction counts of both go to the barriers of the first
 // CTA), warps 2 to 9 drain the accumulators; warp 1 of the first issues the MMAs, whose commits free the stages and announce the
