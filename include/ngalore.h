@@ -40,6 +40,8 @@
  *    a wait inside a GEMM pipeline runs out, the kernel stops issuing work and
  *    ngalore_poll_status returns NGALORE_ERR_TIMEOUT for the state as a whole:
  *    restore it from a checkpoint.  No call traps, aborts or spins for ever.
+ *  - When a launch in the middle of a step fails (NGALORE_ERR_CUDA), parts of W, m and v may have
+ *    advanced; ring position and step index have not, and the next step is a regular one.
  *  - A state is bound to the device that was current in ngalore_create and is
  *    not safe for concurrent calls from several threads.
  */
@@ -234,6 +236,13 @@ ngalore_status ngalore_stream_wait_update(ngalore_state* st, int g, void* stream
  * Not available with s = 0, stream_impl = 1, or for a matrix whose Gram row is formed by gram_fusion.
  */
 ngalore_status ngalore_debug_withhold_solution(ngalore_state* st, int matrix_index, int polls);
+
+/*
+ * Testing aid: the next ngalore_step or ngalore_step_host returns NGALORE_ERR_CUDA after it has launched its projection
+ * (phase 0) or its Gram / solve / moment kernels (phase 1), as it does when a launch or an event fails there.  Not
+ * available on the small-rank path.
+ */
+ngalore_status ngalore_debug_fail_step(ngalore_state* st, int phase);
 
 /* Change the learning rate used from the next step on. */
 ngalore_status ngalore_set_lr(ngalore_state* st, double lr);

@@ -87,16 +87,22 @@ __device__ __forceinline__ unsigned int stochastic_bf16_bits(float x, unsigned i
   return (__float_as_uint(x) + bits16) >> 16;
 }
 
-// The end of a step: ring position, step counters and work counters move on.
-__device__ __forceinline__ void advance_step(Ctrl* ctrl) {
-  ctrl->n_appended += 1;
-  ctrl->k += 1;
+// What the kernels of a step leave behind for the next one to start from.  The epoch moves on too, so that no flag of this step
+// passes for one of the next.
+__device__ __forceinline__ void reset_work(Ctrl* ctrl) {
   ctrl->epoch += 1;
   ctrl->work_counter = 0u;
   ctrl->gemm_counter0 = 0u;
   ctrl->gemm_counter1 = 0u;
   ctrl->spin_limit = 0;
   ctrl->debug_withhold = 0;
+}
+
+// The end of a step: ring position, step counters and work counters move on.
+__device__ __forceinline__ void advance_step(Ctrl* ctrl) {
+  ctrl->n_appended += 1;
+  ctrl->k += 1;
+  reset_work(ctrl);
 }
 
 // Programmatic dependent launch, for the kernels of a short step: a kernel launched so may start while its predecessor in

@@ -251,4 +251,7 @@ __global__ void __launch_bounds__(kStreamThreads) combine_kernel(const MatDesc* 
 
 __global__ void advance_kernel(Ctrl* ctrl) { advance_step(ctrl); }
 
+// Ends a step of which some launches are missing: the next one takes its place in the ring.
+__global__ void abandon_kernel(Ctrl* ctrl) { reset_work(ctrl); }
+
 }  // namespace ngalore

@@ -124,6 +124,7 @@ struct ngalore_state {
   std::vector<cudaEvent_t> ev_upd;
   // profiling
   bool profiling = false;
+  int debug_fail_after = -1;   // >= 0: the next step gives up after this phase (ngalore_debug_fail_step)
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   bool ev_valid = false;
 };
@@ -390,10 +391,11 @@ ngalore_status refresh_impl(ngalore_state* st, const uint16_t* const* G_in, cons
   return finish_refresh(st, st->refresh_tc_idx, true, stream, true, true);
 }
 
-// grouped: the caller delivers W in the groups of ngalore_state::group_part; the back-projection of a group waits
-// for that group's event ev_w_in and records ev_w_done (host-buffer step, tensor-core path only).
-ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* const* G, cudaStream_t stream,
-                         bool grouped = false) {
+// The launches of one step.  begun: set before the first kernel that moves the work counters on; the last one puts them back.
+ngalore_status enqueue_step(ngalore_state* st, float* const* W, const uint16_t* const* G, cudaStream_t stream, bool grouped,
+                            bool& begun) {
+  const int fail_after = st->debug_fail_after;
+  st->debug_fail_after = -1;
   ngalore_status rc;
   if (st->T > 0 && st->k % st->T == 0) {
     std::vector<int> all(st->n);
@@ -407,6 +409,7 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
 
   if (st->sr.ready && !grouped && st->upd_first.size() <= 1) {
     // small-rank path: projection with the Gram row, then solve + moments + weight update (small_rank.cuh)
+    begun = true;
     if (st->profiling) NG_CUDA(cudaEventRecord(st->ev[0], stream));
     if ((rc = sr_project_gram(st->sr, st->d_desc, st->tc.d_Gptr, st->d_ctrl, st->s, stream, &st->launches))) return rc;
     if (st->profiling) {
@@ -429,6 +432,7 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
     }
     return NGALORE_OK;
   }
+  begun = true;
   if (st->profiling) NG_CUDA(cudaEventRecord(st->ev[0], stream));
   // ---- phase 0: R = P^T G into ring slot `cur`
   if (st->opt.gemm_impl == 1) {
@@ -454,6 +458,7 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
   } else {
     if ((rc = tc_project(st->tc, st->d_desc, st->d_ctrl, st->d_hyper, stream, &st->launches))) return rc;
   }
+  if (fail_after == 0) return NGALORE_ERR_CUDA;
   if (st->profiling) NG_CUDA(cudaEventRecord(st->ev[1], stream));
   // ---- phase 1: Gram row, solve, natural gradient + moments
   if (st->opt.stream_impl == 1) {
@@ -464,6 +469,7 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
     if ((rc = fused_stream_launch(st->fused, st->d_desc, st->n, st->d_ctrl, st->d_hyper, st->s, st->tc.short_step, stream, &st->launches))) return rc;
   }
   NG_CUDA(cudaGetLastError());
+  if (fail_after == 1) return NGALORE_ERR_CUDA;
   if (st->profiling) NG_CUDA(cudaEventRecord(st->ev[2], stream));
   // ---- phase 2: W <- (1 - lr wd) W - lr P u
   if (st->opt.gemm_impl == 1) {
@@ -525,6 +531,20 @@ ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* con
     st->n_appended += 1;
   }
   return NGALORE_OK;
+}
+
+// One step.  grouped: the caller delivers W in the groups of ngalore_state::group_part; the back-projection of a group waits
+// for that group's event ev_w_in and records ev_w_done (host-buffer step, tensor-core path only).
+ngalore_status step_impl(ngalore_state* st, float* const* W, const uint16_t* const* G, cudaStream_t stream,
+                         bool grouped = false) {
+  bool begun = false;
+  const ngalore_status rc = enqueue_step(st, W, G, stream, grouped, begun);
+  if (rc != NGALORE_OK && begun) {
+    // the counters stand where the kernels that did go out left them: the next step would take its items for done
+    abandon_kernel<<<1, 1, 0, stream>>>(st->d_ctrl);
+    st->launches += 1;
+  }
+  return rc;
 }
 
 }  // namespace
@@ -1252,6 +1272,12 @@ ngalore_status ngalore_debug_withhold_solution(ngalore_state* st, int matrix_ind
   NG_CUDA(cudaDeviceSynchronize());
   const int v[2] = {polls, matrix_index + 1};
   NG_CUDA(cudaMemcpy(&st->d_ctrl->spin_limit, v, sizeof(v), cudaMemcpyHostToDevice));
+  return NGALORE_OK;
+}
+
+ngalore_status ngalore_debug_fail_step(ngalore_state* st, int phase) {
+  if (st == nullptr || phase < 0 || phase > 1 || st->sr.ready) return NGALORE_ERR_INVALID_ARG;
+  st->debug_fail_after = phase;
   return NGALORE_OK;
 }
 

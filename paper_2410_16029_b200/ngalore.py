@@ -71,6 +71,8 @@ _lib.ngalore_stream_wait_update.restype = ctypes.c_int
 _lib.ngalore_stream_wait_update.argtypes = [_vp, ctypes.c_int, _vp]
 _lib.ngalore_debug_withhold_solution.restype = ctypes.c_int
 _lib.ngalore_debug_withhold_solution.argtypes = [_vp, ctypes.c_int, ctypes.c_int]
+_lib.ngalore_debug_fail_step.restype = ctypes.c_int
+_lib.ngalore_debug_fail_step.argtypes = [_vp, ctypes.c_int]
 _lib.ngalore_set_lr.restype = ctypes.c_int
 _lib.ngalore_set_lr.argtypes = [_vp, ctypes.c_double]
 _lib.ngalore_num_matrices.restype = ctypes.c_int
@@ -243,6 +245,10 @@ class NGaLore:
     def debug_withhold_solution(self, matrix_index: int, polls: int):
         """Testing aid: the next step does not announce matrix_index's solved weights (see include/ngalore.h)."""
         _check(_lib.ngalore_debug_withhold_solution(self._h, matrix_index, polls), "ngalore_debug_withhold_solution")
+
+    def debug_fail_step(self, phase: int):
+        """Testing aid: the next step fails after the launches of `phase` (see include/ngalore.h)."""
+        _check(_lib.ngalore_debug_fail_step(self._h, phase), "ngalore_debug_fail_step")
 
     def set_lr(self, lr: float):
         _check(_lib.ngalore_set_lr(self._h, lr), "ngalore_set_lr")
