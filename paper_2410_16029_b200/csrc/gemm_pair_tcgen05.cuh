@@ -289,9 +289,12 @@ inline bool tc_pair_set_smem() {
 
 // Launch-time setup of the kernels above: the number of pairs that run side by side on this device (0: none).  The tiles are handed out
 // beforehand: a pair that had to wait for another to end would double the time of the launch.  (All four have an SM to themselves, so
-// one of them is asked about.)
+// one of them is asked about.  A call that fails here means no pairs and nothing else: its error is not left for the next launch.)
 inline int tc_pair_init() {
-  if (!tc_pair_set_smem<1, false>() || !tc_pair_set_smem<1, true>() || !tc_pair_set_smem<2, false>() || !tc_pair_set_smem<2, true>()) return 0;
+  if (!tc_pair_set_smem<1, false>() || !tc_pair_set_smem<1, true>() || !tc_pair_set_smem<2, false>() || !tc_pair_set_smem<2, true>()) {
+    cudaGetLastError();
+    return 0;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = 2;
   cfg.blockDim = kPairThreads;
@@ -302,7 +305,9 @@ inline int tc_pair_init() {
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   int pairs = 0;
-  return cudaOccupancyMaxActiveClusters(&pairs, tc_pair_kernel<2, true>, &cfg) == cudaSuccess ? pairs : 0;
+  if (cudaOccupancyMaxActiveClusters(&pairs, tc_pair_kernel<2, true>, &cfg) == cudaSuccess) return pairs;
+  cudaGetLastError();
+  return 0;
 }
 
 template <int NB, bool A_MN>

@@ -137,6 +137,8 @@ namespace {
     if (e__ != cudaSuccess) return NGALORE_ERR_CUDA;    \
   } while (0)
 
+// Around every entry point that has a state: its device is the current one inside, and an error that the runtime has recorded
+// ends with the call that reported it, or the next call would find it after its first launch and take it for that launch's.
 struct DeviceGuard {
   int prev = -1;
   bool ok = true;
@@ -147,6 +149,7 @@ struct DeviceGuard {
   ~DeviceGuard() {
     int cur = -1;
     if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
+    cudaGetLastError();
   }
 };
 

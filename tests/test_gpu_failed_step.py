@@ -1,6 +1,7 @@
-"""A step that fails between its launches leaves no work counter or flag behind that the next step takes for its own.  beta1 = beta2 =
+"""A failed call stays its own.  A step that fails between its launches leaves no work counter or flag behind that the next step takes for its own.  beta1 = beta2 =
 0, so that a step that ran in part and is taken again has the same result; K of the first matrix is split, so that its tiles add to
-a ring slot that has to be cleared.  The bound is that of two orders of the same sums."""
+a ring slot that has to be cleared.  The bound is that of two orders of the same sums.  And a state that does not fit the device is
+refused without an error left over for the next call on another."""
 import pytest
 import torch
 
@@ -42,3 +43,17 @@ def _run(phase, host, s=3, **kw):
 def test_the_step_after_a_failed_one_is_a_regular_one(phase, host, kw):
     for got, want in zip(_run(phase, host, **kw), _run(None, host, **kw)):
         assert (torch.linalg.norm(got - want) / torch.linalg.norm(want)).item() <= 0.1 * TOL_UPDATE
+
+
+def test_a_state_that_does_not_fit_leaves_no_error_for_the_next_step():
+    from paper_2410_16029_b200.ngalore import NGaLore, NGaLoreError
+
+    opt = NGaLore([(300, 136)], R, 3, 0)
+    opt.set_subspace(0, torch.linalg.qr(torch.randn(300, R, device="cuda"))[0])
+    with pytest.raises(NGaLoreError) as refused:
+        NGaLore([(1 << 24, 1 << 24)], 512, 32, 0)      # a history of a terabyte
+    assert refused.value.code == 2
+    W = [torch.zeros(300, 136, device="cuda")]
+    opt.step(W, [torch.randn(300, 136, device="cuda").bfloat16()])
+    torch.cuda.synchronize()
+    assert opt.poll_status()[0] == 0 and opt.step_count == 1 and W[0].abs().max().item() > 0
