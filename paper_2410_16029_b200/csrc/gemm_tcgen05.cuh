@@ -610,6 +610,7 @@ struct TcPlan {
   TcTile* d_tiles_back = nullptr;
   std::vector<int> back_tile0;     // first back-projection tile of every matrix, plus the total (n + 1 entries)
   int n_tiles_proj = 0, n_tiles_back = 0;
+  int proj_bn = 0, back_bn = 0;    // columns of a tile
   int grid_proj = 0, grid_back = 0;
   ClearJob* d_clear = nullptr;     // pieces of the ring slots that tiles of a split K add to
   int n_clear = 0;
@@ -707,21 +708,6 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
     plan.long_k_back = work_long_k * 10 >= work_all * 9;
   }
   const int proj_bm = plan.tall_proj ? 2 * kTcBM : kTcBM;
-  // Tiles of 128 or 64 columns where every one of them still has an SM to itself: with fewer tiles than SMs a step is
-  // the latency of one tile, and half the columns are two thirds of its operands and half of its epilogue.  One 512 x 1376 matrix,
-  // r = 128 (6 projection tiles of 256 columns, 22 of 64; 24 and 88 of the back-projection): 32.7 -> 26.4 us a step.
-  auto tile_width = [&](int widest, auto rows_of, auto cols_of) {
-    int width = widest;
-    while (width > 64) {
-      long long tiles = 0;
-      for (const MatDesc& d : mats) tiles += static_cast<long long>((rows_of(d) + kTcBM - 1) / kTcBM) * ((cols_of(d) + width / 2 - 1) / (width / 2));
-      if (tiles > sm_count) break;
-      width /= 2;
-    }
-    return width;
-  };
-  const int proj_bn = plan.tall_proj ? kProjBN : tile_width(kProjBN, [](const MatDesc& d) { return d.lr_rows; }, [](const MatDesc& d) { return d.lr_cols; });
-  const int back_bn = tile_width(kTcBackBN, [](const MatDesc& d) { return d.M; }, [](const MatDesc& d) { return d.N; });
   std::vector<TcTile> proj, back;
   long long total_kb = 0;
   for (int i = 0; i < n; ++i) {
@@ -732,6 +718,36 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
   const long long per_cta = (total_kb + sm_count - 1) / sm_count;
   long long target_kb = per_cta / 4;
   if (target_kb < 16) target_kb = 16;
+  // K blocks of the projection of a matrix, those of a piece of it, and the pieces
+  struct Split { int kb_total, kb_per, pieces; };
+  auto split_of = [&](const MatDesc& d) {
+    Split k{((d.right ? d.N : d.M) + kTcBK - 1) / kTcBK, 0, 0};
+    const int wanted = std::max(1, static_cast<int>((k.kb_total + target_kb - 1) / target_kb));
+    k.kb_per = (k.kb_total + wanted - 1) / wanted;
+    k.pieces = (k.kb_total + k.kb_per - 1) / k.kb_per;
+    return k;
+  };
+  // Tiles of 128 or 64 columns where every one of them, pieces of a split K included, still has an SM to itself: with fewer
+  // tiles than SMs a step is the latency of one tile, and half the columns are two thirds of its operands and half of its epilogue.
+  // One 512 x 1376 matrix, r = 128 (6 projection tiles of 256 columns, 22 of 64; 24 and 88 of the back-projection): 32.7 -> 26.4 us a step.
+  // Where tiles queue for an SM, narrower ones only stage the operand they share more often (projection, a row of tiles with its
+  // pieces counted once against every one of them: 32000 x 2048, r = 128, 58 -> 46 us; 6000 x 4000, r = 256, 46 -> 34).
+  auto tile_width = [&](int widest, auto tile_rows, auto cols_of) {
+    int width = widest;
+    while (width > 64) {
+      long long tiles = 0;
+      for (const MatDesc& d : mats) tiles += static_cast<long long>(tile_rows(d)) * ((cols_of(d) + width / 2 - 1) / (width / 2));
+      if (tiles > sm_count) break;
+      width /= 2;
+    }
+    return width;
+  };
+  const int proj_bn = plan.tall_proj ? kProjBN
+                                     : tile_width(kProjBN, [&](const MatDesc& d) { return (d.lr_rows + kTcBM - 1) / kTcBM * split_of(d).pieces; },
+                                                  [](const MatDesc& d) { return d.lr_cols; });
+  const int back_bn = tile_width(kTcBackBN, [](const MatDesc& d) { return (d.M + kTcBM - 1) / kTcBM; }, [](const MatDesc& d) { return d.N; });
+  plan.proj_bn = proj_bn;
+  plan.back_bn = back_bn;
   std::vector<ClearJob> clear;
   // Matrices whose Gram row is formed in the projection's epilogue (project_gram_tcgen05.cuh): the workload class
   // of the tall projection tiles (long K, rank 512: there the history read is long enough to hide the MMAs),
@@ -745,11 +761,8 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
   const bool fuse_class = allow_gram_fusion && plan.tall_proj && s >= 1 && s <= kPgSMax;
   for (int i = 0; i < n; ++i) {
     const MatDesc& d = mats[i];
-    const int kb_total = ((d.right ? d.N : d.M) + kTcBK - 1) / kTcBK;
-    int splits = static_cast<int>((kb_total + target_kb - 1) / target_kb);
-    if (splits < 1) splits = 1;
-    const int kb_per = (kb_total + splits - 1) / splits;
-    splits = (kb_total + kb_per - 1) / kb_per;
+    const Split split = split_of(d);
+    const int kb_total = split.kb_total, kb_per = split.kb_per, splits = split.pieces;
     // (a K of up to 128 blocks stays in one piece for it even where the schedule would rather split it)
     if (fuse_class && kb_total <= 128 && !d.right && d.H16 == nullptr && d.s == s && d.lr_rows % 32 == 0 && d.lr_cols % 32 == 0) {
       plan.gram_fused[i] = 1;

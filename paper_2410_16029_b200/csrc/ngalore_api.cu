@@ -1299,6 +1299,18 @@ int64_t ngalore_step_count(const ngalore_state* st) { return st ? st->k : -1; }
 size_t ngalore_device_bytes(const ngalore_state* st) { return st ? st->arena_bytes + st->work_bytes + st->stage_bytes + st->tc.device_bytes + st->refresh.device_bytes + st->sr.device_bytes : 0; }
 int64_t ngalore_launch_count(const ngalore_state* st) { return st ? st->launches : 0; }
 int64_t ngalore_descriptor_uploads(const ngalore_state* st) { return st ? st->tc.bind_uploads : 0; }
+int ngalore_debug_plan(const ngalore_state* st, int what) {
+  if (st == nullptr) return -1;
+  switch (what) {
+    case 0: return st->tc.proj_bn;
+    case 1: return st->tc.n_tiles_proj;
+    case 2: return st->tc.n_clear > 0 ? 1 : 0;
+    case 3: return st->tc.back_bn;
+    case 4: return !st->refresh.ready ? -1 : (st->refresh.pair ? 2 : (st->refresh.tall ? 1 : 0));
+    case 5: return !st->refresh.ready ? -1 : (st->refresh.atomic_mats[RG_Y_FROM_Z].empty() && st->refresh.atomic_mats[RG_Z_FROM_Y].empty() ? 0 : 1);
+  }
+  return -1;
+}
 int ngalore_uses_small_rank_path(const ngalore_state* st) { return (st && st->sr.ready) ? 1 : 0; }
 
 ngalore_status ngalore_set_profiling(ngalore_state* st, int on) {

@@ -73,6 +73,8 @@ _lib.ngalore_debug_withhold_solution.restype = ctypes.c_int
 _lib.ngalore_debug_withhold_solution.argtypes = [_vp, ctypes.c_int, ctypes.c_int]
 _lib.ngalore_debug_fail_step.restype = ctypes.c_int
 _lib.ngalore_debug_fail_step.argtypes = [_vp, ctypes.c_int]
+_lib.ngalore_debug_plan.restype = ctypes.c_int
+_lib.ngalore_debug_plan.argtypes = [_vp, ctypes.c_int]
 _lib.ngalore_set_lr.restype = ctypes.c_int
 _lib.ngalore_set_lr.argtypes = [_vp, ctypes.c_double]
 _lib.ngalore_num_matrices.restype = ctypes.c_int
@@ -249,6 +251,11 @@ class NGaLore:
     def debug_fail_step(self, phase: int):
         """Testing aid: the next step fails after the launches of `phase` (see include/ngalore.h)."""
         _check(_lib.ngalore_debug_fail_step(self._h, phase), "ngalore_debug_fail_step")
+
+    def debug_plan(self, what: str) -> int:
+        """Testing aid: what the state's plan chose (see include/ngalore.h)."""
+        return _lib.ngalore_debug_plan(self._h, ("projection_columns", "projection_tiles", "projection_splits", "update_columns",
+                                                 "refresh_products", "refresh_splits").index(what))
 
     def set_lr(self, lr: float):
         _check(_lib.ngalore_set_lr(self._h, lr), "ngalore_set_lr")

@@ -9,6 +9,32 @@ from tests.parity_util import TOL_UPDATE
 pytestmark = pytest.mark.gpu
 
 
+SETS = [
+    ([(512, 1376)], 128, {}, 64, 0),
+    ([(512, 1376)] * 6, 128, {}, 64, 0),
+    ([(512, 1376)] * 7, 128, {}, 128, 0),
+    ([(512, 1376)] * 24, 128, {}, 256, 0),
+    ([(4000, 2048)], 256, {}, 128, 1),
+    ([(6000, 720)], 200, {}, 64, 1),
+    ([(1024, 4096)], 100, {"projection": "short_side"}, 64, 0),
+    ([(4096, 1400)], 100, {"projection": "short_side"}, 64, 1),
+    ([(32000, 1024)], 128, {}, 256, 1),
+    ([(5000, 2000)] * 3, 128, {}, 256, 1),
+]
+
+
+@pytest.mark.skipif(not torch.cuda.is_available() or torch.cuda.get_device_properties(0).multi_processor_count != 148,
+                    reason="the widths are those of 148 multiprocessors")
+@pytest.mark.parametrize("shapes,r,kw,columns,splits", SETS)
+def test_narrow_tiles_have_a_multiprocessor_each(shapes, r, kw, columns, splits):
+    """With the pieces of a split K counted: where tiles would queue, they stay as wide as they are."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    opt = NGaLore(shapes, r, 2, 0, **kw)
+    assert opt.debug_plan("projection_columns") == 256 or opt.debug_plan("projection_tiles") <= 148
+    assert (opt.debug_plan("projection_columns"), opt.debug_plan("projection_splits")) == (columns, splits)
+
+
 def _steps(shapes, r, gemm_impl, groups=0, **kw):
     from paper_2410_16029_b200.ngalore import NGaLore
 
@@ -34,6 +60,7 @@ def _steps(shapes, r, gemm_impl, groups=0, **kw):
     ([(512, 1376)] * 7, 128, {}),
     ([(128, 72), (130, 328), (257, 1000)], 40, {}),
     ([(4000, 200), (300, 136)], 64, {}),
+    ([(4000, 1000)], 256, {}),
     ([(700, 264), (264, 696)], 100, {"projection": "short_side"}),
     ([(512, 1376)] * 3, 128, {"groups": 2}),
 ])
