@@ -53,16 +53,19 @@ struct StageMeta {
 template <int SMAX, bool HIST16, bool MOM16 = false>
 struct FusedCfg {
   // Elements per stage and slot.  The bf16 history costs more instructions per byte (conversion, two Gram rows),
-  // and the per-stage bookkeeping of a consumer thread weighs as much as its arithmetic on two elements, so its
+  // and the per-stage bookkeeping of a consumer thread weighs as much as its arithmetic on two elements, so up to sixteen slots its
   // threads take four, and its stages are as long as three of them fit: with two, a stage of which is worked on, the SM has too little
-  // under way.  350M shapes, s = 16, bf16 moments: two stages of 2048 elements 950 us, three of 1792 (14 warps) 805.
+  // under way.  350M shapes, s = 16, bf16 moments: two stages of 2048 elements 950 us, three of 1792 (14 warps) 805.  (Beyond
+  // sixteen slots: five stages of 512 elements, two a thread.)
   static constexpr int CE = !HIST16 ? (SMAX <= 16 ? 1024 : 512) : (SMAX <= 8 ? 2048 : (SMAX <= 16 ? (MOM16 ? 1792 : 1536) : 512));
   // Consumer threads: a warp issues the 100 to 250 instructions of a stage one after another, so eight warps take 1 us for it
   // whatever it holds.  The bf16 history costs more instructions per byte (conversion, two Gram rows), and a stage of
   // eight slots at most holds as little as 12 KB (history and moments of s = 0) to 40 KB, which arrive in 0.3 to 0.9 us; they get
   // sixteen warps.  Measured, eight against sixteen, stream phase: s = 5, 11 M elements, 154 -> 125 us; s = 0 on the 60M
-  // shapes 39 -> 35; s = 8 on them 88 either way, as sixteen slots (1.1B shapes, 4.16 ms), which stay with eight warps.
-  static constexpr int kConsumers = HIST16 && SMAX <= 16 ? CE / 4 : (SMAX <= 8 ? 512 : 256);
+  // shapes 39 -> 35; s = 8 on them 88 either way, as sixteen slots (1.1B shapes, 4.16 ms), which stay with eight warps.  So do bf16
+  // moments beside an fp32 history: two elements a thread draw a block of the generator for two of its four words (130M shapes,
+  // s = 5 and 8, 302 -> 308 and 353 -> 361 us; 350M shapes, s = 8, 870 -> 894; s = 0 no difference).
+  static constexpr int kConsumers = HIST16 && SMAX <= 16 ? CE / 4 : (SMAX <= 8 && !MOM16 ? 512 : 256);
   static constexpr int kThreads = kConsumers + 64;  // and the producer and the finishing warp
   static constexpr int kHistBytes = SMAX * CE * (HIST16 ? 2 : 4);
   static constexpr int kCurOff = kHistBytes;                          // HIST16: fp32 gradient of this step
