@@ -73,7 +73,9 @@ __device__ __forceinline__ void tf_dmma(double (&c)[2], double a, double b) {
 
 // 1 / d and 1 / sqrt(d) for d > 0 far from the ends of the range: the hardware's approximation (20 bits) and one step of
 // Householder's third-order iteration, y (1 + e + e^2) with e = 1 - d y and y (1 + e / 2 + 3 e^2 / 8) with e = 1 - d y^2, whose error is
-// of the order of e^3.  No branches, so that the pivots of a block and their square roots overlap.
+// of the order of e^3.  Measured over 1e-280 .. 1e280, they are off by at most 1.001 and 1.24 units of 2^-53 of the value
+// (test_gpu_fp64_scalars.py; half a unit in the last place is up to one of these).  No branches, so that the pivots of a block and their square
+// roots overlap.
 __device__ __forceinline__ double tf_reciprocal(double d) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
