@@ -40,6 +40,7 @@ def _steps(shapes, r, gemm_impl, groups=0, **kw):
 
     gen = torch.Generator(device="cuda").manual_seed(17)
     opt = NGaLore(shapes, r, 3, 0, lam=0.1, lr=1e-2, gemm_impl=gemm_impl, **kw)
+    assert opt.debug_plan("projection_columns") < 256
     if groups:
         opt.set_update_groups(groups)
     for i, (M, N) in enumerate(shapes):

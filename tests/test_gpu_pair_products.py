@@ -11,6 +11,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("r,shapes", [
     (196, [(777, 520), (900, 264)]),
     (256, [(768, 768), (1024, 520)]),
+    (256, [(768, 768), (3000, 264)]),       # (whose K of 3000 is split)
     (260, [(650, 584), (1100, 776), (640, 64)]),
 ])
 def test_products_on_pairs(r, shapes):
@@ -20,6 +21,7 @@ def test_products_on_pairs(r, shapes):
     copies = 60 // len(shapes) + 1        # more than two 256 x 256 tiles for every SM
     G = [g.clone() for g, _ in made for _ in range(copies)]
     opt = NGaLore([s for s in shapes for _ in range(copies)], r, 0, 0)
+    assert opt.debug_plan("refresh_products") == 2 and opt.debug_plan("refresh_splits") == int(max(M for M, _ in shapes) == 3000)
     opt.refresh_subspace(G)
     torch.cuda.synchronize()
     assert opt.poll_status()[0] == 0
