@@ -109,7 +109,8 @@ __device__ __forceinline__ void advance_step(Ctrl* ctrl) {
 // the stream still runs.  pdl_begin lets the successor start in turn and then waits until the predecessor has finished
 // and its writes are visible; what comes before it (barriers, tensor memory) and the launch itself overlap the
 // predecessor's tail.  Every kernel that launch_step is given calls it before it touches global memory that a kernel writes (the
-// tables of a plan, which none does, may be read before: 60M shapes 212.5 -> 211.5 us a step, encoder shapes at r = 8 177.4 -> 176.1);
+// tables of a plan, which none does, may be read before: 60M shapes 213.0 -> 211.7 us a step, encoder shapes at r = 8 177.4 -> 176.3,
+// one 512 x 1376 matrix 26.6 -> 26.3; nothing where an upload of tensor maps goes ahead of the step);
 // after an ordinary launch it returns at once.  What else the launch comes after in its stream, a wait for an event among it, stays a full
 // dependency, so the first kernel of a step may be launched so whatever the caller has put before it.
 __device__ __forceinline__ void pdl_begin() {

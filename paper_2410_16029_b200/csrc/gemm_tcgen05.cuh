@@ -729,7 +729,8 @@ inline ngalore_status tc_plan_create(TcPlan& plan, const std::vector<MatDesc>& m
   };
   // Tiles of 128 or 64 columns where every one of them, pieces of a split K included, still has an SM to itself: with fewer
   // tiles than SMs a step is the latency of one tile, and half the columns are two thirds of its operands and half of its epilogue.
-  // One 512 x 1376 matrix, r = 128 (6 projection tiles of 256 columns, 22 of 64; 24 and 88 of the back-projection): 32.7 -> 26.4 us a step.
+  // One 512 x 1376 matrix, r = 128 (6 projection tiles of 256 columns, 22 of 64; 24 and 88 of the back-projection): with its launch 15.5 -> 11.5
+  // and 12.3 -> 10.2 us.
   // Where tiles queue for an SM, narrower ones only stage the operand they share more often (projection, a row of tiles with its
   // pieces counted once against every one of them: 32000 x 2048, r = 128, 58 -> 46 us; 6000 x 4000, r = 256, 46 -> 34).
   auto tile_width = [&](int widest, auto tile_rows, auto cols_of) {
