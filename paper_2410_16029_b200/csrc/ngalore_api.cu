@@ -257,7 +257,7 @@ ngalore_status apply_gradient(ngalore_state* st, const std::vector<int>& idx, co
 
 // whole_set: this call completes a refresh of every matrix (even when idx lists only part of them).
 // tc_set: idx is the whole list of matrices refreshed on the tensor-core path (ngalore_state::refresh_tc_idx), whose
-// bases sit in Ya: norms and copies of all projectors are two prepared launches.
+// bases sit in Ya (or Yb, as the jobs say): norms and copies of all projectors are two prepared launches.
 ngalore_status finish_refresh(ngalore_state* st, const std::vector<int>& idx, bool basis_in_a, cudaStream_t stream,
                               bool whole_set, bool tc_set = false) {
   ngalore_status rc;
@@ -379,18 +379,6 @@ ngalore_status refresh_impl(ngalore_state* st, const uint16_t* const* G_in, cons
   if ((rc = refresh_tc_run(st->refresh, st->refresh_tc_G.data(), q, st->opt.seed,
                            static_cast<unsigned long long>(st->k) * 65536ull, st->d_ctrl, stream, &st->launches)))
     return rc;
-  // The basis sits in Ya, orthonormal to about 1e-6 where the matrix has enough rows for the bf16-pair rounding
-  // of the last product to average out.  Short matrices get one exact pass (Gram, Cholesky and triangular solve in fp64): Ya -> Yb -> Ya.
-  std::vector<int> small;
-  for (int i : st->refresh_tc_idx)
-    if (st->mats[i].eM < 512) small.push_back(i);
-  if (!small.empty()) {
-    if ((rc = orthonormalise(st, small, 0, true, stream))) return rc;
-    for (int i : small) {
-      const HostMat& hm = st->mats[i];
-      NG_CUDA(cudaMemcpyAsync(hm.Ya, hm.Yb, sizeof(float) * hm.eM * hm.rp, cudaMemcpyDeviceToDevice, stream));
-    }
-  }
   return finish_refresh(st, st->refresh_tc_idx, true, stream, true, true);
 }
 
@@ -842,17 +830,18 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   }
   if (st->opt.gemm_impl != 1) {
     // the refresh plan sees every matrix it takes in the orientation whose left subspace is wanted
-    std::vector<float*> Yf, Zf;
+    std::vector<float*> Yf, Zf, Yshort;
     std::vector<MatDesc> eff;
     for (int i = 0; i < n_matrices; ++i) {
       if (st->mats[i].rp % 4 != 0) { st->refresh_plain_idx.push_back(i); continue; }
       st->refresh_tc_idx.push_back(i);
       Yf.push_back(st->mats[i].Ya); Zf.push_back(st->mats[i].Xa);
+      Yshort.push_back(st->mats[i].Yb);
       eff.push_back(st->h_desc[i]);
       eff.back().M = st->mats[i].eM; eff.back().N = st->mats[i].eN;
     }
     if (!eff.empty()) {
-      rc = refresh_plan_create(st->refresh, eff, Yf, Zf, prop.multiProcessorCount, ritz_columns(st));
+      rc = refresh_plan_create(st->refresh, eff, Yf, Zf, Yshort, prop.multiProcessorCount, ritz_columns(st));
       if (rc != NGALORE_OK) return fail(rc);
       std::vector<WorkingJob> jobs;
       std::vector<int> start(1, 0), nstart(1, 0);
@@ -861,7 +850,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
         const HostMat& hm = st->mats[i];
         const MatDesc& d = st->h_desc[i];
         const int tx = (hm.rp + kEndCols - 1) / kEndCols, ty = (hm.eM + kEndRows - 1) / kEndRows;
-        jobs.push_back(WorkingJob{hm.Ya, st->refresh.mats[k].D, d.P32, d.P16, d.Pt16, st->d_status + i, hm.eM, hm.rp, d.ldp, d.ldpt,
+        jobs.push_back(WorkingJob{st->refresh.is_short[k] ? hm.Yb : hm.Ya, st->refresh.mats[k].D, d.P32, d.P16, d.Pt16, st->d_status + i, hm.eM, hm.rp, d.ldp, d.ldpt,
                                   hm.right ? 0 : 1, tx, end_norm_rows(hm.eM)});
         start.push_back(start.back() + tx * ty);
         nstart.push_back(nstart.back() + tx * ((hm.eM + end_norm_rows(hm.eM) - 1) / end_norm_rows(hm.eM)));

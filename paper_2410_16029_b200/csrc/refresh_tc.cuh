@@ -99,7 +99,8 @@ constexpr int kSyrkRows = 1024, kSyrkRowsFew = 256;
 constexpr int kSyrkFewTiles = 16;   // per SM
 
 struct SyrkMat {
-  const __nv_bfloat16 *hi, *lo;   // rows x ld: the two parts of the basis, L columns of which are valid
+  const __nv_bfloat16 *hi, *lo;   // rows x ld: the two parts of the basis, L columns of which are valid ...
+  const float* f32;               // ... or the basis itself, rows x L
   double* C;       // L x L fp64 accumulator (zeroed before the launch); lower tiles are written
   int rows, L, ld;
 };
@@ -109,7 +110,8 @@ struct SyrkMat {
 // atomics.  On the fp64 tensor cores: bound by their rate, which is that of the vector units (34 TFLOP/s), but reached
 // with a quarter of the instructions and a third of the shared-memory reads; the next 16 rows are fetched and widened
 // while the current ones are multiplied.  156 matrices of the 1.1B shapes, 115 GFLOP: 7.2 ms with 4 x 4 register tiles on
-// the vector units, 4.1 ms so.
+// the vector units, 4.1 ms so.  F32: of a basis in fp32 (refresh_tc_short).
+template <bool F32>
 __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, const SyrkTile* tiles) {
   constexpr int LD = 64 + 8;      // rows 8 modulo 16 doubles apart: fragments without bank conflicts
   __shared__ __align__(16) double As[2][16][LD];
@@ -128,11 +130,19 @@ __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, cons
 #pragma unroll
     for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = 0.0;
   uint2 ah, al, bh, bl;
+  float4 af, bf;
   auto fetch = [&](int k0) {
     const int k = k0 + lk;
+    const bool in_a = k < k1 && i0 + lc < m.L, in_b = k < k1 && j0 + lc < m.L;
+    if constexpr (F32) {
+      const float* row = m.f32 + static_cast<long long>(min(k, k1 - 1)) * m.L;
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      af = in_a ? *reinterpret_cast<const float4*>(row + i0 + lc) : zero;
+      bf = in_b ? *reinterpret_cast<const float4*>(row + j0 + lc) : zero;
+      return;
+    }
     const long long row = static_cast<long long>(min(k, k1 - 1)) * m.ld;
     const uint2 zero = make_uint2(0u, 0u);
-    const bool in_a = k < k1 && i0 + lc < m.L, in_b = k < k1 && j0 + lc < m.L;
     ah = in_a ? *reinterpret_cast<const uint2*>(m.hi + row + i0 + lc) : zero;
     al = in_a ? *reinterpret_cast<const uint2*>(m.lo + row + i0 + lc) : zero;
     bh = in_b ? *reinterpret_cast<const uint2*>(m.hi + row + j0 + lc) : zero;
@@ -145,8 +155,13 @@ __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, cons
   auto put = [&](int buf) {
     double2* a = reinterpret_cast<double2*>(&As[buf][lk][lc]);
     double2* b = reinterpret_cast<double2*>(&Bs[buf][lk][lc]);
-    a[0] = widen(ah.x, al.x); a[1] = widen(ah.y, al.y);
-    b[0] = widen(bh.x, bl.x); b[1] = widen(bh.y, bl.y);
+    if constexpr (F32) {
+      a[0] = make_double2(af.x, af.y); a[1] = make_double2(af.z, af.w);
+      b[0] = make_double2(bf.x, bf.y); b[1] = make_double2(bf.z, bf.w);
+    } else {
+      a[0] = widen(ah.x, al.x); a[1] = widen(ah.y, al.y);
+      b[0] = widen(bh.x, bl.x); b[1] = widen(bh.y, bl.y);
+    }
   };
   fetch(t.k0);
   put(0);
@@ -181,6 +196,81 @@ __global__ void __launch_bounds__(256) syrk_f64_kernel(const SyrkMat* mats, cons
         const int i = i0 + wr + 8 * x + fr, j = j0 + wc + 8 * y + 2 * fk + h;
         if (i < m.L && j <= i) atomicAdd(m.C + static_cast<long long>(i) * m.L + j, acc[x][y][h]);
       }
+}
+
+// Q = Y R^-1 in fp64 from an fp32 basis, rounded to fp32 once: the last pass over matrices with few rows (refresh_tc_short).
+// One CTA per 64 x 64 tile of Q on the fp64 tensor cores; R^-1 is upper triangular, so a tile sums over the rows of R^-1 down to
+// its own last column only.
+struct ShortMat {
+  const float* Y;       // rows x L
+  const double* R;      // L x L
+  float* Q;             // rows x L
+  int rows, L;
+};
+struct ShortTile {
+  int mat, m0, n0;
+};
+__global__ void __launch_bounds__(256) apply_f64_kernel(const ShortMat* mats, const ShortTile* tiles) {
+  constexpr int LD = 64 + 8;      // (as in syrk_f64_kernel)
+  __shared__ __align__(16) double As[2][16][LD];   // [k][row]
+  __shared__ __align__(16) double Bs[2][16][LD];   // [k][column]
+  const ShortTile t = tiles[blockIdx.x];
+  const ShortMat m = mats[t.mat];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
+  const int k1 = min(t.n0 + 64, m.L);
+  const int ar = tid >> 2, ak = (tid & 3) * 4;     // of Y this thread fetches four columns of a row ...
+  const int bk = tid >> 4, bc = (tid & 15) * 4;    // ... and of R^-1 as well
+  const int wr = (warp >> 1) * 16, wc = (warp & 1) * 32;
+  double acc[2][4][2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) acc[x][y][0] = acc[x][y][1] = 0.0;
+  float4 a4;
+  double2 b4[2];
+  auto fetch = [&](int k0) {   // (L is a multiple of 4: four columns are inside together)
+    a4 = t.m0 + ar < m.rows && k0 + ak < k1 ? *reinterpret_cast<const float4*>(m.Y + static_cast<long long>(t.m0 + ar) * m.L + k0 + ak)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool in_b = k0 + bk < k1 && t.n0 + bc < m.L;
+    const double2* row = reinterpret_cast<const double2*>(m.R + static_cast<long long>(k0 + bk) * m.L + t.n0 + bc);
+    b4[0] = in_b ? row[0] : make_double2(0.0, 0.0);
+    b4[1] = in_b ? row[1] : make_double2(0.0, 0.0);
+  };
+  auto put = [&](int buf) {
+    As[buf][ak][ar] = a4.x; As[buf][ak + 1][ar] = a4.y; As[buf][ak + 2][ar] = a4.z; As[buf][ak + 3][ar] = a4.w;
+    double2* b = reinterpret_cast<double2*>(&Bs[buf][bk][bc]);
+    b[0] = b4[0]; b[1] = b4[1];
+  };
+  fetch(0);
+  put(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < k1; k0 += 16, buf ^= 1) {
+    const bool more = k0 + 16 < k1;
+    if (more) fetch(k0 + 16);
+#pragma unroll
+    for (int kk = 0; kk < 16; kk += 4) {
+      double a[2], b[4];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) a[x] = As[buf][kk + fk][wr + 8 * x + fr];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) b[y] = Bs[buf][kk + fk][wc + 8 * y + fr];
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) dmma(acc[x][y], a[x], b[y]);
+    }
+    if (more) put(buf ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const int i = t.m0 + wr + 8 * x + fr, j = t.n0 + wc + 8 * y + 2 * fk;
+      if (i < m.rows && j < m.L)
+        *reinterpret_cast<float2*>(m.Q + static_cast<long long>(i) * m.L + j) = make_float2(static_cast<float>(acc[x][y][0]), static_cast<float>(acc[x][y][1]));
+    }
 }
 
 struct NewtonJob {
@@ -265,6 +355,8 @@ struct RefProduct {
   static constexpr int kSmem = TcSmem<BN, 1, NB, kStages, kEpiWarps, MT>::kTotal;
   static constexpr auto kernel = tc_gemm_kernel<BN, 1, NB, kStages, TC_EPI_STORE, kEpiWarps, MN, false, MT>;
 };
+// Matrices with fewer rows than this end with a pass in fp64 (refresh_tc_short).
+constexpr int kShortRows = 512;
 constexpr int kRefStages2 = 3;  // NA = 2, NB = 2: 64 KB per stage
 
 struct RefreshPlan {
@@ -309,6 +401,15 @@ struct RefreshPlan {
   int sm_count = 0;
   FillJob* d_fill = nullptr;   // the random start Z = Omega of every matrix
   int fill_blocks = 1;         // blocks a matrix: eight entries a thread in the largest
+  // the last exact pass over the matrices with fewer than kShortRows rows (refresh_tc_short)
+  std::vector<char> is_short;
+  int n_short = 0, short_l_max = 0, n_short_syrk = 0, n_short_tiles = 0;
+  SyrkMat* d_short_syrk_mats = nullptr;
+  SyrkTile* d_short_syrk_tiles = nullptr;
+  FactorMat* d_short_factor = nullptr;
+  ShortMat* d_short = nullptr;
+  ShortTile* d_short_tiles = nullptr;
+  ZeroJob* d_short_zero = nullptr;
   ZeroJob* d_zero_d = nullptr;   // clears every matrix's D (as 16-byte words)
 };
 
@@ -321,8 +422,8 @@ inline void refresh_plan_destroy(RefreshPlan& plan) {
 }
 
 inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<MatDesc>& mats,
-                                          const std::vector<float*>& Yf, const std::vector<float*>& Zf, int sm_count,
-                                          int ritz_columns) {
+                                          const std::vector<float*>& Yf, const std::vector<float*>& Zf,
+                                          const std::vector<float*>& Yshort, int sm_count, int ritz_columns) {
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
   if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || fn == nullptr)
@@ -468,9 +569,12 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_factor32 = take(sizeof(FactorMat) * n);
   const size_t o_factor64 = take(sizeof(FactorMat) * n);
   std::vector<SyrkTile> syrk_tiles;
-  auto slabs = [&](int slab) {
+  plan.is_short.resize(n);
+  for (int i = 0; i < n; ++i) plan.is_short[i] = plan.mats[i].M < kShortRows ? 1 : 0;
+  auto slabs = [&](int slab, bool short_only = false) {
     syrk_tiles.clear();
     for (int i = 0; i < n; ++i) {
+      if (short_only && !plan.is_short[i]) continue;
       const int nt = (plan.mats[i].L + 63) / 64, rows = plan.mats[i].M;
       const int step = rows <= 2 * kSyrkRows ? std::max(slab, (rows / 2 + 15) & ~15) : slab;
       for (int k0 = 0; k0 < rows; k0 += step)
@@ -480,6 +584,17 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   };
   slabs(kSyrkRows);
   if (static_cast<int>(syrk_tiles.size()) < kSyrkFewTiles * sm_count) slabs(kSyrkRowsFew);
+  const std::vector<SyrkTile> all_syrk_tiles = syrk_tiles;
+  slabs(kSyrkRowsFew, true);
+  const std::vector<SyrkTile> short_syrk_tiles = syrk_tiles;
+  syrk_tiles = all_syrk_tiles;
+  std::vector<ShortTile> short_tiles;
+  for (int i = 0; i < n; ++i)
+    if (plan.is_short[i])
+      for (int n0 = (plan.mats[i].L - 1) / 64 * 64; n0 >= 0; n0 -= 64)   // (the longest sums first)
+        for (int m0 = 0; m0 < plan.mats[i].M; m0 += 64) short_tiles.push_back(ShortTile{i, m0, n0});
+  plan.n_short_syrk = static_cast<int>(short_syrk_tiles.size());
+  plan.n_short_tiles = static_cast<int>(short_tiles.size());
   plan.n_syrk_tiles = static_cast<int>(syrk_tiles.size());
   const size_t o_syrk_m = take(sizeof(SyrkMat) * n);
   const size_t o_syrk_t = take(sizeof(SyrkTile) * syrk_tiles.size());
@@ -490,6 +605,12 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   const size_t o_eig_redo = take(sizeof(int) * n);
   const size_t o_fill = take(sizeof(FillJob) * n);
   const size_t o_zero_d = take(sizeof(ZeroJob) * n);
+  const size_t o_short_syrk_m = take(sizeof(SyrkMat) * n);
+  const size_t o_short_syrk_t = take(sizeof(SyrkTile) * short_syrk_tiles.size());
+  const size_t o_short_factor = take(sizeof(FactorMat) * n);
+  const size_t o_short_m = take(sizeof(ShortMat) * n);
+  const size_t o_short_t = take(sizeof(ShortTile) * short_tiles.size());
+  const size_t o_short_zero = take(sizeof(ZeroJob) * n);
   std::vector<size_t> o_eig_tri(n);
   for (int i = 0; i < n; ++i) o_eig_tri[i] = take(sizeof(double) * eig_tri_doubles(plan.mats[i].L));
   if (cudaMalloc(&plan.buf, off) != cudaSuccess) { plan.buf = nullptr; return NGALORE_ERR_ALLOC; }
@@ -501,7 +622,10 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   plan.l_max = 0;
   for (const RefreshMat& m : plan.mats) plan.l_max = m.L > plan.l_max ? m.L : plan.l_max;
   std::vector<SplitJob> sy_rest, sz_rest;
-  std::vector<SyrkMat> syrk_m(n);
+  std::vector<SyrkMat> syrk_m(n), short_syrk_m(n);
+  std::vector<FactorMat> short_factor;
+  std::vector<ShortMat> short_m(n);
+  std::vector<ZeroJob> short_zero;
   std::vector<EigMat> eig(n);
   std::vector<FactorMat> eig_factors(n);
   plan.h_maps.resize(static_cast<size_t>(RM_COUNT) * n);
@@ -524,7 +648,14 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     factor64[i] = FactorMat{nullptr, m.X64, m.C64, m.T64, m.Rhi, m.Rlo, m.L, m.ldl};
     m.Y1hi = reinterpret_cast<__nv_bfloat16*>(m.Yf);
     m.Y1lo = m.Y1hi + static_cast<size_t>(m.M) * m.ldl;
-    syrk_m[i] = SyrkMat{m.Y1hi, m.Y1lo, m.X64, m.M, m.L, m.ldl};
+    syrk_m[i] = SyrkMat{m.Y1hi, m.Y1lo, nullptr, m.X64, m.M, m.L, m.ldl};
+    short_syrk_m[i] = SyrkMat{nullptr, nullptr, m.Yf, m.X64, m.M, m.L, m.L};
+    short_m[i] = ShortMat{m.Yf, m.X64, Yshort[i], m.M, m.L};
+    if (plan.is_short[i]) {
+      short_factor.push_back(FactorMat{nullptr, m.X64, m.C64, m.T64, nullptr, nullptr, m.L, 0, m.X64});
+      short_zero.push_back(ZeroJob{reinterpret_cast<float4*>(m.X64), static_cast<long long>(m.L) * m.L * 8 / 16});
+      plan.short_l_max = std::max(plan.short_l_max, m.L);
+    }
     if (std::find(plan.atomic_mats[RG_Y_FROM_Z].begin(), plan.atomic_mats[RG_Y_FROM_Z].end(), i) != plan.atomic_mats[RG_Y_FROM_Z].end())
       sy_rest.push_back(SplitJob{m.Yf, m.Yhi, m.Ylo, static_cast<long long>(m.M) * m.L, m.L, m.ldl});
     if (std::find(plan.atomic_mats[RG_Z_FROM_Y].begin(), plan.atomic_mats[RG_Z_FROM_Y].end(), i) != plan.atomic_mats[RG_Z_FROM_Y].end())
@@ -627,6 +758,24 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_eig, eig.data(), sizeof(EigMat) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(plan.d_eig_factor, eig_factors.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
+
+  plan.n_short = static_cast<int>(short_factor.size());
+  if (plan.n_short > 0) {
+    std::stable_sort(short_factor.begin(), short_factor.end(), wider);
+    bool ok = true;
+    auto put = [&](auto*& dst, size_t at, const auto& src) {
+      using T = typename std::remove_reference_t<decltype(src)>::value_type;
+      dst = reinterpret_cast<T*>(plan.buf + at);
+      ok = ok && cudaMemcpy(dst, src.data(), sizeof(T) * src.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    };
+    put(plan.d_short_syrk_mats, o_short_syrk_m, short_syrk_m);
+    put(plan.d_short_syrk_tiles, o_short_syrk_t, short_syrk_tiles);
+    put(plan.d_short_factor, o_short_factor, short_factor);
+    put(plan.d_short, o_short_m, short_m);
+    put(plan.d_short_tiles, o_short_t, short_tiles);
+    put(plan.d_short_zero, o_short_zero, short_zero);
+    if (!ok) return NGALORE_ERR_CUDA;
+  }
 
   // ---- tables of buffers to clear
   {
@@ -775,7 +924,7 @@ inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStrea
 inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches) {
   zero_jobs_kernel<<<dim3(32, plan.n_zero[RG_COUNT]), 256, 0, stream>>>(plan.d_zero[RG_COUNT]);
   *launches += 1;
-  syrk_f64_kernel<<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
+  syrk_f64_kernel<false><<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
   *launches += 1;
   if (tri_factor_launch(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_10, d_ctrl, stream, launches);
@@ -793,7 +942,23 @@ inline ngalore_status refresh_tc_refine(RefreshPlan& plan, int set, Ctrl* d_ctrl
   return refresh_tc_gemm(plan, RG_APPLY_Y, set == 0 ? RP_APPLY_01 : RP_APPLY_10, d_ctrl, stream, launches);
 }
 
-// Whole-set refresh; leaves the basis in Yf.
+// The matrices with few rows: the rounding of the last product's operands to two bf16 parts does not average out over their
+// rows, so their bases get one more Cholesky QR, all of it in fp64, from Yf to the buffer given for it when the plan was made.  Four
+// launches for all of them; matrix by matrix, on the vector units and with two launches for every 32 columns of a factor, it was most of
+// a refresh: 42 matrices of 328 rows at r' = 328 43.2 ms, now 5.8, of them 0.09 the Gram matrices, 0.21 the factors and 0.11 the
+// product; 36 of 200 rows at r' = 196 11.3 -> 2.6; 49 of 328 rows at r' = 44 8.4 -> 1.3.
+inline ngalore_status refresh_tc_short(RefreshPlan& plan, cudaStream_t stream, int64_t* launches) {
+  if (plan.n_short == 0) return NGALORE_OK;
+  zero_jobs_kernel<<<dim3(8, plan.n_short), 256, 0, stream>>>(plan.d_short_zero);
+  syrk_f64_kernel<true><<<plan.n_short_syrk, 256, 0, stream>>>(plan.d_short_syrk_mats, plan.d_short_syrk_tiles);
+  *launches += 2;
+  if (tri_factor_launch(plan.d_short_factor, plan.n_short, plan.short_l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  apply_f64_kernel<<<plan.n_short_tiles, 256, 0, stream>>>(plan.d_short, plan.d_short_tiles);
+  *launches += 1;
+  return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
+}
+
+// Whole-set refresh; leaves the basis in Yf, of the matrices with few rows (is_short) in the buffer given for it.
 inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G, int q, unsigned long long seed,
                                      unsigned long long stream_base, Ctrl* d_ctrl, cudaStream_t stream,
                                      int64_t* launches) {
@@ -850,6 +1015,7 @@ inline ngalore_status refresh_tc_run(RefreshPlan& plan, const uint16_t* const* G
   // Q orthonormal to about 1e-6 and V orthogonal: so is their product, once its columns are scaled back to unit norm
   // (with the working copies, see finish_refresh; their norms go to D)
   if ((rc = refresh_tc_gemm(plan, RG_APPLY_Y, RP_APPLY_0F, d_ctrl, stream, launches))) return rc;
+  if ((rc = refresh_tc_short(plan, stream, launches))) return rc;
   zero_jobs_kernel<<<dim3(1, plan.n), 256, 0, stream>>>(plan.d_zero_d);
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
