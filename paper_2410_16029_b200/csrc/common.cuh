@@ -40,8 +40,8 @@ struct MatDesc {
   double* gpart;              // per-tile partial Gram rows: ntiles x s
   int* status;                // sticky ngalore_status word
   int* step_bad;              // 1 when this step must leave W, m, v untouched
-  int* gram_done;             // fused kernel: count of finished Gram tiles of this step
-  int* w_ready;               // fused kernel: set to the step epoch once wsol is valid
+  ulonglong2* grow;           // fused kernel: the same rows as tagged words (kernels_stream.cuh)
+  unsigned long long* wpub;   // fused kernel: kMaxHistory tagged weights, valid once they carry this step's tag
   int tile0, ntiles;          // range of streaming tiles owned by this matrix
   int te;                     // elements of one streaming tile of this matrix (multiple of 1024)
 };

@@ -3,18 +3,24 @@
 //
 // Structure: one CTA per SM; a producer warp streams the history (and m, v) through a ring of
 // shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier), eight to sixteen consumer
-// warps compute from shared memory, a finishing warp turns the partial sums of a Gram tile into its partial row
-// and, after a matrix's last one, solves its s x s system while the consumers go on with the next item.  The producer runs ahead of the consumers across tile and
+// warps compute from shared memory, and a finishing warp turns the partial sums of a Gram tile into its partial row,
+// solves the s x s system of the matrices whose last Gram tile the CTA has and fetches the weights of its
+// combination items, each ahead of the consumers.  The producer runs ahead of them across tile and
 // matrix boundaries, so the SM always has several stages of loads in flight.
 //
 // Work items (Gram tiles and combination tiles of all matrices) are fetched in order from a global
-// counter by the producer.  Gram items never wait; the finishing warp of the CTA that has a matrix's last Gram
-// tile solves its s x s system and publishes the weights; the consumers of a combination item wait
-// (bounded) for that flag.  Every item a combination item depends on sits earlier in the list and
+// counter by the producer.  The consumers of a Gram item wait for nothing but its data; the finishing warp of the CTA that has a
+// matrix's last Gram tile waits (bounded) for the partial rows of the others and publishes the weights, that of a
+// CTA with a combination item waits (bounded) for those.  Every item that is waited for sits earlier in the list and
 // has been fetched by a CTA that consumes its items in order, so the kernel cannot deadlock.
 // All Gram items precede all combination items, so the wait is short except at the very end of the Gram items.
+//
+// No consumer reads anything but shared memory before its results go out: where one of them fetched the weights itself (flag, fence,
+// weights, descriptor: 2 to 3 us an item during which nothing left the full ring), a CTA of the 60M shapes, s = 8, spent 12 to 20
+// of 72 us on it, of the encoder shapes at r = 8 13 of 25.
 #pragma once
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/ngalore.h"
@@ -24,11 +30,19 @@
 
 namespace ngalore {
 
-struct FusedItem {
+// All that the producer needs of an item, so that one trip to memory fetches it.
+struct __align__(16) FusedItem {
   int mat;
-  int local;
-  int kind;  // 0 = Gram tile, 1 = combination tile
-  int pad;
+  int kind;        // 0 = Gram tile, 1 = combination tile
+  int solve;       // a Gram tile: whether it is its matrix's last one
+  int count;       // elements
+  long long e0;    // first element
+  long long rn;    // elements of a history slot
+  const void* hist;      // the ring: fp32, or bf16 where the state keeps its history so
+  const float* current;  // bf16 history: the fp32 gradient of this step
+  const void *m, *v;     // moments, fp32 or bf16
+  ulonglong2* rows;      // where the partial rows of a Gram tile go
+  long long pad;
 };
 
 struct FusedPlan {
@@ -42,9 +56,25 @@ struct FusedPlan {
 constexpr long long kSpinLimit = 4000000;  // polls of ~100 ns each before a flag wait is abandoned
 
 struct StageMeta {
-  int mat, kind, local, first, last, count;
-  int cur, c;  // ring position and number of valid slots of this step (the same for every stage of a launch)
+  int kind, last, count, pad;
   long long e0;
+  ulonglong2* rows;
+};
+
+// What the finishing warp is told to do, in the order of the CTA's items: solve for a matrix, or fetch the weights of a combination item
+// (kind < 0: there are no more).
+struct WeightsJob {
+  int mat, kind;
+};
+
+// ... and what it leaves for the consumers of a combination item.
+struct __align__(16) ItemWeights {
+  float w[kMaxHistory];
+  float *m, *v, *cur;
+  __half* u;
+  uint16_t *m16, *v16, *h16;
+  int index;
+  int ok, bad;     // ok 0: the weights never came; bad 1: the step is flagged for the matrix
 };
 
 // Stage layout.  fp32 history: SMAX slots of CE floats, then m, then v.  bf16 history (HIST16): SMAX slots of CE
@@ -75,7 +105,11 @@ struct FusedCfg {
   static constexpr int kStages = HIST16 ? (SMAX <= 16 ? 3 : 5) : (SMAX <= 8 ? 5 : 3);
   static constexpr int kBase = kStages * kStageBytes;
   static constexpr int kFullOff = kBase, kEmptyOff = kBase + 64, kMetaOff = kBase + 128, kFlagOff = kBase + 512;
-  static constexpr int kMeetOff = kBase + 640, kRedBarOff = kBase + 768, kRedMetaOff = kBase + 800, kRedOff = kBase + 896;
+  static constexpr int kJobs = 4;                               // jobs under way to the finishing warp
+  static constexpr int kJobBarOff = kBase + 528, kJobOff = kJobBarOff + 16 * kJobs, kWBarOff = kJobOff + 8 * kJobs;
+  static constexpr int kRedBarOff = kWBarOff + 32, kRedRowsOff = kRedBarOff + 32, kWeightsOff = kBase + 768;
+  static constexpr int kRedOff = kWeightsOff + 2 * static_cast<int>(sizeof(ItemWeights));
+  static_assert(kRedRowsOff + 16 <= kWeightsOff && kRedOff % 8 == 0, "shared memory regions overlap");
   static constexpr int kRows = HIST16 ? 2 : 1;                  // Gram rows per tile
   static constexpr int kRedDoubles = (kConsumers / 32) * SMAX;  // one Gram row per consumer warp
   static constexpr int kTotal = kRedOff + 2 * kRows * kRedDoubles * 8;   // (two tiles in flight to the finishing warp)
@@ -120,11 +154,6 @@ __device__ __forceinline__ double warp_sums(double (&v)[S]) {
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
-
-// What the finishing warp needs to know about a finished Gram tile (mat < 0: the CTA has no more).
-struct RedMeta {
-  int mat, local, cur, c;
-};
 
 template <int THREADS>
 __device__ __forceinline__ void consumer_sync() {
@@ -173,11 +202,15 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   uint64_t* empty_bar = reinterpret_cast<uint64_t*>(fs_smem + C::kEmptyOff);
   StageMeta* meta = reinterpret_cast<StageMeta*>(fs_smem + C::kMetaOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(fs_smem + C::kFlagOff);
-  volatile int* s_flag = abort_flag + 1;                                        // [2] 1: the weights of a combination item came
-  uint64_t* meet_bar = reinterpret_cast<uint64_t*>(fs_smem + C::kMeetOff);      // all consumer warps
+  uint64_t* job_full = reinterpret_cast<uint64_t*>(fs_smem + C::kJobBarOff);    // [kJobs] the producer has left a job
+  uint64_t* job_empty = job_full + C::kJobs;                                    // [kJobs] the finishing warp has taken it
+  WeightsJob* jobs = reinterpret_cast<WeightsJob*>(fs_smem + C::kJobOff);       // [kJobs]
+  uint64_t* w_full = reinterpret_cast<uint64_t*>(fs_smem + C::kWBarOff);        // [2] the weights of a combination item are there
+  uint64_t* w_empty = w_full + 2;                                               // [2] all consumer warps are through with them
+  ItemWeights* weights = reinterpret_cast<ItemWeights*>(fs_smem + C::kWeightsOff);  // [2]
   uint64_t* red_full = reinterpret_cast<uint64_t*>(fs_smem + C::kRedBarOff);   // [2] all consumer warps have left their sums
   uint64_t* red_empty = red_full + 2;                                           // [2] the finishing warp has taken them
-  RedMeta* red_meta = reinterpret_cast<RedMeta*>(fs_smem + C::kRedMetaOff);     // [2]
+  ulonglong2** red_rows = reinterpret_cast<ulonglong2**>(fs_smem + C::kRedRowsOff); // [2] where a tile's rows go (null: there are no more)
   double* red = reinterpret_cast<double*>(fs_smem + C::kRedOff);                // [2][rows][warps][SMAX]
 
   const int tid = threadIdx.x;
@@ -187,143 +220,209 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       mbar_init(empty_bar + s, kConsumerThreads / 32);
     }
     for (int b = 0; b < 2; ++b) { mbar_init(red_full + b, kWarps); mbar_init(red_empty + b, 1); }
-    mbar_init(meet_bar, kWarps);
+    for (int b = 0; b < 2; ++b) { mbar_init(w_full + b, 1); mbar_init(w_empty + b, kWarps); }
+    for (int b = 0; b < C::kJobs; ++b) { mbar_init(job_full + b, 1); mbar_init(job_empty + b, 1); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
-  // (The tables are laid out for good: the item that this CTA will probably claim first, and its matrix, come to the SM ahead of
+  // (The tables are laid out for good: the item that this CTA will probably claim first comes to the SM ahead of
   // the wait for the kernel before.  It is claimed like the others all the same: an item that belonged to a CTA which another kernel
   // keeps from starting could be waited for by that kernel's neighbours for good.)
   if (tid == kConsumerThreads && static_cast<int>(blockIdx.x) < n_items) {
-    const MatDesc& d0 = mats[items[blockIdx.x].mat];
-    asm volatile("" ::"l"(d0.H), "l"(d0.m), "r"(d0.te), "r"(mats[0].s));
+    const FusedItem& i0 = items[blockIdx.x];
+    asm volatile("" ::"r"(i0.mat), "l"(i0.hist), "l"(i0.rows), "r"(mats[0].s));
   }
   pdl_begin();
-  const int tag = ctrl->epoch + 1;
+  int it = 0;      // the producer's item: claimed ahead of everything else
+  if (tid == kConsumerThreads) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
+  const unsigned int tag = static_cast<unsigned int>(ctrl->epoch + 1);
+  const int s_all = mats[0].s;                       // (the same for every matrix, and so are ring position and count)
+  const int c = ring_count(ctrl, s_all), cur = ring_cur(ctrl, s_all);
+  const int prev = HIST16 && c >= 2 ? (cur == 0 ? s_all : cur) - 1 : -1;   // the slot whose row is worked out again
 
   if (tid >= kConsumerThreads + 32) {
     // ------------------------------------------------------------------ finishing warp
+    // Two kinds of work: the partial row of every Gram tile that the consumers leave, and the producer's jobs.  Whatever it
+    // waits for, it looks after the rows meanwhile: another CTA may be waiting for them, or the consumers for their place.
     const int lane = tid & 31;
     const double lambda = hyper->lambda;
-    for (unsigned int n = 0;; ++n) {
-      const int buf = n & 1;
-      if (!mbar_wait_warp(red_full + buf, (n >> 1) & 1u, abort_flag)) break;
-      const RedMeta mt = red_meta[buf];
+    const int withheld = ctrl->debug_withhold - 1;
+    const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
+    bool jobs_open = true, rows_open = true;
+    unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, Gram tiles and combination items so far
+    auto look_after_rows = [&]() {
+      const int buf = tiles & 1;
+      if (!rows_open || !__all_sync(0xffffffffu, mbar_test(red_full + buf, (tiles >> 1) & 1u))) return;
+      ulonglong2* const rows = red_rows[buf];   // [rows][s]: row of `cur` and (HIST16) of `prev`
       double part[C::kRows];
 #pragma unroll
       for (int r = 0; r < C::kRows; ++r) {
-        part[r] = 0.0;
-        if (lane < SMAX) {
-          const double* src = red + (buf * C::kRows + r) * C::kRedDoubles + lane;
-          double t0 = 0.0, t1 = 0.0;
+        const double* src = red + (buf * C::kRows + r) * C::kRedDoubles + min(lane, SMAX - 1);
+        double t0 = 0.0, t1 = 0.0;
 #pragma unroll
-          for (int w = 0; w < kWarps; w += 2) { t0 += src[w * SMAX]; t1 += src[(w + 1) * SMAX]; }
-          part[r] = t0 + t1;
-        }
+        for (int w = 0; w < kWarps; w += 2) { t0 += src[w * SMAX]; t1 += src[(w + 1) * SMAX]; }
+        part[r] = t0 + t1;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(red_empty + buf);
-      if (mt.mat < 0) break;
-      const MatDesc& d = mats[mt.mat];
-      const int cur = mt.cur, c = mt.c;
-      // per-tile partial rows: [tile][s] (fp32 history) or [tile][2][s] (HIST16: row of `cur`, row of `prev`)
-      if (d.ntiles > 1) {
-        int last = 0;
-        if (lane < d.s) {
+      ++tiles;
+      if (rows == nullptr) {
+        rows_open = false;
+      } else if (lane < s_all) {
 #pragma unroll
-          for (int r = 0; r < C::kRows; ++r) __stcg(d.gpart + (static_cast<long long>(mt.local) * C::kRows + r) * d.s + lane, part[r]);
-          __threadfence();
-        }
-        __syncwarp();
-        if (lane == 0) last = atomicAdd(d.gram_done, 1) == d.ntiles - 1 ? 1 : 0;
-        if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-        __threadfence();
+        for (int r = 0; r < C::kRows; ++r) st_tagged(rows + r * s_all + lane, part[r], tag);
       }
-      // the matrix's last tile
-      if (d.ntiles > 1) {
-#pragma unroll
-        for (int r = 0; r < C::kRows; ++r) part[r] = gram_row_sum<SMAX>(d, lane, c, C::kRows, r);
-      }
-      const bool two = HIST16 && c >= 2;
-      solve_matrix<SMAX>(d, cur, c, lambda, lane < c ? part[0] : 0.0, two, two ? (cur == 0 ? d.s : cur) - 1 : 0, part[C::kRows - 1]);
-      __threadfence();
       __syncwarp();
-      if (lane == 0) {
-        *d.gram_done = 0;
-        __threadfence();
-        if (ctrl->debug_withhold != mt.mat + 1) atomicExch(d.w_ready, tag);
+    };
+    // mbar_wait of the whole warp, which looks after the rows between two looks
+    auto wait_for = [&](uint64_t* bar, uint32_t parity) {
+      unsigned long long t0 = 0;
+      for (unsigned int it = 0; !__all_sync(0xffffffffu, mbar_test(bar, parity)); ++it) {
+        look_after_rows();
+        if ((it & 63u) == 63u) {
+          const unsigned long long now = global_timer_ns();
+          if (t0 == 0) t0 = now;
+          if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > kTcWaitLimitNs)) { *abort_flag = 1; return false; }
+        }
       }
+      return true;
+    };
+    while (jobs_open) {
+      const int at = taken % C::kJobs;
+      if (!wait_for(job_full + at, (taken / C::kJobs) & 1u)) break;
+      const WeightsJob job = jobs[at];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(job_empty + at);
+      ++taken;
+      if (job.kind < 0) { jobs_open = false; break; }
+      const MatDesc& d = mats[job.mat];
+      if (job.kind == 0) {
+        GramSolve<SMAX> solve;
+        solve.prepare(d, cur, prev, c, lambda, lane);
+        double row = 0.0, rowp = 0.0;
+        if (!tagged_row_sum<SMAX>(d, lane, c, C::kRows, 0, tag, kSpinLimit, abort_flag, row, look_after_rows)) continue;   // (nobody gets weights, and says so)
+        if (HIST16 && prev >= 0 && !tagged_row_sum<SMAX>(d, lane, c, C::kRows, C::kRows - 1, tag, kSpinLimit, abort_flag, rowp, look_after_rows)) continue;
+        solve.finish(d, cur, prev, c, lambda, lane, row, rowp, tag, withheld == job.mat);
+        continue;
+      }
+      float w;
+      int ok = 1, bad;
+      if (s_all > 0) {
+        unsigned long long word;
+        for (long long spins = 0;; ++spins) {
+          word = ld_relaxed(d.wpub + lane);
+          if (__all_sync(0xffffffffu, static_cast<unsigned int>(word >> 32) >> 1 == (tag & 0x7fffffffu))) break;
+          if (spins >= limit) { ok = 0; break; }
+          look_after_rows();
+          if (spins > 16) __nanosleep(100);
+        }
+        w = __uint_as_float(static_cast<unsigned int>(word));
+        bad = static_cast<int>(word >> 32) & 1;
+        if (!ok && lane == 0) {
+          // The weights never came: this matrix takes no update in this step (the back-projection skips it)
+          // and says why.  Tiles of it that other CTAs did combine have advanced their part of m and v.
+          atomicExch(&ctrl->timeout_flag, 1);
+          atomicExch(d.step_bad, 1);
+          atomicCAS(d.status, 0, 8 /* NGALORE_ERR_TIMEOUT */);
+        }
+      } else {
+        w = __ldcg(d.wsol + lane);
+        bad = __ldcg(d.step_bad) != 0 ? 1 : 0;
+      }
+      const int slot = fetched & 1;
+      if (!wait_for(w_empty + slot, ((fetched >> 1) & 1u) ^ 1u)) break;
+      ++fetched;
+      ItemWeights& o = weights[slot];
+      o.w[lane] = w;
+      if (lane == 0) {
+        o.m = d.m; o.v = d.v; o.cur = current_gradient(d, cur); o.u = d.u16; o.m16 = d.m16; o.v16 = d.v16;
+        o.h16 = HIST16 ? d.H16 + static_cast<long long>(cur) * d.rn : nullptr;
+        o.index = d.index; o.ok = ok; o.bad = bad;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(w_full + slot);
+    }
+    // (the consumers say so when they have left the last Gram tile's sums)
+    while (rows_open) {
+      if (!wait_for(red_full + (tiles & 1), (tiles >> 1) & 1u)) break;
+      look_after_rows();
     }
   } else if (tid >= kConsumerThreads) {
     // ------------------------------------------------------------------ producer warp
     // Lane 0 claims items and arms the barriers; every lane issues the bulk copy of "its" slot (lane j copies
     // history slot j, the next two lanes m and v), so a stage's copies are issued in parallel.  The next item is
-    // claimed and its descriptor fetched while the stages of the current one go out, one round trip to memory per
-    // stage: three round trips in a row between two items cost more than streaming 4096 elements of eight slots.
+    // claimed and fetched while the stages of the current one go out, one round trip to memory per
+    // stage: round trips in a row between two items cost as much as streaming 4096 elements of eight slots.
     const int lane = tid & 31;
-    const int s_all = mats[0].s;                       // (the same for every matrix, and so are ring position and count)
-    const int c = ring_count(ctrl, s_all), cur_slot = ring_cur(ctrl, s_all);
-    struct Source {
-      int mat, kind, local;
-      long long e0, e1;
-      const unsigned char* src[2];                     // this lane's copies: number lane, and lane + 32 where there is one
-    };
-    // copy number k of an item: history slot k, then m and v; its place in a stage and bytes per element
+    // copy number k of an item: history slot k, then m and v; its place in a stage, bytes per element and source
     auto place = [&](int k) {
-      if (k < c) return !HIST16 ? k * CE * 4 : (k == cur_slot ? C::kCurOff : k * CE * 2);
+      if (k < c) return !HIST16 ? k * CE * 4 : (k == cur ? C::kCurOff : k * CE * 2);
       return k == c ? C::kMOff : C::kVOff;
     };
-    auto width = [&](int k) { return k < c ? (HIST16 && k != cur_slot ? 2 : 4) : (MOM16 ? 2 : 4); };
-    auto describe = [&](const FusedItem& item, Source& o) {
-      const MatDesc& d = mats[item.mat];
-      o.mat = item.mat; o.kind = item.kind; o.local = item.local;
-      o.e0 = static_cast<long long>(item.local) * d.te;
-      o.e1 = (o.e0 + d.te < d.rn) ? o.e0 + d.te : d.rn;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int k = lane + 32 * q;
-        const void* base = nullptr;
-        if (k < c) base = !HIST16 ? static_cast<const void*>(d.H + static_cast<long long>(k) * d.rn)
-                                  : (k == cur_slot ? static_cast<const void*>(d.H) : static_cast<const void*>(d.H16 + static_cast<long long>(k) * d.rn));
-        else if (k == c) base = MOM16 ? static_cast<const void*>(d.m16) : static_cast<const void*>(d.m);
-        else if (k == c + 1) base = MOM16 ? static_cast<const void*>(d.v16) : static_cast<const void*>(d.v);
-        o.src[q] = static_cast<const unsigned char*>(base);
-      }
+    auto width = [&](int k) { return k < c ? (HIST16 && k != cur ? 2 : 4) : (MOM16 ? 2 : 4); };
+    auto source = [&](const FusedItem& o, int k) {
+      const void* base = k == c ? o.m : o.v;
+      if (k < c) base = HIST16 && k == cur ? static_cast<const void*>(o.current) : static_cast<const unsigned char*>(o.hist) + k * o.rn * width(k);
+      return static_cast<const unsigned char*>(base);
     };
+    // Tells the finishing warp what this CTA needs of it for an item.  block: wait until there is room (without it, false where
+    // there is none).
+    unsigned int told = 0;
+    bool ok = true;
+    auto tell = [&](int mat, int kind, bool block) {
+      const int at = told % C::kJobs;
+      const uint32_t parity = ((told / C::kJobs) & 1u) ^ 1u;
+      int good = 1;
+      if (lane == 0) {
+        good = block ? (mbar_wait(job_empty + at, parity, abort_flag) ? 1 : 0) : (mbar_test(job_empty + at, parity) ? 1 : 0);
+        if (good) {
+          jobs[at] = WeightsJob{mat, kind};
+          mbar_arrive(job_full + at);
+        }
+      }
+      good = __shfl_sync(0xffffffffu, good, 0);
+      if (good) ++told;
+      else if (block) ok = false;
+      return good != 0;
+    };
+    auto wanted = [](const FusedItem& o) { return o.kind == 1 || o.solve != 0; };
     int stage = 0;
     uint32_t phase = 0;
-    int it = 0;
-    FusedItem item{};
-    Source now{}, next{};
-    if (lane == 0) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
+    FusedItem now{}, next{};
+    bool told_ahead = false;   // the finishing warp knows of the next item
     it = __shfl_sync(0xffffffffu, it, 0);
-    if (it < n_items) { item = items[it]; describe(item, now); }
+    if (it < n_items) now = items[it];
     while (true) {
       if (it >= n_items) {
+        tell(0, -1, true);
         if (lane == 0 && mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag)) {
           meta[stage].kind = -1;
           mbar_arrive(full_bar + stage);
         }
         break;
       }
+      if (wanted(now) && !told_ahead) tell(now.mat, now.kind, true);
+      if (!ok) break;
+      told_ahead = false;
       const int ncopies = c + (now.kind == 1 ? 2 : 0);
-      int step = 0;   // how far the next item is known: 0 claimed, 1 fetched, 2 described
+      const unsigned char* src[2] = {source(now, lane), source(now, lane + 32)};   // this lane's copies
+      int step = 0;   // how far the next item is known: 0 claimed, 1 fetched, 2 on: told to the finishing warp, where that has room
       auto look_ahead = [&]() {
         if (step == 0) {
           if (lane == 0) it = static_cast<int>(atomicAdd(&ctrl->work_counter, 1u));
         } else if (step == 1) {
           it = __shfl_sync(0xffffffffu, it, 0);
-          if (it < n_items) item = items[it];
-        } else if (step == 2) {
-          if (it < n_items) describe(item, next);
+          if (it < n_items) next = items[it];
+        } else if (!told_ahead && it < n_items && wanted(next)) {
+          told_ahead = tell(next.mat, next.kind, false);
         }
         ++step;
       };
-      bool ok = true;
-      for (long long e = now.e0; e < now.e1; e += CE) {
-        const int cnt = (now.e1 - e < CE) ? static_cast<int>(now.e1 - e) : CE;
+      const long long e1 = now.e0 + now.count;
+      for (long long e = now.e0; e < e1; e += CE) {
+        const int cnt = (e1 - e < CE) ? static_cast<int>(e1 - e) : CE;
         int good = 1;
         if (lane == 0) good = mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag) ? 1 : 0;
         good = __shfl_sync(0xffffffffu, good, 0);
@@ -331,11 +430,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         unsigned char* sb = fs_smem + stage * C::kStageBytes;
         const uint32_t bytes = static_cast<uint32_t>(cnt) * 4u;
         if (lane == 0) {
-          StageMeta mt;
-          mt.mat = now.mat; mt.kind = now.kind; mt.local = now.local;
-          mt.first = (e == now.e0) ? 1 : 0; mt.last = (e + CE >= now.e1) ? 1 : 0; mt.count = cnt; mt.e0 = e;
-          mt.cur = cur_slot; mt.c = c;
-          meta[stage] = mt;
+          meta[stage] = StageMeta{now.kind, e + CE >= e1 ? 1 : 0, cnt, 0, e, now.rows};
           const uint32_t hist_bytes = HIST16 ? bytes * static_cast<uint32_t>(c) - (bytes / 2) * static_cast<uint32_t>(c - 1)
                                              : bytes * static_cast<uint32_t>(c);
           const uint32_t mom_bytes = now.kind == 1 ? (MOM16 ? bytes : 2u * bytes) : 0u;
@@ -347,14 +442,14 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           const int k = lane + 32 * q;
           if (k < ncopies) {
             const int w = width(k);
-            bulk_load(sb + place(k), now.src[q] + e * w, static_cast<uint32_t>(cnt * w), full_bar + stage);
+            bulk_load(sb + place(k), src[q] + e * w, static_cast<uint32_t>(cnt * w), full_bar + stage);
           }
         }
         if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         look_ahead();
       }
       if (!ok) break;
-      while (step < 3) look_ahead();
+      while (step < 2) look_ahead();
       now = next;
     }
   } else {
@@ -367,20 +462,19 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     int stage = 0;
     uint32_t phase = 0;
     unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
-    unsigned int combined = 0;     // combination items whose weights have been waited for
-    // Tell the finishing warp that the CTA has no more of them (every Gram item is ahead of every combination item).  That
-    // is done as soon as it is known, so that none of its waits spans more than a Gram tile: a wait is given up after a
-    // time, and the combination items of a CTA may take longer than that without anything being wrong.
+    unsigned int combined = 0;     // combination items whose weights have been taken
+    const unsigned int it_step = static_cast<unsigned int>(ctrl->k);
+    // Tells the finishing warp that the CTA has no more Gram tiles (all of them are ahead of the combination items), as soon as that is
+    // known: at the end of the kernel it would be the last thing everybody waits for.
     bool gram_open = true;
     auto close_gram = [&]() {
-      if (tid == 0) red_meta[tiles_done & 1].mat = -1;
+      if (tid == 0) red_rows[tiles_done & 1] = nullptr;
       __syncwarp();
       if (lane == 0) mbar_arrive(red_full + (tiles_done & 1));
       gram_open = false;
     };
     if (HIST16) {
       // the current slot's place in a stage stays zero for the whole launch: its gradient takes part in fp32 instead
-      const int cur = ring_cur(ctrl, mats[0].s);
       for (int x = 0; x < C::kStages; ++x)
         for (int i = tid; i < CE / 2; i += kConsumerThreads)
           reinterpret_cast<uint32_t*>(fs_smem + x * C::kStageBytes + cur * CE * 2)[i] = 0u;
@@ -430,7 +524,6 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         if (gram_open && mbar_wait_warp(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u, abort_flag)) close_gram();
         break;
       }
-      const int cur = mt.cur, c = mt.c;
       bool alive = true;
       if (mt.kind == 0) {
         // ---- Gram tile
@@ -480,13 +573,13 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           uint64_t axx = 0ull;
 #pragma unroll
           for (int j = 0; j < SMAX; ++j) acc[j] = acc2[j] = 0ull;
-          const int prev = c >= 2 ? (cur == 0 ? mats[mt.mat].s : cur) - 1 : cur;
+          const int old = prev >= 0 ? prev : cur;
           while (true) {
             if (idx < mt.count) {
               float x[VEC];
               uint64_t xx[VEC / 2], xp[VEC / 2];
               load_current(x);
-              load16(prev, xp);            // (a single gradient: the zeros of its own place)
+              load16(old, xp);             // (a single gradient: the zeros of its own place)
 #pragma unroll
               for (int q = 0; q < VEC / 2; ++q) {
                 xx[q] = pack_pair(x[2 * q], x[2 * q + 1]);
@@ -534,55 +627,30 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           }
         }
         ++tiles_done;
-        if (tid == 0) red_meta[buf] = RedMeta{mt.mat, mt.local, cur, c};
+        if (tid == 0) red_rows[buf] = mt.rows;
         __syncwarp();
         if (lane == 0) mbar_arrive(red_full + buf);
       } else {
         // ---- combination tile
         // (where the finishing warp still has two tiles to take, the next item will do)
         if (gram_open && __all_sync(0xffffffffu, mbar_test(red_empty + (tiles_done & 1), ((tiles_done >> 1) & 1u) ^ 1u))) close_gram();
-        const MatDesc& d = mats[mt.mat];
-        bool item_ok = true;
-        if (d.s > 0) {
-          // One thread waits for the weights; the others meet it at a barrier that they leave, like every other wait, when
-          // one of the CTA's warps has given up.  (A bar.sync would wait for good for a warp that is gone.)  What it found
-          // goes through one of two places in turn: nobody is more than one item ahead.
-          if (tid == 0) {
-            const volatile int* flag = d.w_ready;
-            const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
-            long long spins = 0;
-            int ok = 1;
-            while (*flag != tag) {
-              if (++spins > limit) { ok = 0; break; }
-              __nanosleep(100);
-            }
-            if (!ok) {
-              // The weights never came: this matrix takes no update in this step (the back-projection skips it)
-              // and says why.  Tiles of it that other CTAs did combine have advanced their part of m and v.
-              atomicExch(&ctrl->timeout_flag, 1);
-              atomicExch(d.step_bad, 1);
-              atomicCAS(d.status, 0, 8 /* NGALORE_ERR_TIMEOUT */);
-            }
-            s_flag[combined & 1] = ok;
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(meet_bar);
-          if (!mbar_wait_warp(meet_bar, combined & 1, abort_flag)) break;
-          item_ok = s_flag[combined & 1] != 0;
-          ++combined;
-          __threadfence();
-        }
-        const float my_w = __ldcg(d.wsol + lane);
-        const bool item_bad = __ldcg(d.step_bad) != 0;
-        float *const it_m = d.m, *const it_v = d.v, *const it_cur = current_gradient(d, cur);
-        __half* const it_u = d.u16;
-        uint16_t *const it_m16 = d.m16, *const it_v16 = d.v16;
-        uint16_t* const it_h16 = HIST16 ? d.H16 + static_cast<long long>(cur) * d.rn : nullptr;
-        const unsigned int it_mat = static_cast<unsigned int>(d.index), it_step = static_cast<unsigned int>(ctrl->k);
+        const ItemWeights& iw = weights[combined & 1];
+        if (!mbar_wait_warp(w_full + (combined & 1), (combined >> 1) & 1u, abort_flag)) break;
+        const bool item_ok = iw.ok != 0, item_bad = iw.bad != 0;
+        float *const it_m = iw.m, *const it_v = iw.v, *const it_cur = iw.cur;
+        __half* const it_u = iw.u;
+        uint16_t *const it_m16 = iw.m16, *const it_v16 = iw.v16, *const it_h16 = iw.h16;
+        const unsigned int it_mat = static_cast<unsigned int>(iw.index);
         float w[SMAX];
 #pragma unroll
-        for (int j = 0; j < SMAX; ++j) w[j] = __shfl_sync(0xffffffffu, my_w, j);
-        const float wc = HIST16 ? __shfl_sync(0xffffffffu, my_w, cur) : 0.f;
+        for (int j = 0; j < SMAX; j += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(iw.w + j);
+          w[j] = x.x; w[j + 1] = x.y; w[j + 2] = x.z; w[j + 3] = x.w;
+        }
+        const float wc = HIST16 ? iw.w[cur] : 0.f;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(w_empty + (combined & 1));
+        ++combined;
         while (true) {
           if (item_ok && idx < mt.count) {
             const long long e = mt.e0 + idx;
@@ -709,13 +777,29 @@ inline ngalore_status fused_plan_create(FusedPlan& plan, const std::vector<MatDe
   // shapes the phase went from 4.85 ms to 4.2 ms, on the 130M shapes from 0.51 ms to 0.35 ms.
   std::vector<FusedItem> items;
   const int n = static_cast<int>(mats.size());
+  plan.hist16 = !mats.empty() && mats[0].H16 != nullptr;
+  plan.mom16 = !mats.empty() && mats[0].m16 != nullptr;
+  auto add = [&](int i, int t, int kind) {
+    const MatDesc& d = mats[i];
+    FusedItem o{};
+    o.mat = i; o.kind = kind; o.solve = kind == 0 && t == d.ntiles - 1 ? 1 : 0;
+    o.e0 = static_cast<long long>(t) * d.te;
+    o.count = static_cast<int>(std::min<long long>(d.te, d.rn - o.e0));
+    o.rn = d.rn;
+    o.hist = plan.hist16 ? static_cast<const void*>(d.H16) : static_cast<const void*>(d.H);
+    o.current = d.H;
+    o.m = plan.mom16 ? static_cast<const void*>(d.m16) : static_cast<const void*>(d.m);
+    o.v = plan.mom16 ? static_cast<const void*>(d.v16) : static_cast<const void*>(d.v);
+    o.rows = d.grow + static_cast<long long>(t) * (plan.hist16 ? 2 : 1) * s;
+    items.push_back(o);
+  };
   for (int i = 0; i < n; ++i) {
     if (mats[i].s == 0) continue;
     if (skip_gram != nullptr && (*skip_gram)[i]) continue;
-    for (int t = 0; t < mats[i].ntiles; ++t) items.push_back(FusedItem{i, t, 0, 0});
+    for (int t = 0; t < mats[i].ntiles; ++t) add(i, t, 0);
   }
   for (int i = 0; i < n; ++i)
-    for (int t = 0; t < mats[i].ntiles; ++t) items.push_back(FusedItem{i, t, 1, 0});
+    for (int t = 0; t < mats[i].ntiles; ++t) add(i, t, 1);
   plan.n_items = static_cast<int>(items.size());
   if (plan.grid > plan.n_items) plan.grid = plan.n_items;
   if (cudaMalloc(&plan.d_items, sizeof(FusedItem) * items.size()) != cudaSuccess) {
@@ -724,8 +808,6 @@ inline ngalore_status fused_plan_create(FusedPlan& plan, const std::vector<MatDe
   }
   if (cudaMemcpy(plan.d_items, items.data(), sizeof(FusedItem) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
-  plan.hist16 = !mats.empty() && mats[0].H16 != nullptr;
-  plan.mom16 = !mats.empty() && mats[0].m16 != nullptr;
   const cudaError_t e = plan.hist16 ? (plan.mom16 ? fused_set_smem_for<true, true>(s) : fused_set_smem_for<true, false>(s))
                                     : (plan.mom16 ? fused_set_smem_for<false, true>(s) : fused_set_smem_for<false, false>(s));
   return e == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;

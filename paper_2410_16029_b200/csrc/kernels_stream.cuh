@@ -167,6 +167,179 @@ __device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, d
   __syncwarp();
 }
 
+// ---------------------------------------------------------------- the same solve in the fused stream kernel
+//
+// What one warp has for another CTA there (partial rows, weights) goes through words of eight bytes that hold four bytes of the value
+// and the tag of the step: a reader polls the words themselves, so that a value is one trip to L2 behind its writer.  (Value, fence,
+// counter, fence, read took three to four trips each way: one 512 x 1376 matrix, s = 8, waited 10 us from its last Gram tile to its
+// weights, and 4 so.)
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void ld_relaxed_2(const ulonglong2* p, unsigned long long& a, unsigned long long& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned long long tagged(unsigned int value, unsigned int tag) {
+  return static_cast<unsigned long long>(value) | (static_cast<unsigned long long>(tag) << 32);
+}
+__device__ __forceinline__ void st_tagged(ulonglong2* p, double x, unsigned int tag) {
+  const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};"
+               ::"l"(p), "l"(tagged(static_cast<unsigned int>(bits), tag)), "l"(tagged(static_cast<unsigned int>(bits >> 32), tag)) : "memory");
+}
+// Lane j's weight, for the combination tiles (the tag carries whether the step is flagged for the matrix).
+__device__ __forceinline__ void publish_weights(const MatDesc& d, int lane, float w, bool bad, unsigned int tag) {
+  st_relaxed(d.wpub + lane, tagged(__float_as_uint(w), 2u * tag + (bad ? 1u : 0u)));
+}
+
+// gram_row_sum over tagged rows ([tile][rows][s]), each waited for; sums in the same order.  False where they do not come.
+// meanwhile: what the warp does between two looks.
+template <int SMAX, typename F>
+__device__ __forceinline__ bool tagged_row_sum(const MatDesc& d, int lane, int c, int rows, int row, unsigned int tag, long long limit,
+                                               const volatile int* abort_flag, double& out, F&& meanwhile) {
+  constexpr int G = 32 / SMAX, U = 8;   // (sixteen take the registers of eight slots and more: 0.7 us slower for one matrix)
+  const ulonglong2* gp = d.grow + static_cast<long long>(row) * d.s + min(lane % SMAX, c - 1);
+  const long long st = static_cast<long long>(rows) * d.s;
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
+  long long spins = 0;
+  for (int t0 = 0; t0 < d.ntiles; t0 += G * U) {
+    unsigned long long lo[U], hi[U];
+    while (true) {
+#pragma unroll
+      for (int q = 0; q < U; ++q) ld_relaxed_2(gp + min(t0 + q * G + lane / SMAX, d.ntiles - 1) * st, lo[q], hi[q]);
+      bool here = true;
+#pragma unroll
+      for (int q = 0; q < U; ++q) here = here && static_cast<unsigned int>(lo[q] >> 32) == tag && static_cast<unsigned int>(hi[q] >> 32) == tag;
+      if (__all_sync(0xffffffffu, here)) break;
+      if (__any_sync(0xffffffffu, ++spins > limit || *abort_flag != 0)) return false;
+      meanwhile();
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const double v = __longlong_as_double(static_cast<long long>((lo[q] & 0xffffffffull) | (hi[q] << 32)));
+      t[q & 3] += t0 + q * G + lane / SMAX < d.ntiles ? v : 0.0;
+    }
+  }
+  double sum = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+  for (int o = SMAX; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  out = lane < c ? sum : 0.0;
+  return true;
+}
+
+// solve_matrix in two parts.  prepare eliminates the slots whose products are known when the step begins (all but `cur`, and with a
+// bf16 history `prev`) while the Gram tiles are still on their way; finish takes the columns of the new ones through the same
+// steps, two trips through the lanes for each slot (s = 8: 0.3 us where the whole elimination takes 2, s = 16: 0.6 instead of 4), and
+// solves the system of one or two unknowns that is left.  As there, nothing branches on the lane ahead of the shuffles.
+template <int SMAX>
+struct GramSolve {
+  double f[SMAX];    // row `lane`: the multiplier of every step
+  double rdiag;      // one over its pivot
+  double old_prev;   // <H_lane, H_prev> as it was
+  int bad;
+
+  __device__ __forceinline__ static bool known(int j, int cur, int prev, int c) { return j < c && j != cur && j != prev; }
+
+  __device__ __forceinline__ void prepare(const MatDesc& d, int cur, int prev, int c, double lambda, int lane) {
+    const double* old = d.Kraw + min(lane, c - 1) * d.s;
+    const double ic = 1.0 / static_cast<double>(c);
+    const bool mine = known(lane, cur, prev, c);
+    old_prev = __ldcg(old + max(prev, 0));
+#pragma unroll
+    for (int j = 0; j < SMAX; ++j) f[j] = __ldcg(old + min(j, c - 1));
+#pragma unroll
+    for (int j = 0; j < SMAX; ++j) {
+      f[j] = mine && known(j, cur, prev, c) ? f[j] * ic : 0.0;
+      f[j] += j == lane ? (mine ? lambda : 1.0) : 0.0;
+    }
+    double diag = 1.0;
+    bad = 0;
+#pragma unroll
+    for (int k = 0; k < SMAX; ++k) {
+      if (k >= c || bad != 0) break;
+      if (k == cur || k == prev) continue;
+      const double p = __shfl_sync(0xffffffffu, f[k], k);
+      if (!(p > 0.0) || !isfinite(p)) {
+        bad = isfinite(p) ? 6 /* NGALORE_ERR_NOT_SPD */ : 7 /* NGALORE_ERR_NONFINITE */;
+        break;
+      }
+      diag = lane == k ? p : diag;
+      const double ip = 1.0 / p;
+      f[k] = lane == k ? 0.0 : f[k] * ip;
+#pragma unroll
+      for (int j = k + 1; j < SMAX; ++j) f[j] -= f[k] * __shfl_sync(0xffffffffu, f[j], k);
+    }
+    rdiag = 1.0 / diag;
+  }
+
+  // row, rowp: lane j's <H_cur, H_j> and <H_prev, H_j>.  Publishes the weights (unless withheld), then leaves the Gram matrix, the
+  // weights and the status of the matrix for the next kernels and steps.
+  __device__ __forceinline__ void finish(const MatDesc& d, int cur, int prev, int c, double lambda, int lane, double row, double rowp,
+                                         unsigned int tag, bool withhold) {
+    const bool finite = __all_sync(0xffffffffu, lane >= c || isfinite(row));
+    bad = finite ? bad : 7;
+    const double val = finite && lane < c ? row : 0.0;
+    const double ic = 1.0 / static_cast<double>(c);
+    const int use = prev >= 0 && lane < c && lane != cur && isfinite(rowp) ? 1 : 0;
+    const double val_prev = __shfl_sync(0xffffffffu, val, max(prev, 0));   // <H_cur, H_prev>
+    const double valp = lane == cur ? val_prev : (use ? rowp : old_prev);
+    const bool mine = known(lane, cur, prev, c);
+    const double kc = mine ? val * ic : 0.0, kp = mine && prev >= 0 ? valp * ic : 0.0;
+    double yc = kc, yp = kp;
+#pragma unroll
+    for (int k = 0; k < SMAX; ++k) {
+      if (k >= c || bad != 0) break;
+      if (k == cur || k == prev) continue;
+      const double sc = __shfl_sync(0xffffffffu, yc, k);
+      yc -= f[k] * sc;
+      if (prev >= 0) {
+        const double sp = __shfl_sync(0xffffffffu, yp, k);
+        yp -= f[k] * sp;
+      }
+    }
+    const double zc = mine ? yc * rdiag : 0.0, zp = mine ? yp * rdiag : 0.0;
+    const double ccur = __shfl_sync(0xffffffffu, val, cur) * ic + lambda;
+    double xc, xp = 0.0, s_cc;
+    if (prev >= 0) {
+      const double s_pp = __shfl_sync(0xffffffffu, valp, prev) * ic + lambda - warp_sum(kp * zp);
+      const double s_pc = val_prev * ic - warp_sum(kp * zc);
+      const double l = s_pc / s_pp;
+      s_cc = ccur - warp_sum(kc * zc) - l * s_pc;
+      if (bad == 0 && (!(s_pp > 0.0) || !isfinite(s_pp))) bad = isfinite(s_pp) ? 6 : 7;
+      xc = 1.0 / s_cc;
+      xp = -l * xc;
+    } else {
+      s_cc = ccur - warp_sum(kc * zc);
+      xc = 1.0 / s_cc;
+    }
+    if (bad == 0 && (!(s_cc > 0.0) || !isfinite(s_cc))) bad = isfinite(s_cc) ? 6 : 7;
+    const double x = lane == cur ? xc : (lane == prev ? xp : -(zc * xc + zp * xp));
+    const float w = bad == 0 && lane < c ? static_cast<float>(x) : 0.f;
+    if (!withhold) publish_weights(d, lane, w, bad != 0, tag);
+    d.wsol[lane] = w;
+    if (use) {
+      d.Kraw[prev * d.s + lane] = rowp;
+      d.Kraw[lane * d.s + prev] = rowp;
+    }
+    __syncwarp();
+    // (where the step is flagged the poisoned slot becomes a zero gradient: its Gram row and column vanish)
+    if (lane < (bad != 0 ? d.s : c)) {
+      d.Kraw[cur * d.s + lane] = bad != 0 ? 0.0 : val;
+      d.Kraw[lane * d.s + cur] = bad != 0 ? 0.0 : val;
+    }
+    if (lane == 0) {
+      *d.step_bad = bad != 0 ? 1 : 0;
+      if (bad != 0) atomicCAS(d.status, 0, bad);
+    }
+    __syncwarp();
+  }
+};
+
 // N~ = sum_j w_j H_j, then the Adam moments as printed in Sec. 2.2 (eps inside the root, no bias
 // correction), then u rounded to fp16 for the back-projection GEMM.
 template <int SMAX>

@@ -70,7 +70,8 @@ struct ngalore_state {
   Hyper* d_hyper = nullptr;
   int* d_status = nullptr;
   int* d_step_bad = nullptr;
-  int* d_flags = nullptr;            // gram_done / w_ready of every matrix (scratch, not part of a checkpoint)
+  char* d_tagged = nullptr;          // what the stream kernel's warps publish under a step's tag (scratch, not part of a checkpoint)
+  size_t tagged_bytes = 0;
   StreamTile* d_tiles = nullptr;
   int n_tiles = 0;
   std::vector<const uint16_t*> refresh_G;  // the gradients as the refresh reads them (G, or its transposed copy)
@@ -604,11 +605,6 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   st->hyper.seed_lo = static_cast<unsigned int>(st->opt.seed & 0xFFFFFFFFull);
   st->hyper.seed_hi = static_cast<unsigned int>(st->opt.seed >> 32);
 
-  // ---- streaming tile size.  A work item of the persistent stream kernel carries a fixed cost (table and
-  // descriptor loads, the end-of-tile reduction, the completion counter), so tiles are large; measured on the
-  // 1.1B shapes, 65536 to 262144 elements are within 1 % of each other and 16384 costs 4 %.  Tiles shrink only to
-  // keep about two items per pass and SM on small models.  The history is read from HBM twice per step: a big
-  // matrix's history does not survive in L2 between the Gram pass and the combination pass.
   uint64_t hash = 1469598103934665603ull;
   st->mats.resize(n_matrices);
   long long total_rn = 0;
@@ -631,18 +627,20 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     hash = (hash ^ static_cast<uint64_t>((hm.right ? 2 : 1) + (st->opt.history_bf16 ? 4 : 0) + (st->opt.moments_bf16 ? 8 : 0))) * 1099511628211ull;
   }
   st->shape_hash = hash;
-  // Stream tiles: two per SM and pass on large workloads.  Where that would make them short, one per SM: every tile
-  // ends with a block-wide reduction and a handful of global round trips, which on small workloads weigh as much
-  // as its traffic (measured, stream phase: RoBERTa-base shapes r = 8 / r = 4 68 -> 44 us / 52 -> 39 us, 60M shapes
-  // 116 -> 106 us; the 130M shapes and larger are 2 % better with two).  At least 4096 elements, or less where the set has not as
-  // many for every SM: a stage then waits for none before it (one 512 x 1376 matrix, r = 128: 28.2 -> 26.4 us a step).
-  long long te_all = total_rn / (2ll * prop.multiProcessorCount) / 1024 * 1024;
-  if (te_all < 32768) te_all *= 2;
-  if (te_all < 4096) te_all = std::min(4096ll, std::max(1024ll, (total_rn / prop.multiProcessorCount + 1023) / 1024 * 1024));
-  if (te_all > 131072) te_all = 131072;
+  // Stream tiles: about six per SM and pass, so that the SMs end together, of 8192 elements at least, since a tile costs its
+  // CTA some 0.3 us beside its traffic (sums, weights): stream phase of the 60M shapes with tiles of 4096 / 8192 / 12288 / 24576
+  // elements 80 / 78 / 78 / 87 us, of one encoder layer (r = 460, s = 15) 49 / 45 / 51 / 59, of 288-wide layers (s = 3) 49 / 43 /
+  // 43 / 51.  Longer ones up to where they stop to gain: 130M shapes (s = 8) 8192 / 12288 / 24576 / 83968 327 / 319 / 319 / 339,
+  // 1.1B shapes (s = 16) 8192 / 12288 / 40960 / 131072 4110 / 4150 / 4153 / 4200, and with a bf16 history, whose tiles hold half the bytes and
+  // cost more, 350M shapes 8192 / 24576 / 49152 / 131072 881 / 849 / 820 / 834.  Sets with less than 8192 elements for every SM: one
+  // tile each, of 1024 elements at least (a stage then waits for none before it).
+  const long long per_sm = total_rn / prop.multiProcessorCount;
+  const long long te_max = st->opt.history_bf16 == 1 ? 49152 : (s > 8 ? 8192 : 24576);
+  long long te_all = std::min(te_max, std::max(8192ll, per_sm / 6 / 1024 * 1024));
+  if (per_sm < 8192) te_all = per_sm >= 4096 ? per_sm / 1024 * 1024 : std::max(1024ll, (per_sm + 1023) / 1024 * 1024);
   std::vector<int> tile_elems(n_matrices, static_cast<int>(te_all));
-  // The matrices at the end of the item list get tiles a quarter of the size, so that the last wave of the
-  // kernel ends more evenly (the tail of one full-size tile per SM is about 0.1 ms on the 1.1B shapes).
+  // Where tiles are long, the matrices at the end of the item list get tiles a quarter of the size, so that the last wave of
+  // the kernel ends more evenly.
   if (te_all >= 32768) {
     const long long tail_budget = static_cast<long long>(prop.multiProcessorCount) * te_all;
     long long acc = 0;
@@ -683,7 +681,6 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   const size_t o_hyper = take(sizeof(Hyper));
   const size_t o_desc = take(sizeof(MatDesc) * n_matrices);
   const size_t o_chol = take(sizeof(CholProblem) * n_matrices);
-  const size_t o_flags = take(sizeof(int) * 2 * n_matrices);
   const size_t o_eig = take(sizeof(EigMat) * n_matrices);
   const size_t o_eig_factor = take(sizeof(FactorMat) * n_matrices);
   const size_t o_eig_redo = take(sizeof(int) * n_matrices);
@@ -712,6 +709,13 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     woffs[i].Gt = hm.right ? take(sizeof(uint16_t) * hm.N * hm.eN) : 0;
   }
   st->n_tiles = n_tiles;
+  const size_t o_tagged = off;
+  std::vector<size_t> o_wpub(n_matrices), o_grow(n_matrices);
+  for (int i = 0; i < n_matrices; ++i) {
+    o_wpub[i] = take(sizeof(unsigned long long) * kMaxHistory);
+    o_grow[i] = take(sizeof(ulonglong2) * ntl[i] * slots * (hist16 ? 2 : 1));
+  }
+  st->tagged_bytes = off - o_tagged;
   const size_t o_tiles = take(sizeof(StreamTile) * n_tiles);
   st->work_bytes = off;
 
@@ -731,8 +735,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   st->d_desc = reinterpret_cast<MatDesc*>(st->work + o_desc);
   st->d_chol = reinterpret_cast<CholProblem*>(st->work + o_chol);
   st->d_tiles = reinterpret_cast<StreamTile*>(st->work + o_tiles);
-  int* flags = reinterpret_cast<int*>(st->work + o_flags);
-  st->d_flags = flags;
+  st->d_tagged = st->work + o_tagged;
   st->d_eig = reinterpret_cast<EigMat*>(st->work + o_eig);
   st->d_eig_factor = reinterpret_cast<FactorMat*>(st->work + o_eig_factor);
   std::vector<EigMat> eig(n_matrices);
@@ -775,8 +778,8 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     d.gpart = reinterpret_cast<double*>(st->work + woffs[i].gpart);
     d.status = st->d_status + i;
     d.step_bad = st->d_step_bad + i;
-    d.gram_done = flags + 2 * i;
-    d.w_ready = flags + 2 * i + 1;
+    d.wpub = reinterpret_cast<unsigned long long*>(st->work + o_wpub[i]);
+    d.grow = reinterpret_cast<ulonglong2*>(st->work + o_grow[i]);
     d.tile0 = tile0[i]; d.ntiles = ntl[i]; d.te = tile_elems[i];
     hm.Ya = reinterpret_cast<float*>(st->work + woffs[i].Ya);
     hm.Yb = reinterpret_cast<float*>(st->work + woffs[i].Yb);
@@ -1193,10 +1196,10 @@ ngalore_status ngalore_state_import(ngalore_state* st, const void* blob, size_t 
   if (!guard.ok) return NGALORE_ERR_CUDA;
   NG_CUDA(cudaDeviceSynchronize());
   NG_CUDA(cudaMemcpy(st->arena, static_cast<const char*>(blob) + sizeof(h), st->arena_bytes, cudaMemcpyHostToDevice));
-  // The blob brings back the step epoch of the exporting state.  The per-matrix flags of the stream kernel hold
-  // epochs of steps this state ran before the import and could equal the next step's tag by accident (export, step,
-  // import, step): clear them, together with the scheduling counters and anything a testing aid left behind.
-  NG_CUDA(cudaMemset(st->d_flags, 0, sizeof(int) * 2 * st->n));
+  // The blob brings back the step epoch of the exporting state.  What the stream kernel's warps have published carries
+  // tags of steps this state ran before the import, which could equal the next step's by accident (export, step,
+  // import, step): clear it, together with the scheduling counters and anything a testing aid left behind.
+  NG_CUDA(cudaMemset(st->d_tagged, 0, st->tagged_bytes));
   Ctrl c{};
   NG_CUDA(cudaMemcpy(&c, st->d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost));
   c.timeout_flag = 0; c.work_counter = 0u; c.gemm_counter0 = 0u; c.gemm_counter1 = 0u;

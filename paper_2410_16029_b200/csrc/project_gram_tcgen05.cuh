@@ -361,9 +361,7 @@ __global__ void __launch_bounds__(256) pg_solve_kernel(const MatDesc* __restrict
     double row = 0.0;
     for (int q = 0; q < 8; ++q) row += red[q * 32 + threadIdx.x];
     solve_matrix<kPgSMax>(d, ring_cur(ctrl, d.s), c, hyper->lambda, row);
-    __threadfence();
-    __syncwarp();
-    if (threadIdx.x == 0) atomicExch(d.w_ready, ctrl->epoch + 1);
+    publish_weights(d, threadIdx.x, d.wsol[threadIdx.x], *d.step_bad != 0, static_cast<unsigned int>(ctrl->epoch + 1));
   }
 }
 
