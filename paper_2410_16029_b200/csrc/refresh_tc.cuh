@@ -38,6 +38,7 @@ struct SplitJob {
 // All matrices in one launch: blockIdx.y selects the matrix, blockIdx.x strides over its elements, four at a
 // time where the row length allows it (the kernel is a pure stream: 4 bytes in, 4 bytes out per element).
 __global__ void split_hilo_grouped_kernel(const SplitJob* jobs) {
+  pdl_begin();
   const SplitJob jb = jobs[blockIdx.y];
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   const long long t0 = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
@@ -75,6 +76,7 @@ struct ZeroJob {
 };
 
 __global__ void zero_jobs_kernel(const ZeroJob* jobs) {
+  pdl_begin();
   const ZeroJob jb = jobs[blockIdx.y];
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < jb.n16;
        i += static_cast<long long>(gridDim.x) * blockDim.x)
@@ -288,6 +290,7 @@ struct NewtonJob {
 __global__ void __launch_bounds__(256) newton_prep_kernel(const NewtonJob* jobs) {
   __shared__ float tile[32][33];
   const NewtonJob g = jobs[blockIdx.x];
+  pdl_begin();
   const int nb = (g.L + 31) >> 5, lane = threadIdx.x & 31, row = threadIdx.x >> 5;
   auto put = [&](int j, int i, float c) {
     const float f = i == j ? 1.5f - 0.5f * c : -0.5f * c;
@@ -377,6 +380,7 @@ struct RefreshPlan {
   bool wide = false;           // the products with G take tiles of kRefWideBN columns ...
   bool tall = false;           // ... and of 256 rows
   bool pair = false;           // ... on pairs of SMs
+  bool brief = false;          // the kernels between the products are programmatic dependents
   std::vector<int> atomic_mats[RG_COUNT];  // matrices whose K is split for this GEMM (output must be zeroed)
   // buffers to clear before GEMM kind g (the outputs of atomic_mats[g]); entry RG_COUNT: every matrix's X64
   ZeroJob* d_zero[RG_COUNT + 1] = {};
@@ -565,6 +569,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     tc_assign_tiles(tiles[g], plan.grid[g], tile_first[g], g == RG_APPLY_Y || g == RG_APPLY_TRI);
     o_first[g] = take(sizeof(int) * tile_first[g].size());
   }
+  // Programmatic dependents, for what has one wave of CTAs and is short: the start of a kernel (launch, barriers, tensor memory) and
+  // the end of the one before are a third of it.  Refresh, with ordinary launches / so: three small matrices 610 / 490 us, 824-wide
+  // layers at r = 48 943 / 819, 1264-wide at r = 8 1240 / 1069, 60M shapes (5 tiles a CTA in the products with R^-1) 2200 / 2117; 130M
+  // shapes (15) 6777 / 6820.  Not the kernels of the eigensolver: 60M shapes 2200 / 2292.
+  plan.brief = plan.n_tiles[RG_APPLY_TRI] <= 8 * sm_count;
   const size_t o_newton = take(sizeof(NewtonJob) * n);
   const size_t o_factor32 = take(sizeof(FactorMat) * n);
   const size_t o_factor64 = take(sizeof(FactorMat) * n);
@@ -854,7 +863,7 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
                                       bool high_only = false, bool cleared = false) {
   // outputs that several K slices accumulate into start from zero
   if (plan.n_zero[g] > 0 && !cleared) {
-    zero_jobs_kernel<<<dim3(32, plan.n_zero[g]), 256, 0, stream>>>(plan.d_zero[g]);
+    launch_step(plan.brief, zero_jobs_kernel, dim3(32, plan.n_zero[g]), 256, 0, stream, plan.d_zero[g]);
     *launches += 1;
   }
   using L2 = TcSmem<kRefBN, 2, 2, kRefStages2, 8>;
@@ -863,8 +872,8 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
   auto product = [&](auto a_mn) {   // a product with G; a_mn: with G^T
     constexpr bool MN = decltype(a_mn)::value;
     auto run = [&](auto p) {
-      p.kernel<<<plan.grid[g], p.kThreads, p.kSmem, stream>>>(plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl,
-                                                              plan.d_probs[problem], nullptr, 0);
+      launch_step(plan.brief, p.kernel, plan.grid[g], p.kThreads, p.kSmem, stream, plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr,
+                  d_ctrl, plan.d_probs[problem], nullptr, 0);
     };
     if (plan.pair) {
       auto pair = [&](auto parts) {
@@ -886,12 +895,12 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
     case RG_Z_FROM_Y: product(std::true_type{}); break;
     case RG_GRAM_Y:
     case RG_GRAM_Z:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
+      launch_step(plan.brief, tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, true>, plan.grid[g], threads, L2::kTotal, stream,
+                  plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
       break;
     default:
-      tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false><<<plan.grid[g], threads, L2::kTotal, stream>>>(
-          plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
+      launch_step(plan.brief, tc_gemm_kernel<kRefBN, 2, 2, kRefStages2, TC_EPI_STORE, 8, false>, plan.grid[g], threads, L2::kTotal, stream,
+                  plan.d_maps, plan.d_tiles[g], plan.d_first[g], nullptr, d_ctrl, plan.d_probs[problem], nullptr, 0);
       break;
   }
   *launches += 1;
@@ -902,7 +911,7 @@ inline ngalore_status refresh_tc_gemm(RefreshPlan& plan, int g, int problem, Ctr
 inline ngalore_status refresh_tc_split(RefreshPlan& plan, bool y_side, cudaStream_t stream, int64_t* launches) {
   const int n_jobs = y_side ? plan.n_split_y_rest : plan.n_split_z_rest;
   if (n_jobs == 0) return NGALORE_OK;
-  split_hilo_grouped_kernel<<<dim3(64, n_jobs), 256, 0, stream>>>(y_side ? plan.d_split_y_rest : plan.d_split_z_rest);
+  launch_step(plan.brief, split_hilo_grouped_kernel, dim3(64, n_jobs), 256, 0, stream, y_side ? plan.d_split_y_rest : plan.d_split_z_rest);
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
@@ -913,7 +922,7 @@ inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStrea
   ngalore_status rc;
   if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, RP_GRAM_Y0, d_ctrl, stream, launches, false, true))) return rc;
-  if (tri_factor_launch(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches, false, plan.brief) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_01, d_ctrl, stream, launches);
 }
 
@@ -937,7 +946,7 @@ inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStre
 inline ngalore_status refresh_tc_refine(RefreshPlan& plan, int set, Ctrl* d_ctrl, cudaStream_t stream, int64_t* launches) {
   ngalore_status rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, set == 0 ? RP_GRAM_Y0 : RP_GRAM_Y1, d_ctrl, stream, launches))) return rc;
-  newton_prep_kernel<<<dim3(plan.n, 8), 256, 0, stream>>>(plan.d_newton);
+  launch_step(plan.brief, newton_prep_kernel, dim3(plan.n, 8), 256, 0, stream, plan.d_newton);
   *launches += 1;
   return refresh_tc_gemm(plan, RG_APPLY_Y, set == 0 ? RP_APPLY_01 : RP_APPLY_10, d_ctrl, stream, launches);
 }

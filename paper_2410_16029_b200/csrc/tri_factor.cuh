@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
   extern __shared__ __align__(16) unsigned char tf_smem[];
   __shared__ int counter;
   const FactorMat m = mats[blockIdx.x];
+  pdl_begin();
   if (conditional && *m.only_if == 0) return;
   const int L = m.L, nb = (L + NB - 1) / NB, np = nb * NB;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
@@ -396,9 +397,9 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
 constexpr int kTfSmemLimit = 232448 - 256;   // (the kernel has 128 bytes of its own)
 
 // Factor n matrices, the widest l_max wide (widest first in the list: CTAs are handed out in order).  shift_scale: what
-// is added to the unit diagonal, for fp32 matrices in units of L / 65536.
+// is added to the unit diagonal, for fp32 matrices in units of L / 65536.  dependent: launched as a programmatic dependent.
 inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, double shift_scale, cudaStream_t stream,
-                                     int64_t* launches, bool conditional = false) {
+                                     int64_t* launches, bool conditional = false, bool dependent = false) {
   // as much shared memory as the widest matrix that fits with its blocks, and at least what the widest needs without
   size_t smem = tf_base_smem(l_max, false);
   const bool s_global = smem > static_cast<size_t>(kTfSmemLimit);
@@ -412,7 +413,7 @@ inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, 
   auto run = [&](auto kernel) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmemLimit);
     if (e != cudaSuccess) return e;
-    kernel<<<n, kTfThreads, smem, stream>>>(d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
+    launch_step(dependent, kernel, n, kTfThreads, smem, stream, d_mats, static_cast<int>(smem), shift_scale, conditional ? 1 : 0);
     *launches += 1;
     return cudaGetLastError();
   };
