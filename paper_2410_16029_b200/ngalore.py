@@ -22,6 +22,8 @@ if not os.path.exists(LIB_PATH):
 
 _lib = ctypes.CDLL(LIB_PATH)
 
+from . import _bind  # noqa: E402  (built with the library; missing, it fails here)
+
 OK = 0
 STATUS_NAMES = {0: "OK", 1: "INVALID_ARG", 2: "ALLOC", 3: "CUDA", 4: "UNSUPPORTED_DEVICE", 5: "NO_SUBSPACE",
                 6: "NOT_SPD", 7: "NONFINITE", 8: "TIMEOUT"}
@@ -144,6 +146,8 @@ class NGaLore:
         _check(_lib.ngalore_create(arr, len(self.shapes), r, s, T, lam, lr, beta1, beta2, eps, wd,
                                    ctypes.byref(opt), ctypes.byref(handle)), "ngalore_create")
         self._h = handle
+        self._pointer_array = _vp * len(self.shapes)
+        self._flat_shapes = (ctypes.c_int64 * (2 * len(self.shapes)))(*[x for shape in self.shapes for x in shape])
         self.device = torch.device("cuda", torch.cuda.current_device())
 
     def close(self):
@@ -164,11 +168,24 @@ class NGaLore:
             assert w.is_cuda and w.dtype == torch.float32 and w.is_contiguous() and tuple(w.shape) == (M, N)
             assert g.is_cuda and g.dtype == torch.bfloat16 and g.is_contiguous() and tuple(g.shape) == (M, N)
 
+    def _pointers(self, W, G, mode):
+        """The pointers of W and G; mode 0: unchecked, 1: device tensors of the state's shapes, 2: host tensors."""
+        w, g = self._pointer_array(), self._pointer_array()
+        if _bind.collect(W, G, len(self.shapes), ctypes.addressof(self._flat_shapes), ctypes.addressof(w),
+                         ctypes.addressof(g), mode):
+            return w, g
+        # not two lists of plain tensors: other sequences, tensor subclasses
+        if mode == 1:
+            self._check_WG(W, G)
+        elif mode == 2:
+            for x, y in zip(W, G):
+                assert not x.is_cuda and not y.is_cuda and x.is_contiguous() and y.is_contiguous()
+        return _ptr_array(W), _ptr_array(G)
+
     # -- the three calls of the optimizer -------------------------------------------
     def step(self, W: List[torch.Tensor], G: List[torch.Tensor], stream=None, check=True):
-        if check:
-            self._check_WG(W, G)
-        _check(_lib.ngalore_step(self._h, _ptr_array(W), _ptr_array(G), _stream_ptr(stream)), "ngalore_step")
+        w, g = self._pointers(W, G, 1 if check else 0)
+        _check(_lib.ngalore_step(self._h, w, g, _stream_ptr(stream)), "ngalore_step")
 
     def step_ptrs(self, W_ptrs, G_ptrs, stream=None):
         """Step with pre-built pointer arrays (see ``pointer_array``): no per-call marshalling."""
@@ -185,10 +202,8 @@ class NGaLore:
 
     def step_host(self, W_host: List[torch.Tensor], G_host: List[torch.Tensor], stream=None):
         """Step with host tensors (fp32 W updated in place, bf16 G); copies run inside the call."""
-        for w, g in zip(W_host, G_host):
-            assert not w.is_cuda and not g.is_cuda and w.is_contiguous() and g.is_contiguous()
-        _check(_lib.ngalore_step_host(self._h, _ptr_array(W_host), _ptr_array(G_host), _stream_ptr(stream)),
-               "ngalore_step_host")
+        w, g = self._pointers(W_host, G_host, 2)
+        _check(_lib.ngalore_step_host(self._h, w, g, _stream_ptr(stream)), "ngalore_step_host")
 
     # -- state access -----------------------------------------------------------
     def poll_status(self):
