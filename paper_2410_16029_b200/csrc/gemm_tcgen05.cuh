@@ -286,7 +286,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar + s, 1); mbar_init(empty_bar + s, 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, 4 * MT); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, EPI == TC_EPI_PROJECT ? NEPI : 4 * MT); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -422,8 +422,11 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
     float* stg = reinterpret_cast<float*>(smem + STAGES * L::kStageBytes + (warp - 2) * L::kEpiWarpBytes);
     bool ok = true, cleared = EPI != TC_EPI_PROJECT || n_clear == 0;
     if (!cleared) clear_split_slots(mats, clear, n_clear, ctrl);
-    // (of tall tiles, each group drains its half of all of them)
-    constexpr int kStep = MT == 2 ? 1 : kGroups;
+    // (of tall tiles, each group drains its half of all of them; of the step's projection, every second 32 columns: what a CTA does
+    // last is to drain a tile, 6 us for 256 columns with four warps.  60M shapes 199.4 -> 195.8 us a step, one 512 x 1376 matrix
+    // 21.1 -> 20.4, encoder shapes at r = 8 167.5 -> 165.5, 288-wide layers under the short-side rule 76.7 -> 73.1; 130M and more as before)
+    constexpr bool kShareTile = EPI == TC_EPI_PROJECT && kGroups == 2;
+    constexpr int kStep = MT == 2 || kShareTile ? 1 : kGroups;
     const int first = kStep == 2 ? group : 0, half = MT == 2 ? group : 0;
     TcTile tile = tile0;
     if (first > 0 && t_begin + first < t_end) tile = tiles[t_begin + first];
@@ -466,13 +469,19 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
         tile = next;
         continue;
       }
+      const int c_first = kShareTile ? 32 * group : 0, c_step = kShareTile ? 64 : 32;
+      if (kShareTile && c_first >= n_eff) {   // none of the columns are this warp's
+        tc_fence_before();
+        if (lane == 0) mbar_arrive(tempty_bar + buf);
+      }
 #pragma unroll
-      for (int c0 = 0; c0 < BN; c0 += 32) {
+      for (int x = 0; x < BN / (kShareTile ? 64 : 32); ++x) {
+        const int c0 = c_first + x * c_step;
         if (c0 < n_eff) {
           uint32_t r[32];
           tc_ld32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>((buf * MT + half) * BN + c0), r);
           tc_wait_ld();
-          if (c0 + 32 >= n_eff) {
+          if (c0 + c_step >= n_eff) {
             // all TMEM reads of this tile are done: hand the buffer back before the global traffic
             tc_fence_before();
             if (lane == 0) mbar_arrive(tempty_bar + buf);
@@ -547,7 +556,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-constexpr int kProjBN = 256, kProjStages = 4, kProjEpiWarps = 4;
+constexpr int kProjBN = 256, kProjStages = 4, kProjEpiWarps = 8;
 constexpr int kTcBackBN = 256;  // tile width of the back-projection kernel
 
 // Projection with the Gram row in its epilogue (project_gram_tcgen05.cuh): tile width, the longest history that
