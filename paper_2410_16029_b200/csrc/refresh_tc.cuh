@@ -571,9 +571,11 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
   }
   // Programmatic dependents, for what has one wave of CTAs and is short: the start of a kernel (launch, barriers, tensor memory) and
   // the end of the one before are a third of it.  Refresh, with ordinary launches / so: three small matrices 610 / 490 us, 824-wide
-  // layers at r = 48 943 / 819, 1264-wide at r = 8 1240 / 1069, 60M shapes (5 tiles a CTA in the products with R^-1) 2200 / 2117; 130M
-  // shapes (15) 6777 / 6820.  Not the kernels of the eigensolver: 60M shapes 2200 / 2292.
-  plan.brief = plan.n_tiles[RG_APPLY_TRI] <= 8 * sm_count;
+  // layers at r = 48 943 / 819, 1264-wide at r = 8 1240 / 1069, 60M shapes (5 tiles a CTA in the products with R^-1) 2200 / 2117,
+  // 37 and 74 matrices of 768 rows at r = 160 1881 / 1817 and 2427 / 2356.  Not with wide bases, whose factorisations are long: at
+  // r = 224 2974 / 3048 and 3644 / 3658, at r = 256 3660 / 3808 and 4410 / 4452, 130M shapes 6777 / 6820; nor the kernels of the
+  // eigensolver: 60M shapes 2200 / 2292.
+  plan.brief = !plan.wide && plan.n_tiles[RG_APPLY_TRI] <= 8 * sm_count;
   const size_t o_newton = take(sizeof(NewtonJob) * n);
   const size_t o_factor32 = take(sizeof(FactorMat) * n);
   const size_t o_factor64 = take(sizeof(FactorMat) * n);
