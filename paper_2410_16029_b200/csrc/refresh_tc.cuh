@@ -390,6 +390,7 @@ struct RefreshPlan {
   FactorMat* d_factor32 = nullptr;   // R^-1 from C32 (tri_factor.cuh), widest first
   FactorMat* d_factor64 = nullptr;   // R^-1 from the exact Gram matrix in X64
   int l_max = 0;  // largest basis width L of the set
+  int cluster = 1, short_cluster = 1;   // CTAs that factor a matrix together, of all and of the short ones
   // the matrices whose product with G splits K (their result arrives as fp32 and is split afterwards; all others
   // leave the product as bf16 parts already)
   SplitJob* d_split_y_rest = nullptr;
@@ -520,7 +521,7 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
     offs[i].Zhi = take(sizeof(__nv_bfloat16) * m.N * m.ldl);
     offs[i].Zlo = take(sizeof(__nv_bfloat16) * m.N * m.ldl);
     offs[i].C32 = take(sizeof(float) * m.L * m.L);
-    offs[i].C64 = take(sizeof(double) * m.L * m.L);
+    offs[i].C64 = take(std::max(sizeof(double) * m.L * m.L, tf_block_bytes(m.L)));   // (also holds the factor's blocks)
     const size_t l2 = std::max(static_cast<size_t>(m.L) * m.L, tf_spill_doubles(m.L));   // (both also hold the factor's rows)
     offs[i].X64 = take(sizeof(double) * l2);
     offs[i].T64 = take(sizeof(double) * l2);
@@ -770,7 +771,9 @@ inline ngalore_status refresh_plan_create(RefreshPlan& plan, const std::vector<M
       cudaMemcpy(plan.d_eig_factor, eig_factors.data(), sizeof(FactorMat) * n, cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
 
+  plan.cluster = tf_cluster(n, plan.l_max);
   plan.n_short = static_cast<int>(short_factor.size());
+  plan.short_cluster = tf_cluster(plan.n_short, plan.short_l_max);
   if (plan.n_short > 0) {
     std::stable_sort(short_factor.begin(), short_factor.end(), wider);
     bool ok = true;
@@ -924,7 +927,7 @@ inline ngalore_status refresh_tc_orth(RefreshPlan& plan, Ctrl* d_ctrl, cudaStrea
   ngalore_status rc;
   if ((rc = refresh_tc_split(plan, true, stream, launches))) return rc;
   if ((rc = refresh_tc_gemm(plan, RG_GRAM_Y, RP_GRAM_Y0, d_ctrl, stream, launches, false, true))) return rc;
-  if (tri_factor_launch(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches, false, plan.brief) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_factor32, plan.n, plan.l_max, shift_scale, stream, launches, false, plan.brief, plan.cluster) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_01, d_ctrl, stream, launches);
 }
 
@@ -937,7 +940,7 @@ inline ngalore_status refresh_tc_final(RefreshPlan& plan, Ctrl* d_ctrl, cudaStre
   *launches += 1;
   syrk_f64_kernel<false><<<plan.n_syrk_tiles, 256, 0, stream>>>(plan.d_syrk_mats, plan.d_syrk_tiles);
   *launches += 1;
-  if (tri_factor_launch(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_factor64, plan.n, plan.l_max, 1e-12, stream, launches, false, false, plan.cluster) != cudaSuccess) return NGALORE_ERR_CUDA;
   return refresh_tc_gemm(plan, RG_APPLY_TRI, RP_APPLY_10, d_ctrl, stream, launches);
 }
 
@@ -963,7 +966,7 @@ inline ngalore_status refresh_tc_short(RefreshPlan& plan, cudaStream_t stream, i
   zero_jobs_kernel<<<dim3(8, plan.n_short), 256, 0, stream>>>(plan.d_short_zero);
   syrk_f64_kernel<true><<<plan.n_short_syrk, 256, 0, stream>>>(plan.d_short_syrk_mats, plan.d_short_syrk_tiles);
   *launches += 2;
-  if (tri_factor_launch(plan.d_short_factor, plan.n_short, plan.short_l_max, 1e-12, stream, launches) != cudaSuccess) return NGALORE_ERR_CUDA;
+  if (tri_factor_launch(plan.d_short_factor, plan.n_short, plan.short_l_max, 1e-12, stream, launches, false, false, plan.short_cluster) != cudaSuccess) return NGALORE_ERR_CUDA;
   apply_f64_kernel<<<plan.n_short_tiles, 256, 0, stream>>>(plan.d_short, plan.d_short_tiles);
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;

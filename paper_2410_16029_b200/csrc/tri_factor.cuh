@@ -394,12 +394,256 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
   }
 }
 
+// The same with a cluster of CTAs to a matrix, for wide matrices of which there are few: what takes the time of one CTA beyond the
+// chain of diagonal blocks are the fp64 tensor cores of its SM.  Blocks and S live in global memory (L2); rank 0 has the chain, its
+// warps 0, 4, 8 and 12 nothing else, and the other warps of all CTAs share the rest of S and of the update.  Two cluster barriers a step:
+// S is complete (the chain has arrived by then and waits for it later), and the step has ended.  What other SMs write is read past L1.
+constexpr int kTfClusterMax = 4, kTfClusterFrom = 256;
+
+__device__ __forceinline__ void tf_cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void tf_cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kTfThreads, 1) tri_factor_cluster_kernel(const FactorMat* mats, int cluster, double shift_scale, int conditional) {
+  constexpr int NB = kTfNB, LD = kTfLd, WARPS = kTfThreads / 32;
+  extern __shared__ __align__(16) unsigned char tf_smem[];
+  const int rank = static_cast<int>(blockIdx.x) % cluster;
+  const FactorMat m = mats[blockIdx.x / cluster];
+  pdl_begin();
+  if (conditional && *m.only_if == 0) return;   // (all of the cluster)
+  const int L = m.L, nb = (L + NB - 1) / NB, np = nb * NB;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
+  double* Inv0 = reinterpret_cast<double*>(tf_smem);        // [2][NB][LD]
+  double* W = Inv0 + 2 * NB * LD;                           // [NB][LD] the next diagonal block
+  double* I8 = W + NB * LD;                                 // [8][kTfLdS8]
+  double* Sc = I8 + 8 * kTfLdS8;                            // [NB][LD] S of the next diagonal block's rows, for the chain
+  double* rd = Sc + NB * LD;                                // [np] 1 / column norm
+  double *S = m.spill, *B = m.work;
+  auto block = [&](int i, int j) -> double* { return B + (i * (i + 1) / 2 + j) * (NB * NB); };
+  const double tiny = 1e-28, one = 1.0 + (m.C32 != nullptr ? shift_scale * static_cast<double>(L) / 65536.0 : shift_scale);
+  const int all = cluster * WARPS, mine = rank * WARPS + warp;   // all warps, and this one's number
+  // the warps that share a step: all but those on the scheduler of the chain
+  const bool chain_side = rank == 0 && (warp & 3) == 0;
+  const int sharers = all - 4, share = rank == 0 ? warp - 1 - (warp >> 2) : mine - 4;
+
+  // the scaled matrix (beyond L: the identity), 16 rows of a block at a time
+  for (int x = tid; x < np; x += kTfThreads) {
+    const long long o = static_cast<long long>(min(x, L - 1)) * (L + 1);
+    double d = m.C32 != nullptr ? static_cast<double>(m.C32[o]) : m.C64[o];
+    if (x >= L) d = 1.0;
+    if (!(d > 1e-60)) d = d == d ? 1e-60 : d;          // (a NaN stays one, and the basis check finds it)
+    rd[x] = rsqrt(d);
+  }
+  __syncthreads();
+  for (int u = mine; u < nb * (nb + 1); u += all) {
+    const int b = u >> 1, row0 = (u & 1) * 16;
+    int i = static_cast<int>((sqrtf(8.f * b + 1.f) - 1.f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= b) ++i;
+    while (i * (i + 1) / 2 > b) --i;
+    const int j = b - i * (i + 1) / 2;
+    double raw[16];
+    auto rows = [&](const auto* p) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        raw[q] = static_cast<double>(p[static_cast<long long>(min(i * NB + row0 + q, L - 1)) * L + min(j * NB + lane, L - 1)]);
+    };
+    if (m.C32 != nullptr) rows(m.C32); else rows(m.C64);
+    const int c = j * NB + lane;
+    const double scale = rd[c];
+    double* dst = B + b * (NB * NB);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int row = row0 + q, r = i * NB + row;
+      const double v = raw[q] * rd[r] * scale;
+      dst[tf_at(row, lane)] = r == c ? (r < L ? one : 1.0) : (r < L && c < r ? v : 0.0);
+    }
+  }
+  tf_cluster_arrive();
+  tf_cluster_wait();
+
+  for (int k = -1; k < nb; ++k) {
+    double* Inv = Inv0 + (k & 1) * NB * LD;
+    if (k >= 0 && rank != 0) {   // the inverse that the chain has left in the first CTA
+      uint32_t from;
+      asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(from) : "r"(smem_u32(Inv)));
+      for (int x = tid; x < NB * LD / 2; x += kTfThreads) {
+        double2 v;
+        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(from + 16u * x) : "memory");
+        reinterpret_cast<double2*>(Inv)[x] = v;
+      }
+      __syncthreads();
+    }
+    // rows 8 q .. 8 q + 7 of S_i, and of the block (i, k) of R^-1
+    auto form = [&](int i, int q, bool for_chain) {
+      double acc[4][2];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) acc[y][0] = acc[y][1] = 0.0;
+      if (i != k) {
+        const double* blk = i > k ? block(i, k) : block(k, i);
+        double a[8];
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) a[kk] = __ldcg(blk + (i > k ? tf_at(8 * q + fr, 4 * kk + fk) : tf_at(4 * kk + fk, 8 * q + fr)));
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)
+#pragma unroll
+          for (int y = kk / 2; y < 4; ++y) tf_dmma(acc[y], a[kk], Inv[(8 * y + fr) * LD + 4 * kk + fk]);   // (Inv is lower triangular)
+      } else {
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) acc[y][h] = Inv[(8 * y + 2 * fk + h) * LD + 8 * q + fr];
+      }
+      const int row = i * NB + 8 * q + fr;
+      const double scale = rd[row];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const int kk = 8 * y + 2 * fk, col = k * NB + kk;
+        *reinterpret_cast<double2*>(S + row * LD + kk) = make_double2(acc[y][0], acc[y][1]);
+        if (for_chain) *reinterpret_cast<double2*>(Sc + (8 * q + fr) * LD + kk) = make_double2(acc[y][0], acc[y][1]);
+        if (m.R64 != nullptr) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (row < L && col + h < L) m.R64[static_cast<long long>(row) * L + col + h] = i <= k ? acc[y][h] * scale : 0.0;
+        } else if (row < L && col < L) {   // (L is a multiple of 4: the pair is inside together)
+          float f[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float v = i <= k ? static_cast<float>(acc[y][h] * scale) : 0.f;
+            f[h] = v == v ? fminf(fmaxf(v, -1e30f), 1e30f) : v;
+          }
+          const __nv_bfloat162 hv = __floats2bfloat162_rn(f[0], f[1]);
+          const __nv_bfloat162 lv = __floats2bfloat162_rn(f[0] - __low2float(hv), f[1] - __high2float(hv));
+          const long long o = static_cast<long long>(row) * m.ld + col;
+          *reinterpret_cast<__nv_bfloat162*>(m.Rhi + o) = hv;
+          *reinterpret_cast<__nv_bfloat162*>(m.Rlo + o) = lv;
+        }
+      }
+    };
+    if (k + 1 == nb) {   // the last block column of R^-1
+      for (int t = mine; t < 4 * nb; t += all) form(t >> 2, t & 3, false);
+      break;
+    }
+    if (rank == 0 && warp < 4) {
+      double acc[4][2];
+      const double* blk = block(k + 1, k + 1);
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const double2 v = __ldcg(reinterpret_cast<const double2*>(blk + tf_at(8 * warp + fr, 8 * y + 2 * fk)));
+        acc[y][0] = v.x; acc[y][1] = v.y;
+      }
+      if (k >= 0) {
+        form(k + 1, warp, true);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+        for (int kk = 0; kk < NB; kk += 4) {
+          const double a = -Sc[(8 * warp + fr) * LD + kk + fk];
+#pragma unroll
+          for (int y = 0; y < 4; ++y)
+            if (y <= warp) tf_dmma(acc[y], a, Sc[(8 * y + fr) * LD + kk + fk]);
+        }
+      }
+#pragma unroll
+      for (int y = 0; y < 4; ++y)
+        *reinterpret_cast<double2*>(W + (8 * warp + fr) * LD + 8 * y + 2 * fk) = make_double2(acc[y][0], acc[y][1]);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+    }
+    if (chain_side) {
+      tf_cluster_arrive();
+      if (warp == 0) tf_diagonal(W, tiny, I8, Inv0 + ((k + 1) & 1) * NB * LD, lane);
+      tf_cluster_wait();
+    } else {
+      if (k >= 0)
+        for (int t = share; t < 4 * (nb - 1); t += sharers) form((t >> 2) > k ? (t >> 2) + 1 : t >> 2, t & 3, false);
+      tf_cluster_arrive();
+      tf_cluster_wait();
+      // block (i, j) -= S_i S_j^T; block column k starts from zero (its old contents were the panel)
+      const int t0 = (k + 1) * (k + 2) / 2, t1 = nb * (nb + 1) / 2, td = t0 + k + 1;   // td: block (k + 1, k + 1)
+      for (int t = k >= 0 ? t0 + share : t1; t < t1; t += sharers) {
+        if (t == td) continue;
+        int i = static_cast<int>((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+        while ((i + 1) * (i + 2) / 2 <= t) ++i;
+        while (i * (i + 1) / 2 > t) --i;
+        const int j = t - i * (i + 1) / 2;
+        double* blk = block(i, j);
+        double acc[4][4][2];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const double2 v = j == k ? make_double2(0.0, 0.0) : __ldcg(reinterpret_cast<const double2*>(blk + tf_at(8 * x + fr, 8 * y + 2 * fk)));
+            acc[x][y][0] = v.x; acc[x][y][1] = v.y;
+          }
+        const double *Si = S + i * NB * LD + fr * LD + fk, *Sj = S + j * NB * LD + fr * LD + fk;
+#pragma unroll
+        for (int k0 = 0; k0 < NB; k0 += 4) {
+          double a[4], b[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) { a[x] = -__ldcg(Si + 8 * x * LD + k0); b[x] = __ldcg(Sj + 8 * x * LD + k0); }
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            if (j == k && k0 < 8 * y) continue;     // (S_k is the transpose of Inv, upper triangular)
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              if (x >= y || i != j) tf_dmma(acc[x][y], a[x], b[y]);   // (the upper part of a diagonal block is not used)
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y)
+            *reinterpret_cast<double2*>(blk + tf_at(8 * x + fr, 8 * y + 2 * fk)) = make_double2(acc[x][y][0], acc[x][y][1]);
+      }
+    }
+    tf_cluster_arrive();
+    tf_cluster_wait();
+  }
+  // (the first CTA stays until nobody reads its shared memory any more)
+  tf_cluster_arrive();
+  tf_cluster_wait();
+}
+
 constexpr int kTfSmemLimit = 232448 - 256;   // (the kernel has 128 bytes of its own)
 
+inline size_t tf_cluster_smem(int l_max) {
+  return sizeof(double) * (4 * kTfNB * kTfLd + 8 * kTfLdS8 + static_cast<size_t>((l_max + kTfNB - 1) / kTfNB) * kTfNB);
+}
+inline void tf_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int n, int cluster, int l_max) {
+  cfg.gridDim = n * cluster;
+  cfg.blockDim = kTfThreads;
+  cfg.dynamicSmemBytes = tf_cluster_smem(l_max);
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = cluster; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+}
+// CTAs that factor a matrix together, for n matrices, the widest l_max wide: four or two where all matrices still go at once (a cluster
+// has its SMs in one group of them, so that 148 SMs hold fewer than 37 clusters of four; 37 matrices of 480 columns in two waves 8.4 ms a
+// refresh, with one CTA each 7.8) and are so wide that it pays: refresh, one CTA / a cluster, nine matrices of 196 columns 2.24 / 2.23
+// ms, of 256 3.06 / 2.97, of 416 5.24 / 4.19, three of 512 7.13 / 4.80; pairs, 74 of 256 4.40 / 4.40, of 328 6.36 / 6.11, 60 of 480 8.99 / 8.21.
+inline int tf_cluster(int n, int l_max) {
+  if (l_max <= kTfClusterFrom) return 1;
+  for (int c = kTfClusterMax; c > 1; c /= 2) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    tf_cluster_config(cfg, attr, n, c, l_max);
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, tri_factor_cluster_kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    if (n <= fit) return c;
+  }
+  return 1;
+}
+
 // Factor n matrices, the widest l_max wide (widest first in the list: CTAs are handed out in order).  shift_scale: what
-// is added to the unit diagonal, for fp32 matrices in units of L / 65536.  dependent: launched as a programmatic dependent.
+// is added to the unit diagonal, for fp32 matrices in units of L / 65536.  dependent: launched as a programmatic dependent.  cluster: CTAs to a
+// matrix (tf_cluster; more than one: work and spill hold all blocks and rows of S of every matrix).
 inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, double shift_scale, cudaStream_t stream,
-                                     int64_t* launches, bool conditional = false, bool dependent = false) {
+                                     int64_t* launches, bool conditional = false, bool dependent = false, int cluster = 1) {
   // as much shared memory as the widest matrix that fits with its blocks, and at least what the widest needs without
   size_t smem = tf_base_smem(l_max, false);
   const bool s_global = smem > static_cast<size_t>(kTfSmemLimit);
@@ -407,6 +651,18 @@ inline cudaError_t tri_factor_launch(const FactorMat* d_mats, int n, int l_max, 
   for (int l = l_max; l > 0; l -= 4) {
     const size_t need = tf_base_smem(l, s_global) + tf_block_bytes(l);
     if (need <= static_cast<size_t>(kTfSmemLimit)) { smem = need > smem ? need : smem; break; }
+  }
+  if (cluster > 1) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[2]{};
+    tf_cluster_config(cfg, attr[0], n, cluster, l_max);
+    cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 2 : 1;
+    *launches += 1;
+    return cudaLaunchKernelEx(&cfg, tri_factor_cluster_kernel, d_mats, cluster, shift_scale, conditional ? 1 : 0);
   }
   // (the limit to its largest value, since it belongs to the process and not to one state, and here, so that only a kernel
   // that is launched gets loaded)
