@@ -286,7 +286,7 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar + s, 1); mbar_init(empty_bar + s, 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, EPI == TC_EPI_PROJECT ? NEPI : 4 * MT); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar + b, 1); mbar_init(tempty_bar + b, NEPI); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -413,25 +413,23 @@ tc_gemm_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __restrict__
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2 .. 2 + NEPI - 1)
-    // With 8 epilogue warps there are two groups of four; group g drains accumulator buffer g, i.e. the
-    // tiles with (local & 1) == g.  That is for tiles of few K blocks, whose epilogue takes longer than their MMAs
-    // (Q = Y R^-1 of the refresh, K = r': 58 matrices of r' = 128 33 -> 25 us, 84 of r' = 256 81 -> 67 us).
+    // With 8 epilogue warps there are two groups of four, which share a tile: its halves where it is 256 rows tall, else every second 32
+    // columns.  That is for tiles of few K blocks, whose epilogue takes longer than their MMAs (Q = Y R^-1 of the refresh, K = r': 58
+    // matrices of r' = 128 33 -> 25 us, 84 of r' = 256 81 -> 67 us), and because what a CTA does last is to drain a tile, 6 us for 256
+    // columns with four warps: step's projection, 60M shapes 199.4 -> 195.8 us a step, one 512 x 1376 matrix 21.1 -> 20.4, encoder
+    // shapes at r = 8 167.5 -> 165.5, 288-wide layers under the short-side rule 76.7 -> 73.1; 130M and more as before.  Kernels of a refresh,
+    // where the groups used to take tiles in turn, or there was one: 60M shapes 2094 -> 2047, 824-wide layers at r = 48 820 -> 795.
     const int quarter = warp & 3;  // TMEM lanes 32 * quarter .. + 31 belong to this warp
     constexpr int kGroups = NEPI / 4;
     const int group = (warp - 2) >> 2;
     float* stg = reinterpret_cast<float*>(smem + STAGES * L::kStageBytes + (warp - 2) * L::kEpiWarpBytes);
     bool ok = true, cleared = EPI != TC_EPI_PROJECT || n_clear == 0;
     if (!cleared) clear_split_slots(mats, clear, n_clear, ctrl);
-    // (of tall tiles, each group drains its half of all of them; of the step's projection, every second 32 columns: what a CTA does
-    // last is to drain a tile, 6 us for 256 columns with four warps.  60M shapes 199.4 -> 195.8 us a step, one 512 x 1376 matrix
-    // 21.1 -> 20.4, encoder shapes at r = 8 167.5 -> 165.5, 288-wide layers under the short-side rule 76.7 -> 73.1; 130M and more as before)
-    constexpr bool kShareTile = EPI == TC_EPI_PROJECT && kGroups == 2;
-    constexpr int kStep = MT == 2 || kShareTile ? 1 : kGroups;
-    const int first = kStep == 2 ? group : 0, half = MT == 2 ? group : 0;
+    constexpr bool kShareTile = MT == 1 && kGroups == 2;
+    const int half = MT == 2 ? group : 0;
     TcTile tile = tile0;
-    if (first > 0 && t_begin + first < t_end) tile = tiles[t_begin + first];
-    for (int local = first; t_begin + local < t_end && ok; local += kStep) {
-      const TcTile next = tiles[min(t_begin + local + kStep, t_end - 1)];
+    for (int local = 0; t_begin + local < t_end && ok; ++local) {
+      const TcTile next = tiles[min(t_begin + local + 1, t_end - 1)];
       float* out;
       __nv_bfloat16 *out_hi = nullptr, *out_lo = nullptr;
       int rows_total, out_cols, ld_out, ld16 = 0;

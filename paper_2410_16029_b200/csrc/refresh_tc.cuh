@@ -353,7 +353,7 @@ constexpr int kRefWideBN = 256;
 // A product with G (one part of A, NB parts of B): 192 KB of stages, as many as go.
 template <int BN, int NB, int MT, bool MN>
 struct RefProduct {
-  static constexpr int kEpiWarps = 4 * MT, kThreads = 64 + 32 * kEpiWarps;
+  static constexpr int kEpiWarps = 8, kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kStages = 192 / (16 * MT + NB * BN / 8);
   static constexpr int kSmem = TcSmem<BN, 1, NB, kStages, kEpiWarps, MT>::kTotal;
   static constexpr auto kernel = tc_gemm_kernel<BN, 1, NB, kStages, TC_EPI_STORE, kEpiWarps, MN, false, MT>;
