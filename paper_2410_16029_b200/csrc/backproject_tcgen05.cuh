@@ -225,7 +225,15 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
         }
         for (int c = 0; c < wchunks; ++c) {
           if ((c & 1) == parity) {
-            if (!__all_sync(0xffffffffu, mbar_wait(wfull_bar + slot, phase, abort_flag))) { ok = false; break; }
+            // The slot's previous use may have been the other group's (a tile with an odd number of chunks, or five slots), and its load
+            // still on the way while those of later chunks have landed: one phase bit cannot tell that from this chunk's arrival, and a
+            // warp that took the slot then would store what is not there and release it while its barrier expects no one (an
+            // unspecified launch failure, 1312-column matrices at r = 37, ten thousand tiles a step).  So first that use has been released
+            // (at most 0.3 % of a step).
+            if (!__all_sync(0xffffffffu, mbar_wait(wempty_bar + slot, phase ^ 1u, abort_flag) && mbar_wait(wfull_bar + slot, phase, abort_flag))) {
+              ok = false;
+              break;
+            }
             uint32_t r[32];
             tc_ld32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * kBpBN + c * 32), r);
             tc_wait_ld();
