@@ -230,7 +230,7 @@ ngalore_status ngalore_stream_wait_update(ngalore_state* st, int g, void* stream
 /*
  * Testing aid (no counterpart in the paper): in the next ngalore_step only, the solved weights of matrix
  * `matrix_index` are computed but not announced, and the tiles that wait for them give up after `polls` polls
- * (1 .. 1000000, about 100 ns each) instead of the default limit.  The step then ends normally with
+ * (1 .. 1000000, about 0.3 us each) or, with 0, after the 0.9 s after which they give up by themselves.  The step then ends normally with
  * NGALORE_ERR_TIMEOUT in that matrix's status word and its W unchanged; the following step is a regular one.
  * This is how the tests exercise a bounded wait that runs out; nothing hangs or traps.  Synchronises the device.
  * Not available with s = 0, stream_impl = 1, or for a matrix whose Gram row is formed by gram_fusion.

@@ -57,7 +57,7 @@ struct Ctrl {
   // Testing aids, both cleared at the end of every step.  They exist so that a test can make a bounded wait run
   // out without hanging or trapping anything: the solution of one matrix is computed but not published, and the
   // tiles that wait for it give up after a few polls.
-  int spin_limit;             // > 0: polls before a flag wait of the stream kernel is abandoned (0: the default)
+  int spin_limit;             // > 0: polls before a wait for weights is abandoned (0: after a time, like everywhere else)
   int debug_withhold;         // > 0: the weights of matrix (debug_withhold - 1) are not published in this step
 };
 
@@ -131,6 +131,12 @@ inline cudaError_t launch_step(bool dependent, void (*kernel)(P...), dim3 grid, 
   cfg.attrs = &attr;
   cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+__device__ __forceinline__ unsigned long long global_timer_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
 }
 
 struct StreamTile {

@@ -53,7 +53,13 @@ struct FusedPlan {
   bool mom16 = false;   // the state keeps its moments in bf16
 };
 
-constexpr long long kSpinLimit = 4000000;  // polls of ~100 ns each before a flag wait is abandoned
+// The finishing warp's waits for what other CTAs publish, the partial rows of a matrix and its weights, in time, since what a poll takes
+// depends on what else goes on (0.33 us for a weight that nothing writes).  The consumers and the producer wait for this warp in turn, until
+// kTcWaitLimitNs, and give the whole CTA up then, with items of matrices that have nothing to do with it: so all that it may spend
+// before a combination item has its weights, the rows of two slots and the weights themselves, has to be less.  And the rows are given up before the
+// weights that depend on them, so that no solve ends after somebody has flagged its matrix.
+constexpr unsigned long long kRowsLimitNs = 300000000ull, kWeightsLimitNs = 900000000ull;
+static_assert(2 * kRowsLimitNs < kWeightsLimitNs && 2 * kRowsLimitNs + kWeightsLimitNs <= kTcWaitLimitNs / 4 * 3, "waits that depend on each other end in turn");
 
 struct StageMeta {
   int kind, last, count, pad;
@@ -249,7 +255,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const int lane = tid & 31;
     const double lambda = hyper->lambda;
     const int withheld = ctrl->debug_withhold - 1;
-    const long long limit = ctrl->spin_limit > 0 ? ctrl->spin_limit : kSpinLimit;
+    const unsigned int polls = static_cast<unsigned int>(ctrl->spin_limit);   // (testing aid; 0: the limit in time alone)
+    unsigned long long rows_limit = kRowsLimitNs;   // (what did not come in time for one matrix is not waited for again)
     bool jobs_open = true, rows_open = true;
     unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, Gram tiles and combination items so far
     auto look_after_rows = [&]() {
@@ -302,19 +309,26 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         GramSolve<SMAX> solve;
         solve.prepare(d, cur, prev, c, lambda, lane);
         double row = 0.0, rowp = 0.0;
-        if (!tagged_row_sum<SMAX>(d, lane, c, C::kRows, 0, tag, kSpinLimit, abort_flag, row, look_after_rows)) continue;   // (nobody gets weights, and says so)
-        if (HIST16 && prev >= 0 && !tagged_row_sum<SMAX>(d, lane, c, C::kRows, C::kRows - 1, tag, kSpinLimit, abort_flag, rowp, look_after_rows)) continue;
+        bool here = tagged_row_sum<SMAX>(d, lane, c, C::kRows, 0, tag, rows_limit, abort_flag, row, look_after_rows);
+        if (HIST16 && prev >= 0 && here) here = tagged_row_sum<SMAX>(d, lane, c, C::kRows, C::kRows - 1, tag, rows_limit, abort_flag, rowp, look_after_rows);
+        if (!here) { rows_limit = 0; continue; }   // (nobody gets weights, and says so)
         solve.finish(d, cur, prev, c, lambda, lane, row, rowp, tag, withheld == job.mat);
         continue;
       }
       float w;
       int ok = 1, bad;
       if (s_all > 0) {
-        unsigned long long word;
-        for (long long spins = 0;; ++spins) {
+        unsigned long long word, t0 = 0;
+        for (unsigned int spins = 0;; ++spins) {
           word = ld_relaxed(d.wpub + lane);
           if (__all_sync(0xffffffffu, static_cast<unsigned int>(word >> 32) >> 1 == (tag & 0x7fffffffu))) break;
-          if (spins >= limit) { ok = 0; break; }
+          if (polls != 0 && spins >= polls) ok = 0;
+          if ((spins & 63u) == 63u) {
+            const unsigned long long now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > kWeightsLimitNs)) ok = 0;
+          }
+          if (!ok) break;
           look_after_rows();
           if (spins > 16) __nanosleep(100);
         }

@@ -197,16 +197,18 @@ __device__ __forceinline__ void publish_weights(const MatDesc& d, int lane, floa
   st_relaxed(d.wpub + lane, tagged(__float_as_uint(w), 2u * tag + (bad ? 1u : 0u)));
 }
 
-// gram_row_sum over tagged rows ([tile][rows][s]), each waited for; sums in the same order.  False where they do not come.
+// gram_row_sum over tagged rows ([tile][rows][s]), each waited for; sums in the same order.  False where they do not come within
+// limit_ns.
 // meanwhile: what the warp does between two looks.
 template <int SMAX, typename F>
-__device__ __forceinline__ bool tagged_row_sum(const MatDesc& d, int lane, int c, int rows, int row, unsigned int tag, long long limit,
+__device__ __forceinline__ bool tagged_row_sum(const MatDesc& d, int lane, int c, int rows, int row, unsigned int tag, unsigned long long limit_ns,
                                                const volatile int* abort_flag, double& out, F&& meanwhile) {
   constexpr int G = 32 / SMAX, U = 8;   // (sixteen take the registers of eight slots and more: 0.7 us slower for one matrix)
   const ulonglong2* gp = d.grow + static_cast<long long>(row) * d.s + min(lane % SMAX, c - 1);
   const long long st = static_cast<long long>(rows) * d.s;
   double t[4] = {0.0, 0.0, 0.0, 0.0};
-  long long spins = 0;
+  unsigned int spins = 0;
+  unsigned long long begin = 0;
   for (int t0 = 0; t0 < d.ntiles; t0 += G * U) {
     unsigned long long lo[U], hi[U];
     while (true) {
@@ -216,7 +218,11 @@ __device__ __forceinline__ bool tagged_row_sum(const MatDesc& d, int lane, int c
 #pragma unroll
       for (int q = 0; q < U; ++q) here = here && static_cast<unsigned int>(lo[q] >> 32) == tag && static_cast<unsigned int>(hi[q] >> 32) == tag;
       if (__all_sync(0xffffffffu, here)) break;
-      if (__any_sync(0xffffffffu, ++spins > limit || *abort_flag != 0)) return false;
+      if ((++spins & 63u) == 0u) {
+        const unsigned long long now = global_timer_ns();
+        if (begin == 0) begin = now;
+        if (__any_sync(0xffffffffu, *abort_flag != 0 || now - begin > limit_ns)) return false;
+      }
       meanwhile();
     }
 #pragma unroll

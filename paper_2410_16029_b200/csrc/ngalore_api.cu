@@ -1258,7 +1258,7 @@ ngalore_status ngalore_stream_wait_update(ngalore_state* st, int g, void* stream
 }
 
 ngalore_status ngalore_debug_withhold_solution(ngalore_state* st, int matrix_index, int polls) {
-  if (st == nullptr || matrix_index < 0 || matrix_index >= st->n || polls < 1 || polls > 1000000) return NGALORE_ERR_INVALID_ARG;
+  if (st == nullptr || matrix_index < 0 || matrix_index >= st->n || polls < 0 || polls > 1000000) return NGALORE_ERR_INVALID_ARG;
   if (st->s < 1 || st->opt.stream_impl == 1) return NGALORE_ERR_INVALID_ARG;
   if (!st->tc.gram_fused.empty() && st->tc.gram_fused[matrix_index]) return NGALORE_ERR_INVALID_ARG;
   if (st->sr.ready) return NGALORE_ERR_INVALID_ARG;   // the small-rank path has no wait to run out
