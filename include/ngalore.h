@@ -261,7 +261,8 @@ int64_t ngalore_launch_count(const ngalore_state* st);
 int ngalore_uses_small_rank_path(const ngalore_state* st);  /* 1 if the state takes the small-rank path (see options) */
 /* Testing aid: what a state's plan chose.  what: 0 columns of a projection tile, 1 projection tiles (pieces of a split K counted),
  * 2 whether a projection splits K, 3 columns of a back-projection tile, 4 the products of a refresh with G (0: a tile to a CTA,
- * 1: two accumulators a CTA, 2: pairs of SMs, -1: no tensor-core refresh), 5 whether one of those products splits K.  -1 for any other. */
+ * 1: two accumulators a CTA, 2: pairs of SMs, -1: no tensor-core refresh), 5 whether one of those products splits K, 6 the most stream tiles that
+ * a matrix has.  -1 for any other. */
 int ngalore_debug_plan(const ngalore_state* st, int what);
 /* How many times ngalore_step had to encode and upload the TMA descriptors of a (W, G) pair of pointer arrays
  * (see ngalore_step: once per distinct pair while it stays cached). */

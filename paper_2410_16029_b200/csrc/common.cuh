@@ -44,6 +44,7 @@ struct MatDesc {
   unsigned long long* wpub;   // fused kernel: kMaxHistory tagged weights, valid once they carry this step's tag
   int tile0, ntiles;          // range of streaming tiles owned by this matrix
   int te;                     // elements of one streaming tile of this matrix (multiple of 1024)
+  int run;                    // fused kernel: elements of a tile whose products are summed in fp32 (te at most)
 };
 
 struct Ctrl {

@@ -35,14 +35,15 @@ struct __align__(16) FusedItem {
   int mat;
   int kind;        // 0 = Gram tile, 1 = combination tile
   int solve;       // a Gram tile: whether it is its matrix's last one
-  int count;       // elements
+  int count;       // elements, of a run at most
   long long e0;    // first element
   long long rn;    // elements of a history slot
   const void* hist;      // the ring: fp32, or bf16 where the state keeps its history so
   const float* current;  // bf16 history: the fp32 gradient of this step
   const void *m, *v;     // moments, fp32 or bf16
-  ulonglong2* rows;      // where the partial rows of a Gram tile go
-  long long pad;
+  uintptr_t rows;        // where the partial rows of a Gram tile go (StageMeta)
+  int rest;              // elements of a Gram tile beyond its first run: products are summed in fp32 run by run, runs in fp64
+  int pad;
 };
 
 struct FusedPlan {
@@ -62,9 +63,9 @@ constexpr unsigned long long kRowsLimitNs = 300000000ull, kWeightsLimitNs = 9000
 static_assert(2 * kRowsLimitNs < kWeightsLimitNs && 2 * kRowsLimitNs + kWeightsLimitNs <= kTcWaitLimitNs / 4 * 3, "waits that depend on each other end in turn");
 
 struct StageMeta {
-  int kind, last, count, pad;
+  int kind, last, count, pad;   // last: the sums of a Gram tile's run are complete, or a combination item is
   long long e0;
-  ulonglong2* rows;
+  uintptr_t rows;               // where the rows of the Gram tile go; odd: its next run is still to come
 };
 
 // What the finishing warp is told to do, in the order of the CTA's items: solve for a matrix, or fetch the weights of a combination item
@@ -118,7 +119,8 @@ struct FusedCfg {
   static_assert(kRedRowsOff + 16 <= kWeightsOff && kRedOff % 8 == 0, "shared memory regions overlap");
   static constexpr int kRows = HIST16 ? 2 : 1;                  // Gram rows per tile
   static constexpr int kRedDoubles = (kConsumers / 32) * SMAX;  // one Gram row per consumer warp
-  static constexpr int kTotal = kRedOff + 2 * kRows * kRedDoubles * 8;   // (two tiles in flight to the finishing warp)
+  static constexpr int kSumOff = kRedOff + 2 * kRows * kRedDoubles * 8;  // (two tiles in flight to the finishing warp)
+  static constexpr int kTotal = kSumOff + kRows * SMAX * 8;
   static_assert(kStages * sizeof(StageMeta) <= 384, "stage metadata overflows its slot");
   static_assert(kTotal <= 232448, "shared memory budget of one CTA exceeded");
 };
@@ -216,7 +218,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   ItemWeights* weights = reinterpret_cast<ItemWeights*>(fs_smem + C::kWeightsOff);  // [2]
   uint64_t* red_full = reinterpret_cast<uint64_t*>(fs_smem + C::kRedBarOff);   // [2] all consumer warps have left their sums
   uint64_t* red_empty = red_full + 2;                                           // [2] the finishing warp has taken them
-  ulonglong2** red_rows = reinterpret_cast<ulonglong2**>(fs_smem + C::kRedRowsOff); // [2] where a tile's rows go (null: there are no more)
+  uintptr_t* red_rows = reinterpret_cast<uintptr_t*>(fs_smem + C::kRedRowsOff); // [2] where a tile's rows go (StageMeta; 0: there are no more)
   double* red = reinterpret_cast<double*>(fs_smem + C::kRedOff);                // [2][rows][warps][SMAX]
 
   const int tid = threadIdx.x;
@@ -258,11 +260,13 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const unsigned int polls = static_cast<unsigned int>(ctrl->spin_limit);   // (testing aid; 0: the limit in time alone)
     unsigned long long rows_limit = kRowsLimitNs;   // (what did not come in time for one matrix is not waited for again)
     bool jobs_open = true, rows_open = true;
-    unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, Gram tiles and combination items so far
+    unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, runs of Gram tiles and combination items so far
+    double* const before = reinterpret_cast<double*>(fs_smem + C::kSumOff) + min(lane, SMAX - 1);   // where pending: the runs of the tile so far
+    bool pending = false;
     auto look_after_rows = [&]() {
       const int buf = tiles & 1;
       if (!rows_open || !__all_sync(0xffffffffu, mbar_test(red_full + buf, (tiles >> 1) & 1u))) return;
-      ulonglong2* const rows = red_rows[buf];   // [rows][s]: row of `cur` and (HIST16) of `prev`
+      const uintptr_t at = red_rows[buf];   // [rows][s]: row of `cur` and (HIST16) of `prev`
       double part[C::kRows];
 #pragma unroll
       for (int r = 0; r < C::kRows; ++r) {
@@ -275,11 +279,23 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       __syncwarp();
       if (lane == 0) mbar_arrive(red_empty + buf);
       ++tiles;
-      if (rows == nullptr) {
-        rows_open = false;
-      } else if (lane < s_all) {
+      if (pending) {
 #pragma unroll
-        for (int r = 0; r < C::kRows; ++r) st_tagged(rows + r * s_all + lane, part[r], tag);
+        for (int r = 0; r < C::kRows; ++r) part[r] += before[r * SMAX];
+        __syncwarp();
+      }
+      if (at == 0) {
+        rows_open = false;
+      } else if ((at & 1) != 0) {   // (lanes that share an address have the same sum)
+#pragma unroll
+        for (int r = 0; r < C::kRows; ++r) before[r * SMAX] = part[r];
+        pending = true;
+      } else {
+        pending = false;
+        if (lane < s_all) {
+#pragma unroll
+          for (int r = 0; r < C::kRows; ++r) st_tagged(reinterpret_cast<ulonglong2*>(at) + r * s_all + lane, part[r], tag);
+        }
       }
       __syncwarp();
     };
@@ -434,33 +450,41 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
         }
         ++step;
       };
-      const long long e1 = now.e0 + now.count;
-      for (long long e = now.e0; e < e1; e += CE) {
-        const int cnt = (e1 - e < CE) ? static_cast<int>(e1 - e) : CE;
-        int good = 1;
-        if (lane == 0) good = mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag) ? 1 : 0;
-        good = __shfl_sync(0xffffffffu, good, 0);
-        if (!good) { ok = false; break; }
-        unsigned char* sb = fs_smem + stage * C::kStageBytes;
-        const uint32_t bytes = static_cast<uint32_t>(cnt) * 4u;
-        if (lane == 0) {
-          meta[stage] = StageMeta{now.kind, e + CE >= e1 ? 1 : 0, cnt, 0, e, now.rows};
-          const uint32_t hist_bytes = HIST16 ? bytes * static_cast<uint32_t>(c) - (bytes / 2) * static_cast<uint32_t>(c - 1)
-                                             : bytes * static_cast<uint32_t>(c);
-          const uint32_t mom_bytes = now.kind == 1 ? (MOM16 ? bytes : 2u * bytes) : 0u;
-          mbar_expect_tx(full_bar + stage, hist_bytes + mom_bytes);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int k = lane + 32 * q;
-          if (k < ncopies) {
-            const int w = width(k);
-            bulk_load(sb + place(k), src[q] + e * w, static_cast<uint32_t>(cnt * w), full_bar + stage);
+      while (true) {
+        const long long e1 = now.e0 + now.count;
+        for (long long e = now.e0; e < e1; e += CE) {
+          const int cnt = (e1 - e < CE) ? static_cast<int>(e1 - e) : CE;
+          int good = 1;
+          if (lane == 0) good = mbar_wait(empty_bar + stage, phase ^ 1u, abort_flag) ? 1 : 0;
+          good = __shfl_sync(0xffffffffu, good, 0);
+          if (!good) { ok = false; break; }
+          unsigned char* sb = fs_smem + stage * C::kStageBytes;
+          const uint32_t bytes = static_cast<uint32_t>(cnt) * 4u;
+          if (lane == 0) {
+            meta[stage] = StageMeta{now.kind, e + CE >= e1 ? 1 : 0, cnt, 0, e, now.rows};
+            const uint32_t hist_bytes = HIST16 ? bytes * static_cast<uint32_t>(c) - (bytes / 2) * static_cast<uint32_t>(c - 1)
+                                               : bytes * static_cast<uint32_t>(c);
+            const uint32_t mom_bytes = now.kind == 1 ? (MOM16 ? bytes : 2u * bytes) : 0u;
+            mbar_expect_tx(full_bar + stage, hist_bytes + mom_bytes);
           }
+          __syncwarp();
+  #pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int k = lane + 32 * q;
+            if (k < ncopies) {
+              const int w = width(k);
+              bulk_load(sb + place(k), src[q] + e * w, static_cast<uint32_t>(cnt * w), full_bar + stage);
+            }
+          }
+          if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
+          look_ahead();
         }
-        if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
-        look_ahead();
+        // (the next run of the tile, like one of its own to the consumers)
+        if (!ok || now.rest == 0) break;
+        now.e0 += now.count;
+        now.count = min(now.count, now.rest);
+        now.rest -= now.count;
+        if (now.rest == 0) now.rows &= ~static_cast<uintptr_t>(1);
       }
       if (!ok) break;
       while (step < 2) look_ahead();
@@ -475,14 +499,14 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const int idx = tid * VEC;     // this thread's elements of a stage
     int stage = 0;
     uint32_t phase = 0;
-    unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
+    unsigned int tiles_done = 0;   // runs of Gram tiles handed to the finishing warp
     unsigned int combined = 0;     // combination items whose weights have been taken
     const unsigned int it_step = static_cast<unsigned int>(ctrl->k);
     // Tells the finishing warp that the CTA has no more Gram tiles (all of them are ahead of the combination items), as soon as that is
     // known: at the end of the kernel it would be the last thing everybody waits for.
     bool gram_open = true;
     auto close_gram = [&]() {
-      if (tid == 0) red_rows[tiles_done & 1] = nullptr;
+      if (tid == 0) red_rows[tiles_done & 1] = 0;
       __syncwarp();
       if (lane == 0) mbar_arrive(red_full + (tiles_done & 1));
       gram_open = false;
@@ -540,7 +564,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       }
       bool alive = true;
       if (mt.kind == 0) {
-        // ---- Gram tile
+        // ---- Gram tile, or a run of one
         const int buf = tiles_done & 1;
         // this warp's sums of row r over its lanes, into the buffer of the finishing warp
         auto hand_over = [&](int r, double (&v)[SMAX]) {
@@ -804,7 +828,8 @@ inline ngalore_status fused_plan_create(FusedPlan& plan, const std::vector<MatDe
     o.current = d.H;
     o.m = plan.mom16 ? static_cast<const void*>(d.m16) : static_cast<const void*>(d.m);
     o.v = plan.mom16 ? static_cast<const void*>(d.v16) : static_cast<const void*>(d.v);
-    o.rows = d.grow + static_cast<long long>(t) * (plan.hist16 ? 2 : 1) * s;
+    o.rows = reinterpret_cast<uintptr_t>(d.grow + static_cast<long long>(t) * (plan.hist16 ? 2 : 1) * s);
+    if (kind == 0 && o.count > d.run) { o.rest = o.count - d.run; o.count = d.run; o.rows |= 1; }
     items.push_back(o);
   };
   for (int i = 0; i < n; ++i) {

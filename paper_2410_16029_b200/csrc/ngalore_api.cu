@@ -649,6 +649,18 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
       acc += st->mats[i].rn;
     }
   }
+  // And no matrix has more than six of them for every SM, or three with a bf16 history (two partial rows a tile): the warp that solves for it
+  // reads the rows of all after the last one, 16 tiles a look of 0.7 us (8 for s > 16, 32 up to 8), and in a set of one or a few such
+  // matrices nothing else goes on meanwhile.  Step without / with this limit, us, r = 512: one 2048 x 32000 matrix, s = 16 655 / 600; 64000
+  // columns, s = 24 1799 / 1531; 128000 columns, s = 16 2540 / 2238, s = 8 1666 / 1660, with 16-bit state 2150 / 1700; seven layers of width 2048 before
+  // one of 32000 columns, bf16 history, 875 / 730.  Stream phase of the first with four, five, six, seven and ten a SM 383 / 373 / 375 / 392 / 414 (six: a
+  // multiple of the SMs also where tiles are long: 128000 columns 1553 / 1402 / 1383 / 1414 / 1451); two, three and four with a bf16 history 266 / 266 /
+  // 289, 128000 columns 1144 / 861 / 1023.
+  // A longer tile is summed in runs of what the rules above say, so that no more products meet in fp32.  (The plain kernels have no runs.)
+  const std::vector<int> run_elems = tile_elems;
+  const long long most = (st->opt.history_bf16 == 1 ? 3 : 6) * prop.multiProcessorCount;
+  for (int i = 0; s > 0 && st->opt.stream_impl != 1 && i < n_matrices; ++i)
+    tile_elems[i] = static_cast<int>(std::max<long long>(tile_elems[i], ((st->mats[i].rn + most - 1) / most + 1023) / 1024 * 1024));
 
   // ---- arena layout
   const int slots = s > 0 ? s : 1;
@@ -780,7 +792,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     d.step_bad = st->d_step_bad + i;
     d.wpub = reinterpret_cast<unsigned long long*>(st->work + o_wpub[i]);
     d.grow = reinterpret_cast<ulonglong2*>(st->work + o_grow[i]);
-    d.tile0 = tile0[i]; d.ntiles = ntl[i]; d.te = tile_elems[i];
+    d.tile0 = tile0[i]; d.ntiles = ntl[i]; d.te = tile_elems[i]; d.run = run_elems[i];
     hm.Ya = reinterpret_cast<float*>(st->work + woffs[i].Ya);
     hm.Yb = reinterpret_cast<float*>(st->work + woffs[i].Yb);
     hm.Xa = reinterpret_cast<float*>(st->work + woffs[i].Xa);
@@ -1300,6 +1312,7 @@ int ngalore_debug_plan(const ngalore_state* st, int what) {
     case 3: return st->tc.back_bn;
     case 4: return !st->refresh.ready ? -1 : (st->refresh.pair ? 2 : (st->refresh.tall ? 1 : 0));
     case 5: return !st->refresh.ready ? -1 : (st->refresh.atomic_mats[RG_Y_FROM_Z].empty() && st->refresh.atomic_mats[RG_Z_FROM_Y].empty() ? 0 : 1);
+    case 6: { int most = 0; for (const MatDesc& d : st->h_desc) most = std::max(most, d.ntiles); return most; }
   }
   return -1;
 }

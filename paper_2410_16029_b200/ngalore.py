@@ -270,7 +270,7 @@ class NGaLore:
     def debug_plan(self, what: str) -> int:
         """Testing aid: what the state's plan chose (see include/ngalore.h)."""
         return _lib.ngalore_debug_plan(self._h, ("projection_columns", "projection_tiles", "projection_splits", "update_columns",
-                                                 "refresh_products", "refresh_splits").index(what))
+                                                 "refresh_products", "refresh_splits", "stream_tiles").index(what))
 
     def set_lr(self, lr: float):
         _check(_lib.ngalore_set_lr(self._h, lr), "ngalore_set_lr")
