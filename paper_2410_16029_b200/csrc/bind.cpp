@@ -21,6 +21,14 @@ bool device_ok(const at::Tensor& t, at::ScalarType dtype, const int64_t* shape) 
   return t.is_cuda() && t.scalar_type() == dtype && t.dim() == 2 && t.size(0) == shape[0] && t.size(1) == shape[1] && t.is_contiguous();
 }
 
+// A buffer that a step on host memory reads and writes as rows x cols floats or bf16 values, whatever its shape: it has to hold that many.
+// (Gradients may come as the bits of their values.)
+bool host_ok(const at::Tensor& t, bool weights, const int64_t* shape) {
+  const at::ScalarType type = t.scalar_type();
+  const bool typed = weights ? type == at::kFloat : type == at::kBFloat16 || type == at::kShort || type == at::kUInt16;
+  return t.is_cpu() && typed && t.is_contiguous() && t.numel() >= shape[0] * shape[1];
+}
+
 // collect(W, G, n, shapes, W_out, G_out, mode): shapes, W_out and G_out are addresses (2 n int64, n pointers each).  True: the pointers are
 // there.  False: something else than n plain tensors each, which the caller has to look at itself.  AssertionError: a tensor that
 // is not what a step takes.
@@ -44,8 +52,8 @@ PyObject* collect(PyObject*, PyObject* args) {
         PyErr_Format(PyExc_AssertionError, "matrix %zd: a step takes contiguous CUDA tensors of its shape, W float32 and G bfloat16", i);
         return nullptr;
       }
-      if (mode == kHost && (w->is_cuda() || g->is_cuda() || !w->is_contiguous() || !g->is_contiguous())) {
-        PyErr_Format(PyExc_AssertionError, "matrix %zd: a step on host buffers takes contiguous CPU tensors", i);
+      if (mode == kHost && !(host_ok(*w, true, shapes + 2 * i) && host_ok(*g, false, shapes + 2 * i))) {
+        PyErr_Format(PyExc_AssertionError, "matrix %zd: a step on host buffers takes contiguous CPU tensors of its size, W float32 and G bfloat16", i);
         return nullptr;
       }
       w_out[i] = w->data_ptr();

@@ -129,6 +129,19 @@ def _ptr_array(tensors: Sequence[torch.Tensor]):
     return arr
 
 
+def _check_buffers(shapes, W, G, host: bool) -> None:
+    """A pointer for every matrix and, for a step on host buffers, as many values behind it as the step reads and writes."""
+    n = len(shapes)
+    if len(W) < n or len(G) < n:
+        raise AssertionError(f"a step takes W and G of all {n} matrices, not of {len(W)} and {len(G)}")
+    bits = (torch.bfloat16, torch.int16, torch.uint16)
+    for i, ((M, N), w, g) in enumerate(zip(shapes, W, G) if host else ()):
+        if not (all(t.device.type == "cpu" and t.is_contiguous() and t.numel() >= M * N for t in (w, g))
+                and w.dtype == torch.float32 and g.dtype in bits):
+            raise AssertionError(f"matrix {i}: a step on host buffers takes contiguous CPU tensors of its size, "
+                                 "W float32 and G bfloat16")
+
+
 class NGaLore:
     """Optimizer state for a list of (rows, cols) weight matrices on the current CUDA device."""
 
@@ -177,9 +190,8 @@ class NGaLore:
         # not two lists of plain tensors: other sequences, tensor subclasses
         if mode == 1:
             self._check_WG(W, G)
-        elif mode == 2:
-            for x, y in zip(W, G):
-                assert not x.is_cuda and not y.is_cuda and x.is_contiguous() and y.is_contiguous()
+        else:
+            _check_buffers(self.shapes, W, G, host=mode == 2)
         return _ptr_array(W), _ptr_array(G)
 
     # -- the three calls of the optimizer -------------------------------------------
