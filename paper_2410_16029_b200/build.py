@@ -25,8 +25,25 @@ def _sources():
     return [os.path.join(d, f) for f in os.listdir(d) if f.endswith((".cu", ".cuh"))] + [inc]
 
 
+def _bind_stamp() -> str:
+    """What _bind.so depends on beside its source."""
+    import torch
+
+    return "torch %s, Python %s" % (torch.__version__, ".".join(map(str, sys.version_info[:3])))
+
+
+def _bind_current(out: str, stamp: str) -> bool:
+    """Whether `out` is newer than its source and was built with what `stamp` says."""
+    try:
+        with open(out + ".stamp") as f:
+            return f.read() == stamp and os.path.getmtime(out) >= os.path.getmtime(BIND_SRC)
+    except OSError:
+        return False
+
+
 def _build_bind(force: bool) -> None:
-    if not force and os.path.exists(BIND_OUT) and os.path.getmtime(BIND_OUT) >= os.path.getmtime(BIND_SRC):
+    stamp = _bind_stamp()
+    if not force and _bind_current(BIND_OUT, stamp):
         return
     import torch
 
@@ -38,6 +55,8 @@ def _build_bind(force: bool) -> None:
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("host compiler failed: " + " ".join(cmd))
+    with open(BIND_OUT + ".stamp", "w") as f:
+        f.write(stamp)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:

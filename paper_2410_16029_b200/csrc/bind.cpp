@@ -4,6 +4,7 @@
 #include <Python.h>
 
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/version.h>
 
 namespace {
 
@@ -71,4 +72,12 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_bind", nullptr, -1, methods, null
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__bind() { return PyModule_Create(&module); }
+// (built_for: the tensor's layout that is compiled in belongs to one torch and one Python, see ngalore.py)
+PyMODINIT_FUNC PyInit__bind() {
+  PyObject* m = PyModule_Create(&module);
+  if (m != nullptr && PyModule_AddObject(m, "built_for", Py_BuildValue("(sii)", TORCH_VERSION, PY_MAJOR_VERSION, PY_MINOR_VERSION)) != 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}

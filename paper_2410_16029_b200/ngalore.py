@@ -1,13 +1,16 @@
-"""Thin ctypes binding over the C-ABI library ``libngalore.so`` (see include/ngalore.h).
+"""Binding over the C-ABI library ``libngalore.so`` (see include/ngalore.h): ctypes, and ``_bind.so`` for the
+pointers of a step's tensors.
 
 Argument marshalling only: every step of the optimizer runs in the library's
 CUDA kernels.  torch is used for device memory and streams.  Importing this
-module fails loudly when the library has not been built; there is no fallback.
+module fails loudly when either has not been built, or ``_bind.so`` was for
+another torch or Python; there is no fallback.
 """
 from __future__ import annotations
 
 import ctypes
 import os
+import sys
 from typing import List, Optional, Sequence
 
 import torch
@@ -15,14 +18,28 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libngalore.so")
 
-if not os.path.exists(LIB_PATH):
-    raise ImportError(
-        f"{LIB_PATH} is missing: build it first (python -c 'import __graft_entry__ as g; g.build()' "
+_HOW = ("build it first (python -c 'import __graft_entry__ as g; g.build()' "
         "or python -m paper_2410_16029_b200.build). There is no CPU fallback.")
+
+if not os.path.exists(LIB_PATH):
+    raise ImportError(f"{LIB_PATH} is missing: {_HOW}")
 
 _lib = ctypes.CDLL(LIB_PATH)
 
-from . import _bind  # noqa: E402  (built with the library; missing, it fails here)
+try:
+    from . import _bind  # noqa: E402
+except ImportError as e:
+    raise ImportError(f"{os.path.join(_HERE, '_bind.so')} is missing or does not fit this torch and Python ({e}): {_HOW}") from e
+
+
+def _check_built_for(built_for) -> None:
+    """The layout of a tensor that is compiled into _bind.so is that of one torch, its module object that of one Python."""
+    here = (torch.__version__.split("+")[0], *sys.version_info[:2])
+    if tuple(built_for) != here:
+        raise ImportError(f"_bind.so was built for torch and Python {tuple(built_for)}, this is {here}: {_HOW}")
+
+
+_check_built_for(getattr(_bind, "built_for", ()))
 
 OK = 0
 STATUS_NAMES = {0: "OK", 1: "INVALID_ARG", 2: "ALLOC", 3: "CUDA", 4: "UNSUPPORTED_DEVICE", 5: "NO_SUBSPACE",
