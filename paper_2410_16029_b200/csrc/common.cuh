@@ -37,10 +37,10 @@ struct MatDesc {
   float* P32;                 // fp32 master of the projector, pr x rp row-major
   double* Kraw;               // s x s raw inner products <H_i, H_j>
   float* wsol;                // kMaxHistory solution weights of (lambda I + K) w = e_cur
-  double* gpart;              // per-tile partial Gram rows: ntiles x s
+  double* gpart;              // plain kernels: per-tile partial Gram rows, ntiles x s
   int* status;                // sticky ngalore_status word
   int* step_bad;              // 1 when this step must leave W, m, v untouched
-  ulonglong2* grow;           // fused kernel: the same rows as tagged words (kernels_stream.cuh)
+  ulonglong2* grow;           // fused kernel: such rows as tagged words (kernels_stream.cuh), two a tile with a bf16 history
   unsigned long long* wpub;   // fused kernel: kMaxHistory tagged weights, valid once they carry this step's tag
   int tile0, ntiles;          // range of streaming tiles owned by this matrix
   int te;                     // elements of one streaming tile of this matrix (multiple of 1024)

@@ -468,7 +468,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
             mbar_expect_tx(full_bar + stage, hist_bytes + mom_bytes);
           }
           __syncwarp();
-  #pragma unroll
+#pragma unroll
           for (int q = 0; q < 2; ++q) {
             const int k = lane + 32 * q;
             if (k < ncopies) {

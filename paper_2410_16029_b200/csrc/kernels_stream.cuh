@@ -57,14 +57,14 @@ __device__ __forceinline__ void gram_tile(const MatDesc& d, int local, int cur, 
 }
 
 // Lane j's share of the Gram row (zero from lane c on): the sum over the matrix's tiles of partial product j, in a fixed
-// order, so that the result is reproducible.  rows: partial rows per tile, row: which of them.
+// order, so that the result is reproducible.
 // The partial rows of early tiles have left L2 by then, so it is the number of loads under way that decides: 32 / SMAX lanes
 // share a column, sixteen loads each (352 tiles, s = 16: 37 us with one lane a column and eight loads, 19 us so).
 template <int SMAX>
-__device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c, int rows = 1, int row = 0) {
+__device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c) {
   constexpr int G = 32 / SMAX, U = 16;
-  const double* gp = d.gpart + static_cast<long long>(row) * d.s + min(lane % SMAX, c - 1);
-  const long long st = static_cast<long long>(rows) * d.s;
+  const double* gp = d.gpart + min(lane % SMAX, c - 1);
+  const long long st = d.s;
   double t[4] = {0.0, 0.0, 0.0, 0.0};
   for (int t0 = 0; t0 < d.ntiles; t0 += G * U) {
     double x[U];
@@ -95,10 +95,8 @@ __device__ __forceinline__ double gram_row_sum(const MatDesc& d, int lane, int c
 // together by a shuffle that all of them take part in: each one then costs two turns of the scheduler, 500 cycles instead of
 // 30 (one 1024 x 1024 matrix, s = 20: 125 us a solve, 10 so).  So nothing ahead of the elimination, here and in
 // gram_row_sum, branches on the lane, and what is stored is stored after it.
-// have_prev: lane j also holds <H_prev, H_j> for the slot that was current one step ago (bf16 history).
 template <int SMAX>
-__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double row,
-                                             bool have_prev = false, int prev = 0, double rowp = 0.0) {
+__device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, double lambda, double row) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
   double a[SMAX];
@@ -108,17 +106,6 @@ __device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, d
     for (int j = 0; j < SMAX; ++j) {
       const double v = __ldcg(old + min(j, c - 1));
       a[j] = lane < c && j < c ? v : 0.0;
-    }
-  }
-  // row and column `prev` against the stored (rounded) values; the entry with `cur` follows below
-  const int use = have_prev && lane < c && lane != cur && isfinite(rowp) ? 1 : 0;
-  if (have_prev) {
-#pragma unroll
-    for (int j = 0; j < SMAX; ++j) {
-      const double v = __shfl_sync(0xffffffffu, rowp, j);
-      const int uj = __shfl_sync(0xffffffffu, use, j);
-      a[j] = lane == prev && uj ? v : a[j];
-      a[j] = j == prev && use ? rowp : a[j];
     }
   }
   const bool finite = __all_sync(0xffffffffu, lane >= c || isfinite(row));
@@ -150,11 +137,6 @@ __device__ __forceinline__ void solve_matrix(const MatDesc& d, int cur, int c, d
     b -= f * __shfl_sync(0xffffffffu, b, k);
   }
   d.wsol[lane] = bad == 0 && lane < c ? static_cast<float>(b / diag) : 0.f;
-  if (use) {
-    d.Kraw[prev * d.s + lane] = rowp;
-    d.Kraw[lane * d.s + prev] = rowp;
-  }
-  __syncwarp();
   // (where the step is flagged the poisoned slot becomes a zero gradient: its Gram row and column vanish)
   if (lane < (bad != 0 ? d.s : c)) {
     d.Kraw[cur * d.s + lane] = bad != 0 ? 0.0 : val;
@@ -197,7 +179,7 @@ __device__ __forceinline__ void publish_weights(const MatDesc& d, int lane, floa
   st_relaxed(d.wpub + lane, tagged(__float_as_uint(w), 2u * tag + (bad ? 1u : 0u)));
 }
 
-// gram_row_sum over tagged rows ([tile][rows][s]), each waited for; sums in the same order.  False where they do not come within
+// gram_row_sum over tagged rows ([tile][rows][s]; row: which of them), each waited for; sums in the same order.  False where they do not come within
 // limit_ns.
 // meanwhile: what the warp does between two looks.
 template <int SMAX, typename F>

@@ -711,7 +711,7 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
     for (int t = 0; t < ntl[i]; ++t) tiles.push_back(StreamTile{i, t});
     n_tiles += ntl[i];
     woffs[i].u16 = take(sizeof(__half) * hm.rn);
-    woffs[i].gpart = take(sizeof(double) * ntl[i] * slots * (hist16 ? 2 : 1));
+    woffs[i].gpart = take(st->opt.stream_impl == 1 ? sizeof(double) * ntl[i] * slots : 0);
     woffs[i].Rcur = hist16 ? take(sizeof(float) * hm.rn) : 0;
     woffs[i].Ya = take(sizeof(float) * hm.eM * ((hm.rp + 7) / 8 * 8));   // (also two bf16 parts with padded rows)
     woffs[i].Yb = take(sizeof(float) * hm.eM * hm.rp);

@@ -27,3 +27,16 @@ def test_tiles_of_a_large_matrix_are_bounded(shapes, s, kw, per_sm):
 def test_steps_of_a_large_matrix_agree_with_64_bits(s, rounded):
     worst, scale = largest_errors(BEHIND, 256, s, s + 2, rounded)
     assert worst <= 1.0 and scale <= 1.0
+
+
+def test_rows_of_the_plain_kernels_are_not_held_beside_them():
+    """A state holds the partial Gram rows that its kernels use: 16 bytes an entry in the stream kernel, and 8 more for the plain ones only."""
+    from paper_2410_16029_b200.ngalore import NGaLore
+
+    shapes, s = [(256, 24 * 1024)], 16          # 6 M elements, at least 700 tiles of 8192
+    held = []
+    for kw in ({}, {"stream_impl": 1}):
+        opt = NGaLore(shapes, 256, s, 0, **kw)
+        held.append((opt.device_bytes, opt.debug_plan("stream_tiles")))
+        opt.close()
+    assert held[0][1] == held[1][1] and held[1][0] - held[0][0] >= 8 * s * held[0][1]
