@@ -21,6 +21,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/ngalore.h"
@@ -52,6 +53,7 @@ struct FusedPlan {
   int grid = 0;
   bool hist16 = false;  // the state keeps its history ring in bf16
   bool mom16 = false;   // the state keeps its moments in bf16
+  bool runs = false;    // some Gram tile has more than one run
 };
 
 // The finishing warp's waits for what other CTAs publish, the partial rows of a matrix and its weights, in time, since what a poll takes
@@ -119,8 +121,7 @@ struct FusedCfg {
   static_assert(kRedRowsOff + 16 <= kWeightsOff && kRedOff % 8 == 0, "shared memory regions overlap");
   static constexpr int kRows = HIST16 ? 2 : 1;                  // Gram rows per tile
   static constexpr int kRedDoubles = (kConsumers / 32) * SMAX;  // one Gram row per consumer warp
-  static constexpr int kSumOff = kRedOff + 2 * kRows * kRedDoubles * 8;  // (two tiles in flight to the finishing warp)
-  static constexpr int kTotal = kSumOff + kRows * SMAX * 8;
+  static constexpr int kTotal = kRedOff + 2 * kRows * kRedDoubles * 8;   // (two tiles in flight to the finishing warp)
   static_assert(kStages * sizeof(StageMeta) <= 384, "stage metadata overflows its slot");
   static_assert(kTotal <= 232448, "shared memory budget of one CTA exceeded");
 };
@@ -195,7 +196,9 @@ __device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c)
 // v by a relative 1 - beta2, less than half a bf16 unit, so rounding to nearest would freeze it) with bits from a
 // counter-based generator keyed by (element group, matrix, step index); the direction u of the step comes from
 // the unrounded values.
-template <int SMAX, bool HIST16, bool MOM16>
+// RUNS: some Gram tile has more than one run.  An instance of its own, since the code for it costs sets without 0.2 us of 20.6 (one 512 x 1376
+// matrix) to 0.3 of 196.5 (60M shapes).
+template <int SMAX, bool HIST16, bool MOM16, bool RUNS>
 __global__ void __launch_bounds__((FusedCfg<SMAX, HIST16, MOM16>::kThreads), 1)
 fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restrict__ items, int n_items, Ctrl* ctrl,
                     const Hyper* __restrict__ hyper) {
@@ -218,7 +221,7 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   ItemWeights* weights = reinterpret_cast<ItemWeights*>(fs_smem + C::kWeightsOff);  // [2]
   uint64_t* red_full = reinterpret_cast<uint64_t*>(fs_smem + C::kRedBarOff);   // [2] all consumer warps have left their sums
   uint64_t* red_empty = red_full + 2;                                           // [2] the finishing warp has taken them
-  uintptr_t* red_rows = reinterpret_cast<uintptr_t*>(fs_smem + C::kRedRowsOff); // [2] where a tile's rows go (StageMeta; 0: there are no more)
+  ulonglong2** red_rows = reinterpret_cast<ulonglong2**>(fs_smem + C::kRedRowsOff); // [2] where a tile's rows go (null: there are no more)
   double* red = reinterpret_cast<double*>(fs_smem + C::kRedOff);                // [2][rows][warps][SMAX]
 
   const int tid = threadIdx.x;
@@ -260,13 +263,11 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const unsigned int polls = static_cast<unsigned int>(ctrl->spin_limit);   // (testing aid; 0: the limit in time alone)
     unsigned long long rows_limit = kRowsLimitNs;   // (what did not come in time for one matrix is not waited for again)
     bool jobs_open = true, rows_open = true;
-    unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, runs of Gram tiles and combination items so far
-    double* const before = reinterpret_cast<double*>(fs_smem + C::kSumOff) + min(lane, SMAX - 1);   // where pending: the runs of the tile so far
-    bool pending = false;
+    unsigned int taken = 0, tiles = 0, fetched = 0;   // jobs, Gram tiles and combination items so far
     auto look_after_rows = [&]() {
       const int buf = tiles & 1;
       if (!rows_open || !__all_sync(0xffffffffu, mbar_test(red_full + buf, (tiles >> 1) & 1u))) return;
-      const uintptr_t at = red_rows[buf];   // [rows][s]: row of `cur` and (HIST16) of `prev`
+      ulonglong2* const rows = red_rows[buf];   // [rows][s]: row of `cur` and (HIST16) of `prev`
       double part[C::kRows];
 #pragma unroll
       for (int r = 0; r < C::kRows; ++r) {
@@ -279,23 +280,11 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       __syncwarp();
       if (lane == 0) mbar_arrive(red_empty + buf);
       ++tiles;
-      if (pending) {
-#pragma unroll
-        for (int r = 0; r < C::kRows; ++r) part[r] += before[r * SMAX];
-        __syncwarp();
-      }
-      if (at == 0) {
+      if (rows == nullptr) {
         rows_open = false;
-      } else if ((at & 1) != 0) {   // (lanes that share an address have the same sum)
+      } else if (lane < s_all) {
 #pragma unroll
-        for (int r = 0; r < C::kRows; ++r) before[r * SMAX] = part[r];
-        pending = true;
-      } else {
-        pending = false;
-        if (lane < s_all) {
-#pragma unroll
-          for (int r = 0; r < C::kRows; ++r) st_tagged(reinterpret_cast<ulonglong2*>(at) + r * s_all + lane, part[r], tag);
-        }
+        for (int r = 0; r < C::kRows; ++r) st_tagged(rows + r * s_all + lane, part[r], tag);
       }
       __syncwarp();
     };
@@ -479,8 +468,8 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
           look_ahead();
         }
-        // (the next run of the tile, like one of its own to the consumers)
-        if (!ok || now.rest == 0) break;
+        if (!RUNS || !ok || now.rest == 0) break;
+        // the next run of the tile, like one of its own to the consumers
         now.e0 += now.count;
         now.count = min(now.count, now.rest);
         now.rest -= now.count;
@@ -499,14 +488,15 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
     const int idx = tid * VEC;     // this thread's elements of a stage
     int stage = 0;
     uint32_t phase = 0;
-    unsigned int tiles_done = 0;   // runs of Gram tiles handed to the finishing warp
+    unsigned int tiles_done = 0;   // Gram tiles handed to the finishing warp
+    bool later = false;            // this run of a Gram tile is not its first
     unsigned int combined = 0;     // combination items whose weights have been taken
     const unsigned int it_step = static_cast<unsigned int>(ctrl->k);
     // Tells the finishing warp that the CTA has no more Gram tiles (all of them are ahead of the combination items), as soon as that is
     // known: at the end of the kernel it would be the last thing everybody waits for.
     bool gram_open = true;
     auto close_gram = [&]() {
-      if (tid == 0) red_rows[tiles_done & 1] = 0;
+      if (tid == 0) red_rows[tiles_done & 1] = nullptr;
       __syncwarp();
       if (lane == 0) mbar_arrive(red_full + (tiles_done & 1));
       gram_open = false;
@@ -566,10 +556,11 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
       if (mt.kind == 0) {
         // ---- Gram tile, or a run of one
         const int buf = tiles_done & 1;
-        // this warp's sums of row r over its lanes, into the buffer of the finishing warp
+        // this warp's sums of row r over its lanes, into the buffer of the finishing warp (runs of a tile one after another)
         auto hand_over = [&](int r, double (&v)[SMAX]) {
           const double t = warp_sums<SMAX>(v);
-          if ((lane & (32 / SMAX - 1)) == 0) red[((buf * C::kRows + r) * kWarps + warp) * SMAX + lane / (32 / SMAX)] = t;
+          double* const at = red + ((buf * C::kRows + r) * kWarps + warp) * SMAX + lane / (32 / SMAX);
+          if ((lane & (32 / SMAX - 1)) == 0) *at = RUNS && later ? *at + t : t;
         };
         if constexpr (!HIST16) {
           float acc[SMAX];
@@ -664,8 +655,10 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
             hand_over(C::kRows - 1, v);
           }
         }
+        later = RUNS && (mt.rows & 1) != 0;
+        if (later) continue;
         ++tiles_done;
-        if (tid == 0) red_rows[buf] = mt.rows;
+        if (tid == 0) red_rows[buf] = reinterpret_cast<ulonglong2*>(mt.rows);
         __syncwarp();
         if (lane == 0) mbar_arrive(red_full + buf);
       } else {
@@ -792,15 +785,23 @@ fused_stream_kernel(const MatDesc* __restrict__ mats, const FusedItem* __restric
   }
 }
 
-template <int SMAX, bool HIST16, bool MOM16>
-inline cudaError_t fused_set_smem() {
-  return cudaFuncSetAttribute(fused_stream_kernel<SMAX, HIST16, MOM16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              FusedCfg<SMAX, HIST16, MOM16>::kTotal);
-}
-
-template <bool HIST16, bool MOM16>
-inline cudaError_t fused_set_smem_for(int s) {
-  return s <= 8 ? fused_set_smem<8, HIST16, MOM16>() : (s <= 16 ? fused_set_smem<16, HIST16, MOM16>() : fused_set_smem<32, HIST16, MOM16>());
+template <int SMAX, bool HIST16, bool MOM16, bool RUNS>
+struct FusedKernel {
+  using C = FusedCfg<SMAX, HIST16, MOM16>;
+  static constexpr auto kernel = fused_stream_kernel<SMAX, HIST16, MOM16, RUNS>;
+};
+// f with the kernel of a plan
+template <typename F>
+inline auto fused_with_kernel(const FusedPlan& plan, int s, F&& f) {
+  auto instance = [&](auto hist16, auto mom16, auto runs) {
+    constexpr bool H = decltype(hist16)::value, M = decltype(mom16)::value, R = decltype(runs)::value;
+    return s <= 8 ? f(FusedKernel<8, H, M, R>{}) : (s <= 16 ? f(FusedKernel<16, H, M, R>{}) : f(FusedKernel<32, H, M, R>{}));
+  };
+  auto moments = [&](auto hist16, auto mom16) {
+    return plan.runs ? instance(hist16, mom16, std::true_type{}) : instance(hist16, mom16, std::false_type{});
+  };
+  auto history = [&](auto hist16) { return plan.mom16 ? moments(hist16, std::true_type{}) : moments(hist16, std::false_type{}); };
+  return plan.hist16 ? history(std::true_type{}) : history(std::false_type{});
 }
 
 // skip_gram (optional, one entry per matrix): 1 where the Gram row and the solve of a matrix are done before this
@@ -829,7 +830,10 @@ inline ngalore_status fused_plan_create(FusedPlan& plan, const std::vector<MatDe
     o.m = plan.mom16 ? static_cast<const void*>(d.m16) : static_cast<const void*>(d.m);
     o.v = plan.mom16 ? static_cast<const void*>(d.v16) : static_cast<const void*>(d.v);
     o.rows = reinterpret_cast<uintptr_t>(d.grow + static_cast<long long>(t) * (plan.hist16 ? 2 : 1) * s);
-    if (kind == 0 && o.count > d.run) { o.rest = o.count - d.run; o.count = d.run; o.rows |= 1; }
+    if (kind == 0 && o.count > d.run) {
+      o.rest = o.count - d.run; o.count = d.run; o.rows |= 1;
+      plan.runs = true;
+    }
     items.push_back(o);
   };
   for (int i = 0; i < n; ++i) {
@@ -847,8 +851,9 @@ inline ngalore_status fused_plan_create(FusedPlan& plan, const std::vector<MatDe
   }
   if (cudaMemcpy(plan.d_items, items.data(), sizeof(FusedItem) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return NGALORE_ERR_CUDA;
-  const cudaError_t e = plan.hist16 ? (plan.mom16 ? fused_set_smem_for<true, true>(s) : fused_set_smem_for<true, false>(s))
-                                    : (plan.mom16 ? fused_set_smem_for<false, true>(s) : fused_set_smem_for<false, false>(s));
+  const cudaError_t e = fused_with_kernel(plan, s, [](auto k) {
+    return cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, decltype(k)::C::kTotal);
+  });
   return e == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }
 
@@ -857,31 +862,12 @@ inline void fused_plan_destroy(FusedPlan& plan) {
   plan.d_items = nullptr;
 }
 
-template <int SMAX, bool HIST16, bool MOM16>
-inline void fused_launch_one(const FusedPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper,
-                             bool short_step, cudaStream_t stream) {
-  using C = FusedCfg<SMAX, HIST16, MOM16>;
-  launch_step(short_step, fused_stream_kernel<SMAX, HIST16, MOM16>, plan.grid, C::kThreads, C::kTotal, stream, d_mats, plan.d_items,
-              plan.n_items, d_ctrl, d_hyper);
-}
-
-template <bool HIST16, bool MOM16>
-inline void fused_launch_for(const FusedPlan& plan, const MatDesc* d_mats, Ctrl* d_ctrl, const Hyper* d_hyper, int s,
-                             bool short_step, cudaStream_t stream) {
-  if (s <= 8) fused_launch_one<8, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
-  else if (s <= 16) fused_launch_one<16, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
-  else fused_launch_one<32, HIST16, MOM16>(plan, d_mats, d_ctrl, d_hyper, short_step, stream);
-}
-
 inline ngalore_status fused_stream_launch(FusedPlan& plan, const MatDesc* d_mats, int /*n_mats*/, Ctrl* d_ctrl,
                                           const Hyper* d_hyper, int s, bool short_step, cudaStream_t stream, int64_t* launches) {
-  if (plan.hist16) {
-    if (plan.mom16) fused_launch_for<true, true>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
-    else fused_launch_for<true, false>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
-  } else {
-    if (plan.mom16) fused_launch_for<false, true>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
-    else fused_launch_for<false, false>(plan, d_mats, d_ctrl, d_hyper, s, short_step, stream);
-  }
+  fused_with_kernel(plan, s, [&](auto k) {
+    using C = typename decltype(k)::C;
+    return launch_step(short_step, k.kernel, plan.grid, C::kThreads, C::kTotal, stream, d_mats, plan.d_items, plan.n_items, d_ctrl, d_hyper);
+  });
   *launches += 1;
   return cudaGetLastError() == cudaSuccess ? NGALORE_OK : NGALORE_ERR_CUDA;
 }

@@ -651,9 +651,9 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   }
   // And no matrix has more than six of them for every SM, or three with a bf16 history (two partial rows a tile): the warp that solves for it
   // reads the rows of all after the last one, 16 tiles a look of 0.7 us (8 for s > 16, 32 up to 8), and in a set of one or a few such
-  // matrices nothing else goes on meanwhile.  Step without / with this limit, us, r = 512: one 2048 x 32000 matrix, s = 16 655 / 600; 64000
-  // columns, s = 24 1799 / 1531; 128000 columns, s = 16 2540 / 2238, s = 8 1666 / 1660, with 16-bit state 2150 / 1700; seven layers of width 2048 before
-  // one of 32000 columns, bf16 history, 875 / 730.  Stream phase of the first with four, five, six, seven and ten a SM 383 / 373 / 375 / 392 / 414 (six: a
+  // matrices nothing else goes on meanwhile.  Step without / with this limit, us, r = 512: one 2048 x 32000 matrix, s = 16 656 / 598; 64000
+  // columns, s = 24 1804 / 1471; 128000 columns, s = 16 2518 / 2222, s = 8 1658 / 1650, with 16-bit state 2150 / 1678; seven layers of width 2048 before
+  // one of 32000 columns, bf16 history, 877 / 724.  Stream phase of the first with four, five, six, seven and ten a SM 383 / 373 / 375 / 392 / 414 (six: a
   // multiple of the SMs also where tiles are long: 128000 columns 1553 / 1402 / 1383 / 1414 / 1451); two, three and four with a bf16 history 266 / 266 /
   // 289, 128000 columns 1144 / 861 / 1023.
   // A longer tile is summed in runs of what the rules above say, so that no more products meet in fp32.  (The plain kernels have no runs.)
