@@ -230,6 +230,11 @@ tc_backproject_kernel(const CUtensorMap* __restrict__ tmaps, const TcTile* __res
             // warp that took the slot then would store what is not there and release it while its barrier expects no one (an
             // unspecified launch failure, 1312-column matrices at r = 37, ten thousand tiles a step).  So first that use has been released
             // (at most 0.3 % of a step).
+            // One bit is enough for that wait, because the use before the previous one has been released already: loads are issued in order, each
+            // after its slot's last release, and a chunk at most four before this one has landed (two before, in this tile or, with one more,
+            // the tile before, this warp's own; where that tile had one chunk and this is the odd group, the last even chunk of the tile before
+            // that, which the other group had taken when it handed the accumulator back that this tile's MMAs waited for).
+            static_assert(kBpSlots > 4, "a chunk that landed four chunks ago was loaded after the slot's use before the previous one");
             if (!__all_sync(0xffffffffu, mbar_wait(wempty_bar + slot, phase ^ 1u, abort_flag) && mbar_wait(wfull_bar + slot, phase, abort_flag))) {
               ok = false;
               break;
