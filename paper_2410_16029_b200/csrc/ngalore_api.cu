@@ -633,7 +633,8 @@ ngalore_status ngalore_create(const ngalore_shape* shapes, int n_matrices, int r
   // 43 / 51.  Longer ones up to where they stop to gain: 130M shapes (s = 8) 8192 / 12288 / 24576 / 83968 327 / 319 / 319 / 339,
   // 1.1B shapes (s = 16) 8192 / 12288 / 40960 / 131072 4110 / 4150 / 4153 / 4200, and with a bf16 history, whose tiles hold half the bytes and
   // cost more, 350M shapes 8192 / 24576 / 49152 / 131072 881 / 849 / 820 / 834.  Sets with less than 8192 elements for every SM: one
-  // tile each, of 1024 elements at least (a stage then waits for none before it).
+  // tile each up to 4096, of 1024 elements at least (a stage then waits for none before it); above, tiles rounded down to 1024 elements, of which
+  // some SMs have two (rounded up, one each: four 512 x 1376 matrices, r = 128, s = 8 22.5 / 20.5 us, seven of 1024 x 1024, r = 96, s = 16 30.7 / 28.7; not taken so far).
   const long long per_sm = total_rn / prop.multiProcessorCount;
   const long long te_max = st->opt.history_bf16 == 1 ? 49152 : (s > 8 ? 8192 : 24576);
   long long te_all = std::min(te_max, std::max(8192ll, per_sm / 6 / 1024 * 1024));

@@ -399,6 +399,7 @@ __global__ void __launch_bounds__(kTfThreads, 1) tri_factor_kernel(const FactorM
 // warps 0, 4, 8 and 12 nothing else, and the other warps of all CTAs share the rest of S and of the update.  Two cluster barriers a step:
 // S is complete (the chain has arrived by then and waits for it later), and the step has ended.  What other SMs write is read past L1.
 constexpr int kTfClusterMax = 4, kTfClusterFrom = 256;
+constexpr size_t kTfClusterSmem = 49152;   // without raising the kernel's limit
 
 __device__ __forceinline__ void tf_cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
@@ -623,8 +624,10 @@ inline void tf_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr
 // has its SMs in one group of them, so that 148 SMs hold fewer than 37 clusters of four; 37 matrices of 480 columns in two waves 8.4 ms a
 // refresh, with one CTA each 7.8) and are so wide that it pays: refresh, one CTA / a cluster, nine matrices of 196 columns 2.24 / 2.23
 // ms, of 256 3.06 / 2.97, of 416 5.24 / 4.19, three of 512 7.13 / 4.80; pairs, 74 of 256 4.40 / 4.40, of 328 6.36 / 6.11, 60 of 480 8.99 / 8.21.
+// Beyond 1440 columns the norms of a matrix's columns no longer fit beside the blocks in the 48 KB that every kernel has, and one CTA takes it as
+// before: what a cluster would give there has not been measured.
 inline int tf_cluster(int n, int l_max) {
-  if (l_max <= kTfClusterFrom) return 1;
+  if (l_max <= kTfClusterFrom || tf_cluster_smem(l_max) > kTfClusterSmem) return 1;
   for (int c = kTfClusterMax; c > 1; c /= 2) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr{};
